@@ -328,21 +328,16 @@ int amgd_graph_launch(amgd_handle h);
  *   contiguous run of rows, each warp asking the L2 for the row pointers
  *   and CSR lines of its next row groups ahead of use and loading the CSR
  *   with an evict-first and the vectors with an evict-last cache policy.
- *   For the distance pass, staged selects 0 the row
- *   kernel (G lanes per row), 1 the tile kernel (one thread per stored
- *   entry), 2 the row kernel reading the vectors in the sweeps' row order
- *   in place (search depth 1: no caller-order copy of the vectors; U in
- *   {2,4}; the default) or 3 the warp-staged kernel on that order (each
- *   warp gathers its rows' neighbour vectors once, G lanes per row, into a
- *   shared-memory window and fits one stored entry per lane; U in {4,8}).
- *   With search depth d > 1 a stage-2 or stage-3 shape runs as stage 0.  Shapes change speed only, never results beyond the order of
- *   the K-term LS sums.  kernel: AMGD_KERNEL_RELAX (the sweeps) or
+ *   The distance pass has one kernel, chosen by the row's size alone: every
+ *   shape in the range above (stage 2 with U in {2,4}, stage 3 with U in
+ *   {4,8}) is accepted and kept, and all of them run it.  Shapes change speed
+ *   only, never results beyond the order of the K-term LS sums.  kernel: AMGD_KERNEL_RELAX (the sweeps) or
  *   AMGD_KERNEL_EDGE (the distance pass); the shape applies to the current
  *   storage precision.
- * amgd_autotune times every valid shape of both kernels on the handle's own
+ * amgd_autotune times every valid shape of the sweeps on the handle's own
  *   matrix and vectors (one sweep of sweep_type/omega into the spare vector
- *   buffer -- the current vectors are kept -- and one distance pass;
- *   computed distances are invalidated) and keeps the fastest.  cache_path
+ *   buffer -- the current vectors are kept) and keeps the fastest, and times
+ *   the distance pass for the record (computed distances are invalidated).  cache_path
  *   (may be NULL): a text file of earlier results keyed by GPU name,
  *   storage, K, size buckets, sweep type and color count; a matching line
  *   is used without timing, a new result is appended.

@@ -126,8 +126,7 @@ struct amgd_ctx {
     bool async_pending = false;
     struct PendingOut { int64_t *rp; int mem; int64_t cap; };
     std::vector<PendingOut> pending_out;         // strength outputs checked at amgd_sync
-    int32_t *edge_tiles = nullptr;               // row tiles of the edge pass (over the pattern)
-    int32_t n_edge_tiles = 0;
+    void *norms = nullptr;                       // distance pass: S_xx of every vector row
     // pattern of the fits, threshold and strength graph: the graph G_d of A^d
     // (search depth d); for d = 1 these alias A's caller-order pattern
     int32_t depth = 1;
@@ -500,12 +499,11 @@ int run_relax_recorded(amgd_ctx *h, int32_t nu, double omega, cudaStream_t s)
 
 int run_edge(amgd_ctx *h, double theta, cudaStream_t s)
 {
-    Shape sh = h->edge_shape[h->storage];
-    if (sh.stage >= 2 && h->depth > 1) sh.stage = 0;    // stages 2 and 3 cover A's own pattern
-    // stages 0 and 1 run on the caller's numbering: bring a row-permuted vector
-    // block back to caller order first; stages 2 and 3 read the sweeps' row order
+    // A's own pattern (search depth 1) is fitted on the vectors in the sweeps'
+    // row order, in place; G_d on a caller-order copy
+    const bool in_place = h->depth == 1;
     const void *xc = h->x[h->cur];
-    if (h->perm && sh.stage < 2) {
+    if (h->perm && !in_place) {
         if (!h->x_caller) return fail(h, AMGD_ERR_STATE, "caller-order vector buffer missing");
         CK(h, launch_unpermute(h->storage, h->x[h->cur], h->x_caller, h->perm, (int32_t)h->n,
                                Kp_of(h->storage, h->K), s));
@@ -528,14 +526,14 @@ int run_edge(amgd_ctx *h, double theta, cudaStream_t s)
     a.defer_list = h->defer_list;
     a.prp = h->prp;
     a.pcol = h->pcol;
-    a.tiles = h->edge_tiles;
-    a.ntiles = h->n_edge_tiles;
+    a.norms = h->norms;
+    a.nnz_p = h->nnz_p;
+    a.K = h->K;
     a.n = (int32_t)h->n;
     a.Kp = Kp_of(h->storage, h->K);
     a.target = h->target;
     a.theta = theta;
-    if (sh.stage >= 2) {
-        a.x = h->x[h->cur];                  // the sweeps' row order, read in place
+    if (in_place) {
         a.xrow = h->perm ? h->pinv : nullptr;
         a.xcol = h->perm ? h->colx : h->col_o;
     }
@@ -543,7 +541,7 @@ int run_edge(amgd_ctx *h, double theta, cudaStream_t s)
     a.status = h->status;
     bool unit_w = true;
     for (double wk : h->h_w) unit_w = unit_w && wk == 1.0;
-    CK(h, launch_edge(h->storage, sh, unit_w, a, s));
+    CK(h, launch_edge(h->storage, in_place, unit_w, a, s));
     h->have_dist = true;
     return AMGD_OK;
 }
@@ -557,30 +555,6 @@ int alloc_slot_outputs(amgd_ctx *h, int st)
     const size_t es = st == ST_FP64 ? 8 : 4;
     CK(h, cudaMalloc(&h->a, (h->nnz_p ? h->nnz_p : 1) * es));
     CK(h, cudaMalloc(&h->ls, (h->nnz_p ? h->nnz_p : 1) * es));
-    return AMGD_OK;
-}
-
-// row tiles of the edge pass over a caller-order pattern row pointer (host)
-int build_edge_tiles(amgd_ctx *h, const std::vector<int32_t> &prp)
-{
-    std::vector<int32_t> tiles(1, 0);
-    int64_t rows = 0, slots = 0;
-    const int64_t n = h->n;
-    for (int64_t i = 0; i < n; ++i) {
-        const int64_t len = prp[(size_t)i + 1] - prp[(size_t)i];
-        if (rows > 0 && (rows == kEdgeTileRows || slots + len > kEdgeTileSlots)) {
-            tiles.push_back((int32_t)i);
-            rows = slots = 0;
-        }
-        ++rows;
-        slots += len;
-    }
-    if (n > 0) tiles.push_back((int32_t)n);
-    dfree(h->edge_tiles);
-    h->edge_tiles = nullptr;
-    h->n_edge_tiles = (int32_t)tiles.size() - 1;
-    CK(h, dalloc(&h->edge_tiles, tiles.size()));
-    CK(h, cudaMemcpy(h->edge_tiles, tiles.data(), tiles.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     return AMGD_OK;
 }
 
@@ -689,7 +663,6 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
     h->pcol = h->col_o;
     h->nnz_p = h->nnz;
     h->E_p = h->E;
-    if ((rc = build_edge_tiles(h, h->h_rp)) != AMGD_OK) return bail(rc);
     h->rp_p = h->rp_o;
     h->col_p = h->col_o;
     h->val64 = h->val_o;
@@ -707,6 +680,7 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
     }
     h->color_start = {0, n};
     TRY(dalloc(&h->flag, (size_t)h->nnz_p + 16));   // 16-byte loads past the end
+    TRY(cudaMalloc(&h->norms, (size_t)(n ? n : 1) * 16));
     TRY(dalloc(&h->defer_count, 1));
     TRY(dalloc(&h->defer_list, (size_t)n));
     TRY(dalloc(&h->count, (size_t)n));
@@ -1431,9 +1405,9 @@ int amgd_autotune(amgd_handle h, int sweep_type, double omega, const char *cache
                 if (P % NV == 0 && shape_ok(h->storage, h->K, Shape{P / NV, NV, U, stage}) &&
                     relax_shape_available(h->storage, Shape{P / NV, NV, U, stage}))
                     cands.push_back(Shape{P / NV, NV, U, stage});
-    const Shape keep_r = h->relax_shape[h->storage], keep_e = h->edge_shape[h->storage];
+    const Shape keep_r = h->relax_shape[h->storage], best_e = h->edge_shape[h->storage];
     const int cur = h->cur;
-    Shape best_r = keep_r, best_e = keep_e;
+    Shape best_r = keep_r;
     float tr = 1e30f, te = 1e30f;
     for (const Shape &c : cands) {
         float ms = 0.f;
@@ -1448,21 +1422,11 @@ int amgd_autotune(amgd_handle h, int sweep_type, double omega, const char *cache
             if (prc != AMGD_OK) { h->relax_shape[h->storage] = keep_r; return prc; }
         }
     }
-    // edge pass: stage 0 row kernel, stage 1 tile kernel, stage 2 the row
-    // kernel and stage 3 the warp-staged kernel on the sweeps' row order
-    // (search depth 1)
-    for (int stage : {0, 1, 2, 3})
-        for (int NV : {1, 2, 4})
-            for (int U : {2, 4, 8}) {
-                const Shape c{P / NV, NV, U, stage};
-                if (P % NV != 0 || !shape_ok(h->storage, h->K, c) || !edge_shape_ok(c)) continue;
-                if (stage >= 2 && h->depth > 1) continue;
-                float ms = 0.f;
-                h->edge_shape[h->storage] = c;
-                const int rc = time_ms(h, [&]() { return run_edge(h, 0.5, h->stream); }, 5, ms);
-                if (rc != AMGD_OK) { h->edge_shape[h->storage] = keep_e; return rc; }
-                if (ms < te) { te = ms; best_e = c; }
-            }
+    // the distance pass has one kernel for every shape: timed once for the record
+    {
+        const int rc = time_ms(h, [&]() { return run_edge(h, 0.5, h->stream); }, 5, te);
+        if (rc != AMGD_OK) return rc;
+    }
     h->relax_shape[h->storage] = best_r;
     h->edge_shape[h->storage] = best_e;
     h->cur = cur;
@@ -1585,8 +1549,7 @@ int amgd_set_search_depth(amgd_handle h, int32_t d)
         h->depth = d;
     }
     h->E_p = h->nnz_p - h->n;
-    int rc = build_edge_tiles(h, d > 1 ? prp : h->h_rp);
-    if (rc != AMGD_OK) return rc;
+    int rc;
     if ((rc = alloc_slot_outputs(h, h->storage)) != AMGD_OK) return rc;
     dfree(h->flag);
     h->flag = nullptr;
@@ -2197,7 +2160,7 @@ int amgd_destroy(amgd_handle h)
                     h->val32, h->x[0], h->x[1],
                     h->w64, h->w32, h->a, h->ls, h->flag, h->count, h->tile, h->s_rp_tmp,
                     h->s_col_tmp, h->tmp64, h->ckpt, h->seg, h->adj_vec, h->adj_slot, h->lsb,
-                    h->adj_part, h->at_rp, h->at_row, h->at_slot, h->edge_tiles, h->mirror,
+                    h->adj_part, h->at_rp, h->at_row, h->at_slot, h->norms, h->mirror,
                     h->ip_coarse, h->ip_sel_col, h->ip_cnt, h->ip_sel_val, h->ip_ls, h->ip_rp,
                     h->ip_out, h->ip_pos, h->ip_list, h->ip_bcnt, h->ip_bkt, h->cr_u[0], h->cr_u[1], h->cr_coarse, h->cr_coarse_p, h->cr_cdiag, h->stage[0], h->stage[1], h->res_rp[0],
                     h->res_rp[1], h->res_col[0], h->res_col[1], h->async_err, h->cr_state,

@@ -129,6 +129,41 @@ __device__ __forceinline__ void ldg32(const void *p, uint4 &a, uint4 &b)
                  : "l"(p));
 }
 
+// Plain (coherent) loads of data that an earlier kernel of the stream writes:
+// a chained kernel (launch_chained) may be running while its predecessor still
+// writes, so the read-only path, which asks that the data stay unchanged for
+// the kernel's whole life, is left to the pattern arrays.
+__device__ __forceinline__ uint4 ld16(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void ld32(const void *p, uint4 &a, uint4 &b)
+{
+    asm volatile("ld.global.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p));
+}
+__device__ __forceinline__ float ld_plain(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_plain(const double *p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_plain(const double2 *p)
+{
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0,%1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+
 // a lane that owns a whole row (G = 1) of an even number of chunks reads them
 // in pairs; the rows must then start on 32-byte boundaries, which the
 // handle's buffers do (a row is P chunks, P even).  Launchers refuse other
@@ -145,8 +180,7 @@ struct Shape {
     int G, NV, U;
     int stage = 0;   // relaxation: 0 direct, 1 TMA-staged CSR, 2 cp.async pipelined,
                      // 3 chunked (one block per SM, L2 prefetch of the CSR ahead of use);
-                     // edge pass: 0 row kernel, 1 tile kernel, 2 row kernel on the
-                     // sweeps' row order in place
+                     // the distance pass accepts 0..3, all of them the same kernel
 };
 
 // per-device record of a one-time host setting of a kernel (a shared-memory
@@ -164,6 +198,35 @@ inline int current_device_index()
     int d = -1;
     if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= kMaxDevices) return -1;
     return d;
+}
+
+// Programmatic dependent launch.  A kernel launched with launch_chained may
+// start while the kernel before it in the stream finishes: until its
+// chain_wait() it reads nothing but the pattern arrays (row pointers, column
+// indices, row maps), which are written under a stream synchronisation and
+// never change under queued work -- no values, vectors or outputs -- and it
+// writes nothing.  chain_wait() returns when every earlier kernel of the stream
+// has completed and its writes are visible; each chained kernel calls it before
+// chain_release(), so the kernels before its predecessor are complete when it
+// starts.  chain_release() lets the next kernel start as soon as every block
+// has called it.  What it saves is the launch gap of the short kernels.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... Args>
+inline cudaError_t launch_chained(void (*kern)(P...), unsigned grid, int threads, size_t smem, cudaStream_t s,
+                                  Args... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, P(args)...);
 }
 
 // device status bits: a bounded wait that gave up; an index that failed its
@@ -217,7 +280,7 @@ struct RelaxArgs {
 struct EdgeArgs {                // everything in the caller's numbering
     const int32_t *rp, *col;     // CSR pattern of A (targets)
     const int32_t *prp, *pcol;   // pattern of the fits: G_d (= rp, col for d = 1); every
-                                 // per-slot output and the tiles follow this pattern
+                                 // per-slot output follows this pattern
     const void *val;             // values, arithmetic type
     const void *diag;            // diagonal a_ii, arithmetic type
     const double *val64;         // values in FP64 (mixed-path fallback)
@@ -229,23 +292,18 @@ struct EdgeArgs {                // everything in the caller's numbering
     int32_t *count_out;          // per row
     uint32_t *defer_count;       // rows appended to defer_list (mixed paths)
     int32_t *defer_list;         // rows to redo in FP64 (capacity n)
-    const int32_t *tiles;        // ntiles + 1 first rows of the row tiles
-    int32_t ntiles;
     int32_t n, Kp, target;       // target: 0 residual, 1 plain
     double theta;
-    // edge stage 2 (search depth 1): x is the vector block in the sweeps' row
+    // in place (search depth 1): x is the vector block in the sweeps' row
     // order; xrow[i] is the vector row of caller row i (NULL: i) and xcol[p]
     // the vector row of the column of caller slot p
     const int32_t *xrow = nullptr, *xcol = nullptr;
-    bool compensated = false;    // mixed paths of stage 2: compensated FP32 LS sums
+    int32_t K = 0;               // components in use (the others are padding)
+    int64_t nnz_p = 0;           // entries of the fits' pattern
+    void *norms = nullptr;       // workspace, n rows: S_xx (FP32), or S_xx and 1 / S_xx (FP64)
+    bool compensated = false;    // mixed paths: compensated FP32 LS sums
     uint32_t *status = nullptr;  // device status word (checked build: index range)
 };
-
-// row tiles of the edge pass: consecutive rows, at most kEdgeTileRows rows and
-// kEdgeTileSlots stored entries per tile (a row with more entries is a tile
-// of its own)
-constexpr int kEdgeTileRows = 256;
-constexpr int kEdgeTileSlots = 4096;
 
 struct InitArgs {
     void *x;                   // n x Kp, permuted rows
@@ -262,7 +320,8 @@ struct InitArgs {
 cudaError_t launch_relax(int storage, Shape sh, const RelaxArgs &a, cudaStream_t s);
 // false for a staged shape whose shared memory exceeds the per-block limit
 bool relax_shape_available(int storage, Shape sh);
-cudaError_t launch_edge(int storage, Shape sh, bool unit_w, const EdgeArgs &a, cudaStream_t s);
+// in_place: read the vectors in the sweeps' row order (search depth 1)
+cudaError_t launch_edge(int storage, bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s);
 
 // scatter caller-order n x K doubles into permuted, padded storage and back

@@ -21,16 +21,13 @@
 //      cancellation never decides a distance.
 //   3. m_i = min_p LS_ip; slot p is strong iff LS_p = 0 or theta LS_p < m_i
 //      (§4.2, Eq. (4.4), r = 1/LS); per-row strong count.
-// The pass works in the caller's numbering, so every output lands where the
-// caller expects it.  Its kernels compute the same thing (the edge shape's
-// stage selects one; the autotuner times them): stage 0, k_edge_rows, G
-// lanes per row through all steps, on a caller-order copy of a row-permuted
-// vector block; stage 1, k_edge_tiles, rows cut into tiles with one thread
-// per stored entry for the fits, on the same copy; stage 2, k_edge_rows
-// reading the permuted block in place through renumbered column indices
-// (no copy; search depth 1); stage 3, k_edge_warp (k_edge_warp.cuh), on the
-// same in-place order, gathering every neighbour row once into a per-warp
-// shared-memory window and fitting one stored entry per lane.
+// Outputs are in the caller's numbering.  The vectors are read in the
+// sweeps' row order in place (renumbered column indices) for search depth 1,
+// from a caller-order copy otherwise.
+//
+// Two kernels.  S_xx depends on the neighbour alone, so k_norms forms it once
+// per row instead of once per entry; k_edge_fit does the rest with a few
+// lanes per row.
 #pragma once
 #include <type_traits>
 
@@ -40,7 +37,7 @@
 namespace amgd {
 namespace edge_impl {
 
-constexpr int kEdgeThreads = 256;
+constexpr int kFitThreads = 128;
 
 template <int G, class T>
 __device__ __forceinline__ T group_sum(T v, unsigned mask)
@@ -50,67 +47,27 @@ __device__ __forceinline__ T group_sum(T v, unsigned mask)
     return v;
 }
 
-template <class C> __device__ __forceinline__ C divide(C a, C b) { return a / b; }
 // the mixed path's coefficient only needs FP32 relative accuracy (its error
 // enters LS at second order): the fast division is enough
-template <> __device__ __forceinline__ float divide<float>(float a, float b)
+__device__ __forceinline__ float divide(float a, float b) { return __fdividef(a, b); }
+
+// ---------------------------------------------------------------------------
+// Order of the K-term sums.  A row is P pieces of V components (16 bytes).
+// Every piece has its own partial sum, in component order, and the pieces are
+// joined by the binary tree that adds piece q and piece q + P/2, then q and
+// q + P/4, ... (the order of a shuffle butterfly over P lanes that hold one
+// piece each, which is how k_norms forms S_xx).  tree_sum walks that tree
+// depth first, so that at most log2(P) partial sums are live.
+// ---------------------------------------------------------------------------
+template <int L, int H, int END, class Leaf, class Join>
+__device__ __forceinline__ auto tree_sum(Leaf &leaf, Join &join)
 {
-    return __fdividef(a, b);
-}
-
-// sums over one 16-byte piece of (w) x x and (w) y x; FP32 pieces in packed pairs
-template <class C, int V, bool UW> struct PieceSums;
-
-template <int V, bool UW> struct PieceSums<double, V, UW> {
-    double xx = 0.0, yx = 0.0;
-    __device__ __forceinline__ void add(const double (&x)[V], const double (&y)[V], const double (&w)[V]) {
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-            const double wx = UW ? x[e] : w[e] * x[e];
-            xx = fma(wx, x[e], xx);
-            yx = fma(wx, y[e], yx);
-        }
-    }
-    __device__ __forceinline__ double sxx() const { return xx; }
-    __device__ __forceinline__ double syx() const { return yx; }
-};
-
-template <int V, bool UW> struct PieceSums<float, V, UW> {
-    float2 xx = make_float2(0.f, 0.f), yx = make_float2(0.f, 0.f);
-    __device__ __forceinline__ void add(const float (&x)[V], const float (&y)[V], const float (&w)[V]) {
-#pragma unroll
-        for (int e = 0; e < V / 2; ++e) {
-            float2 x2 = make_float2(x[2 * e], x[2 * e + 1]);
-            const float2 wx = UW ? x2 : make_float2(w[2 * e] * x2.x, w[2 * e + 1] * x2.y);
-            xx = __ffma2_rn(wx, x2, xx);
-            yx = __ffma2_rn(wx, make_float2(y[2 * e], y[2 * e + 1]), yx);
-        }
-    }
-    __device__ __forceinline__ float sxx() const { return xx.x + xx.y; }
-    __device__ __forceinline__ float syx() const { return yx.x + yx.y; }
-};
-
-// sum over one piece of w (y - a x)^2, each residual one fused multiply-add
-template <class C, int V, bool UW>
-__device__ __forceinline__ void residual_add(C a, const C (&x)[V], const C (&y)[V], const C (&w)[V], C &res)
-{
-    if constexpr (std::is_same<C, float>::value) {
-        const float2 na = make_float2(-a, -a);
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int e = 0; e < V / 2; ++e) {
-            const float2 d = __ffma2_rn(na, make_float2(x[2 * e], x[2 * e + 1]),
-                                        make_float2(y[2 * e], y[2 * e + 1]));
-            const float2 wd = UW ? d : make_float2(w[2 * e] * d.x, w[2 * e + 1] * d.y);
-            acc = __ffma2_rn(wd, d, acc);
-        }
-        res += acc.x + acc.y;
+    if constexpr (H == END) {
+        return leaf(L);
     } else {
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-            const C d = fma(-a, x[e], y[e]);
-            res = fma(UW ? d : w[e] * d, d, res);
-        }
+        const auto a = tree_sum<L, 2 * H, END>(leaf, join);
+        const auto b = tree_sum<L + H, 2 * H, END>(leaf, join);
+        return join(a, b);
     }
 }
 
@@ -118,11 +75,10 @@ __device__ __forceinline__ void residual_add(C a, const C (&x)[V], const C (&y)[
 // Compensated FP32 sums (mixed paths, AMGD_SUM_COMPENSATED).  Each sum is two
 // FP32 words: a running sum and the exact rounding error of every addition,
 // taken by TwoSum (six IEEE additions, no fusion) -- the Kahan-Babuska-
-// Neumaier scheme.  S_xx and S_yx travel together as one packed pair; the LS
-// terms of even and odd components as the halves of another (FP32x2
-// instructions).  Lanes combine their pairs in the shuffle butterfly with
-// TwoSum again, adding the error words; the two words are added once at the
-// end.
+// Neumaier scheme; two partial sums are joined by TwoSum again, adding the
+// error words, and the two words are added once at the end.  Two independent
+// chains share the FP32x2 instructions: two pieces of S_yx, the even and odd
+// components of an LS piece.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float2 sub2(float2 a, float2 b)
 {
@@ -143,590 +99,584 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     const float ap = __fsub_rn(s, bp);
     e = __fadd_rn(__fsub_rn(a, ap), __fsub_rn(b, bp));
 }
+struct Comp {
+    float s, c;
+};
+// two sums side by side
 struct Comp2 {
-    float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
-    __device__ __forceinline__ void add(float2 t)
-    {
+    float2 s, c;
+};
+__device__ __forceinline__ Comp2 comp2_join(const Comp2 &a, const Comp2 &b)
+{
+    Comp2 r;
+    float2 e;
+    two_sum2(a.s, b.s, r.s, e);
+    r.c = __fadd2_rn(__fadd2_rn(a.c, b.c), e);
+    return r;
+}
+// the chain t(0), t(1), ..., t(N - 1): the first term is exact
+template <int N, class Term>
+__device__ __forceinline__ Comp2 comp2_chain(const Term &t)
+{
+    Comp2 r{t(0), make_float2(0.f, 0.f)};
+#pragma unroll
+    for (int k = 1; k < N; ++k) {
         float2 sn, e;
-        two_sum2(s, t, sn, e);
-        s = sn;
-        c = __fadd2_rn(c, e);
+        two_sum2(r.s, t(k), sn, e);
+        r.s = sn;
+        r.c = k == 1 ? e : __fadd2_rn(r.c, e);
+    }
+    return r;
+}
+struct CompJoin {
+    __device__ __forceinline__ Comp operator()(const Comp &a, const Comp &b) const
+    {
+        Comp r;
+        float e;
+        two_sum(a.s, b.s, r.s, e);
+        r.c = __fadd_rn(__fadd_rn(a.c, b.c), e);
+        return r;
     }
 };
-// pairs of the G lanes of a row combined (xor butterfly: every lane ends with
-// the total)
-template <int G>
-__device__ __forceinline__ void comp2_allreduce(Comp2 &v, unsigned mask)
+
+// ---------------------------------------------------------------------------
+// S_xx of every vector row: on the mixed paths FP32 sums in the order above
+// (P lanes per row, one piece each); FP64 with its reciprocal, so that a fit
+// needs no FP64 division (nine operations of the FP64 pipe, which retires two
+// per clock and SM), one thread per row (K + 10 operations; P lanes would run
+// the division P times: 25 against 6 us at 111k rows, K = 13).  The reciprocal
+// is NaN where S_xx or 1/S_xx leaves the range in which the quotient's
+// correction is exact: those fits divide.  Bound: one read of the vectors,
+// most of it from the L2 that the last sweep left them in.
+// ---------------------------------------------------------------------------
+constexpr int kNormThreads = 256;
+
+template <class TS, int P, bool UW, bool COMP>
+__global__ void __launch_bounds__(kNormThreads) k_norms(const TS *X, const void *wv, int32_t n,
+                                                        void *out)
 {
+    using S = Store<TS>;
+    using C = typename S::C;
+    constexpr int V = S::V;
+    if constexpr (std::is_same<C, double>::value) {
+        const int64_t r = (int64_t)blockIdx.x * kNormThreads + threadIdx.x;
+        chain_wait();
+        chain_release();
+        if (r >= n) return;
+        double s = 0.0, s1 = 0.0;
+#pragma unroll 4
+        for (int q = 0; q < P; ++q) {
+            double x[V];
+            S::unpack(ld16(X + (r * P + q) * V), x);
+            const double2 w = UW ? make_double2(1.0, 1.0) : ld_plain((const double2 *)wv + q);
+            s = fma(UW ? x[0] : w.x * x[0], x[0], s);
+            s1 = fma(UW ? x[1] : w.y * x[1], x[1], s1);
+        }
+        s += s1;
+        ((double2 *)out)[r] = make_double2(s, s > 1e-290 && s < 1e290 ? 1.0 / s : NAN);
+    } else {
+        const int lane = threadIdx.x % P;
+        const int64_t r0 = (int64_t)blockIdx.x * (kNormThreads / P) + threadIdx.x / P;
+        const int64_t r = r0 < n ? r0 : n - 1;          // every lane takes part in the shuffles
+        chain_wait();
+        chain_release();
+        C x[V];
+        S::unpack(ld16(X + (r * P + lane) * V), x);
+        float wx[V];
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        float2 so, co;
-        so.x = __shfl_xor_sync(mask, v.s.x, o, G);
-        so.y = __shfl_xor_sync(mask, v.s.y, o, G);
-        co.x = __shfl_xor_sync(mask, v.c.x, o, G);
-        co.y = __shfl_xor_sync(mask, v.c.y, o, G);
-        float2 sn, e;
-        two_sum2(v.s, so, sn, e);
-        v.s = sn;
-        v.c = __fadd2_rn(__fadd2_rn(v.c, co), e);
-    }
-}
-// (S_xx, S_yx) of one piece, added to a compensated pair
-template <int V, bool UW>
-__device__ __forceinline__ void comp_piece_sums(const float (&x)[V], const float (&y)[V],
-                                                const float (&w)[V], Comp2 &acc)
-{
+        for (int e = 0; e < V; ++e) wx[e] = UW ? x[e] : ((const float *)wv)[lane * V + e] * x[e];
+        float total;
+        if constexpr (COMP) {
+            Comp v{__fmul_rn(wx[0], x[0]), 0.f};
+            CompJoin join;
 #pragma unroll
-    for (int e = 0; e < V; ++e) {
-        const float wx = UW ? x[e] : w[e] * x[e];
-        acc.add(__fmul2_rn(make_float2(wx, wx), make_float2(x[e], y[e])));
-    }
-}
-// w (y - a x)^2 of one piece, even and odd components as the pair's halves
-template <int V, bool UW>
-__device__ __forceinline__ void comp_residual(float a, const float (&x)[V], const float (&y)[V],
-                                              const float (&w)[V], Comp2 &acc)
-{
-    const float2 na = make_float2(-a, -a);
+            for (int e = 1; e < V; ++e) {
+                float s, err;
+                two_sum(v.s, __fmul_rn(wx[e], x[e]), s, err);
+                v.s = s;
+                v.c = __fadd_rn(v.c, err);
+            }
 #pragma unroll
-    for (int e = 0; e < V; e += 2) {
-        const float2 d = __ffma2_rn(na, make_float2(x[e], x[e + 1]), make_float2(y[e], y[e + 1]));
-        const float2 wd = UW ? d : make_float2(w[e] * d.x, w[e + 1] * d.y);
-        acc.add(__fmul2_rn(wd, d));
+            for (int o = P / 2; o > 0; o >>= 1) {
+                const Comp other{__shfl_xor_sync(0xffffffffu, v.s, o, P), __shfl_xor_sync(0xffffffffu, v.c, o, P)};
+                v = join(v, other);
+            }
+            total = v.s + v.c;
+        } else {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < V; e += 2)
+                s = __ffma2_rn(make_float2(wx[e], wx[e + 1]), make_float2(x[e], x[e + 1]), s);
+            total = group_sum<P>(s.x + s.y, 0xffffffffu);
+        }
+        if (r0 < n && lane == 0) ((float *)out)[r] = total;
     }
-}
-// the LS pair's two halves joined, then the lanes: one FP32 value
-template <int G>
-__device__ __forceinline__ float comp_ls_total(const Comp2 &acc, unsigned mask)
-{
-    float s, e;
-    two_sum(acc.s.x, acc.s.y, s, e);
-    Comp2 one;
-    one.s = make_float2(s, 0.f);
-    one.c = make_float2(__fadd_rn(__fadd_rn(acc.c.x, acc.c.y), e), 0.f);
-    comp2_allreduce<G>(one, mask);
-    return one.s.x + one.c.x;
 }
 
 // ---------------------------------------------------------------------------
-// Row kernel (edge shape stages 0 and 2).  G lanes own one row through all three
-// steps: the target from the row's gathers, then the fits with the row's
-// neighbours gathered again (mostly L1/L2 hits), K-component sums reduced
-// across the G lanes with shuffles, then the flags.
-// Stage 2 (PX): the vectors stay in the sweeps' row order (no caller-order
-// copy is made); row i's own vector is read at xrow[i] and the neighbour of
-// slot p at xcol[p] -- the caller CSR with every column index mapped to the
-// sweeps' numbering -- and the mixed paths may sum with compensation (COMP).
-// Per-warp output staging: a warp owns 32/G consecutive rows of the caller's
-// numbering, i.e. one contiguous run of CSR slots.  a, LS and the flags of
-// that run are collected in shared memory and written out with coalesced
-// stores (a run wider than warp_slots<G>() -- 16 slots per row on average --
-// is written directly).
+// G lanes share a row.  A lane holds NP = P / G of its pieces: the pairs
+// (2m, 2m + 1) with m = t G + lane, t = 0 .. NP/2 - 1, so that each of its
+// 32-byte loads lies beside its neighbours' (P = 1: the one piece).  The two
+// pieces of a pair run side by side in the FP32x2 instructions, through the
+// levels of the tree inside the lane (over t), then across the lanes, and are
+// joined last.
+// ---------------------------------------------------------------------------
+template <int G, int NP>
+__device__ __forceinline__ int fit_piece(int lane, int q)
+{
+    return NP == 1 ? q : 2 * ((q / 2) * G + lane) + (q & 1);
+}
+
 template <int G>
-constexpr int warp_slots()
+__device__ __forceinline__ float comp_total(Comp2 v, unsigned mask)
 {
-    return (32 / G) * 16;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        Comp2 w;
+        w.s.x = __shfl_xor_sync(mask, v.s.x, o, G);
+        w.s.y = __shfl_xor_sync(mask, v.s.y, o, G);
+        w.c.x = __shfl_xor_sync(mask, v.c.x, o, G);
+        w.c.y = __shfl_xor_sync(mask, v.c.y, o, G);
+        v = comp2_join(v, w);
+    }
+    float s, e;
+    two_sum(v.s.x, v.s.y, s, e);
+    return s + __fadd_rn(__fadd_rn(v.c.x, v.c.y), e);
+}
+template <int G>
+__device__ __forceinline__ float plain_total(float2 v, unsigned mask)
+{
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1)
+        v = __fadd2_rn(v, make_float2(__shfl_xor_sync(mask, v.x, o, G), __shfl_xor_sync(mask, v.y, o, G)));
+    return v.x + v.y;
 }
 
-template <class C, int G>
-constexpr int edge_smem_bytes()
+// S_xx (FP32) or S_xx and its reciprocal (FP64) as k_norms left them
+template <class C> struct Norm { using T = float; };
+template <> struct Norm<double> { using T = double2; };
+
+// One fit: S_yx, a_ij and LS_ij from the lane's pieces of x_j (as stored), of
+// the target and of the weights (w, UW: unused), the first np of them not all
+// padding; every lane of the row ends with the result.
+template <class TS, int G, int NP, bool UW, bool COMP, class W>
+__device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
+                                          const typename Store<TS>::C (&y)[NP][Store<TS>::V], const W &w,
+                                          const typename Norm<typename Store<TS>::C>::T &nr, int np, unsigned mask,
+                                          typename Store<TS>::C &a_, typename Store<TS>::C &ls_)
 {
-    return (kEdgeThreads / 32) * warp_slots<G>() * (2 * (int)sizeof(C) + 1);
+    using S = Store<TS>;
+    using C = typename S::C;
+    constexpr int V = S::V;
+    if constexpr (std::is_same<C, double>::value) {
+        // two chains (even and odd components), joined once
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            if (q >= np) break;
+            C x[V];
+            S::unpack(raw[q], x);
+            s0 = fma(UW ? x[0] : w(q, 0) * x[0], y[q][0], s0);
+            s1 = fma(UW ? x[1] : w(q, 1) * x[1], y[q][1], s1);
+        }
+        const double syx = group_sum<G>(s0 + s1, mask);
+        // a = S_yx / S_xx: the product with the reciprocal, corrected by its
+        // exact remainder; operands outside its range divide
+        a_ = syx * nr.y;
+        if ((__double2hiint(a_) & 0x7fffffff) < 0x7f000000) a_ = fma(fma(-a_, nr.x, syx), nr.y, a_);
+        else a_ = nr.x == 0.0 ? 0.0 : syx / nr.x;
+        double r0 = 0.0, r1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            if (q >= np) break;
+            C x[V];
+            S::unpack(raw[q], x);
+            const double d0 = fma(-a_, x[0], y[q][0]), d1 = fma(-a_, x[1], y[q][1]);
+            r0 = fma(UW ? d0 : w(q, 0) * d0, d0, r0);
+            r1 = fma(UW ? d1 : w(q, 1) * d1, d1, r1);
+        }
+        ls_ = group_sum<G>(r0 + r1, mask);
+    } else if constexpr (NP == 1) {
+        C x[V];
+        S::unpack(raw[0], x);
+        auto wx = [&](int e) { return UW ? x[e] : w(0, e) * x[e]; };
+        float syx;
+        if constexpr (COMP) {
+            Comp v{__fmul_rn(wx(0), y[0][0]), 0.f};
+#pragma unroll
+            for (int e = 1; e < V; ++e) {
+                float s, err;
+                two_sum(v.s, __fmul_rn(wx(e), y[0][e]), s, err);
+                v.s = s;
+                v.c = __fadd_rn(v.c, err);
+            }
+            syx = v.s + v.c;
+        } else {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < V; e += 2)
+                s = __ffma2_rn(make_float2(wx(e), wx(e + 1)), make_float2(y[0][e], y[0][e + 1]), s);
+            syx = s.x + s.y;
+        }
+        a_ = (nr == 0.f) ? 0.f : divide(syx, nr);
+        auto d2 = [&](int e) { return make_float2(fmaf(-a_, x[e], y[0][e]), fmaf(-a_, x[e + 1], y[0][e + 1])); };
+        auto wd2 = [&](int e, float2 d) { return UW ? d : make_float2(w(0, e) * d.x, w(0, e + 1) * d.y); };
+        if constexpr (COMP) {
+            const Comp2 v = comp2_chain<V / 2>([&](int k) {
+                const float2 d = d2(2 * k);
+                return __fmul2_rn(wd2(2 * k, d), d);
+            });
+            ls_ = comp_total<1>(v, mask);
+        } else {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < V; e += 2) {
+                const float2 d = d2(e);
+                s = __ffma2_rn(wd2(e, d), d, s);
+            }
+            ls_ = s.x + s.y;
+        }
+    } else {
+        float syx;
+        // products w x y of component e of the pair's two pieces
+        auto xy = [&](const C (&x0)[V], const C (&x1)[V], int q, int e) {
+            return make_float2(__fmul_rn(UW ? x0[e] : w(q, e) * x0[e], y[q][e]),
+                               __fmul_rn(UW ? x1[e] : w(q + 1, e) * x1[e], y[q + 1][e]));
+        };
+        if constexpr (COMP) {
+            auto leaf = [&](int t) {
+                C x0[V], x1[V];
+                S::unpack(raw[2 * t], x0);
+                S::unpack(raw[2 * t + 1], x1);
+                return comp2_chain<V>([&](int e) { return xy(x0, x1, 2 * t, e); });
+            };
+            auto join = [](const Comp2 &a, const Comp2 &b) { return comp2_join(a, b); };
+            syx = comp_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
+        } else {
+            auto piece = [&](int q) {
+                C x[V];
+                S::unpack(raw[q], x);
+                float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int e = 0; e < V; e += 2)
+                    s = __ffma2_rn(UW ? make_float2(x[e], x[e + 1]) : make_float2(w(q, e) * x[e], w(q, e + 1) * x[e + 1]),
+                                   make_float2(y[q][e], y[q][e + 1]), s);
+                return s.x + s.y;
+            };
+            auto leaf = [&](int t) { return make_float2(piece(2 * t), piece(2 * t + 1)); };
+            auto join = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
+            syx = plain_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
+        }
+        a_ = (nr == 0.f) ? 0.f : divide(syx, nr);
+        // residuals of component e of a pair's two pieces, times the weights
+        auto terms = [&](int t, float2 (&d)[V], float2 (&wd)[V]) {
+            C x0[V], x1[V];
+            S::unpack(raw[2 * t], x0);
+            S::unpack(raw[2 * t + 1], x1);
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                d[e] = make_float2(fmaf(-a_, x0[e], y[2 * t][e]), fmaf(-a_, x1[e], y[2 * t + 1][e]));
+                wd[e] = UW ? d[e] : make_float2(w(2 * t, e) * d[e].x, w(2 * t + 1, e) * d[e].y);
+            }
+        };
+        if constexpr (COMP) {
+            // even and odd components of a piece are separate chains
+            auto leaf = [&](int t) {
+                float2 d[V], wd[V];
+                terms(t, d, wd);
+                const Comp2 even = comp2_chain<V / 2>([&](int k) { return __fmul2_rn(wd[2 * k], d[2 * k]); });
+                const Comp2 odd = comp2_chain<V / 2>([&](int k) { return __fmul2_rn(wd[2 * k + 1], d[2 * k + 1]); });
+                return comp2_join(even, odd);
+            };
+            auto join = [](const Comp2 &a, const Comp2 &b) { return comp2_join(a, b); };
+            ls_ = comp_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
+        } else {
+            auto leaf = [&](int t) {
+                float2 d[V], wd[V];
+                terms(t, d, wd);
+                float2 even = make_float2(0.f, 0.f), odd = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < V / 2; ++k) {
+                    even = __ffma2_rn(wd[2 * k], d[2 * k], even);
+                    odd = __ffma2_rn(wd[2 * k + 1], d[2 * k + 1], odd);
+                }
+                return __fadd2_rn(even, odd);
+            };
+            auto join = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
+            ls_ = plain_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
+        }
+    }
 }
 
-// resident blocks per SM asked of the compiler: three for the plain sums
-// (occupancy hides the gathers), two for the compensated ones (their extra
-// live words would otherwise spill)
-template <bool COMP>
-constexpr int edge_rows_min_blocks()
-{
-    return COMP ? 2 : 3;
-}
+// ---------------------------------------------------------------------------
+// G lanes per row, a block per run of consecutive rows.  The block's stored
+// entries are one contiguous run of slots: their gather indices and values
+// come into shared memory with coalesced loads, the fits replace them there
+// (a over the values; LS over the indices where the sizes agree), and a, LS
+// and the flags leave with coalesced stores.  A block whose run exceeds `cap`
+// slots works on global memory directly.  The neighbour row of the next entry
+// is in flight while an entry is fitted.
+//
+// Bound: the FP32 pipe on the compensated mixed paths (8 FP32 operations per
+// component for S_yx and 9 for LS), the FP64 pipe on FP64 (3K + 3 operations
+// per entry at two per clock and SM).  Few lanes per row keep y_i in registers
+// for all its entries and spend little on reductions; a lane per entry (y_i
+// from shared memory, row minima by shuffles) issued twice the instructions.
+//
+// Lanes per row, entries in flight and resident blocks (measured, us per pass,
+// K = 16 FP32 9-point 1024^2 / K = 32 FP32 7-point 128^3): a share of 16
+// components per lane 174 / 623, of 8 281 / 897 (the joins across lanes), of 32
+// - / 699 (a 32-byte load of a lane is an L1 wavefront of its own unless its
+// neighbours read the same 128-byte line).  One entry at a time with seven
+// resident blocks beats two with five (193 / 689) and a double-buffered one
+// with four (204 / 784): warps hide the gathers better than registers do.
+// BF16 rows of 64 bytes and more keep 32 components per lane (7-point 96^3,
+// K = 32: 231 against 268).  FP64 is at 70-80 % of its pipe whatever the shape.
+// Before (G = P lanes per row, S_xx per entry) the two workloads took 193 (with
+// the best shape) and 1331 us (752 with the best), K = 13 FP64 7-point 333^2
+// 385 (150 now), 25 entries per row of BF16 K = 16 (512^2) 236 (92 now).
+// ---------------------------------------------------------------------------
+template <class TS, int P>
+struct FitLayout {
+    using C = typename Store<TS>::C;
+    static constexpr int V = Store<TS>::V, KP = P * V;
+    static constexpr int CL = sizeof(TS) == 2 ? 32 : 16;               // components per lane
+    static constexpr int G = KP <= CL ? 1 : KP / CL;
+    static constexpr int NP = P / G;
+    static constexpr int U = sizeof(TS) == 8 && NP <= 4 ? 4 : 1;      // entries gathered at a time
+    static constexpr int MINB = sizeof(TS) == 8 ? 4 : sizeof(TS) == 4 ? 7 : NP * V <= 16 ? 6 : 5;   // resident blocks
+    static constexpr int WB = KP * (int)sizeof(C);                    // weights of the block
+    static constexpr bool LS_OVER = sizeof(C) == 4;                    // LS replaces the gather index
+    static constexpr int SLOT = 4 + (LS_OVER ? 1 : 2) * (int)sizeof(C) + 1;
+    static constexpr int UT = NP <= 2 || (sizeof(TS) == 8 && NP <= 4) ? 4 : (NP <= 4 ? 2 : 1);   // and in the target
+    static int bytes(int cap, bool unit_w) { return (unit_w ? 0 : WB) + cap * SLOT; }
+    static_assert(NP == 1 ? G == 1 : NP % 2 == 0, "pairs of pieces");
+};
 
-template <class TS, int G, int NV, int U, bool UW, bool PX, bool COMP>
-__global__ void __launch_bounds__(kEdgeThreads, edge_rows_min_blocks<COMP>()) k_edge_rows(EdgeArgs A)
+// SHARED: several shares per row (el of them; else one)
+template <class TS, int P, bool UW, bool PX, bool COMP, bool SHARED>
+__global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fit(EdgeArgs A, int cap, int shares)
 {
     using S = Store<TS>;
     using C = typename S::C;
     using AV = typename S::A;
-    constexpr int V = S::V;
+    using L = FitLayout<TS, P>;
+    constexpr int V = S::V, KP = L::KP, G = L::G, NP = L::NP, UT = L::UT, U = L::U;
     constexpr bool kMixed = !std::is_same<C, double>::value;
-    constexpr int kWarpSlots = warp_slots<G>();
     extern __shared__ __align__(16) unsigned char esm[];
+    const int T = blockDim.x, tid = threadIdx.x;
+    // el shares of a row's entries, G lanes each; gmask: the lanes of a share,
+    // rmask: of the row
+    const int el = SHARED ? shares : 1;
+    const int gl = tid % G, sub = tid / G % el, width = G * el;
+    const unsigned gmask = G == 1 ? 1u << (tid % 32) : ((1u << G) - 1u) << ((tid % 32) / G * G);
+    const unsigned rmask = width == 32 ? 0xffffffffu : ((1u << width) - 1u) << ((tid % 32) / width * width);
+    C *ws = reinterpret_cast<C *>(esm);                              // weights (UW: none)
+    C *a_s = reinterpret_cast<C *>(esm + (UW ? 0 : L::WB));           // values, then a
+    C *lsep = a_s + cap;                                             // LS where it has its own place
+    int32_t *x_s = reinterpret_cast<int32_t *>(L::LS_OVER ? lsep : lsep + cap);   // gather indices
+    C *ls_s = L::LS_OVER ? reinterpret_cast<C *>(x_s) : lsep;
+    uint8_t *fl_s = reinterpret_cast<uint8_t *>(x_s + cap);
 
-    const int lane = threadIdx.x % G, lane32 = threadIdx.x % 32, warp = threadIdx.x / 32;
-    const int grp_in_warp = lane32 / G;
-    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (grp_in_warp * G));
-    const int64_t r = (int64_t)blockIdx.x * (kEdgeThreads / G) + threadIdx.x / G;
-    const int64_t wr0 = (int64_t)blockIdx.x * (kEdgeThreads / G) + (int64_t)warp * (32 / G);
-    if (wr0 >= A.n) return;                      // whole warp past the end
-    const bool active = r < A.n;
-
-    C *a_s = reinterpret_cast<C *>(esm) + (size_t)warp * kWarpSlots;
-    C *ls_s = reinterpret_cast<C *>(esm) + (size_t)(kEdgeThreads / 32) * kWarpSlots + (size_t)warp * kWarpSlots;
-    uint8_t *fl_s = esm + (size_t)(kEdgeThreads / 32) * kWarpSlots * 2 * sizeof(C) + (size_t)warp * kWarpSlots;
-
-    const int32_t *__restrict__ col = A.col;
-    const int32_t *__restrict__ xcol = PX ? A.xcol : A.col;   // gather index of each slot
-    const AV *__restrict__ val = (const AV *)A.val;
-    const TS *__restrict__ X = (const TS *)A.x;
-    const int Kp = A.Kp;
-    const int64_t wr1 = min((int64_t)A.n, wr0 + 32 / G);
-    const int wbase = __ldg(A.prp + wr0), wend = __ldg(A.prp + wr1);
-    const bool staged = wend - wbase <= kWarpSlots;
+    const int np = G == 1 ? (A.K + V - 1) / V : NP;                   // pieces that are not all padding
+    const int rows = T / width;
+    const int64_t R0 = (int64_t)blockIdx.x * rows;
+    const int nr = (int)min((int64_t)rows, A.n - R0);
+    const int S0 = __ldg(A.prp + R0), S1 = __ldg(A.prp + R0 + nr);
+    const bool staged = S1 - S0 <= cap;
+    const int32_t *__restrict__ xcol = PX ? A.xcol : A.col;          // gather index of A's slots
+    const int32_t *__restrict__ fcol = PX ? A.xcol : A.pcol;         // and of the fits' slots
+    const AV *val = (const AV *)A.val;
+    const TS *X = (const TS *)A.x;
     C *a_out = (C *)A.a_out;
     C *ls_out = (C *)A.ls_out;
+    if (staged)
+        for (int q = tid; q < S1 - S0; q += T) x_s[q] = __ldg(fcol + S0 + q);
+    chain_wait();
+    chain_release();
+    if constexpr (!UW)
+        for (int k = tid; k < KP; k += T) ws[k] = ((const C *)A.w)[k];
+    if (PX && staged)                                                // d = 1: the fits' slots are A's
+        for (int q = tid; q < S1 - S0; q += T) a_s[q] = (C)ld_plain(val + S0 + q);
+    __syncthreads();
 
-    C w[NV][V];
-    if constexpr (!UW) {
+    if (tid / width < nr) {
+        const int64_t r = R0 + tid / width;
+        const int q0 = __ldg(A.prp + r), q1 = __ldg(A.prp + r + 1);
+        const int p0 = PX ? q0 : __ldg(A.rp + r), p1 = PX ? q1 : __ldg(A.rp + r + 1);
+        const int64_t xr = (PX && A.xrow) ? checked_row(__ldg(A.xrow + r), A.n, A.status) : r;
+        const C diag = (C)ld_plain((const AV *)A.diag + r);
+        auto gather = [&](int64_t j, uint4 (&raw)[NP]) {
+            const TS *src = X + checked_row(j, A.n, A.status) * KP;
+            if constexpr (NP == 1) {
+                raw[0] = ld16(src);
+            } else {
 #pragma unroll
-        for (int t = 0; t < NV; ++t)
-#pragma unroll
-            for (int e = 0; e < V; ++e) w[t][e] = ((const C *)A.w)[piece_of<G, NV>(lane, t) * V + e];
-    }
+                for (int q = 0; q < NP; q += 2) ld32(src + fit_piece<G, NP>(gl, q) * V, raw[q], raw[q + 1]);
+            }
+        };
+        auto w = [&](int q, int e) { return UW ? C(1) : ws[fit_piece<G, NP>(gl, q) * V + e]; };
 
-    int q0 = 0, q1 = 0;       // the row's entries in the pattern of the fits
-    C m = C(INFINITY), diag = C(1);
-    bool defer = false;       // a fit of this row cancelled in FP32: redo the row in FP64
-    if (active) {
-        const int p0 = __ldg(A.rp + r), p1 = __ldg(A.rp + r + 1);
-        q0 = __ldg(A.prp + r);
-        q1 = __ldg(A.prp + r + 1);
-        diag = (C)__ldg((const AV *)A.diag + r);
-
-        // ---- 1. target --------------------------------------------------
-        C y[NV][V];
+        // ---- 1. target ------------------------------------------------------------
+        C y[NP][V];
+        float syy = 0.f;
+        int j1 = -1;                 // exact rule: the row's one off-diagonal (gather index)
+        C a1 = C(0);
         {
-            Acc<C, V> acc[NV];
-            row_sum<TS, G, NV, U, false>(xcol, val, X, X, 0, Kp, lane, p0, p1, acc, A.n, A.status);
-            const C d = C(1) / diag;
-            const int64_t xr = (PX && A.xrow) ? checked_row(__ldg(A.xrow + r), A.n, A.status) : r;
+            Acc<C, V> acc[NP];
 #pragma unroll
-            for (int t = 0; t < NV; ++t) {
-                S::unpack(ldg16(X + xr * Kp + piece_of<G, NV>(lane, t) * V), y[t]);     // x_i
+            for (int t = 0; t < NP; ++t) acc[t].zero();
+            if (A.target == 0) {
+                for (int pb = p0; pb < p1; pb += UT) {
+                    int jj[UT];
+                    C vv[UT];
+#pragma unroll
+                    for (int u = 0; u < UT; ++u) {
+                        const int p = pb + u;
+                        const bool ok = p < p1;
+                        if (PX && staged) {
+                            jj[u] = ok ? x_s[p - S0] : -1;
+                            vv[u] = ok ? a_s[p - S0] : C(0);
+                        } else {
+                            jj[u] = ok ? __ldg(xcol + p) : -1;
+                            vv[u] = ok ? (C)ld_plain(val + p) : C(0);
+                        }
+                    }
+                    uint4 raw[UT][NP];
+#pragma unroll
+                    for (int u = 0; u < UT; ++u)
+                        if (jj[u] >= 0) gather(jj[u], raw[u]);
+#pragma unroll
+                    for (int u = 0; u < UT; ++u) {
+                        if (jj[u] < 0) break;
+#pragma unroll
+                        for (int t = 0; t < NP; ++t) {
+                            if (sizeof(C) == 8 && t >= np) break;
+                            C x[V];
+                            S::unpack(raw[u][t], x);
+                            acc[t].fma_piece(vv[u], x);
+                        }
+                    }
+                }
+            }
+            uint4 own[NP];
+            gather(xr, own);
+            const C d = C(1) / diag;
+#pragma unroll
+            for (int t = 0; t < NP; ++t) {
+                S::unpack(own[t], y[t]);
                 if (A.target == 0) {
 #pragma unroll
                     for (int e = 0; e < V; ++e) y[t][e] = fma(-d, acc[t].get(e), y[t][e]);
                 }
             }
-        }
-        C syy = C(0);
-        if constexpr (kMixed) {
+            if constexpr (kMixed) {
+                // S_yy, in the order of the other sums
+                auto piece = [&](int q) {
+                    float s = 0.f;
 #pragma unroll
-            for (int t = 0; t < NV; ++t)
-#pragma unroll
-                for (int e = 0; e < V; ++e)
-                    syy = fma(UW ? y[t][e] : w[t][e] * y[t][e], y[t][e], syy);
-            syy = group_sum<G>(syy, gmask);
-        }
-        // a residual-target row of A with one off-diagonal j1: y_i is exactly
-        // -(a_ij1 / a_ii) x_j1
-        int j1 = -1;
-        C v1 = C(0);
-        if (A.target == 0 && p1 - p0 == 2) {
-            const int pj = __ldg(col + p0) == r ? p0 + 1 : p0;
-            j1 = __ldg(col + pj);
-            v1 = (C)__ldg(val + pj);
-        }
-
-        // ---- 2. one-point LS per off-diagonal -----------------------------
-        for (int pb = q0; pb < q1; pb += U) {
-            int jj[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) jj[u] = (pb + u < q1) ? __ldg(A.pcol + pb + u) : -1;
-            uint4 raw[U][NV];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (jj[u] >= 0 && jj[u] != r) {
-                    const int64_t xj = checked_row(PX ? (int64_t)__ldg(xcol + pb + u) : (int64_t)jj[u],
-                                                   A.n, A.status);
-                    if constexpr (NV % 2 == 0) {                 // side-by-side pieces: 32-byte pairs
-#pragma unroll
-                        for (int t = 0; t < NV; t += 2)
-                            ldg32(X + xj * Kp + piece_of<G, NV>(lane, t) * V, raw[u][t], raw[u][t + 1]);
-                    } else {
-#pragma unroll
-                        for (int t = 0; t < NV; ++t)
-                            raw[u][t] = ldg16(X + xj * Kp + piece_of<G, NV>(lane, t) * V);
-                    }
+                    for (int e = 0; e < V; ++e) s = fmaf(UW ? y[q][e] : w(q, e) * y[q][e], y[q][e], s);
+                    return s;
+                };
+                if constexpr (NP == 1) {
+                    syy = piece(0);
+                } else {
+                    auto leaf = [&](int t) { return make_float2(piece(2 * t), piece(2 * t + 1)); };
+                    auto join = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
+                    syy = plain_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), gmask);
                 }
+            }
+            if (A.target == 0 && p1 - p0 == 2) {
+                // one off-diagonal j1: y_i is exactly -(a_ij1 / a_ii) x_j1
+                const int pj = __ldg(xcol + p0) == xr ? p0 + 1 : p0;
+                j1 = __ldg(xcol + pj);
+                a1 = -(C)ld_plain(val + pj) / diag;
+            }
+        }
+        if constexpr (G > 1 || SHARED) __syncwarp(rmask);   // the row's values and indices are read out
+
+        // ---- 2. one-point fits ------------------------------------------------------
+        C m = C(INFINITY);
+        bool defer = false;          // a fit of this row cancelled in FP32: redo the row in FP64
+        for (int pb = q0 + sub; pb < q1; pb += U * el) {
+            int jj[U];
+            uint4 raw[U][NP];
+            typename Norm<C>::T nr_j[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int p = pb + u * el;
+                jj[u] = p < q1 ? (staged ? x_s[p - S0] : __ldg(fcol + p)) : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (jj[u] < 0 || jj[u] == xr) continue;
+                nr_j[u] = ld_plain((const typename Norm<C>::T *)A.norms + checked_row(jj[u], A.n, A.status));
+                gather(jj[u], raw[u]);
+            }
+            if constexpr (G > 1) __syncwarp(gmask);      // every lane has read these entries' indices
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (jj[u] < 0) break;
-                const int p = pb + u;
-                C a_, ls_;
-                if (jj[u] == r) {
-                    a_ = C(0);
-                    ls_ = C(NAN);
+                const int p = pb + u * el;
+                C a_ = C(0), ls_ = C(NAN);
+                if (jj[u] == xr) {
                 } else if (jj[u] == j1) {
-                    a_ = -v1 / diag;
+                    a_ = a1;
                     ls_ = C(0);
-                } else if constexpr (COMP && kMixed) {
-                    Comp2 sx;
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        C xj[V];
-                        S::unpack(raw[u][t], xj);
-                        comp_piece_sums<V, UW>(xj, y[t], w[t], sx);
-                    }
-                    comp2_allreduce<G>(sx, gmask);
-                    const C sxx = sx.s.x + sx.c.x, syx = sx.s.y + sx.c.y;
-                    a_ = (sxx == C(0)) ? C(0) : divide(syx, sxx);
-                    Comp2 sl;
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        C xj[V];
-                        S::unpack(raw[u][t], xj);
-                        comp_residual<V, UW>(a_, xj, y[t], w[t], sl);
-                    }
-                    ls_ = comp_ls_total<G>(sl, gmask);
-                    defer = defer || ls_ < C(1e-4) * syy;
+                    m = fmin(m, ls_);
                 } else {
-                    // x_j is unpacked from the gathered bits once per use, so only one
-                    // 16-byte piece of it is live in registers at a time
-                    PieceSums<C, V, UW> ps;
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        C xj[V];
-                        S::unpack(raw[u][t], xj);
-                        ps.add(xj, y[t], w[t]);
-                    }
-                    const C sxx = group_sum<G>(ps.sxx(), gmask);
-                    const C syx = group_sum<G>(ps.syx(), gmask);
-                    a_ = (sxx == C(0)) ? C(0) : divide(syx, sxx);
-                    C res = C(0);
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        C xj[V];
-                        S::unpack(raw[u][t], xj);
-                        residual_add<C, V, UW>(a_, xj, y[t], w[t], res);
-                    }
-                    ls_ = group_sum<G>(res, gmask);
+                    fit_entry<TS, G, NP, UW, COMP>(raw[u], y, w, nr_j[u], np, gmask, a_, ls_);
+                    m = fmin(m, ls_);
                     if constexpr (kMixed) defer = defer || ls_ < C(1e-4) * syy;
                 }
-                if (jj[u] != r) m = fmin(m, ls_);
-                if (lane == 0) {
-                    if (staged) { a_s[p - wbase] = a_; ls_s[p - wbase] = ls_; }
+                if (gl == 0) {
+                    if (staged) { a_s[p - S0] = a_; ls_s[p - S0] = ls_; }
                     else { a_out[p] = a_; ls_out[p] = ls_; }
                 }
             }
         }
-    }
-    __syncwarp();
+        // the shares' minima and marks joined; every lane's stores are visible to the row's
+        if constexpr (G > 1 || SHARED) __syncwarp(rmask);
+        if constexpr (SHARED) {
+            for (int o = G; o < width; o <<= 1) m = fmin(m, __shfl_xor_sync(rmask, m, o));
+            if constexpr (kMixed) defer = __any_sync(rmask, defer);
+        }
 
-    // ---- 3. strength flags (from the LS values just produced) ----------------
-    const C theta = (C)A.theta;
-    int cnt = 0;
-    if (active) {
-        for (int p = q0 + lane; p < q1; p += G) {
-            const int j = __ldg(A.pcol + p);
-            const C l = staged ? ls_s[p - wbase] : ls_out[p];
-            const int strong = (j != r) && (l == C(0) || theta * l < m);
-            if (staged) fl_s[p - wbase] = (uint8_t)strong;
+        // ---- 3. strength flags (Eq. (4.4) in LS form) and counts --------------------
+        const C theta = (C)A.theta;
+        int cnt = 0;
+        for (int p = q0 + tid % width; p < q1; p += width) {
+            const C l = staged ? ls_s[p - S0] : ls_out[p];            // NaN on the diagonal
+            const bool strong = l == C(0) || theta * l < m;
+            if (staged) fl_s[p - S0] = (uint8_t)strong;
             else A.flag_out[p] = (uint8_t)strong;
             cnt += strong;
         }
-        cnt = group_sum<G>(cnt, gmask);
-        if (lane == 0) A.count_out[r] = cnt;
-        if (kMixed && defer && lane == 0) A.defer_list[atomicAdd(A.defer_count, 1u)] = (int32_t)r;
+        for (int o = 1; o < width; o <<= 1) cnt += __shfl_xor_sync(rmask, cnt, o);
+        if (tid % width == 0) {
+            A.count_out[r] = cnt;
+            if (kMixed && defer) A.defer_list[atomicAdd(A.defer_count, 1u)] = (int32_t)r;
+        }
     }
-    __syncwarp();
-
-    // ---- coalesced write-out of the warp's slot run --------------------------
     if (staged) {
-        for (int q = lane32; q < wend - wbase; q += 32) {
-            a_out[wbase + q] = a_s[q];
-            ls_out[wbase + q] = ls_s[q];
-            A.flag_out[wbase + q] = fl_s[q];
+        __syncthreads();
+        for (int q = tid; q < S1 - S0; q += T) {
+            a_out[S0 + q] = a_s[q];
+            ls_out[S0 + q] = ls_s[q];
+            A.flag_out[S0 + q] = fl_s[q];
         }
     }
 }
 
-// ---------------------------------------------------------------------------
-// Tile kernel (edge shape stage 1).  A block owns one tile of consecutive caller rows (at most
-// kEdgeTileRows rows and kEdgeTileSlots stored entries; a longer row is a
-// tile of its own), i.e. one contiguous run of CSR slots:
-//   A. targets: G lanes per row form y_i (the same row sums and rounding as
-//      the sweeps) into shared memory, plus S_yy per row on the mixed paths;
-//   B. fits: one thread per stored entry gathers x_j once, reads y_i from
-//      shared memory and forms S_xx, S_yx, a_ij and the residual sum LS_ij
-//      over all K components itself -- no cross-lane reductions, whole-warp
-//      use for the per-edge scalar work, coalesced a/LS writes; the row
-//      minimum of LS is an atomic minimum on the (non-negative) bit patterns
-//      in shared memory, which is order independent;
-//   C. flags and per-row counts from the row minima.
-// ---------------------------------------------------------------------------
-template <class C> struct MinBits;
-template <> struct MinBits<float> {
-    using T = unsigned int;
-    static constexpr T kInf = 0x7f800000u;
-    __device__ __forceinline__ static T bits(float v) { return __float_as_uint(v); }
-    __device__ __forceinline__ static float value(T b) { return __uint_as_float(b); }
-};
-template <> struct MinBits<double> {
-    using T = unsigned long long;
-    static constexpr T kInf = 0x7ff0000000000000ull;
-    __device__ __forceinline__ static T bits(double v) { return (T)__double_as_longlong(v); }
-    __device__ __forceinline__ static double value(T b) { return __longlong_as_double((long long)b); }
-};
-
-// shared-memory layout of one tile
-template <class TS, int KP>
-struct EdgeTileLayout {
-    using C = typename Store<TS>::C;
-    using M = typename MinBits<C>::T;
-    static constexpr int TR = kEdgeTileRows;
-    static constexpr int YS = 0;                                        // TR x KP targets
-    static constexpr int DG = YS + TR * KP * (int)sizeof(C);            // TR diagonals
-    static constexpr int SY = DG + TR * (int)sizeof(C);                 // TR S_yy
-    static constexpr int MN = (SY + TR * (int)sizeof(C) + 7) & ~7;      // TR row minima (bits)
-    static constexpr int RP = MN + TR * (int)sizeof(M);                 // TR + 1 slot offsets
-    static constexpr int CN = RP + (TR + 1) * 4;                        // TR strong counts
-    static constexpr int DF = CN + TR * 4;                              // TR defer marks
-    static constexpr int J1 = DF + TR * 4;                              // TR exact-rule neighbours
-    static constexpr int V1 = (J1 + TR * 4 + 7) & ~7;                   // TR their values a_ij1
-    static constexpr int SR = V1 + TR * (int)sizeof(C);                 // slot -> local row (u8)
-    static constexpr int BYTES = SR + kEdgeTileSlots;
-};
-
-template <class TS, int G, int NV, int U, bool UW, bool COMP>
-__global__ void __launch_bounds__(kEdgeThreads) k_edge_tiles(EdgeArgs A)
-{
-    using S = Store<TS>;
-    using C = typename S::C;
-    using AV = typename S::A;
-    using MB = MinBits<C>;
-    constexpr int V = S::V;
-    constexpr int P = G * NV;           // 16-byte pieces per row
-    constexpr int KP = P * V;           // padded components per row
-    using L = EdgeTileLayout<TS, KP>;
-    constexpr bool kMixed = !std::is_same<C, double>::value;
-    constexpr int HOLD = P <= 4 ? P : 1;     // pieces of x_j kept in registers between the sums
-    extern __shared__ __align__(16) unsigned char esm[];
-    C *ys = reinterpret_cast<C *>(esm + L::YS);
-    C *dg = reinterpret_cast<C *>(esm + L::DG);
-    C *syy = reinterpret_cast<C *>(esm + L::SY);
-    typename MB::T *rmin = reinterpret_cast<typename MB::T *>(esm + L::MN);
-    int32_t *rps = reinterpret_cast<int32_t *>(esm + L::RP);
-    int32_t *cnt = reinterpret_cast<int32_t *>(esm + L::CN);
-    int32_t *dfr = reinterpret_cast<int32_t *>(esm + L::DF);
-    int32_t *j1s = reinterpret_cast<int32_t *>(esm + L::J1);
-    C *v1s = reinterpret_cast<C *>(esm + L::V1);
-    uint8_t *srow = esm + L::SR;
-
-    const int32_t R0 = __ldg(A.tiles + blockIdx.x), R1 = __ldg(A.tiles + blockIdx.x + 1);
-    const int nr = R1 - R0;
-    const bool single = nr == 1;                 // possibly longer than kEdgeTileSlots
-    const int32_t *__restrict__ col = A.col;
-    const AV *__restrict__ val = (const AV *)A.val;
-    const TS *__restrict__ X = (const TS *)A.x;
-    const C *__restrict__ wv = (const C *)A.w;
-
-    for (int q = threadIdx.x; q <= nr; q += kEdgeThreads) rps[q] = __ldg(A.prp + R0 + q);
-    for (int q = threadIdx.x; q < nr; q += kEdgeThreads) {
-        dg[q] = (C)__ldg((const AV *)A.diag + R0 + q);
-        rmin[q] = MB::kInf;
-        cnt[q] = 0;
-        dfr[q] = 0;
-    }
-    __syncthreads();
-    const int S0 = rps[0], S1 = rps[nr];
-
-    // ---- A. targets -----------------------------------------------------------
-    {
-        const int lane = threadIdx.x % G;
-        const unsigned gmask = (G == 32) ? 0xffffffffu
-                                         : (((1u << G) - 1u) << ((threadIdx.x % 32) / G * G));
-        for (int rl = threadIdx.x / G; rl < nr; rl += kEdgeThreads / G) {
-            const int64_t r = R0 + rl;
-            if (!single)
-                for (int q = rps[rl] + lane; q < rps[rl + 1]; q += G) srow[q - S0] = (uint8_t)rl;
-            const int p0 = __ldg(A.rp + r), p1 = __ldg(A.rp + r + 1);   // row of A
-            if (lane == 0) {
-                // a residual-target row of A with one off-diagonal j1: y_i is
-                // exactly -(a_ij1 / a_ii) x_j1
-                int j1 = -1;
-                C v1 = C(0);
-                if (A.target == 0 && p1 - p0 == 2) {
-                    const int pj = __ldg(col + p0) == r ? p0 + 1 : p0;
-                    j1 = __ldg(col + pj);
-                    v1 = (C)__ldg(val + pj);
-                }
-                j1s[rl] = j1;
-                v1s[rl] = v1;
-            }
-            C y[NV][V];
-#pragma unroll
-            for (int t = 0; t < NV; ++t) S::unpack(ldg16(X + r * KP + piece_of<G, NV>(lane, t) * V), y[t]);
-            if (A.target == 0) {
-                Acc<C, V> acc[NV];
-                row_sum<TS, G, NV, U, false>(col, val, X, X, 0, KP, lane, p0, p1, acc, A.n, A.status);
-                const C d = C(1) / dg[rl];
-#pragma unroll
-                for (int t = 0; t < NV; ++t)
-#pragma unroll
-                    for (int e = 0; e < V; ++e) y[t][e] = fma(-d, acc[t].get(e), y[t][e]);
-            }
-            C s = C(0);
-#pragma unroll
-            for (int t = 0; t < NV; ++t) {
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    ys[rl * KP + piece_of<G, NV>(lane, t) * V + e] = y[t][e];
-                    if constexpr (kMixed)
-                        s = fma(UW ? y[t][e] : wv[piece_of<G, NV>(lane, t) * V + e] * y[t][e], y[t][e], s);
-                }
-            }
-            if constexpr (kMixed) {
-                s = group_sum<G>(s, gmask);
-                if (lane == 0) syy[rl] = s;
-            }
-        }
-    }
-    __syncthreads();
-
-    // ---- B. one-point fits, one stored entry per thread -------------------------
-    // one entry of a thread at a time (two in flight, their x_j gathered together,
-    // measured slower: the registers cost more occupancy than the overlap gains)
-    constexpr int E = 1;
-    C *a_out = (C *)A.a_out;
-    C *ls_out = (C *)A.ls_out;
-    // the fit of slot p (row rl, column j) from the pieces `hold` of x_j
-    auto fit = [&](int rl, int j, const uint4 (&hold)[HOLD], C &a_, C &ls_) {
-        const TS *xj = X + checked_row(j, A.n, A.status) * KP;
-        const C *yr = ys + rl * KP;
-        if constexpr (COMP && kMixed) {
-            // compensated sums over all K components in this thread
-            Comp2 sx;
-#pragma unroll
-            for (int c = 0; c < P; ++c) {
-                const uint4 raw = (P <= 4) ? hold[c < HOLD ? c : 0] : ldg16(xj + c * V);
-                C x[V], y[V], w[V];
-                S::unpack(raw, x);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    y[e] = yr[c * V + e];
-                    w[e] = UW ? C(1) : wv[c * V + e];
-                }
-                comp_piece_sums<V, UW>(x, y, w, sx);
-            }
-            const C sxx = sx.s.x + sx.c.x, syx = sx.s.y + sx.c.y;
-            a_ = (sxx == C(0)) ? C(0) : divide(syx, sxx);
-            Comp2 sl;
-#pragma unroll
-            for (int c = 0; c < P; ++c) {
-                const uint4 raw = (P <= 4) ? hold[c < HOLD ? c : 0] : ldg16(xj + c * V);
-                C x[V], y[V], w[V];
-                S::unpack(raw, x);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    y[e] = yr[c * V + e];
-                    w[e] = UW ? C(1) : wv[c * V + e];
-                }
-                comp_residual<V, UW>(a_, x, y, w, sl);
-            }
-            ls_ = comp_ls_total<1>(sl, 0xffffffffu);
-        } else {
-            PieceSums<C, V, UW> ps;
-#pragma unroll
-            for (int c = 0; c < P; ++c) {
-                const uint4 raw = (P <= 4) ? hold[c < HOLD ? c : 0] : ldg16(xj + c * V);
-                C x[V], y[V], w[V];
-                S::unpack(raw, x);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    y[e] = yr[c * V + e];
-                    w[e] = UW ? C(1) : wv[c * V + e];
-                }
-                ps.add(x, y, w);
-            }
-            const C sxx = ps.sxx(), syx = ps.syx();
-            a_ = (sxx == C(0)) ? C(0) : divide(syx, sxx);
-            C res = C(0);
-#pragma unroll
-            for (int c = 0; c < P; ++c) {
-                const uint4 raw = (P <= 4) ? hold[c < HOLD ? c : 0] : ldg16(xj + c * V);
-                C x[V], y[V], w[V];
-                S::unpack(raw, x);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    y[e] = yr[c * V + e];
-                    w[e] = UW ? C(1) : wv[c * V + e];
-                }
-                residual_add<C, V, UW>(a_, x, y, w, res);
-            }
-            ls_ = res;
-        }
-    };
-    for (int pb = S0 + threadIdx.x; pb < S1; pb += E * kEdgeThreads) {
-        int rls[E], js[E];
-        uint4 hold[E][HOLD];
-#pragma unroll
-        for (int q = 0; q < E; ++q) {
-            const int p = pb + q * kEdgeThreads;
-            js[q] = -1;
-            if (p < S1) {
-                rls[q] = single ? 0 : srow[p - S0];
-                js[q] = __ldg(A.pcol + p);
-                if (P <= 4 && js[q] != R0 + rls[q] && js[q] != j1s[rls[q]]) {
-                    const TS *xj = X + checked_row(js[q], A.n, A.status) * KP;
-                    if constexpr (HOLD % 2 == 0) {                  // 32-byte pairs
-#pragma unroll
-                        for (int c = 0; c < HOLD; c += 2) ldg32(xj + c * V, hold[q][c], hold[q][c + 1]);
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < HOLD; ++c) hold[q][c] = ldg16(xj + c * V);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < E; ++q) {
-            if (js[q] < 0) break;
-            const int p = pb + q * kEdgeThreads;
-            const int rl = rls[q], j = js[q];
-            const int64_t r = R0 + rl;
-            C a_, ls_;
-            if (j == r) {
-                a_ = C(0);
-                ls_ = C(NAN);
-            } else if (j == j1s[rl]) {
-                a_ = -v1s[rl] / dg[rl];                 // y_i = -(a_ij/a_ii) x_j exactly
-                ls_ = C(0);
-            } else {
-                fit(rl, j, hold[q], a_, ls_);
-                if constexpr (kMixed)
-                    if (ls_ < C(1e-4) * syy[rl]) dfr[rl] = 1;    // cancellation: redo the row in FP64
-            }
-            a_out[p] = a_;
-            ls_out[p] = ls_;
-            if (j != r) atomicMin(&rmin[rl], MB::bits(ls_));
-        }
-    }
-    __syncthreads();
-
-    // ---- C. strength flags (Eq. (4.4) in LS form) and counts -------------------
-    const C theta = (C)A.theta;
-    for (int p = S0 + threadIdx.x; p < S1; p += kEdgeThreads) {
-        const int rl = single ? 0 : srow[p - S0];
-        const C l = ls_out[p];                       // written by this block in B; NaN on the diagonal
-        const C m = MB::value(rmin[rl]);
-        const int strong = l == C(0) || theta * l < m;   // false for the diagonal's NaN
-        A.flag_out[p] = (uint8_t)strong;
-        if (strong) atomicAdd(&cnt[rl], 1);
-    }
-    __syncthreads();
-    for (int rl = threadIdx.x; rl < nr; rl += kEdgeThreads) {
-        A.count_out[R0 + rl] = cnt[rl];
-        if (kMixed && dfr[rl]) A.defer_list[atomicAdd(A.defer_count, 1u)] = R0 + rl;
-    }
-}
-
-// Mixed paths: rows listed by k_edge (a fit cancelled in FP32, LS < 1e-4 S_yy)
-// are recomputed here entirely in FP64 from the stored vectors (widened
+// Mixed paths: rows listed by k_edge_fit (a fit cancelled in FP32, LS < 1e-4
+// S_yy) are recomputed here entirely in FP64 from the stored vectors (widened
 // exactly) and the FP64 values of A: target with the FP64 path's rounding,
-// every one-point fit, the row minimum, flags and count.  One warp per row,
-// lanes over the K components (K <= 64: two per lane).
+// every one-point fit, the row minimum, flags and count.  One warp per row:
+// lanes over the components for the target (two per lane for K > 32), then one
+// stored entry per lane for the fits, the K-term sums in the order of a
+// butterfly over 32 lanes that hold a component each.  Bound: the FP64 pipe
+// (a fit in one lane is 7K FP64 operations; the lanes of a butterfly would
+// repeat every addition).
 template <class TS>
 __device__ __forceinline__ double elem64(const TS *p)
 {
@@ -736,45 +686,71 @@ __device__ __forceinline__ double elem64(const TS *p)
         return (double)*p;
 }
 
-template <class TS, bool PX>
-__global__ void __launch_bounds__(256) k_edge_fixup(EdgeArgs A)
+constexpr int kFixThreads = 256;
+
+template <class TS, int P, bool PX>
+__global__ void __launch_bounds__(kFixThreads) k_edge_fixup(EdgeArgs A)
 {
     using C = typename Store<TS>::C;
+    constexpr int KP = P * Store<TS>::V;
+    constexpr int LEAVES = KP < 32 ? KP : 32;
+    __shared__ double ysm[kFixThreads / 32][KP], wsm[KP];
+    chain_wait();
+    chain_release();
     const unsigned count = *A.defer_count;
     const int lane = threadIdx.x % 32;
+    double *ys = ysm[threadIdx.x / 32];
     const TS *X = (const TS *)A.x;
-    const int Kp = A.Kp;
-    // vector row of caller row i and of the neighbour of slot p (stage 2: the
-    // sweeps' row order; search depth 1, so the fit slots are A's slots)
+    if ((unsigned)blockIdx.x * (kFixThreads / 32) >= count) return;
+    for (int k = threadIdx.x; k < KP; k += kFixThreads) wsm[k] = A.w64[k];
+    __syncthreads();
+    // vector row of caller row i (in place: the sweeps' row order; search
+    // depth 1, so the fit slots are A's slots)
     auto xrow = [&](int64_t i) -> int64_t { return (PX && A.xrow) ? checked_row(A.xrow[i], A.n, A.status) : i; };
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
-    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; q < count; q += warps) {
+    const int64_t warps = (int64_t)gridDim.x * (kFixThreads / 32);
+    for (int64_t q = (int64_t)blockIdx.x * (kFixThreads / 32) + threadIdx.x / 32; q < count; q += warps) {
         const int64_t r = A.defer_list[q];
         const int p0 = A.rp[r], p1 = A.rp[r + 1];         // row of A: target
         const int q0 = A.prp[r], q1 = A.prp[r + 1];       // entries of the fits
         double diag = 1.0;
         int j1 = -1;
         double v1 = 0.0;
-        for (int p = p0; p < p1; ++p) {
-            if (A.col[p] == r) diag = A.val64[p];
-            else if (A.target == 0 && p1 - p0 == 2) { j1 = A.col[p]; v1 = A.val64[p]; }
+        double acc[2] = {0.0, 0.0};
+        for (int pb = p0; pb < p1; pb += 4) {
+            // four entries' gathers in flight
+            double v[4], x[4][2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (pb + u >= p1) break;
+                const int p = pb + u;
+                v[u] = A.val64[p];
+                if (A.col[p] == r) diag = v[u];
+                else if (A.target == 0 && p1 - p0 == 2) { j1 = A.col[p]; v1 = v[u]; }
+                const TS *src = X + checked_row(PX ? A.xcol[p] : A.col[p], A.n, A.status) * KP;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) x[u][h] = lane + 32 * h < KP ? elem64(src + lane + 32 * h) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (pb + u >= p1) break;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) acc[h] = fma(v[u], x[u][h], acc[h]);
+            }
         }
         const double d = 1.0 / diag;
-        double y[2], w[2];
+        __syncwarp();                                     // the last row's targets are read out
+#pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int k = lane + 32 * h;
-            w[h] = k < Kp ? A.w64[k] : 0.0;
-            double acc = 0.0;
-            const double xi = k < Kp ? elem64(X + xrow(r) * Kp + k) : 0.0;
-            if (k < Kp)
-                for (int p = p0; p < p1; ++p)
-                    acc = fma(A.val64[p], elem64(X + checked_row(PX ? A.xcol[p] : A.col[p], A.n, A.status) * Kp + k), acc);
-            y[h] = (A.target == 0) ? fma(-d, acc, xi) : xi;
+            if (k >= KP) break;
+            const double xi = elem64(X + xrow(r) * KP + k);
+            ys[k] = (A.target == 0) ? fma(-d, acc[h], xi) : xi;
         }
+        __syncwarp();
         double m = INFINITY;
         C *a_out = (C *)A.a_out;
         C *ls_out = (C *)A.ls_out;
-        for (int p = q0; p < q1; ++p) {
+        for (int p = q0 + lane; p < q1; p += 32) {
             const int64_t j = A.pcol[p];
             double a64, ls64;
             if (j == r) {
@@ -784,34 +760,31 @@ __global__ void __launch_bounds__(256) k_edge_fixup(EdgeArgs A)
                 a64 = -v1 / diag;
                 ls64 = 0.0;
             } else {
-                double xj[2], sxx = 0.0, syx = 0.0;
-                const int64_t xjr = checked_row(PX ? (int64_t)A.xcol[p] : j, A.n, A.status);
-                for (int h = 0; h < 2; ++h) {
-                    const int k = lane + 32 * h;
-                    xj[h] = k < Kp ? elem64(X + xjr * Kp + k) : 0.0;
-                    sxx = fma(w[h] * xj[h], xj[h], sxx);
-                    syx = fma(w[h] * xj[h], y[h], syx);
-                }
-                for (int o = 16; o > 0; o >>= 1) {
-                    sxx += __shfl_xor_sync(0xffffffffu, sxx, o);
-                    syx += __shfl_xor_sync(0xffffffffu, syx, o);
-                }
+                const TS *xj = X + checked_row(PX ? (int64_t)A.xcol[p] : j, A.n, A.status) * KP;
+                auto add = [](double a, double b) { return a + b; };
+                // component l of the sum (and l + 32 for K > 32): f(w, x, y)
+                auto over = [&](auto f) {
+                    auto leaf = [&](int l) {
+                        double s = f(0.0, wsm[l], elem64(xj + l), ys[l]);
+                        if constexpr (KP > 32) s = f(s, wsm[l + 32], elem64(xj + l + 32), ys[l + 32]);
+                        return s;
+                    };
+                    return tree_sum<0, 1, LEAVES>(leaf, add);
+                };
+                const double sxx = over([](double s, double w, double x, double) { return fma(w * x, x, s); });
+                const double syx = over([](double s, double w, double x, double y) { return fma(w * x, y, s); });
                 a64 = (sxx == 0.0) ? 0.0 : syx / sxx;
-                double res = 0.0;
-                for (int h = 0; h < 2; ++h) {
-                    const double e = fma(-a64, xj[h], y[h]);
-                    res = fma(w[h] * e, e, res);
-                }
-                for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
-                ls64 = res;
+                ls64 = over([&](double s, double w, double x, double y) {
+                    const double e = fma(-a64, x, y);
+                    return fma(w * e, e, s);
+                });
             }
             if (j != r) m = fmin(m, ls64);
-            if (lane == 0) {
-                a_out[p] = (C)a64;
-                ls_out[p] = (C)ls64;
-            }
+            a_out[p] = (C)a64;
+            ls_out[p] = (C)ls64;
         }
-        __syncwarp();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
         int cnt = 0;
         for (int p = q0 + lane; p < q1; p += 32) {
             const double l = (double)ls_out[p];
@@ -821,114 +794,84 @@ __global__ void __launch_bounds__(256) k_edge_fixup(EdgeArgs A)
         }
         for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
         if (lane == 0) A.count_out[r] = cnt;
-        __syncwarp();
     }
 }
 
-template <class TS, int G, int NV, int U, bool UW, bool PX, bool COMP>
-cudaError_t go_rows(const EdgeArgs &a, cudaStream_t s)
+// Shares of a row's entries and threads of a block.  A small matrix leaves most
+// of the chip idle at one lane group per row, and the pass is then the latency
+// of a row's entries one after the other: up to four shares (each forms the
+// target of its own) while the lanes fit in two warps per scheduler, and
+// blocks of down to 32 threads while there are fewer than four per SM (64 x 64
+// 5-point, K = 8, FP64: 12.9 us with one share, 8.7 with four).
+inline int fit_shares(int64_t lanes, int G)
 {
-    if constexpr (NV % 2 == 0)
-        if (!rows_aligned32(a.x, a.Kp, sizeof(TS))) return cudaErrorMisalignedAddress;
-    const int rows_per_block = kEdgeThreads / G;
-    const unsigned grid = (unsigned)(((int64_t)a.n + rows_per_block - 1) / rows_per_block);
-    constexpr int smem = edge_smem_bytes<typename Store<TS>::C, G>();
-    static PerDevice opted;                  // shared-memory opt-in made on each device
-    const int dev = current_device_index();
-    if (smem > 48 * 1024 && opted.get(dev) == 0) {
-        const cudaError_t e = cudaFuncSetAttribute(k_edge_rows<TS, G, NV, U, UW, PX, COMP>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        opted.set(dev, 1);
-    }
-    k_edge_rows<TS, G, NV, U, UW, PX, COMP><<<grid, kEdgeThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    int el = 1;
+    while (el < 4 && G * el < 32 && lanes * el < (int64_t)152 * 256) el *= 2;
+    return el;
 }
-
-template <class TS, int G, int NV, int U, bool UW, bool COMP>
-cudaError_t go_tiles(const EdgeArgs &a, cudaStream_t s)
+inline int fit_threads(int64_t lanes)
 {
-    constexpr int KP = G * NV * Store<TS>::V;
-    if (a.Kp != KP || a.ntiles <= 0) return cudaErrorInvalidValue;
-    if constexpr ((G * NV) % 2 == 0)          // 32-byte row reads (row sums at G = 1, fits)
-        if (!rows_aligned32(a.x, a.Kp, sizeof(TS))) return cudaErrorMisalignedAddress;
-    constexpr int smem = EdgeTileLayout<TS, KP>::BYTES;
-    static PerDevice opted;                  // shared-memory opt-in made on each device
-    const int dev = current_device_index();
-    if (smem > 48 * 1024 && opted.get(dev) == 0) {
-        const cudaError_t e = cudaFuncSetAttribute(k_edge_tiles<TS, G, NV, U, UW, COMP>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        opted.set(dev, 1);
-    }
-    k_edge_tiles<TS, G, NV, U, UW, COMP><<<(unsigned)a.ntiles, kEdgeThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    int t = kFitThreads;
+    while (t > 32 && lanes < (int64_t)152 * 4 * t) t /= 2;
+    return t;
 }
 
-}  // namespace edge_impl
-}  // namespace amgd
+template <class TS, int P, bool UW, bool PX, bool COMP>
+cudaError_t go_fit(const EdgeArgs &a, cudaStream_t s)
+{
+    using L = FitLayout<TS, P>;
+    if (a.Kp != L::KP || !a.norms) return cudaErrorInvalidValue;
+    if constexpr (P % 2 == 0)                      // 32-byte row reads
+        if (!rows_aligned32(a.x, a.Kp, sizeof(TS))) return cudaErrorMisalignedAddress;
+    constexpr int per = sizeof(TS) == 8 ? kNormThreads : kNormThreads / P;    // rows per block
+    cudaError_t e = launch_chained(k_norms<TS, P, UW, COMP>, (unsigned)(((int64_t)a.n + per - 1) / per), kNormThreads,
+                                   0, s, (const TS *)a.x, a.w, a.n, a.norms);
+    if (e != cudaSuccess) return e;
+    // slots staged per block: the average rows' entries and a quarter more
+    // (a block with longer rows works on global memory), at most 96 KB
+    const int el = fit_shares((int64_t)a.n * L::G, L::G);
+    const int T = fit_threads((int64_t)a.n * L::G * el);
+    const int rows = T / (L::G * el);
+    int64_t cap = (int64_t)((double)a.nnz_p / a.n * rows * 1.25) + 32;
+    const int64_t most = (96 * 1024 - L::bytes(0, UW)) / L::SLOT;
+    cap = (cap < most ? cap : most) & ~(int64_t)15;
+    const int smem = L::bytes((int)cap, UW);
+    const auto kern = el > 1 ? k_edge_fit<TS, P, UW, PX, COMP, true> : k_edge_fit<TS, P, UW, PX, COMP, false>;
+    static PerDevice opted[2];               // shared-memory opt-in made on each device
+    const int dev = current_device_index();
+    if (opted[el > 1].get(dev) == 0) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+        if (e != cudaSuccess) return e;
+        opted[el > 1].set(dev, 1);
+    }
+    e = launch_chained(kern, (unsigned)(((int64_t)a.n + rows - 1) / rows), T, smem, s, a, (int)cap, el);
+    if (e != cudaSuccess) return e;
+    if constexpr (!std::is_same<TS, double>::value)
+        e = launch_chained(k_edge_fixup<TS, P, PX>, 152, kFixThreads, 0, s, a);
+    return e;
+}
 
-#include "k_edge_warp.cuh"
+template <class TS, bool COMP, int P>
+cudaError_t dispatch_w(bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s)
+{
+    if (in_place) return unit_w ? go_fit<TS, P, true, true, COMP>(a, s) : go_fit<TS, P, false, true, COMP>(a, s);
+    return unit_w ? go_fit<TS, P, true, false, COMP>(a, s) : go_fit<TS, P, false, false, COMP>(a, s);
+}
 
-namespace amgd {
-namespace edge_impl {
-
-// one storage type and summation form; the plain and the compensated forms
-// are instantiated in separate translation units (parallel compilation)
-template <class TS, bool COMP, int G, int NV, int U, bool UW>
-cudaError_t go(int stage, const EdgeArgs &a, cudaStream_t s)
+// one storage type and summation form per translation unit (parallel
+// compilation)
+template <class TS, bool COMP>
+cudaError_t dispatch(bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s)
 {
     if (a.n <= 0) return cudaSuccess;
-    if (stage == 1) return go_tiles<TS, G, NV, U, UW, COMP>(a, s);
-    if (stage == 2) return go_rows<TS, G, NV, U, UW, true, COMP>(a, s);
-    if (stage == 3) {
-        if constexpr (U >= 4) return go_warp<TS, G, NV, U, UW, COMP>(a, s);
-        return cudaErrorInvalidValue;
-    }
-    return go_rows<TS, G, NV, U, UW, false, COMP>(a, s);
-}
-
-template <class TS, bool COMP, int G, int NV, bool UW>
-cudaError_t dispatch_u(int stage, int U, const EdgeArgs &a, cudaStream_t s)
-{
-    switch (U) {
-    case 2: return go<TS, COMP, G, NV, 2, UW>(stage, a, s);
-    case 4: return go<TS, COMP, G, NV, 4, UW>(stage, a, s);
-    case 8: return go<TS, COMP, G, NV, 8, UW>(stage, a, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
-template <class TS, bool COMP, int G, int NV>
-cudaError_t dispatch_w(int stage, int U, bool unit_w, const EdgeArgs &a, cudaStream_t s)
-{
-    return unit_w ? dispatch_u<TS, COMP, G, NV, true>(stage, U, a, s)
-                  : dispatch_u<TS, COMP, G, NV, false>(stage, U, a, s);
-}
-
-template <class TS, bool COMP, int G>
-cudaError_t dispatch_nv(int stage, int NV, int U, bool unit_w, const EdgeArgs &a, cudaStream_t s)
-{
     constexpr int V = Store<TS>::V;
-    switch (NV) {
-    case 1: return dispatch_w<TS, COMP, G, 1>(stage, U, unit_w, a, s);
-    case 2: if constexpr (G * 2 * V <= 64) return dispatch_w<TS, COMP, G, 2>(stage, U, unit_w, a, s); break;
-    case 4: if constexpr (G * 4 * V <= 64) return dispatch_w<TS, COMP, G, 4>(stage, U, unit_w, a, s); break;
-    }
-    return cudaErrorInvalidValue;
-}
-
-template <class TS, bool COMP>
-cudaError_t dispatch_g(Shape sh, bool unit_w, const EdgeArgs &a, cudaStream_t s)
-{
-    constexpr int V = Store<TS>::V;
-    switch (sh.G) {
-    case 1: return dispatch_nv<TS, COMP, 1>(sh.stage, sh.NV, sh.U, unit_w, a, s);
-    case 2: return dispatch_nv<TS, COMP, 2>(sh.stage, sh.NV, sh.U, unit_w, a, s);
-    case 4: return dispatch_nv<TS, COMP, 4>(sh.stage, sh.NV, sh.U, unit_w, a, s);
-    case 8: if constexpr (8 * V <= 64) return dispatch_nv<TS, COMP, 8>(sh.stage, sh.NV, sh.U, unit_w, a, s); break;
-    case 16: if constexpr (16 * V <= 64) return dispatch_nv<TS, COMP, 16>(sh.stage, sh.NV, sh.U, unit_w, a, s); break;
-    case 32: if constexpr (32 * V <= 64) return dispatch_nv<TS, COMP, 32>(sh.stage, sh.NV, sh.U, unit_w, a, s); break;
+    switch (a.Kp / V) {
+    case 1: return dispatch_w<TS, COMP, 1>(in_place, unit_w, a, s);
+    case 2: return dispatch_w<TS, COMP, 2>(in_place, unit_w, a, s);
+    case 4: return dispatch_w<TS, COMP, 4>(in_place, unit_w, a, s);
+    case 8: return dispatch_w<TS, COMP, 8>(in_place, unit_w, a, s);
+    case 16: if constexpr (16 * V <= 64) return dispatch_w<TS, COMP, 16>(in_place, unit_w, a, s); break;
+    case 32: if constexpr (32 * V <= 64) return dispatch_w<TS, COMP, 32>(in_place, unit_w, a, s); break;
     }
     return cudaErrorInvalidValue;
 }

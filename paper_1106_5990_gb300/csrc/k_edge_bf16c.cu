@@ -4,9 +4,9 @@
 
 namespace amgd {
 
-cudaError_t launch_edge_bf16_comp(Shape sh, bool unit_w, const EdgeArgs &a, cudaStream_t s)
+cudaError_t launch_edge_bf16_comp(bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s)
 {
-    return edge_impl::dispatch_g<__nv_bfloat16, true>(sh, unit_w, a, s);
+    return edge_impl::dispatch<__nv_bfloat16, true>(in_place, unit_w, a, s);
 }
 
 }  // namespace amgd

@@ -4,9 +4,9 @@
 
 namespace amgd {
 
-cudaError_t launch_edge_f32_comp(Shape sh, bool unit_w, const EdgeArgs &a, cudaStream_t s)
+cudaError_t launch_edge_f32_comp(bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s)
 {
-    return edge_impl::dispatch_g<float, true>(sh, unit_w, a, s);
+    return edge_impl::dispatch<float, true>(in_place, unit_w, a, s);
 }
 
 }  // namespace amgd

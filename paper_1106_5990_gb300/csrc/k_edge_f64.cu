@@ -3,9 +3,9 @@
 
 namespace amgd {
 
-cudaError_t launch_edge_f64(Shape sh, bool unit_w, const EdgeArgs &a, cudaStream_t s)
+cudaError_t launch_edge_f64(bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s)
 {
-    return edge_impl::dispatch_g<double, false>(sh, unit_w, a, s);
+    return edge_impl::dispatch<double, false>(in_place, unit_w, a, s);
 }
 
 }  // namespace amgd
