@@ -19,7 +19,7 @@ LIB = os.path.join(LIBDIR, "libamgd.so")
 # the checked build: every gather index of the sweep and distance kernels is
 # bounds-tested in the kernel (AMGD_CHECKS); for tests, loaded with AMGD_CHECKED=1
 LIB_CHECKED = os.path.join(LIBDIR, "libamgd_checked.so")
-SOURCES = ["amgd_api.cu", "k_relax.cu", "k_edge.cu", "k_edge_f64.cu", "k_edge_f32.cu",
+SOURCES = ["amgd_api.cu", "k_relax.cu", "k_sell.cu", "k_edge.cu", "k_edge_f64.cu", "k_edge_f32.cu",
            "k_edge_f32c.cu", "k_edge_bf16.cu", "k_edge_bf16c.cu", "k_init.cu", "k_compact.cu",
            "amgd_noalloc.cu", "k_adjoint.cu", "k_interp.cu", "k_cr.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -55,6 +55,19 @@ struct amgd_ctx {
     uint32_t *defer_count = nullptr;             // rows the mixed edge pass redoes in FP64
     int32_t *defer_list = nullptr;
     std::vector<int64_t> color_start;           // permuted row start of each color
+    // sliced copy of the permuted matrix (built by ensure_sell for the sweeps)
+    int64_t sweep_calls = 0;                     // sweep calls prepared so far
+    bool sell_tried = false;                     // for the current coloring
+    bool sell_ok = false;                        // the copy exists (else its padding was too much)
+    int64_t sell_entries = 0;
+    int64_t *sell_ptr = nullptr, *sell_tab = nullptr;   // tab: first rows, then first slices of the colors
+    int32_t *sell_col = nullptr, *sell_slot = nullptr, *sell_map = nullptr;
+    double *sell_val64 = nullptr;
+    float *sell_val32 = nullptr;
+    std::vector<int64_t> color_slice;            // first slice of each color
+    bool perm32_stale = false;                   // row-permuted FP32 values out of date
+    bool graph_csr = false;                      // the captured graph reads the row-permuted CSR values
+    void *weight = nullptr;                      // omega / a_ii of a relaxation (8 bytes per row)
     // vectors
     void *x[2] = {nullptr, nullptr};
     int cur = 0;
@@ -330,26 +343,37 @@ int upload_weights(amgd_ctx *h)
     return AMGD_OK;
 }
 
-// Values from src (caller order; NULL: h->val_o itself) into every copy the
-// kernels read -- the caller FP64 array, the FP32 copies and, with a
-// coloring, the row-permuted arrays -- in one coalesced pass, then the
-// diagonals in caller and permuted order.
-// Every value copy from the caller-order values (src, or the handle's own
-// FP64 copy when NULL).  The row-permuted FP64 copy and diagonal feed only the
-// FP64 sweeps and the coarsening; with mixed storage they are left stale here
-// and refreshed by refresh_perm64 when one of those next runs.  err (NULL:
-// none) collects the value checks of an asynchronous update.
+// whether the sweeps read the row-permuted CSR (the staged kernels, or no sliced
+// copy) instead of the sliced copy
+bool sweeps_use_csr(const amgd_ctx *h)
+{
+    const int st = h->relax_shape[h->storage].stage;
+    return st == 1 || st == 2 || !h->sell_ok;
+}
+
+// Every value copy that queued work reads, from the caller-order values (src,
+// or the handle's own FP64 copy when NULL), in one coalesced pass, then the
+// diagonals in caller and permuted order: the caller FP64 and FP32 arrays, the
+// sliced copy of the sweeps, and the row-permuted CSR arrays only where a sweep
+// kernel reads them.  Those are otherwise left stale, to be refreshed from the
+// caller-order FP64 copy when a staged sweep (refresh_perm32 / 64) or the
+// coarsening (refresh_perm64) next runs.  err (NULL: none) collects the value
+// checks of an asynchronous update.
 int permute_values(amgd_ctx *h, const double *src = nullptr, uint32_t *err = nullptr)
 {
     const bool in_place = src == nullptr;
     const bool mixed = h->storage != ST_FP64;
-    float *v32o = (h->val32_o && h->val32_o != h->val32) ? h->val32_o : nullptr;
-    double *vp64 = (h->perm && !mixed) ? h->val64 : nullptr;   // without a coloring val64 is val_o
+    const bool csr = sweeps_use_csr(h) || (h->gexec && h->graph_csr);
+    float *v32o = mixed ? h->val32_o : nullptr;
+    double *vp64 = (h->perm && !mixed && csr) ? h->val64 : nullptr;   // without a coloring val64 is val_o
+    float *vp32 = (h->perm && mixed && csr) ? h->val32 : nullptr;     // and val32 is not read
     CK(h, launch_scatter_values(in_place ? h->val_o : src, h->nnz, h->perm ? h->slot_perm : nullptr,
-                                in_place ? nullptr : h->val_o, v32o, vp64, h->val32, h->stream, err));
+                                h->sell_ok ? h->sell_slot : nullptr, in_place ? nullptr : h->val_o, v32o, vp64, vp32,
+                                mixed ? nullptr : h->sell_val64, mixed ? h->sell_val32 : nullptr, h->stream, err));
     CK(h, launch_diag_values(h->val_o, h->diag_slot, h->perm, (int32_t)h->n, h->diag64_o,
                              h->diag32_o, mixed ? nullptr : h->diag64, h->diag32, h->stream, err));
-    h->perm64_stale = mixed;
+    h->perm64_stale = mixed || !csr;
+    h->perm32_stale = !(mixed && csr);
     return AMGD_OK;
 }
 
@@ -358,12 +382,173 @@ int refresh_perm64(amgd_ctx *h, cudaStream_t s)
 {
     if (!h->perm64_stale) return AMGD_OK;
     if (h->perm)
-        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, h->val64,
-                                    nullptr, s));
+        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, nullptr, h->val64,
+                                    nullptr, nullptr, nullptr, s));
     CK(h, launch_diag_values(h->val_o, h->diag_slot, h->perm, (int32_t)h->n, nullptr, nullptr,
                              h->diag64, nullptr, s));
     h->perm64_stale = false;
     return AMGD_OK;
+}
+
+// and the row-permuted FP32 values
+int refresh_perm32(amgd_ctx *h, cudaStream_t s)
+{
+    if (!h->perm32_stale) return AMGD_OK;
+    if (h->perm)
+        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, nullptr, nullptr, h->val32,
+                                    nullptr, nullptr, s));
+    h->perm32_stale = false;
+    return AMGD_OK;
+}
+
+void drop_sell(amgd_ctx *h)
+{
+    void *ptrs[] = {h->sell_ptr, h->sell_tab, h->sell_col, h->sell_slot, h->sell_map, h->sell_val64, h->sell_val32};
+    for (void *p : ptrs) dfree(p);
+    h->sell_ptr = h->sell_tab = nullptr;
+    h->sell_col = h->sell_slot = h->sell_map = nullptr;
+    h->sell_val64 = nullptr;
+    h->sell_val32 = nullptr;
+    h->sell_tried = h->sell_ok = false;
+}
+
+// The sliced copy of the current row order, and its values for the current
+// storage.  Synchronises the handle's stream when something has to be built,
+// so it runs before a capture, never inside one.  Where the copy would be more
+// than half as large again as the matrix (rows of very uneven length), or does
+// not fit the device, the sweeps read the row-permuted CSR.
+int ensure_sell(amgd_ctx *h)
+{
+    if (h->n == 0) return AMGD_OK;
+    cudaStream_t s = h->stream;
+    cudaError_t e = cudaSuccess;
+    // gives the copy up; an allocation that fails leaves the CSR in use
+    auto without = [&](cudaError_t err) {
+        drop_sell(h);
+        h->sell_tried = true;
+        if (err == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            return AMGD_OK;
+        }
+        if (err == cudaSuccess) return AMGD_OK;
+        h->sell_tried = false;
+        return cuda_fail(h, err, "the sweeps' copy of the matrix");
+    };
+    if (!h->sell_tried) {
+        const int nc = (int)h->color_start.size() - 1;
+        h->color_slice.assign((size_t)nc + 1, 0);
+        for (int c = 0; c < nc; ++c)
+            h->color_slice[(size_t)c + 1] = h->color_slice[(size_t)c] +
+                (h->color_start[(size_t)c + 1] - h->color_start[(size_t)c] + kSellRows - 1) / kSellRows;
+        const int64_t nsl = h->color_slice[(size_t)nc];
+        std::vector<int64_t> tab(h->color_start.begin(), h->color_start.end());
+        tab.insert(tab.end(), h->color_slice.begin(), h->color_slice.end());
+        // scratch: widths (padded for 16-byte loads), their tile sums, the total
+        const size_t wn = ((size_t)nsl + 8) & ~(size_t)7, tn = (size_t)(nsl / kTileRows + 2) & ~(size_t)1;
+        int32_t *scratch = nullptr;
+        e = dalloc(&h->sell_tab, tab.size());
+        if (e == cudaSuccess) e = dalloc(&h->sell_ptr, (size_t)nsl + 1);
+        if (e == cudaSuccess) e = dalloc(&scratch, wn + tn + 4);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->sell_tab, tab.data(), tab.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
+        int32_t *width = scratch, *tile = scratch + wn;
+        unsigned long long *dtotal = (unsigned long long *)(scratch + wn + tn), total = 0;
+        const SellArgs a{h->rp_p, h->col_p, h->rp_o, h->perm, h->sell_tab, h->sell_tab + nc + 1, nc, nsl, (int32_t)h->n};
+        auto measure = [&]() {
+            if (e == cudaSuccess) e = launch_sell_width(a, h->sell_map, width, dtotal, s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&total, dtotal, sizeof total, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        };
+        measure();
+        // rows of uneven length: sorted inside windows where the rows in order
+        // would store an eighth more than the matrix
+        const unsigned long long nnz = (unsigned long long)h->nnz;
+        if (e == cudaSuccess && total > nnz + nnz / 8 + 8192) {
+            e = dalloc(&h->sell_map, (size_t)nsl * kSellRows);
+            if (e == cudaSuccess) e = launch_sell_sort(a, h->sell_map, s);
+            measure();
+        }
+        const bool fits = total <= nnz + nnz / 2 + 32768 && total < (1ull << 31) - 64;
+        if (e == cudaSuccess && fits) {
+            e = launch_row_ptr(width, (int32_t)nsl, tile, h->sell_ptr, s);
+            if (e == cudaSuccess) e = dalloc(&h->sell_col, (size_t)total);
+            if (e == cudaSuccess) e = dalloc(&h->sell_slot, (size_t)h->nnz);
+            if (e == cudaSuccess) e = launch_sell_fill(a, h->sell_map, h->sell_ptr, h->sell_col, h->sell_slot, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        }
+        dfree(scratch);
+        if (e != cudaSuccess || !fits) return without(e);
+        h->sell_entries = (int64_t)total;
+        h->sell_tried = h->sell_ok = true;
+    }
+    if (!h->sell_ok) return AMGD_OK;
+    const bool mixed = h->storage != ST_FP64;
+    if (mixed ? !h->sell_val32 : !h->sell_val64) {
+        e = mixed ? dalloc(&h->sell_val32, (size_t)h->sell_entries) : dalloc(&h->sell_val64, (size_t)h->sell_entries);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(mixed ? (void *)h->sell_val32 : (void *)h->sell_val64, 0,
+                                (size_t)h->sell_entries * (mixed ? 4 : 8), s);
+        if (e == cudaSuccess)
+            e = launch_scatter_values(h->val_o, h->nnz, nullptr, h->sell_slot, nullptr, nullptr, nullptr, nullptr,
+                                      mixed ? nullptr : h->sell_val64, mixed ? h->sell_val32 : nullptr, s);
+        if (e != cudaSuccess) return without(e);
+    }
+    if (!h->weight) CK(h, cudaMalloc(&h->weight, (size_t)h->n * sizeof(double)));
+    return AMGD_OK;
+}
+
+// What a sweep launch needs before it is queued or captured: the sliced copy,
+// or current CSR values for the kernels that read those.  `bytes`: vector bytes
+// the caller's sweeps gather.  Building the copy costs some 200 us and a pass
+// over the matrix, a sweep saves about a quarter of its time: it is built once a
+// handle's sweeps have gathered 2 GB, or when they are called a second time
+// (128 x 128 7-point, K = 8, FP64, one call of 4 sweeps: 30 us of sweeps).
+int prepare_sweeps(amgd_ctx *h, size_t bytes, cudaStream_t s)
+{
+    constexpr size_t kWorth = (size_t)2 << 30;
+    const int stage = h->relax_shape[h->storage].stage;
+    const bool repeated = h->sweep_calls > 0 || bytes >= kWorth;
+    ++h->sweep_calls;
+    if ((stage == 0 || stage == 3) && (repeated || h->sell_ok)) {
+        const int rc = ensure_sell(h);
+        if (rc != AMGD_OK) return rc;
+    }
+    if (!sweeps_use_csr(h)) return AMGD_OK;
+    return h->storage == ST_FP64 ? refresh_perm64(h, s) : refresh_perm32(h, s);
+}
+// of a captured graph or a tuned handle, whose sweeps repeat
+int prepare_sweeps(amgd_ctx *h, cudaStream_t s) { return prepare_sweeps(h, ~(size_t)0, s); }
+// vector bytes that nu sweeps gather
+size_t sweep_bytes(const amgd_ctx *h, int32_t nu)
+{
+    return (size_t)h->nnz * Kp_of(h->storage, h->K) * esize(h->storage) * (size_t)nu;
+}
+
+// the arguments shared by every sweep of the handle
+RelaxArgs sweep_args(amgd_ctx *h, double omega)
+{
+    const bool f64 = h->storage == ST_FP64;
+    RelaxArgs a;
+    a.status = h->status;
+    a.wait_limit = h->wait_limit;
+    a.extra_tx = h->test_extra_tx;
+    a.rp = h->rp_p;
+    a.col = h->col_p;
+    a.val = f64 ? (const void *)h->val64 : (const void *)(h->perm ? h->val32 : h->val32_o);
+    a.diag = f64 ? (const void *)h->diag64 : (const void *)h->diag32;
+    a.Kp = Kp_of(h->storage, h->K);
+    a.omega = omega;
+    a.avg_nnz = h->n ? (float)((double)h->nnz / (double)h->n) : 0.f;
+    a.nrows = (int32_t)h->n;
+    if (h->sell_ok) {
+        a.sell_ptr = h->sell_ptr;
+        a.sell_col = h->sell_col;
+        a.sell_val = f64 ? (const void *)h->sell_val64 : (const void *)h->sell_val32;
+        a.rowmap = h->sell_map;
+        a.weight = h->weight;
+        a.sell_width = (int32_t)((h->sell_entries + 32 * h->color_slice.back() - 1) / (32 * h->color_slice.back()));
+    }
+    return a;
 }
 
 int run_init(amgd_ctx *h, uint64_t seed, cudaStream_t s)
@@ -387,22 +572,9 @@ int run_init(amgd_ctx *h, uint64_t seed, cudaStream_t s)
 int run_relax(amgd_ctx *h, int32_t nu, double omega, int sweep, cudaStream_t s)
 {
     const Shape sh = h->relax_shape[h->storage];
-    if (h->storage == ST_FP64 && nu > 0) {
-        const int rc = refresh_perm64(h, s);
-        if (rc != AMGD_OK) return rc;
-    }
-    RelaxArgs a;
-    a.status = h->status;
-    a.wait_limit = h->wait_limit;
-    a.extra_tx = h->test_extra_tx;
-    a.rp = h->rp_p;
-    a.col = h->col_p;
-    a.val = h->storage == ST_FP64 ? (const void *)h->val64 : (const void *)h->val32;
-    a.diag = h->storage == ST_FP64 ? (const void *)h->diag64 : (const void *)h->diag32;
-    a.Kp = Kp_of(h->storage, h->K);
-    a.omega = omega;
-    a.avg_nnz = h->n ? (float)((double)h->nnz / (double)h->n) : 0.f;
-    a.nrows = (int32_t)h->n;
+    RelaxArgs a = sweep_args(h, omega);
+    const bool sliced = !sweeps_use_csr(h);
+    if (sliced && nu > 0) CK(h, launch_weights(h->storage, a.diag, omega, h->weight, (int32_t)h->n, s));
     for (int32_t it = 0; it < nu; ++it) {
         a.xold = h->x[h->cur];
         a.xnew = h->x[1 - h->cur];
@@ -416,6 +588,7 @@ int run_relax(amgd_ctx *h, int32_t nu, double omega, int sweep, cudaStream_t s)
                 a.r0 = (int32_t)h->color_start[c];
                 a.r1 = (int32_t)h->color_start[c + 1];
                 a.split = a.r0;
+                if (sliced) a.slice0 = h->color_slice.empty() ? 0 : h->color_slice[c];
                 CK(h, launch_relax(h->storage, sh, a, s));
             }
         }
@@ -439,25 +612,11 @@ cudaError_t ensure_buf(void **p, size_t &have, size_t bytes)
 }
 
 // One Jacobi sweep X_dst = X_src - omega D^{-1} A X_src with the handle's
-// relaxation shape (bit-identical to the sweeps of run_relax).
+// relaxation shape (bit-identical to the sweeps of run_relax); the caller has
+// queued the weights (launch_weights) for omega.
 int jacobi_step(amgd_ctx *h, const void *src, void *dst, double omega, cudaStream_t s)
 {
-    if (h->storage == ST_FP64) {
-        const int rc = refresh_perm64(h, s);
-        if (rc != AMGD_OK) return rc;
-    }
-    RelaxArgs a;
-    a.status = h->status;
-    a.wait_limit = h->wait_limit;
-    a.extra_tx = h->test_extra_tx;
-    a.rp = h->rp_p;
-    a.col = h->col_p;
-    a.val = h->storage == ST_FP64 ? (const void *)h->val64 : (const void *)h->val32;
-    a.diag = h->storage == ST_FP64 ? (const void *)h->diag64 : (const void *)h->diag32;
-    a.Kp = Kp_of(h->storage, h->K);
-    a.omega = omega;
-    a.avg_nnz = h->n ? (float)((double)h->nnz / (double)h->n) : 0.f;
-    a.nrows = (int32_t)h->n;
+    RelaxArgs a = sweep_args(h, omega);
     a.xold = src;
     a.xnew = dst;
     a.r0 = 0;
@@ -485,6 +644,8 @@ int run_relax_recorded(amgd_ctx *h, int32_t nu, double omega, cudaStream_t s)
         return h->x[(c0 + m) & 1];
     };
     if (nck > 0) CK(h, cudaMemcpyAsync(h->ckpt, h->x[c0], xb, cudaMemcpyDeviceToDevice, s));
+    if (nu > 0 && !sweeps_use_csr(h))
+        CK(h, launch_weights(h->storage, sweep_args(h, omega).diag, omega, h->weight, (int32_t)h->n, s));
     for (int32_t k = 0; k < nu; ++k) {
         const int rc = jacobi_step(h, loc(k), loc(k + 1), omega, s);
         if (rc != AMGD_OK) return rc;
@@ -763,12 +924,10 @@ int amgd_set_precision(amgd_handle h, int storage)
     if (storage == h->storage) return AMGD_OK;
     CK(h, cudaStreamSynchronize(h->stream));
     drop_graph(h);                       // vector and output buffers are reallocated
-    if (storage != ST_FP64 && !h->val32) {
-        CK(h, dalloc(&h->val32, (size_t)h->nnz + 4));
+    if (storage != ST_FP64 && !h->val32_o) {
         CK(h, dalloc(&h->val32_o, (size_t)h->nnz + 4));
-        int rc = permute_values(h);
-        if (rc != AMGD_OK) return rc;
     }
+    if (storage != ST_FP64 && h->perm && !h->val32) CK(h, dalloc(&h->val32, (size_t)h->nnz + 4));
     // re-layout the current vectors: export to caller-order doubles, import
     CK(h, ensure_tmp64(h, (size_t)h->n * h->K));
     CK(h, launch_export(h->storage, h->x[h->cur], h->tmp64, h->perm, (int32_t)h->n, h->K,
@@ -798,6 +957,14 @@ int amgd_set_precision(amgd_handle h, int storage)
     h->cur = 0;
     h->storage = storage;
     if (slot_type_changes) {
+        // the value copies of the new arithmetic type (the sliced one is remade
+        // when a sweep next runs)
+        dfree(h->sell_val64);
+        dfree(h->sell_val32);
+        h->sell_val64 = nullptr;
+        h->sell_val32 = nullptr;
+        rc = permute_values(h);
+        if (rc != AMGD_OK) return rc;
         rc = alloc_slot_outputs(h, storage);
         if (rc != AMGD_OK) return rc;
     }
@@ -891,6 +1058,7 @@ int amgd_set_coloring(amgd_handle h, const int32_t *color, int32_t ncolors, int 
         CK(h, dalloc(&h->col_p, (size_t)h->nnz + 4));
         CK(h, dalloc(&h->val64, (size_t)h->nnz + 4));
     }
+    if (h->val32_o && !h->val32) CK(h, dalloc(&h->val32, (size_t)h->nnz + 4));
     if (!h->x_caller) {
         const size_t bytes = (size_t)n * Kp_of(h->storage, h->K) * esize(h->storage);
         CK(h, cudaMalloc(&h->x_caller, bytes ? bytes : 16));
@@ -919,6 +1087,7 @@ int amgd_set_coloring(amgd_handle h, const int32_t *color, int32_t ncolors, int 
         if (h->nnz)
             CK(h, cudaMemcpy(h->slot_perm, sp.data(), h->nnz * sizeof(int32_t), cudaMemcpyHostToDevice));
     }
+    drop_sell(h);                        // of the former row order
     int rc = permute_values(h);
     if (rc != AMGD_OK) return rc;
     CK(h, launch_import(h->storage, h->tmp64, h->x[h->cur], h->perm, (int32_t)n, h->K,
@@ -1155,6 +1324,10 @@ int amgd_relax(amgd_handle h, int32_t nu, double omega, int sweep_type)
         return fail(h, AMGD_ERR_ARG, "unknown sweep type");
     if (sweep_type == AMGD_SWEEP_MCGS && !h->perm)
         return fail(h, AMGD_ERR_STATE, "MCGS needs amgd_set_coloring first");
+    if (nu > 0) {
+        const int rc = prepare_sweeps(h, sweep_bytes(h, nu), h->stream);
+        if (rc != AMGD_OK) return rc;
+    }
     if (h->ckpt_every > 0 && sweep_type == AMGD_SWEEP_JACOBI && !h->perm)
         return run_relax_recorded(h, nu, omega, h->stream);
     return run_relax(h, nu, omega, sweep_type, h->stream);
@@ -1240,6 +1413,11 @@ int amgd_graph_capture(amgd_handle h, uint64_t seed, int32_t nu, double omega, i
     if (!h->cap_stream) CK(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
     if (h->graph) { cudaGraphDestroy(h->graph); h->graph = nullptr; }
+    {
+        const int rc = prepare_sweeps(h, h->stream);
+        if (rc != AMGD_OK) return rc;
+    }
+    h->graph_csr = sweeps_use_csr(h);
     CK(h, cudaStreamSynchronize(h->stream));
     const int cur0 = h->cur;
     h->cur = 0;
@@ -1412,6 +1590,10 @@ int amgd_autotune(amgd_handle h, int sweep_type, double omega, const char *cache
     for (const Shape &c : cands) {
         float ms = 0.f;
         h->relax_shape[h->storage] = c;
+        {
+            const int prc = prepare_sweeps(h, h->stream);
+            if (prc != AMGD_OK) { h->relax_shape[h->storage] = keep_r; return prc; }
+        }
         // one sweep from the current vectors into the spare buffer (the
         // current vectors are not touched), then restore the buffer index
         int rc = time_ms(h, [&]() { int q = run_relax(h, 1, omega, sweep_type, h->stream); h->cur = cur; return q; }, 5, ms);
@@ -1888,6 +2070,7 @@ int prepare_backward(amgd_ctx *h)
     const int32_t S = h->ckpt_every > 0 ? h->ckpt_every : 1;
     int rc = ensure_transpose(h);
     if (rc != AMGD_OK) return rc;
+    if ((rc = prepare_sweeps(h, h->stream)) != AMGD_OK) return rc;
     CK(h, ensure_buf(&h->adj_vec, h->adj_vec_bytes, 4 * nk * cs));
     CK(h, ensure_buf(&h->adj_slot, h->adj_slot_bytes, 6 * (size_t)(h->nnz ? h->nnz : 1) * cs));
     CK(h, ensure_buf(&h->seg, h->seg_bytes, (size_t)(S - 1) * xb));
@@ -1966,6 +2149,8 @@ int run_backward(amgd_ctx *h, const double *lsb_in, double *vb, cudaStream_t s)
 
     // sweeps, last to first, one checkpoint segment at a time: the iterates
     // between two checkpoints are recomputed by the forward kernel
+    if (nu > 0 && !sweeps_use_csr(h))
+        CK(h, launch_weights(st, sweep_args(h, h->traj_omega).diag, h->traj_omega, h->weight, n, s));
     int xc = 0;
     const int32_t nseg = (nu + S - 1) / S;
     for (int32_t c = nseg - 1; c >= 0; --c) {
@@ -2079,6 +2264,11 @@ int amgd_graph_capture_backward(amgd_handle h, uint64_t seed, int32_t nu, double
     if (!h->cap_stream) CK(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
     if (h->graph) { cudaGraphDestroy(h->graph); h->graph = nullptr; }
+    {
+        const int rc = prepare_sweeps(h, h->stream);
+        if (rc != AMGD_OK) return rc;
+    }
+    h->graph_csr = sweeps_use_csr(h);
     CK(h, cudaStreamSynchronize(h->stream));
     const int cur0 = h->cur;
     h->cur = 0;
@@ -2149,6 +2339,8 @@ int amgd_destroy(amgd_handle h)
         dfree(h->pinv);
         dfree(h->colx);
     }
+    drop_sell(h);
+    dfree(h->weight);
     dfree(h->mat_id);
     if (h->depth > 1) {
         dfree(h->prp);

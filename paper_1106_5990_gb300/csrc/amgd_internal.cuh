@@ -275,6 +275,15 @@ struct RelaxArgs {
     double omega;
     float avg_nnz = 0.f;  // stored entries per row of the whole matrix
     int32_t nrows = 0;    // rows of the vector block (the range of a gather index)
+    // sliced copy of the permuted matrix (NULL: none): slice q holds 32 rows of one
+    // color, entry k of its row l at sell_ptr[q] + 32 k + l, column -1 past the row's end
+    const int64_t *sell_ptr = nullptr;
+    const int32_t *sell_col = nullptr;
+    const void *sell_val = nullptr;       // same type as val
+    const int32_t *rowmap = nullptr;      // row of (q, l) at 32 q + l, -1: none (NULL: in order)
+    int32_t sell_width = 0;               // entries of an average row of the sliced copy, padding included
+    int64_t slice0 = 0;                   // first slice of this color phase
+    const void *weight = nullptr;         // omega / a_ii per row
 };
 
 struct EdgeArgs {                // everything in the caller's numbering
@@ -320,6 +329,29 @@ struct InitArgs {
 cudaError_t launch_relax(int storage, Shape sh, const RelaxArgs &a, cudaStream_t s);
 // false for a staged shape whose shared memory exceeds the per-block limit
 bool relax_shape_available(int storage, Shape sh);
+// w[r] = omega / diag[r] in the arithmetic type
+cudaError_t launch_weights(int storage, const void *diag, double omega, void *w, int32_t n, cudaStream_t s);
+
+// sliced copy of the row-permuted matrix (k_sell.cu)
+constexpr int kSellRows = 32;           // rows of a slice
+constexpr int kSellWindow = 512;        // rows sorted by length together
+struct SellArgs {
+    const int32_t *rp, *col;            // row-permuted CSR
+    const int32_t *rp_o, *perm;         // caller row pointers; caller row of a permuted row (NULL: itself)
+    const int64_t *color_row, *color_slice;   // ncolors + 1 first rows / slices of the colors (device)
+    int32_t ncolors;
+    int64_t nslices;
+    int32_t n;
+};
+// rowmap (sorted by length inside windows of kSellWindow rows; ties in row order)
+cudaError_t launch_sell_sort(const SellArgs &a, int32_t *rowmap, cudaStream_t s);
+// entries of every slice (rowmap NULL: rows in order), width[nslices], and their sum
+cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t *width, unsigned long long *total,
+                              cudaStream_t s);
+// columns (-1: padding) and the position of every caller slot
+cudaError_t launch_sell_fill(const SellArgs &a, const int32_t *rowmap, const int64_t *ptr, int32_t *sell_col,
+                             int32_t *slot, cudaStream_t s);
+
 // in_place: read the vectors in the sweeps' row order (search depth 1)
 cudaError_t launch_edge(int storage, bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s);
@@ -348,11 +380,12 @@ cudaError_t launch_permute_values(const double *v, const int32_t *rp_orig,
                                   float *vp32, int32_t n, cudaStream_t s);
 
 // one coalesced pass over caller-order values src[nnz] into the caller FP64 /
-// FP32 copies and the row-permuted FP64 / FP32 copies (NULL targets skipped;
-// slot_perm NULL = identity); err (NULL: none) |= 1 for a non-finite value
-cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *slot_perm,
-                                  double *val_o, float *val32_o, double *vp64, float *vp32,
-                                  cudaStream_t s, uint32_t *err = nullptr);
+// FP32 copies, the row-permuted FP64 / FP32 copies (at slot_perm, NULL =
+// identity) and the sweeps' sliced copy (at slot_sell); NULL targets skipped;
+// err (NULL: none) |= 1 for a non-finite value
+cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *slot_perm, const int32_t *slot_sell,
+                                  double *val_o, float *val32_o, double *vp64, float *vp32, double *vs64,
+                                  float *vs32, cudaStream_t s, uint32_t *err = nullptr);
 // diagonals (diag_slot = caller slot of each row's diagonal) in caller order
 // and in permuted order (NULL targets skipped); err (NULL: none) |= 2 for a
 // zero diagonal

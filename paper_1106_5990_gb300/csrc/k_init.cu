@@ -272,13 +272,15 @@ __global__ void k_check_values(const double *__restrict__ v, int64_t nnz,
 }
 
 // one pass over the stored values in caller order (coalesced): the FP64
-// caller copy, the FP32 caller copy and the row-permuted FP64 / FP32 copies
-// (slot_perm[p] = permuted slot of caller slot p); NULL targets are skipped.
-// err (NULL: no check): bit 0 set when a value is not finite.
+// caller copy, the FP32 caller copy, the row-permuted FP64 / FP32 copies
+// (slot_perm[p] = permuted slot of caller slot p) and the sliced copy
+// (slot_sell[p] = its position); NULL targets are skipped.  err (NULL: no
+// check): bit 0 set when a value is not finite.
 __global__ void k_scatter_values(const double *__restrict__ src, int64_t nnz,
-                                 const int32_t *__restrict__ slot_perm, double *__restrict__ val_o,
-                                 float *__restrict__ val32_o, double *__restrict__ vp64,
-                                 float *__restrict__ vp32, uint32_t *__restrict__ err)
+                                 const int32_t *__restrict__ slot_perm, const int32_t *__restrict__ slot_sell,
+                                 double *__restrict__ val_o, float *__restrict__ val32_o, double *__restrict__ vp64,
+                                 float *__restrict__ vp32, double *__restrict__ vs64, float *__restrict__ vs32,
+                                 uint32_t *__restrict__ err)
 {
     bool bad = false;
     for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < nnz;
@@ -288,9 +290,16 @@ __global__ void k_scatter_values(const double *__restrict__ src, int64_t nnz,
         const float f = (float)x;
         if (val_o) val_o[p] = x;
         if (val32_o) val32_o[p] = f;
-        const int64_t q = slot_perm ? slot_perm[p] : p;
-        if (vp64) vp64[q] = x;
-        if (vp32) vp32[q] = f;
+        if (vp64 || vp32) {
+            const int64_t q = slot_perm ? slot_perm[p] : p;
+            if (vp64) vp64[q] = x;
+            if (vp32) vp32[q] = f;
+        }
+        if (vs64 || vs32) {
+            const int64_t q = slot_sell[p];
+            if (vs64) vs64[q] = x;
+            if (vs32) vs32[q] = f;
+        }
     }
     if (err && __any_sync(0xffffffffu, bad) && (threadIdx.x % 32) == 0) atomicOr(err, 1u);
 }
@@ -460,14 +469,14 @@ cudaError_t launch_check_values(const double *v, int64_t nnz, const int32_t *dia
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *slot_perm,
-                                  double *val_o, float *val32_o, double *vp64, float *vp32,
-                                  cudaStream_t s, uint32_t *err)
+cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *slot_perm, const int32_t *slot_sell,
+                                  double *val_o, float *val32_o, double *vp64, float *vp32, double *vs64,
+                                  float *vs32, cudaStream_t s, uint32_t *err)
 {
     if (nnz == 0) return cudaSuccess;
     const int64_t want = (nnz + kThreads - 1) / kThreads;
     k_scatter_values<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), kThreads, 0, s>>>(
-        src, nnz, slot_perm, val_o, val32_o, vp64, vp32, err);
+        src, nnz, slot_perm, slot_sell, val_o, val32_o, vp64, vp32, vs64, vs32, err);
     return cudaGetLastError();
 }
 

@@ -472,177 +472,206 @@ k_relax_pipe(RelaxArgs A, int64_t chunk)
     cp_async_wait<0>();
 }
 
-// Chunked persistent variant (stage 3).  One block of kChunkThreads threads
-// per SM owns one contiguous chunk of rows; its warps walk the chunk side by
-// side in groups of RW = 32/G rows (group g of the chunk goes to warp g mod W),
-// so the whole SM moves through consecutive rows together.  On matrices whose
-// neighbours are close in the row order (stencils on grid lines, banded and
-// mesh orderings) the rows an SM gathers are then the few grid lines around
-// its current position, and a line fetched into L1 for one row serves the
-// rows of the next lines too: the L2 -> L1 traffic of the gathers drops from
-// one copy of each vector row per block that touches it towards one per SM.
-// Each warp also asks the L2 for the row-pointer line of its group after next
-// and for the column-index and value lines of its next group (their bounds
-// come from the row pointers prefetched one group earlier), so a row's first
-// two dependent round trips hit L2.  L2 policy: the test-vector block (read
-// by the gathers, written by the update) is loaded and stored with an
-// evict-last hint and the CSR, which streams through once per sweep, with an
-// evict-first hint, so the vectors of the next color phase and sweep tend to
-// stay in the 129 MB L2 instead of being pushed out by the matrix.  Same row
-// sums in the same order as k_relax: same bits.  896 threads (28 warps): the
-// register budget of 72 per thread holds a batch of four 64-byte rows per lane
-// pair without spilling (at 1024 threads, 64 registers spilled and the sweep
-// was 10% slower; 768 threads were 4% slower, and at 640 the direct kernel
-// wins).
-constexpr int kChunkThreads = 896;
+// ---------------------------------------------------------------------------
+// Sweep over the sliced copy of A (stages 0 and 3).  A slice is 32 consecutive
+// rows of one color phase; entry k of the slice's row l lies at
+// ptr[slice] + 32 k + l (column -1 where the row is shorter), so the lanes of a
+// warp read column indices and values of consecutive rows as one line and
+// without row pointers.  MAP: the slice's rows are rowmap[32 slice + l] (rows
+// sorted by length inside windows, where that saves padding); -1: none.
+//
+// G lanes per row, each with accesses of 32 bytes side by side with its
+// neighbours' (NV pieces; one 16-byte piece for the shortest rows).  U entries are
+// gathered at a time, and while they are in flight the columns and values of the
+// next batch -- of the warp's next group of rows after the last -- are loaded from
+// the L2, which was asked for them a group earlier: a warp waits once per batch.
+// A block owns `chunk` consecutive groups of 32 / G rows and its warps walk them
+// side by side, so that the rows an SM gathers are the few grid lines around its
+// position.  Same row sums in the same order as a sequential evaluation: same bits.
+//
+// Bound: latency of the gathers and instruction issue on the mixed paths (at one
+// block per SM, 20 warps), the FP64 pipe on FP64.  Eight sweeps, us, before (CSR
+// kernels, untuned / best shape) -> now: 9-point 1024^2 K = 16 FP32 704 / 521 ->
+// 521; 128^3 7-point K = 32 FP32 2012 / 1541 -> 1585; 600k-row graph BF16 538 / 524
+// -> 430; 9-point 700^2 FP64 1657 / 1329 -> 1155; 64^2 5-point K = 8 FP64 49 -> 24.
+// Slices on their own gain little: without the look-ahead the first took 614, with
+// evict-last hints on the vectors 650, with 4 entries instead of 5 at a time 571.
+// ---------------------------------------------------------------------------
+template <class TS, int P>
+struct SellShape {
+    // 32 bytes per lane for rows up to 64 bytes, 64 bytes per lane beyond (fewer
+    // lanes that all read the row's indices)
+    static constexpr int NV = P >= 8 ? 4 : (P >= 2 ? 2 : 1), G = P / NV;
+    static constexpr int UMAX = NV == 4 ? 4 : 5;                        // most entries gathered at a time
+    static constexpr int THREADS = NV == 4 ? 512 : 640;                 // one block per SM
+};
 
 __device__ __forceinline__ void prefetch_l2(const void *p)
 {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
-__device__ __forceinline__ uint64_t policy_evict_last()
+__device__ __forceinline__ void st32(void *p, const uint4 &a, const uint4 &b)
 {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ uint64_t policy_evict_first()
-{
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ uint4 ldg16_hint(const void *p, uint64_t pol)
-{
-    uint4 v;
-    asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p), "l"(pol));
-    return v;
-}
-__device__ __forceinline__ void st16_hint(void *p, const uint4 &v, uint64_t pol)
-{
-    asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(p), "r"(v.x),
-                 "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
+    asm volatile("st.global.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
+                 "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
                  : "memory");
 }
-// 32-byte vector load / store (sm_100 and later; the address is 32-byte aligned)
-__device__ __forceinline__ void ldg32_hint(const void *p, uint64_t pol, uint4 &a, uint4 &b)
-{
-    asm volatile("ld.global.nc.L2::cache_hint.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
-                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                 : "l"(p), "l"(pol));
-}
-__device__ __forceinline__ void st32_hint(void *p, const uint4 &a, const uint4 &b, uint64_t pol)
-{
-    asm volatile("st.global.L2::cache_hint.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;" ::"l"(p),
-                 "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "l"(pol)
-                 : "memory");
-}
-__device__ __forceinline__ int32_t ld32_hint(const int32_t *p, uint64_t pol)
+// entry K of a slice's row: column index (a pattern array: read-only path) and
+// value (written by other kernels); the offset is an immediate
+template <int K>
+__device__ __forceinline__ int32_t ld_col(const int32_t *p)
 {
     int32_t v;
-    asm volatile("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    asm volatile("ld.global.nc.L1::no_allocate.b32 %0, [%1+%2];" : "=r"(v) : "l"(p), "n"(K * 32 * 4));
     return v;
 }
-__device__ __forceinline__ float ldv_hint(const float *p, uint64_t pol)
+template <int K>
+__device__ __forceinline__ float ld_val(const float *p)
 {
     float v;
-    asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    asm volatile("ld.global.L1::no_allocate.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(K * 32 * 4));
     return v;
 }
-__device__ __forceinline__ double ldv_hint(const double *p, uint64_t pol)
+template <int K>
+__device__ __forceinline__ double ld_val(const double *p)
 {
     double v;
-    asm volatile("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
+    asm volatile("ld.global.L1::no_allocate.f64 %0, [%1+%2];" : "=d"(v) : "l"(p), "n"(K * 32 * 8));
     return v;
 }
+// the first `left` of U columns (-1 past them) and values
+template <int U, int K = 0>
+__device__ __forceinline__ void ld_cols(const int32_t *pc, int left, int (&jj)[U])
+{
+    if constexpr (K < U) {
+        jj[K] = -1;
+        if (K < left) jj[K] = ld_col<K>(pc);
+        ld_cols<U, K + 1>(pc, left, jj);
+    }
+}
+template <int U, class AV, class C, int K = 0>
+__device__ __forceinline__ void ld_vals(const AV *pv, int left, C (&vv)[U])
+{
+    if constexpr (K < U) {
+        vv[K] = C(0);
+        if (K < left) vv[K] = (C)ld_val<K>(pv);
+        ld_vals<U, AV, C, K + 1>(pv, left, vv);
+    }
+}
 
-template <class TS, int G, int NV, int U, bool SPLIT>
-__global__ void __launch_bounds__(kChunkThreads, 1) k_relax_chunk(RelaxArgs A, int32_t chunk)
+template <class TS, int P, int U, bool SPLIT, bool MAP>
+__global__ void __launch_bounds__(SellShape<TS, P>::THREADS, 1) k_relax_sell(RelaxArgs A, int32_t chunk)
 {
     using S = Store<TS>;
     using C = typename S::C;
     using AV = typename S::A;
-    constexpr int V = S::V, RW = 32 / G, NW = kChunkThreads / 32;
-    constexpr int64_t STEP = (int64_t)NW * RW;            // rows between a warp's groups
-    const int warp = threadIdx.x / 32, lane32 = threadIdx.x % 32;
-    const int lane = lane32 % G, rig = lane32 / G;
-    const TS *xold = (const TS *)A.xold;
-    TS *xnew = (TS *)A.xnew;
-    const AV *val = (const AV *)A.val;
-    const int32_t *col = A.col;
-    const int Kp = A.Kp;
-    const int64_t c0 = (int64_t)A.r0 + (int64_t)blockIdx.x * chunk;
-    const int64_t c1 = min((int64_t)A.r1, c0 + chunk);
-    const uint64_t keep = policy_evict_last(), stream = policy_evict_first();
-    // a lane holding an even number of pieces holds them side by side and moves
-    // them two at a time (32-byte accesses: half the load instructions and
-    // cache wavefronts of a gather); otherwise the pieces interleave over the
-    // G lanes.  Every component keeps its own FMA chain, so both layouts give
-    // the same bits.
-    constexpr bool W32 = NV % 2 == 0;
-    auto piece = [&](int tt) { return W32 ? lane * NV + tt : tt * G + lane; };
+    using L = SellShape<TS, P>;
+    constexpr int V = S::V, G = L::G, NV = L::NV, RW = 32 / G, KP = P * V, PER = 32 / RW;
+    constexpr int PV = NV >= 2 ? 2 * V : V;              // components of one access
+    const int lane32 = threadIdx.x % 32, lane = lane32 % G, rig = lane32 / G;
+    const TS *xold = (const TS *)A.xold + lane * PV;
+    TS *xnew = (TS *)A.xnew + lane * PV;
+    const int split = A.split;
+    // row groups of this warp: [g, gend) in steps of the block's warps
+    const int ngroups = (A.r1 - A.r0 + RW - 1) / RW, step = blockDim.x / 32;
+    const int gend = min(ngroups, ((int)blockIdx.x + 1) * chunk);
+    int g = blockIdx.x * chunk + threadIdx.x / 32;
+    if (g >= gend) {
+        chain_wait();
+        return;
+    }
+    const int64_t *ptr = A.sell_ptr + A.slice0;
+    // first entry of a group's rows in their slice, and the slice's width
+    auto slice_of = [&](int grp, int64_t &base, int &w) {
+        const int64_t b0 = __ldg(ptr + grp / PER);
+        w = (int)(__ldg(ptr + grp / PER + 1) - b0) / 32;
+        base = b0 + (grp % PER) * RW;
+    };
+    int64_t base, nbase = 0;
+    int w, nw = 0;
+    slice_of(g, base, w);
+    const int32_t *pc = A.sell_col + base + rig;
+    const AV *pv = (const AV *)A.sell_val + base + rig;
+    int jj[U];
+    C vv[U];
+    ld_cols<U>(pc, w, jj);
+    chain_wait();
+    chain_release();
+    ld_vals<U, AV, C>(pv, w, vv);
+    if (g + step < gend) slice_of(g + step, nbase, nw);
 
-    for (int64_t wr0 = c0 + (int64_t)warp * RW; wr0 < c1; wr0 += STEP) {
-        // row pointers of this warp's group after next, into L2
-        if (lane32 == 0 && wr0 + 2 * STEP < c1) prefetch_l2(A.rp + wr0 + 2 * STEP);
-        // bounds of this warp's next group (its row pointers were prefetched)
-        int n0 = 0, n1 = 0;
-        if (wr0 + STEP < c1) {
-            n0 = ld32_hint(A.rp + wr0 + STEP, stream);
-            n1 = ld32_hint(A.rp + min(wr0 + STEP + RW, c1), stream);
+    for (; g < gend; g += step) {
+        int r = A.r0 + g * RW + rig;
+        if constexpr (MAP) r = __ldg(A.rowmap + (A.slice0 * 32 + g * RW + rig));
+        const bool live = MAP ? r >= 0 : r < A.r1;
+        int64_t fbase = 0;
+        int fw = 0;
+        if (g + 2 * step < gend) {
+            // the group after next: its lines into L2
+            slice_of(g + 2 * step, fbase, fw);
+            for (int q = lane32; q < fw; q += 32) {
+                prefetch_l2(A.sell_col + fbase + 32 * q);
+                prefetch_l2((const AV *)A.sell_val + fbase + 32 * q);
+                if constexpr (sizeof(AV) == 8) prefetch_l2((const AV *)A.sell_val + fbase + 32 * q + 16);
+            }
         }
-        const int64_t r = wr0 + rig;
-        if (r < c1) {
-            const int p0 = ld32_hint(A.rp + r, stream), p1 = ld32_hint(A.rp + r + 1, stream);
-            Acc<C, V> acc[NV];
+        Acc<C, V> acc[NV];
 #pragma unroll
-            for (int tt = 0; tt < NV; ++tt) acc[tt].zero();
-            for (int pb = p0; pb < p1; pb += U) {
-                int jj[U];
-                C vv[U];
+        for (int t = 0; t < NV; ++t) acc[t].zero();
+        for (int left = w; left > 0; left -= U) {
+            uint4 raw[U][NV];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const bool ok = pb + u < p1;
-                    jj[u] = ok ? ld32_hint(col + pb + u, stream) : -1;
-                    vv[u] = ok ? (C)ldv_hint(val + pb + u, stream) : C(0);
-                }
-                uint4 raw[U][NV];
+            for (int u = 0; u < U; ++u) {
+                if (jj[u] < 0) continue;
+                const TS *src = (SPLIT && jj[u] < split ? (const TS *)xnew : xold) +
+                                checked_row(jj[u], A.nrows, A.status) * KP;
+                if constexpr (NV >= 2) {
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (jj[u] >= 0) {
-                        const TS *src = (SPLIT && jj[u] < A.split ? (const TS *)xnew : xold) +
-                                        checked_row(jj[u], A.nrows, A.status) * Kp;
-                        if constexpr (W32) {
-#pragma unroll
-                            for (int tt = 0; tt < NV; tt += 2)
-                                ldg32_hint(src + piece(tt) * V, keep, raw[u][tt], raw[u][tt + 1]);
-                        } else {
-#pragma unroll
-                            for (int tt = 0; tt < NV; ++tt) raw[u][tt] = ldg16_hint(src + piece(tt) * V, keep);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (jj[u] < 0) break;
-#pragma unroll
-                    for (int tt = 0; tt < NV; ++tt) {
-                        C x[V];
-                        S::unpack(raw[u][tt], x);
-                        acc[tt].fma_piece(vv[u], x);
-                    }
+                    for (int t = 0; t < NV; t += 2) ld32(src + t / 2 * G * PV, raw[u][t], raw[u][t + 1]);
+                } else {
+                    raw[u][0] = ld16(src);
                 }
             }
-            const C c = (C)A.omega / ldv_hint((const AV *)A.diag + r, stream);
-            // x_i - (omega / a_ii) s_i, a pair of pieces (W32) or one piece at a time
-            constexpr int PW = W32 ? 2 : 1;
+            // the next batch's columns and values, of the next group after the last
+            int jn[U];
+            C vn[U];
+            int nleft = left - U;
+            if (nleft > 0) {
+                pc += 32 * U;
+                pv += 32 * U;
+            } else {
+                pc = A.sell_col + nbase + rig;
+                pv = (const AV *)A.sell_val + nbase + rig;
+                nleft = nw;
+            }
+            ld_cols<U>(pc, nleft, jn);
+            ld_vals<U, AV, C>(pv, nleft, vn);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (jj[u] < 0) continue;
+#pragma unroll
+                for (int t = 0; t < NV; ++t) {
+                    C x[V];
+                    S::unpack(raw[u][t], x);
+                    acc[t].fma_piece(vv[u], x);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                jj[u] = jn[u];
+                vv[u] = vn[u];
+            }
+        }
+        if (live) {
+            // the row itself (never of an earlier color), weighted
+            const C c = ld_plain((const C *)A.weight + r);
+            constexpr int PW = NV >= 2 ? 2 : 1;
 #pragma unroll
             for (int t0 = 0; t0 < NV; t0 += PW) {
+                const int64_t o = (int64_t)r * KP + t0 / 2 * G * PV;
                 uint4 own[PW];
-                if constexpr (W32) ldg32_hint(xold + r * Kp + piece(t0) * V, keep, own[0], own[1]);
-                else own[0] = ldg16_hint(xold + r * Kp + piece(t0) * V, keep);
+                if constexpr (NV >= 2) ld32(xold + o, own[0], own[1]);
+                else own[0] = ld16(xold + o);
 #pragma unroll
                 for (int h = 0; h < PW; ++h) {
                     C xi[V], out[V];
@@ -651,50 +680,85 @@ __global__ void __launch_bounds__(kChunkThreads, 1) k_relax_chunk(RelaxArgs A, i
                     for (int e = 0; e < V; ++e) out[e] = fma(-c, acc[t0 + h].get(e), xi[e]);
                     own[h] = S::pack(out);
                 }
-                if constexpr (W32) st32_hint(xnew + r * Kp + piece(t0) * V, own[0], own[1], keep);
-                else st16_hint(xnew + r * Kp + piece(t0) * V, own[0], keep);
+                if constexpr (NV >= 2) st32(xnew + o, own[0], own[1]);
+                else *reinterpret_cast<uint4 *>(xnew + o) = own[0];
             }
         }
-        // column-index and value lines of this warp's next group, into L2
-        if (n1 > n0) {
-            const int64_t q0 = n0 & ~31, nq = ((int64_t)n1 - q0 + 31) / 32;     // 128-byte lines
-            for (int64_t q = lane32; q < nq; q += 32) prefetch_l2(col + q0 + 32 * q);
-            constexpr int EPL = 128 / (int)sizeof(AV);                          // values per line
-            const int64_t v0 = n0 & ~(int64_t)(EPL - 1), nv = ((int64_t)n1 - v0 + EPL - 1) / EPL;
-            for (int64_t q = lane32; q < nv; q += 32) prefetch_l2(val + v0 + EPL * q);
-        }
+        w = nw;
+        nbase = fbase;
+        nw = fw;
     }
 }
 
-template <class TS, int G, int NV, int U>
-cudaError_t go_chunk(const RelaxArgs &a, cudaStream_t s)
+// Groups per block and threads of a block.  Small phases spread over the SMs in
+// blocks of two warps; otherwise one block per SM takes one chunk (one wave, with
+// as many warps as share its groups evenly),
+// or, beyond kSellSpan rows per SM, several: the blocks run in order, so the
+// rows in work at a time then stay within a window that the L2 holds (7-point
+// 112^3, K = 32: one chunk per SM read 637 MB from DRAM, the rows in order 264).
+constexpr int kSellSpan = 4096;
+
+template <class TS, int P, int U, bool SPLIT, bool MAP>
+cudaError_t go_sell_typed(const RelaxArgs &a, cudaStream_t s)
 {
-    const int64_t rows = (int64_t)a.r1 - a.r0;
-    if (rows <= 0) return cudaSuccess;
-    constexpr int RW = 32 / G;
-    auto kern = a.split > 0 ? k_relax_chunk<TS, G, NV, U, true> : k_relax_chunk<TS, G, NV, U, false>;
-    static PerDevice sm_count;
-    const int dev = current_device_index();
-    int sms = sm_count.get(dev);
-    if (sms == 0) {
-        int d = 0;
-        cudaGetDevice(&d);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
-        if (sms <= 0) sms = 1;
-        sm_count.set(dev, sms);
+    using L = SellShape<TS, P>;
+    constexpr int RW = 32 / L::G, SMS = 152;
+    const int64_t rows = (int64_t)a.r1 - a.r0, groups = (rows + RW - 1) / RW;
+    int threads = L::THREADS;
+    int64_t chunk;
+    if (groups <= (int64_t)SMS * 8) {
+        threads = 64;
+        chunk = 2;
+    } else {
+        const int64_t waves = (rows + (int64_t)SMS * kSellSpan - 1) / ((int64_t)SMS * kSellSpan);
+        chunk = (groups + SMS * waves - 1) / (SMS * waves);
+        const int64_t rounds = (chunk + threads / 32 - 1) / (threads / 32);
+        threads = 32 * (int)((chunk + rounds - 1) / rounds);
     }
-    // 32-byte accesses (NV even) need 32-byte aligned rows: always true of the
-    // handle's buffers (P even), refused rather than faulted otherwise
-    if constexpr (NV % 2 == 0) {
+    return launch_chained(k_relax_sell<TS, P, U, SPLIT, MAP>, (unsigned)((groups + chunk - 1) / chunk), threads, 0, s, a,
+                          (int32_t)chunk);
+}
+
+template <class TS, int P, int U>
+cudaError_t go_sell_u(const RelaxArgs &a, cudaStream_t s)
+{
+    if (a.rowmap)
+        return a.split > 0 ? go_sell_typed<TS, P, U, true, true>(a, s) : go_sell_typed<TS, P, U, false, true>(a, s);
+    return a.split > 0 ? go_sell_typed<TS, P, U, true, false>(a, s) : go_sell_typed<TS, P, U, false, false>(a, s);
+}
+
+template <class TS, int P>
+cudaError_t go_sell(const RelaxArgs &a, cudaStream_t s)
+{
+    if (a.r1 <= a.r0) return cudaSuccess;
+    // 32-byte accesses need 32-byte aligned rows: always true of the handle's
+    // buffers (P even), refused rather than faulted otherwise
+    if constexpr (P >= 2) {
         if (!rows_aligned32(a.xold, a.Kp, sizeof(TS)) || !rows_aligned32(a.xnew, a.Kp, sizeof(TS)))
             return cudaErrorMisalignedAddress;
     }
-    // one chunk per SM, a whole number of warp groups each
-    int64_t chunk = (rows + sms - 1) / sms;
-    chunk = (chunk + RW - 1) / RW * RW;
-    const int64_t blocks = (rows + chunk - 1) / chunk;
-    kern<<<(unsigned)blocks, kChunkThreads, 0, s>>>(a, (int32_t)chunk);
-    return cudaGetLastError();
+    // the average slice in the fewest batches, and those as even as they go
+    constexpr int UMAX = SellShape<TS, P>::UMAX;
+    const int w = a.sell_width > 1 ? a.sell_width : 1, batches = (w + UMAX - 1) / UMAX, u = (w + batches - 1) / batches;
+    if (u <= 3) return go_sell_u<TS, P, 3>(a, s);
+    if (u == 4 || UMAX == 4) return go_sell_u<TS, P, 4>(a, s);
+    if constexpr (UMAX >= 5) return go_sell_u<TS, P, 5>(a, s);
+    return cudaErrorInvalidValue;
+}
+
+template <class TS>
+cudaError_t dispatch_sell(const RelaxArgs &a, cudaStream_t s)
+{
+    constexpr int V = Store<TS>::V;
+    switch (a.Kp / V) {
+    case 1: return go_sell<TS, 1>(a, s);
+    case 2: return go_sell<TS, 2>(a, s);
+    case 4: return go_sell<TS, 4>(a, s);
+    case 8: return go_sell<TS, 8>(a, s);
+    case 16: if constexpr (16 * V <= 64) return go_sell<TS, 16>(a, s); break;
+    case 32: if constexpr (32 * V <= 64) return go_sell<TS, 32>(a, s); break;
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <class TS, int G, int NV>
@@ -806,13 +870,7 @@ cudaError_t go(const RelaxArgs &a, cudaStream_t s)
 template <class TS, int G, int NV>
 cudaError_t dispatch_u(int U, int stage, const RelaxArgs &a, cudaStream_t s)
 {
-    if (stage == 3) {
-        switch (U) {
-        case 4: return go_chunk<TS, G, NV, 4>(a, s);
-        case 8: return go_chunk<TS, G, NV, 8>(a, s);
-        }
-        return cudaErrorInvalidValue;
-    }
+    if (stage == 3) stage = 0;        // no sliced copy: the direct kernel
     switch (U) {
     case 4: return stage == 2 ? go_pipe<TS, G, NV>(a, s)
                  : stage ? go_staged<TS, G, NV, 4>(a, s) : go<TS, G, NV, 4>(a, s);
@@ -849,7 +907,28 @@ cudaError_t dispatch_g(Shape sh, const RelaxArgs &a, cudaStream_t s)
     return cudaErrorInvalidValue;
 }
 
+// omega / a_ii of every row, once per call of nu sweeps (a division is nine
+// operations of the narrow FP64 pipe, some fifteen instructions in FP32, and every
+// lane of a row would make it in every sweep)
+template <class C>
+__global__ void __launch_bounds__(256) k_weights(const C *diag, double omega, C *w, int32_t n)
+{
+    chain_wait();
+    chain_release();
+    const int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (r < n) w[r] = (C)omega / ld_plain(diag + r);
+}
+
 }  // namespace
+
+cudaError_t launch_weights(int storage, const void *diag, double omega, void *w, int32_t n, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    const unsigned grid = (unsigned)(((int64_t)n + 255) / 256);
+    if (storage == ST_FP64)
+        return launch_chained(k_weights<double>, grid, 256, 0, s, (const double *)diag, omega, (double *)w, n);
+    return launch_chained(k_weights<float>, grid, 256, 0, s, (const float *)diag, omega, (float *)w, n);
+}
 
 // shared memory of the pipelined kernel for a shape (0 if not instantiated)
 template <class TS>
@@ -884,6 +963,14 @@ bool relax_shape_available(int storage, Shape sh)
 
 cudaError_t launch_relax(int storage, Shape sh, const RelaxArgs &a, cudaStream_t s)
 {
+    if (a.sell_ptr && (sh.stage == 0 || sh.stage == 3)) {
+        switch (storage) {
+        case ST_FP64: return dispatch_sell<double>(a, s);
+        case ST_FP32: return dispatch_sell<float>(a, s);
+        case ST_BF16: return dispatch_sell<__nv_bfloat16>(a, s);
+        }
+        return cudaErrorInvalidValue;
+    }
     switch (storage) {
     case ST_FP64: return dispatch_g<double>(sh, a, s);
     case ST_FP32: return dispatch_g<float>(sh, a, s);
