@@ -213,10 +213,10 @@ int amgd_set_values(amgd_handle h, const double *val, int mem);
  * so that the upload of the next values and the download of the last strength
  * graph overlap the build between them.
  * amgd_set_values_async -- like amgd_set_values: val[nnz] (host: page-locked
- *   memory for the copy to be asynchronous; or device) is copied into one of
- *   two staging buffers, checked on the device (finite, nonzero diagonal) and
- *   applied in the handle's stream order.  val must stay valid and unchanged
- *   until amgd_sync returns.  Values that fail the check are applied all the
+ *   memory for the copy to be asynchronous; or device) is checked on the device
+ *   (finite, nonzero diagonal) and applied in the handle's stream order: host
+ *   values through one of two staging buffers, device values read in place.
+ *   val must stay valid and unchanged until amgd_sync returns.  Values that fail the check are applied all the
  *   same (results computed from them are meaningless) and the next amgd_sync
  *   returns the error.
  * amgd_strength_async -- the current strength graph M^d (§4.2) as CSR, like
@@ -324,10 +324,8 @@ int amgd_graph_launch(amgd_handle h);
  *   use (waits bounded to about one second; a wait that runs out makes the
  *   next synchronising call return AMGD_ERR_TIMEOUT); 2 warp-pipelined, CSR
  *   slices and neighbour rows copied with cp.async two and one row groups
- *   ahead (U must be 4); 3 chunked, one 896-thread block per SM owning a
- *   contiguous run of rows, each warp asking the L2 for the row pointers
- *   and CSR lines of its next row groups ahead of use and loading the CSR
- *   with an evict-first and the vectors with an evict-last cache policy.
+ *   ahead (U must be 4); 3 accepted and kept, the same kernel as 0, which
+ *   chooses its lanes, batch and blocks by the row's size and the matrix.
  *   The distance pass has one kernel, chosen by the row's size alone: every
  *   shape in the range above (stage 2 with U in {2,4}, stage 3 with U in
  *   {4,8}) is accepted and kept, and all of them run it.  Shapes change speed

@@ -364,14 +364,25 @@ int permute_values(amgd_ctx *h, const double *src = nullptr, uint32_t *err = nul
     const bool in_place = src == nullptr;
     const bool mixed = h->storage != ST_FP64;
     const bool csr = sweeps_use_csr(h) || (h->gexec && h->graph_csr);
-    float *v32o = mixed ? h->val32_o : nullptr;
-    double *vp64 = (h->perm && !mixed && csr) ? h->val64 : nullptr;   // without a coloring val64 is val_o
-    float *vp32 = (h->perm && mixed && csr) ? h->val32 : nullptr;     // and val32 is not read
-    CK(h, launch_scatter_values(in_place ? h->val_o : src, h->nnz, h->perm ? h->slot_perm : nullptr,
-                                h->sell_ok ? h->sell_slot : nullptr, in_place ? nullptr : h->val_o, v32o, vp64, vp32,
-                                mixed ? nullptr : h->sell_val64, mixed ? h->sell_val32 : nullptr, h->stream, err));
-    CK(h, launch_diag_values(h->val_o, h->diag_slot, h->perm, (int32_t)h->n, h->diag64_o,
-                             h->diag32_o, mixed ? nullptr : h->diag64, h->diag32, h->stream, err));
+    ValueArgs a = {};
+    a.src = in_place ? h->val_o : src;
+    a.rp = h->rp_o;
+    a.diag_slot = h->diag_slot;
+    a.pinv = h->perm ? h->pinv : nullptr;
+    a.slot_perm = h->perm ? h->slot_perm : nullptr;
+    a.slot_sell = h->sell_slot;
+    a.val_o = in_place ? nullptr : h->val_o;
+    a.val32_o = mixed ? h->val32_o : nullptr;
+    // without a coloring val64 is val_o, and val32 is not read
+    a.perm_val = !(h->perm && csr) ? nullptr : mixed ? (void *)h->val32 : (void *)h->val64;
+    a.sell = !h->sell_ok ? nullptr : mixed ? (void *)h->sell_val32 : (void *)h->sell_val64;
+    a.d64_o = h->diag64_o;
+    a.d32_o = h->diag32_o;
+    a.d64_p = mixed ? nullptr : h->diag64;
+    a.d32_p = h->diag32;
+    a.err = err;
+    a.n = (int32_t)h->n;
+    CK(h, launch_values(a, !mixed, h->nnz, h->stream));
     h->perm64_stale = mixed || !csr;
     h->perm32_stale = !(mixed && csr);
     return AMGD_OK;
@@ -1219,24 +1230,28 @@ int amgd_set_values_async(amgd_handle h, const double *val, int mem)
     if (mem != AMGD_MEM_HOST && mem != AMGD_MEM_DEVICE) return fail(h, AMGD_ERR_ARG, "bad mem");
     int rc = async_setup(h);
     if (rc != AMGD_OK) return rc;
-    if (!h->stage[0]) {
-        CK(h, dalloc(&h->stage[0], (size_t)h->nnz + 4));
-        CK(h, dalloc(&h->stage[1], (size_t)h->nnz + 4));
+    if (mem == AMGD_MEM_DEVICE) {
+        // read in place, in stream order: val stays unchanged until amgd_sync
+        rc = permute_values(h, val, h->async_err);
+        if (rc != AMGD_OK) return rc;
+    } else {
+        if (!h->stage[0]) {
+            CK(h, dalloc(&h->stage[0], (size_t)h->nnz + 4));
+            CK(h, dalloc(&h->stage[1], (size_t)h->nnz + 4));
+        }
+        const int k = h->up_slot;
+        h->up_slot ^= 1;
+        // the slot's previous contents must have been applied before it is refilled
+        CK(h, cudaStreamWaitEvent(h->up_stream, h->ev_used[k], 0));
+        CK(h, cudaMemcpyAsync(h->stage[k], val, h->nnz * sizeof(double), cudaMemcpyHostToDevice, h->up_stream));
+        CK(h, cudaEventRecord(h->ev_up[k], h->up_stream));
+        CK(h, cudaStreamWaitEvent(h->stream, h->ev_up[k], 0));
+        // the value checks ride on the copies (their bits land in the error word
+        // the next synchronising call reads)
+        rc = permute_values(h, h->stage[k], h->async_err);
+        if (rc != AMGD_OK) return rc;
+        CK(h, cudaEventRecord(h->ev_used[k], h->stream));
     }
-    const int k = h->up_slot;
-    h->up_slot ^= 1;
-    // the slot's previous contents must have been applied before it is refilled
-    CK(h, cudaStreamWaitEvent(h->up_stream, h->ev_used[k], 0));
-    CK(h, cudaMemcpyAsync(h->stage[k], val, h->nnz * sizeof(double),
-                          mem == AMGD_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                          h->up_stream));
-    CK(h, cudaEventRecord(h->ev_up[k], h->up_stream));
-    CK(h, cudaStreamWaitEvent(h->stream, h->ev_up[k], 0));
-    // the value checks ride on the copies (their bits land in the error word
-    // the next synchronising call reads)
-    rc = permute_values(h, h->stage[k], h->async_err);
-    if (rc != AMGD_OK) return rc;
-    CK(h, cudaEventRecord(h->ev_used[k], h->stream));
     h->async_pending = true;
     h->have_dist = false;
     h->traj_valid = false;

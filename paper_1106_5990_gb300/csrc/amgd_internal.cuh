@@ -379,6 +379,22 @@ cudaError_t launch_permute_values(const double *v, const int32_t *rp_orig,
                                   const int32_t *perm, const int32_t *rp_perm, double *vp64,
                                   float *vp32, int32_t n, cudaStream_t s);
 
+// every value copy that the queued kernels read, from caller-order values in
+// device memory, with the diagonals; NULL targets skipped; err (NULL: none) |= 1
+// for a non-finite value, |= 2 for a zero diagonal.  "VS": FP64 (f64) or FP32.
+struct ValueArgs {
+    const double *src;
+    const int32_t *rp, *diag_slot, *pinv;           // caller rows; slot of each diagonal; permuted row (NULL: itself)
+    const int32_t *slot_perm, *slot_sell;           // CSR slot (NULL: itself) and sliced position of a caller slot
+    double *val_o;                                  // caller FP64 and FP32 copies
+    float *val32_o;
+    void *perm_val, *sell;                          // row-permuted CSR and sliced copy, VS
+    double *d64_o, *d64_p;
+    float *d32_o, *d32_p;
+    uint32_t *err;
+    int32_t n;
+};
+cudaError_t launch_values(const ValueArgs &a, bool f64, int64_t nnz, cudaStream_t s);
 // one coalesced pass over caller-order values src[nnz] into the caller FP64 /
 // FP32 copies, the row-permuted FP64 / FP32 copies (at slot_perm, NULL =
 // identity) and the sweeps' sliced copy (at slot_sell); NULL targets skipped;

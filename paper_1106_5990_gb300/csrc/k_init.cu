@@ -328,6 +328,61 @@ __global__ void k_diag_values(const double *__restrict__ v, const int32_t *__res
     if (err && __any_sync(0xffffffffu, zero) && (threadIdx.x % 32) == 0) atomicOr(err, 2u);
 }
 
+// Every copy of the values in one pass over them (launch_values).  A block takes
+// kThreads consecutive caller rows: their values come in and the caller-order
+// copies go out as one contiguous run, and the run waits in shared memory (in the
+// type VS of the sweeps) for the sliced copy, where one thread per row writes
+// entry k of consecutive rows side by side -- a scatter slot by slot would write
+// each value to a line of its own -- and for the diagonals.  Bound: HBM.
+template <class VS>
+__global__ void __launch_bounds__(kThreads) k_values(ValueArgs A, int cap)
+{
+    extern __shared__ __align__(16) unsigned char vsm[];
+    VS *sv = reinterpret_cast<VS *>(vsm);
+    int32_t *sp = reinterpret_cast<int32_t *>(sv + cap);
+    const int64_t R0 = (int64_t)blockIdx.x * kThreads;
+    const int nr = (int)min((int64_t)kThreads, A.n - R0), tid = threadIdx.x;
+    const int S0 = A.rp[R0], S1 = A.rp[R0 + nr];
+    const bool fits = S1 - S0 <= cap;
+    VS *sell = (VS *)A.sell;
+    if (sell && fits)
+        for (int q = tid; q < S1 - S0; q += kThreads) sp[q] = __ldg(A.slot_sell + S0 + q);
+    chain_wait();
+    bool bad = false;
+    for (int p = S0 + tid; p < S1; p += kThreads) {
+        const double x = ld_plain(A.src + p);
+        bad = bad || !isfinite(x);
+        if (A.val_o) A.val_o[p] = x;
+        const VS v = (VS)x;
+        if (A.val32_o) A.val32_o[p] = (float)v;
+        if (A.perm_val) ((VS *)A.perm_val)[A.slot_perm ? A.slot_perm[p] : p] = v;
+        if (sell) {
+            if (fits) sv[p - S0] = v;
+            else sell[A.slot_sell[p]] = v;
+        }
+    }
+    __syncthreads();
+    bool zero = false;
+    if (tid < nr) {
+        const int64_t o = R0 + tid;
+        if (sell && fits) {
+            const int q1 = A.rp[o + 1] - S0;
+            for (int q = A.rp[o] - S0; q < q1; ++q) sell[sp[q]] = sv[q];
+        }
+        const double d = ld_plain(A.src + A.diag_slot[o]);
+        zero = d == 0.0;
+        const int64_t r = A.pinv ? A.pinv[o] : o;
+        A.d64_o[o] = d;
+        A.d32_o[o] = (float)d;
+        if (A.d64_p) A.d64_p[r] = d;
+        A.d32_p[r] = (float)d;
+    }
+    if (A.err) {
+        const uint32_t e = (__any_sync(0xffffffffu, bad) ? 1u : 0u) | (__any_sync(0xffffffffu, zero) ? 2u : 0u);
+        if (e && tid % 32 == 0) atomicOr(A.err, e);
+    }
+}
+
 inline unsigned blocks(int64_t work) { return (unsigned)((work + kThreads - 1) / kThreads); }
 
 // priority keys of the coarse-point selection: one Philox4x64-10 block per
@@ -478,6 +533,18 @@ cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t 
     k_scatter_values<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), kThreads, 0, s>>>(
         src, nnz, slot_perm, slot_sell, val_o, val32_o, vp64, vp32, vs64, vs32, err);
     return cudaGetLastError();
+}
+
+cudaError_t launch_values(const ValueArgs &a, bool f64, int64_t nnz, cudaStream_t s)
+{
+    if (a.n == 0) return cudaSuccess;
+    // a block's average run and a quarter more, within the default shared memory
+    const int slot = (f64 ? 8 : 4) + 4;
+    int64_t cap = (int64_t)((double)nnz / a.n * kThreads * 1.25) + 64;
+    if (cap * slot > 48 * 1024) cap = 48 * 1024 / slot;
+    cap &= ~(int64_t)3;
+    if (f64) return launch_chained(k_values<double>, blocks(a.n), kThreads, (size_t)cap * slot, s, a, (int)cap);
+    return launch_chained(k_values<float>, blocks(a.n), kThreads, (size_t)cap * slot, s, a, (int)cap);
 }
 
 cudaError_t launch_diag_values(const double *v, const int32_t *diag_slot, const int32_t *perm,
