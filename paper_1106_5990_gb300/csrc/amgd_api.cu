@@ -26,8 +26,9 @@ struct amgd_ctx {
     int32_t K = 0, nmat = 1;
     int storage = ST_FP64, target = AMGD_TARGET_RESIDUAL;
     std::vector<int64_t> row_off, slot_off;
-    std::vector<int32_t> h_rp, h_col;          // caller CSR pattern (int32)
-    std::vector<int32_t> h_diag_slot;           // slot of each row's diagonal
+    std::vector<int32_t> h_rp, h_col;          // caller CSR pattern (int32); see ensure_host_csr
+    bool host_csr = false;                      // they hold it
+    void *slab = nullptr;                       // one allocation: the arrays that live as long as the handle
     // device: caller numbering
     int32_t *rp_o = nullptr, *col_o = nullptr;
     double *val_o = nullptr;
@@ -307,6 +308,19 @@ int check_csr(const int64_t *rp, const int32_t *col, const double *val, int64_t 
     return AMGD_OK;
 }
 
+// the pattern on the host, for the set-ups that run there (a matrix created
+// from device memory leaves it on the device)
+int ensure_host_csr(amgd_ctx *h)
+{
+    if (h->host_csr) return AMGD_OK;
+    h->h_rp.resize((size_t)h->n + 1);
+    h->h_col.resize((size_t)h->nnz);
+    CK(h, cudaMemcpy(h->h_rp.data(), h->rp_o, ((size_t)h->n + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    if (h->nnz) CK(h, cudaMemcpy(h->h_col.data(), h->col_o, (size_t)h->nnz * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    h->host_csr = true;
+    return AMGD_OK;
+}
+
 cudaError_t ensure_tmp64(amgd_ctx *h, size_t count)
 {
     if (h->tmp64_len >= count && h->tmp64) return cudaSuccess;
@@ -335,8 +349,6 @@ int upload_weights(amgd_ctx *h)
     std::vector<double> w64((size_t)KpMax, 0.0);
     std::vector<float> w32((size_t)KpMax, 0.0f);
     for (int k = 0; k < h->K; ++k) { w64[(size_t)k] = h->h_w[(size_t)k]; w32[(size_t)k] = (float)h->h_w[(size_t)k]; }
-    if (!h->w64) CK(h, dalloc(&h->w64, (size_t)KpMax));
-    if (!h->w32) CK(h, dalloc(&h->w32, (size_t)KpMax));
     CK(h, cudaMemcpyAsync(h->w64, w64.data(), KpMax * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemcpyAsync(h->w32, w32.data(), KpMax * sizeof(float), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
@@ -749,36 +761,64 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
     }
     const int64_t n = row_off.back();
     if (n >= (int64_t)1 << 31) return fail(nullptr, AMGD_ERR_UNSUPPORTED, "n >= 2^31");
-    std::vector<int32_t> h_rp(1, 0), h_col, diag_slot;
+    // host copies of the concatenated matrix, validated (matrices in host memory,
+    // and device matrices that the device check does not pass: the message names
+    // the first fault)
+    std::vector<int32_t> h_rp, h_col, diag_slot;
     std::vector<double> h_val;
-    std::vector<int32_t> marker, dslot;
-    for (int32_t b = 0; b < nmat; ++b) {
-        const int64_t nb = n_in[b];
-        if (!rp_in[b]) return fail(nullptr, AMGD_ERR_ARG, "NULL row_ptr");
-        std::vector<int64_t> rp((size_t)nb + 1);
-        cudaError_t e = fetch(rp.data(), rp_in[b], (nb + 1) * sizeof(int64_t), mem);
-        if (e != cudaSuccess) return cuda_fail(nullptr, e, "copy row_ptr");
-        if (rp[0] != 0) return fail(nullptr, AMGD_ERR_CSR, "row_ptr[0] != 0");
-        const int64_t nnzb = rp[(size_t)nb];
-        if (nnzb < 0) return fail(nullptr, AMGD_ERR_CSR, "negative nnz");
-        if (slot_off.back() + nnzb >= ((int64_t)1 << 31) - 16)
-            return fail(nullptr, AMGD_ERR_UNSUPPORTED, "nnz >= 2^31");
-        if (nnzb > 0 && (!col_in[b] || !val_in[b])) return fail(nullptr, AMGD_ERR_ARG, "NULL col/val");
-        std::vector<int32_t> col((size_t)nnzb);
-        std::vector<double> val((size_t)nnzb);
-        e = fetch(col.data(), col_in[b], nnzb * sizeof(int32_t), mem);
-        if (e == cudaSuccess) e = fetch(val.data(), val_in[b], nnzb * sizeof(double), mem);
-        if (e != cudaSuccess) return cuda_fail(nullptr, e, "copy col/val");
-        std::string msg;
-        const int rc = check_csr(rp.data(), col.data(), val.data(), nb, marker, dslot,
-                                 slot_off.back(), msg);
-        if (rc != AMGD_OK) return fail(nullptr, rc, "matrix " + std::to_string(b) + ": " + msg);
-        const int64_t ro = row_off[(size_t)b], so = slot_off.back();
-        for (int64_t i = 1; i <= nb; ++i) h_rp.push_back((int32_t)(so + rp[(size_t)i]));
-        for (int64_t p = 0; p < nnzb; ++p) h_col.push_back((int32_t)(ro + col[(size_t)p]));
-        h_val.insert(h_val.end(), val.begin(), val.end());
-        diag_slot.insert(diag_slot.end(), dslot.begin(), dslot.end());
-        slot_off.push_back(so + nnzb);
+    auto load_host = [&]() -> int {
+        std::vector<int32_t> marker, dslot;
+        slot_off.assign(1, 0);
+        h_rp.assign(1, 0);
+        for (int32_t b = 0; b < nmat; ++b) {
+            const int64_t nb = n_in[b];
+            if (!rp_in[b]) return fail(nullptr, AMGD_ERR_ARG, "NULL row_ptr");
+            std::vector<int64_t> rp((size_t)nb + 1);
+            cudaError_t e = fetch(rp.data(), rp_in[b], (nb + 1) * sizeof(int64_t), mem);
+            if (e != cudaSuccess) return cuda_fail(nullptr, e, "copy row_ptr");
+            if (rp[0] != 0) return fail(nullptr, AMGD_ERR_CSR, "row_ptr[0] != 0");
+            const int64_t nnzb = rp[(size_t)nb];
+            if (nnzb < 0) return fail(nullptr, AMGD_ERR_CSR, "negative nnz");
+            if (slot_off.back() + nnzb >= ((int64_t)1 << 31) - 16)
+                return fail(nullptr, AMGD_ERR_UNSUPPORTED, "nnz >= 2^31");
+            if (nnzb > 0 && (!col_in[b] || !val_in[b])) return fail(nullptr, AMGD_ERR_ARG, "NULL col/val");
+            std::vector<int32_t> col((size_t)nnzb);
+            std::vector<double> val((size_t)nnzb);
+            e = fetch(col.data(), col_in[b], nnzb * sizeof(int32_t), mem);
+            if (e == cudaSuccess) e = fetch(val.data(), val_in[b], nnzb * sizeof(double), mem);
+            if (e != cudaSuccess) return cuda_fail(nullptr, e, "copy col/val");
+            std::string msg;
+            const int rc = check_csr(rp.data(), col.data(), val.data(), nb, marker, dslot,
+                                     slot_off.back(), msg);
+            if (rc != AMGD_OK) return fail(nullptr, rc, "matrix " + std::to_string(b) + ": " + msg);
+            const int64_t ro = row_off[(size_t)b], so = slot_off.back();
+            for (int64_t i = 1; i <= nb; ++i) h_rp.push_back((int32_t)(so + rp[(size_t)i]));
+            for (int64_t p = 0; p < nnzb; ++p) h_col.push_back((int32_t)(ro + col[(size_t)p]));
+            h_val.insert(h_val.end(), val.begin(), val.end());
+            diag_slot.insert(diag_slot.end(), dslot.begin(), dslot.end());
+            slot_off.push_back(so + nnzb);
+        }
+        return AMGD_OK;
+    };
+    bool on_device = mem == AMGD_MEM_DEVICE;
+    if (on_device) {
+        // the entry counts; the rest of the matrix stays where it is
+        for (int32_t b = 0; b < nmat; ++b) {
+            if (!rp_in[b]) return fail(nullptr, AMGD_ERR_ARG, "NULL row_ptr");
+            int64_t ends[2] = {0, 0};
+            cudaError_t e = fetch(&ends[0], rp_in[b], sizeof(int64_t), mem);
+            if (e == cudaSuccess) e = fetch(&ends[1], rp_in[b] + n_in[b], sizeof(int64_t), mem);
+            if (e != cudaSuccess) return cuda_fail(nullptr, e, "copy row_ptr");
+            if (ends[0] != 0) return fail(nullptr, AMGD_ERR_CSR, "row_ptr[0] != 0");
+            if (ends[1] < 0) return fail(nullptr, AMGD_ERR_CSR, "negative nnz");
+            if (slot_off.back() + ends[1] >= ((int64_t)1 << 31) - 16)
+                return fail(nullptr, AMGD_ERR_UNSUPPORTED, "nnz >= 2^31");
+            if (ends[1] > 0 && (!col_in[b] || !val_in[b])) return fail(nullptr, AMGD_ERR_ARG, "NULL col/val");
+            slot_off.push_back(slot_off.back() + ends[1]);
+        }
+    } else {
+        const int rc = load_host();
+        if (rc != AMGD_OK) return rc;
     }
 
     amgd_ctx *h = new amgd_ctx();
@@ -789,9 +829,6 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
     h->nmat = nmat;
     h->row_off = row_off;
     h->slot_off = slot_off;
-    h->h_rp = std::move(h_rp);
-    h->h_col = std::move(h_col);
-    h->h_diag_slot = std::move(diag_slot);
     h->h_w.assign((size_t)K, 1.0);
     for (int st = 0; st < 3; ++st) {
         h->relax_shape[st] = default_shape(st, K);
@@ -811,38 +848,67 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
         cudaError_t e__ = (expr);                                          \
         if (e__ != cudaSuccess) return bail(cuda_fail(h, e__, #expr));     \
     } while (0)
-    TRY(dalloc(&h->rp_o, (size_t)n + 1 + 4));      // +16 bytes: widened bulk copies
-    TRY(dalloc(&h->col_o, (size_t)h->nnz + 16));  // +64 bytes: widened bulk copies, 16-slot loads
-    TRY(dalloc(&h->val_o, (size_t)h->nnz + 4));
-    TRY(dalloc(&h->mat_off, (size_t)nmat + 1));
-    TRY(cudaMemcpy(h->rp_o, h->h_rp.data(), (n + 1) * sizeof(int32_t), cudaMemcpyHostToDevice));
-    if (h->nnz) {
-        TRY(cudaMemcpy(h->col_o, h->h_col.data(), h->nnz * sizeof(int32_t), cudaMemcpyHostToDevice));
-        TRY(cudaMemcpy(h->val_o, h_val.data(), h->nnz * sizeof(double), cudaMemcpyHostToDevice));
+    // the arrays that are never replaced, in one allocation (an allocation and its
+    // release cost 25 us, and a handle made for one build has them all)
+    {
+        struct Part { void **p; size_t bytes; };
+        auto part = [](auto **p, size_t count) {
+            return Part{(void **)p, ((count ? count : 1) * sizeof(**p) + 255) & ~(size_t)255};
+        };
+        const size_t N = (size_t)n, Z = (size_t)h->nnz;
+        double *norms = nullptr;
+        const Part parts[] = {
+            part(&h->rp_o, N + 1 + 4),       // +16 bytes: widened bulk copies
+            part(&h->col_o, Z + 16),         // +64 bytes: widened bulk copies, 16-slot loads
+            part(&h->val_o, Z + 4), part(&h->mat_off, (size_t)nmat + 1), part(&h->diag_slot, N),
+            part(&h->err_word, 1), part(&h->status, 1), part(&h->diag64, N), part(&h->diag32, N),
+            part(&h->diag64_o, N), part(&h->diag32_o, N), part(&norms, 2 * N), part(&h->defer_count, 1),
+            part(&h->defer_list, N), part(&h->count, N), part(&h->tile, N / kTileRows + 2),
+            part(&h->w64, 64), part(&h->w32, 64)};
+        size_t total = 0;
+        for (const Part &q : parts) total += q.bytes;
+        TRY(cudaMalloc(&h->slab, total));
+        char *at = (char *)h->slab;
+        for (const Part &q : parts) { *q.p = at; at += q.bytes; }
+        h->norms = norms;
     }
-    TRY(cudaMemcpy(h->mat_off, row_off.data(), (nmat + 1) * sizeof(int64_t), cudaMemcpyHostToDevice));
-    TRY(dalloc(&h->diag_slot, (size_t)n));
-    TRY(dalloc(&h->err_word, 1));
-    TRY(dalloc(&h->status, 1));
-    TRY(cudaMemset(h->status, 0, sizeof(uint32_t)));
-    // test hooks for the bounded-wait path (never set in normal use):
-    // AMGD_TEST_STAGING_EXTRA_TX declares bytes that no copy delivers, so the
-    // first staged wait runs out; AMGD_TEST_WAIT_LIMIT shortens the waits.
-    if (const char *e = getenv("AMGD_TEST_STAGING_EXTRA_TX")) h->test_extra_tx = (uint32_t)atoi(e);
-    if (const char *e = getenv("AMGD_TEST_WAIT_LIMIT")) h->wait_limit = atoll(e);
-    if (n) TRY(cudaMemcpy(h->diag_slot, h->h_diag_slot.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
-    h->prp = h->rp_o;
-    h->pcol = h->col_o;
-    h->nnz_p = h->nnz;
-    h->E_p = h->E;
+    TRY(cudaMemcpyAsync(h->mat_off, row_off.data(), (nmat + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
+    TRY(cudaMemsetAsync(h->status, 0, sizeof(uint32_t), h->stream));
     h->rp_p = h->rp_o;
     h->col_p = h->col_o;
     h->val64 = h->val_o;
-    TRY(dalloc(&h->diag64, (size_t)n));
-    TRY(dalloc(&h->diag32, (size_t)n));
-    TRY(dalloc(&h->diag64_o, (size_t)n));
-    TRY(dalloc(&h->diag32_o, (size_t)n));
-    {
+    if (on_device) {
+        // checked, renumbered and copied by one pass over each matrix on the device
+        TRY(cudaMemsetAsync(h->err_word, 0, sizeof(uint32_t), h->stream));
+        for (int32_t b = 0; b < nmat; ++b) {
+            const CreateArgs ca{rp_in[b], col_in[b], val_in[b], n_in[b], slot_off[(size_t)b + 1] - slot_off[(size_t)b],
+                                row_off[(size_t)b], slot_off[(size_t)b], h->rp_o, h->col_o, h->val_o, h->diag_slot,
+                                h->diag64, h->diag64_o, h->diag32, h->diag32_o, h->err_word};
+            TRY(launch_create(ca, h->stream));
+        }
+        if (n == 0) TRY(cudaMemsetAsync(h->rp_o, 0, sizeof(int32_t), h->stream));
+        uint32_t err = 0;
+        TRY(cudaMemcpyAsync(&err, h->err_word, sizeof err, cudaMemcpyDeviceToHost, h->stream));
+        TRY(cudaStreamSynchronize(h->stream));
+        if (err) {
+            // a fault, or a long row in no order: the host check decides
+            on_device = false;
+            if ((rc = load_host()) != AMGD_OK) {
+                h->err = g_create_err;
+                return bail(rc);
+            }
+        }
+    }
+    if (!on_device) {
+        TRY(cudaMemcpy(h->rp_o, h_rp.data(), (n + 1) * sizeof(int32_t), cudaMemcpyHostToDevice));
+        if (h->nnz) {
+            TRY(cudaMemcpy(h->col_o, h_col.data(), h->nnz * sizeof(int32_t), cudaMemcpyHostToDevice));
+            TRY(cudaMemcpy(h->val_o, h_val.data(), h->nnz * sizeof(double), cudaMemcpyHostToDevice));
+        }
+        if (n) TRY(cudaMemcpy(h->diag_slot, diag_slot.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
+        h->h_rp = std::move(h_rp);
+        h->h_col = std::move(h_col);
+        h->host_csr = true;
         cudaError_t e = launch_diagonal(h->rp_p, h->col_p, h->val64, h->diag64, h->diag32,
                                         (int32_t)n, h->stream);
         if (e == cudaSuccess)
@@ -850,13 +916,17 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
                                 h->stream);
         if (e != cudaSuccess) return bail(cuda_fail(h, e, "launch_diagonal"));
     }
+    // test hooks for the bounded-wait path (never set in normal use):
+    // AMGD_TEST_STAGING_EXTRA_TX declares bytes that no copy delivers, so the
+    // first staged wait runs out; AMGD_TEST_WAIT_LIMIT shortens the waits.
+    if (const char *e = getenv("AMGD_TEST_STAGING_EXTRA_TX")) h->test_extra_tx = (uint32_t)atoi(e);
+    if (const char *e = getenv("AMGD_TEST_WAIT_LIMIT")) h->wait_limit = atoll(e);
+    h->prp = h->rp_o;
+    h->pcol = h->col_o;
+    h->nnz_p = h->nnz;
+    h->E_p = h->E;
     h->color_start = {0, n};
     TRY(dalloc(&h->flag, (size_t)h->nnz_p + 16));   // 16-byte loads past the end
-    TRY(cudaMalloc(&h->norms, (size_t)(n ? n : 1) * 16));
-    TRY(dalloc(&h->defer_count, 1));
-    TRY(dalloc(&h->defer_list, (size_t)n));
-    TRY(dalloc(&h->count, (size_t)n));
-    TRY(dalloc(&h->tile, (size_t)(n / kTileRows + 2)));
     if ((rc = alloc_slot_outputs(h, ST_FP64)) != AMGD_OK) return bail(rc);
     if ((rc = alloc_vectors(h, ST_FP64, &h->x[0], &h->x[1])) != AMGD_OK) return bail(rc);
     if ((rc = upload_weights(h)) != AMGD_OK) return bail(rc);
@@ -868,6 +938,7 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
     // setup kernel has run, so a test can watch a gather's bounds test fire
     // (the next synchronising call returns AMGD_ERR_CHECK)
     if (const char *e = getenv("AMGD_TEST_BAD_COLUMN")) {
+        if ((rc = ensure_host_csr(h)) != AMGD_OK) return bail(rc);
         const long long slot = atoll(e);
         if (slot >= 0 && slot < h->nnz) {
             const int32_t bad = (int32_t)n + 1000;
@@ -1032,6 +1103,10 @@ int amgd_set_coloring(amgd_handle h, const int32_t *color, int32_t ncolors, int 
     if (h->async_pending) return fail(h, AMGD_ERR_STATE, "asynchronous work pending: call amgd_sync first");
     if (ncolors < 1 || (!color && h->n > 0)) return fail(h, AMGD_ERR_ARG, "bad coloring arguments");
     const int64_t n = h->n;
+    {
+        const int rc = ensure_host_csr(h);
+        if (rc != AMGD_OK) return rc;
+    }
     std::vector<int32_t> c((size_t)n);
     CK(h, fetch(c.data(), color, n * sizeof(int32_t), mem));
     std::vector<int64_t> start((size_t)ncolors + 1, 0);
@@ -1719,6 +1794,10 @@ int amgd_set_search_depth(amgd_handle h, int32_t d)
     if (h->async_pending) return fail(h, AMGD_ERR_STATE, "asynchronous work pending: call amgd_sync first");
     if (d < 1 || d > 16) return fail(h, AMGD_ERR_ARG, "search depth must be in 1..16");
     if (d == h->depth) return AMGD_OK;
+    if (d > 1) {
+        const int rc = ensure_host_csr(h);
+        if (rc != AMGD_OK) return rc;
+    }
     std::vector<int32_t> prp, pcol;
     if (d > 1 && !depth_pattern(h->h_rp, h->h_col, h->n, d, ((int64_t)1 << 31) - 64, prp, pcol))
         return fail(h, AMGD_ERR_UNSUPPORTED, "the graph of A^d has 2^31 entries or more");
@@ -2032,6 +2111,10 @@ namespace {
 int ensure_transpose(amgd_ctx *h)
 {
     if (h->at_rp) return AMGD_OK;
+    {
+        const int rc = ensure_host_csr(h);
+        if (rc != AMGD_OK) return rc;
+    }
     const int64_t n = h->n, nnz = h->nnz;
     std::vector<int32_t> trp((size_t)n + 1, 0), trow((size_t)nnz), tslot((size_t)nnz);
     for (int64_t p = 0; p < nnz; ++p) ++trp[(size_t)h->h_col[(size_t)p] + 1];
@@ -2361,13 +2444,9 @@ int amgd_destroy(amgd_handle h)
         dfree(h->prp);
         dfree(h->pcol);
     }
-    void *ptrs[] = {h->rp_o, h->col_o, h->val_o, h->mat_off, h->diag_slot, h->err_word, h->status,
-                    h->diag64, h->diag32, h->val32_o, h->diag64_o, h->diag32_o, h->x_caller,
-                    h->defer_count, h->defer_list,
-                    h->val32, h->x[0], h->x[1],
-                    h->w64, h->w32, h->a, h->ls, h->flag, h->count, h->tile, h->s_rp_tmp,
-                    h->s_col_tmp, h->tmp64, h->ckpt, h->seg, h->adj_vec, h->adj_slot, h->lsb,
-                    h->adj_part, h->at_rp, h->at_row, h->at_slot, h->norms, h->mirror,
+    void *ptrs[] = {h->slab, h->val32_o, h->x_caller, h->val32, h->x[0], h->x[1], h->a, h->ls, h->flag,
+                    h->s_rp_tmp, h->s_col_tmp, h->tmp64, h->ckpt, h->seg, h->adj_vec, h->adj_slot, h->lsb,
+                    h->adj_part, h->at_rp, h->at_row, h->at_slot, h->mirror,
                     h->ip_coarse, h->ip_sel_col, h->ip_cnt, h->ip_sel_val, h->ip_ls, h->ip_rp,
                     h->ip_out, h->ip_pos, h->ip_list, h->ip_bcnt, h->ip_bkt, h->cr_u[0], h->cr_u[1], h->cr_coarse, h->cr_coarse_p, h->cr_cdiag, h->stage[0], h->stage[1], h->res_rp[0],
                     h->res_rp[1], h->res_col[0], h->res_col[1], h->async_err, h->cr_state,

@@ -356,6 +356,24 @@ cudaError_t launch_sell_fill(const SellArgs &a, const int32_t *rowmap, const int
 cudaError_t launch_edge(int storage, bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s);
 
+// one matrix of a handle created from device memory, checked and copied into the
+// handle's arrays (rows from row0, slots from slot0); err |= 1: row pointers out
+// of order, a column out of range or twice in a row, a value not finite, a
+// diagonal missing or zero; |= 2: a row too long to check for duplicates here
+struct CreateArgs {
+    const int64_t *rp;
+    const int32_t *col;
+    const double *val;
+    int64_t n, nnz, row0, slot0;
+    int32_t *rp_o, *col_o;
+    double *val_o;
+    int32_t *diag_slot;
+    double *d64_p, *d64_o;
+    float *d32_p, *d32_o;
+    uint32_t *err;
+};
+cudaError_t launch_create(const CreateArgs &a, cudaStream_t s);
+
 // scatter caller-order n x K doubles into permuted, padded storage and back
 cudaError_t launch_import(int storage, const double *src, void *x, const int32_t *perm,
                           int32_t n, int32_t K, int32_t Kp, cudaStream_t s);
