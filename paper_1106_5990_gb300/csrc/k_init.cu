@@ -433,8 +433,10 @@ inline unsigned blocks(int64_t work) { return (unsigned)((work + kThreads - 1) /
 // priority keys of the coarse-point selection: one Philox4x64-10 block per
 // point, counter (i, stage, 1, 0) (word 2 = 1 keeps them apart from the
 // test-vector draws), key (seed, 0); word 0 is the key
-__global__ void k_cr_keys(int32_t n, int32_t stage, uint64_t seed, uint64_t *__restrict__ key)
+__global__ void k_cr_keys(int32_t n, int32_t stage, uint64_t seed, uint64_t *key)
 {
+    chain_wait();
+    chain_release();
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         key[i] = philox4x64_10((uint64_t)i, (uint64_t)stage, 1ull, 0ull, seed, 0ull).v[0];
 }
@@ -444,8 +446,7 @@ __global__ void k_cr_keys(int32_t n, int32_t stage, uint64_t seed, uint64_t *__r
 cudaError_t launch_cr_keys(int32_t n, int32_t stage, uint64_t seed, uint64_t *key, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    k_cr_keys<<<blocks(n), kThreads, 0, s>>>(n, stage, seed, key);
-    return cudaGetLastError();
+    return launch_chained(k_cr_keys, blocks(n), kThreads, 0, s, n, stage, seed, key);
 }
 
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s)
