@@ -129,7 +129,10 @@ __global__ void __launch_bounds__(kThreads) k_tv_init(InitArgs A, int lq)
     using SB = StartBits<TS>;
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int64_t r = t >> lq;
-    if (r >= A.n) return;
+    if (r >= A.n) {
+        chain_wait();
+        return;
+    }
     const int q = (int)(t & ((1 << lq) - 1));
     const int64_t o = A.perm ? A.perm[r] : r;
     int lo = 0, hi = A.nmat;                 // matrix b with mat_off[b] <= o < mat_off[b+1]
@@ -146,6 +149,8 @@ __global__ void __launch_bounds__(kThreads) k_tv_init(InitArgs A, int lq)
         const uint32_t m = (k & 1) ? (uint32_t)(u.v[k / 2] >> 32) : (uint32_t)u.v[k / 2];
         v[k] = 8 * q + k < A.K ? SB::get(m) : 0;     // padding: +0
     }
+    chain_wait();                  // the vectors may still be in use; the draws did not depend on them
+    chain_release();
     TS *x = (TS *)A.x + r * A.Kp + 8 * q;
     if (A.Kp >= 8) {
         uint4 *x4 = reinterpret_cast<uint4 *>(x);
@@ -457,9 +462,9 @@ cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s)
     const int64_t work = (int64_t)a.n << lq;
     if (work == 0) return cudaSuccess;
     switch (storage) {
-    case ST_FP64: k_tv_init<double><<<blocks(work), kThreads, 0, s>>>(a, lq); break;
-    case ST_FP32: k_tv_init<float><<<blocks(work), kThreads, 0, s>>>(a, lq); break;
-    case ST_BF16: k_tv_init<__nv_bfloat16><<<blocks(work), kThreads, 0, s>>>(a, lq); break;
+    case ST_FP64: return launch_chained(k_tv_init<double>, blocks(work), kThreads, 0, s, a, lq);
+    case ST_FP32: return launch_chained(k_tv_init<float>, blocks(work), kThreads, 0, s, a, lq);
+    case ST_BF16: return launch_chained(k_tv_init<__nv_bfloat16>, blocks(work), kThreads, 0, s, a, lq);
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
