@@ -2170,7 +2170,7 @@ int prepare_backward(amgd_ctx *h)
     if (rc != AMGD_OK) return rc;
     if ((rc = prepare_sweeps(h, h->stream)) != AMGD_OK) return rc;
     CK(h, ensure_buf(&h->adj_vec, h->adj_vec_bytes, 4 * nk * cs));
-    CK(h, ensure_buf(&h->adj_slot, h->adj_slot_bytes, 6 * (size_t)(h->nnz ? h->nnz : 1) * cs));
+    CK(h, ensure_buf(&h->adj_slot, h->adj_slot_bytes, (6 * (size_t)(h->nnz ? h->nnz : 1) + (size_t)h->n) * cs));
     CK(h, ensure_buf(&h->seg, h->seg_bytes, (size_t)(S - 1) * xb));
     if (!h->lsb) CK(h, dalloc(&h->lsb, (size_t)(h->nnz ? h->nnz : 1)));
     if (!h->adj_part) CK(h, dalloc(&h->adj_part, (size_t)2 * kAdjReduceBlocks + 2));
@@ -2200,6 +2200,7 @@ int run_backward(amgd_ctx *h, const double *lsb_in, double *vb, cudaStream_t s)
     void *gs = slots, *gt = slots + nnz * cs, *at_b = slots + 2 * nnz * cs;
     void *bm = slots + 3 * nnz * cs;
     double *a64 = (double *)(slots + 4 * nnz * cs), *ls64 = (double *)(slots + 5 * nnz * cs);
+    double *inv64 = (double *)(slots + 6 * nnz * cs);
 
     AdjArgs a;
     a.rp = h->rp_o;
@@ -2223,13 +2224,20 @@ int run_backward(amgd_ctx *h, const double *lsb_in, double *vb, cudaStream_t s)
     a.unit_w = true;
     for (double wk : h->h_w) a.unit_w = a.unit_w && wk == 1.0;
     a.y = Y;                             // the refit leaves the FP64 target here for the adjoint
+    a.inv = inv64;
+    CK(h, launch_adj_inverse(h->diag64_o, inv64, n, s));
     // the fits of X_nu in FP64 (the forward pass's own a and LS may be FP32)
     CK(h, launch_adj_refit(st, a, s));
     CK(h, launch_adj_upstream(st, h->rp_o, h->col_o, ls64, h->flag, lsb_in, h->lsb, h->adj_part,
                               nb, n, h->target, s));
-    CK(h, launch_adj_bvals(st, h->val_o, h->diag64_o, h->at_row, h->at_slot, at_b, nnz, s));
-    if (h->mirror)   // per slot (j, i): a_ij / a_ii, the mirror entry over its row's diagonal
-        CK(h, launch_adj_bvals(st, h->val_o, h->diag64_o, h->col_o, h->mirror, bm, nnz, s));
+    if (h->mirror) {
+        // per slot (j, i): a_ij / a_ii, the mirror entry over its row's diagonal; a
+        // symmetric pattern's transposed entries are these slots in the same order
+        CK(h, launch_adj_bvals(st, h->val_o, h->diag64_o, inv64, h->col_o, h->mirror, bm, nnz, s));
+        a.at_b = bm;
+    } else {
+        CK(h, launch_adj_bvals(st, h->val_o, h->diag64_o, inv64, h->at_row, h->at_slot, at_b, nnz, s));
+    }
 
     a.y = Y;
     a.ybar = Ybar;

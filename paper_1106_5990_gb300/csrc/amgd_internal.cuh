@@ -164,6 +164,19 @@ __device__ __forceinline__ double2 ld_plain(const double2 *p)
     return v;
 }
 
+// exact widening to double.  Normal BF16/FP32 numbers are re-biased by bit
+// manipulation on the integer pipe (exponent + 1023 - 127, mantissa shifted
+// to the top of the 52-bit field); zeros, subnormals, infinities and NaNs
+// take the conversion instruction.
+__device__ __forceinline__ double widen_f32_bits(uint32_t u)
+{
+    const uint32_t e = (u >> 23) & 0xffu;
+    if (e == 0u || e == 0xffu) return (double)__uint_as_float(u);
+    const uint64_t bits = ((uint64_t)(u >> 31) << 63) | ((uint64_t)(e + 896u) << 52) |
+                          ((uint64_t)(u & 0x7fffffu) << 29);
+    return __longlong_as_double((long long)bits);
+}
+
 // a lane that owns a whole row (G = 1) of an even number of chunks reads them
 // in pairs; the rows must then start on 32-byte boundaries, which the
 // handle's buffers do (a row is P chunks, P even).  Launchers refuse other
@@ -446,6 +459,7 @@ cudaError_t launch_strength(const int32_t *count, const int32_t *rp_orig, const 
 struct AdjArgs {
     const int32_t *rp, *col;          // CSR pattern of A
     const void *val, *diag;           // values and diagonal, C
+    const double *inv;                // 1 / diagonal
     const int32_t *at_rp;             // transpose: column j owns entries [at_rp[j], at_rp[j+1])
     const int32_t *at_row, *at_slot;  // row i and slot p of each entry (rows ascending)
     const void *at_b;                 // b_q = a(i,j) / a_ii per entry, C
@@ -473,7 +487,9 @@ cudaError_t launch_adj_upstream(int storage, const int32_t *rp, const int32_t *c
                                 double *lsb, double *partial, int32_t nblocks, int32_t n,
                                 int32_t target, cudaStream_t s);
 // b_q = val[at_slot[q]] / a_ii, i = at_row[q], for every transposed entry (C)
-cudaError_t launch_adj_bvals(int storage, const double *val64, const double *diag64,
+// (inv64: 1 / diag64 of every row, from launch_adj_inverse)
+cudaError_t launch_adj_inverse(const double *diag64, double *inv64, int32_t n, cudaStream_t s);
+cudaError_t launch_adj_bvals(int storage, const double *val64, const double *diag64, const double *inv64,
                              const int32_t *at_row, const int32_t *at_slot, void *at_b,
                              int64_t nnz, cudaStream_t s);
 // a and LS of every slot refitted in FP64 from the stored X_nu

@@ -102,10 +102,50 @@ __device__ __forceinline__ void stc(C *p, const C (&x)[V])
 template <class TS, int V>
 __device__ __forceinline__ void unpack64(const uint4 &raw, double (&x)[V])
 {
+    // (on the integer pipe: a conversion costs as much as an FP64 multiply-add)
     typename Store<TS>::C t[V];
     Store<TS>::unpack(raw, t);
 #pragma unroll
-    for (int e = 0; e < V; ++e) x[e] = (double)t[e];
+    for (int e = 0; e < V; ++e) {
+        if constexpr (sizeof(t[0]) == 8) x[e] = t[e];
+        else x[e] = widen_f32_bits(__float_as_uint(t[e]));
+    }
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) { return widen_f32_bits(__float_as_uint(x)); }
+
+// v[u] with a lane-dependent u, without local memory
+template <int U, class T>
+__device__ __forceinline__ T pick(const T (&v)[U], int u)
+{
+    T r = v[0];
+#pragma unroll
+    for (int k = 1; k < U; ++k) r = u == k ? v[k] : r;
+    return r;
+}
+
+// the sums of U <= G values over the G lanes of a row, the one of value lane % U in
+// each lane: the last log2 U halvings exchange values instead of copying them, which
+// takes U - 1 additions and exchanges instead of U log2 U.  Pairs as group_sum's.
+// (5-point 512^2, K = 16 FP32: a reverse sweep 32.0 -> 28.7 us, k_edge_bwd 172 -> 156)
+template <int G, int U, class T>
+__device__ __forceinline__ T lane_sums(T (&v)[U], int lane, unsigned mask)
+{
+    static_assert(U <= G, "a lane per value");
+#pragma unroll
+    for (int o = G / 2; o >= U; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < U; ++k) v[k] += __shfl_xor_sync(mask, v[k], o, G);
+#pragma unroll
+    for (int o = U / 2; o > 0; o >>= 1) {
+        const bool upper = lane & o;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const T send = upper ? v[k] : v[k + o], keep = upper ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(mask, send, o, G);
+        }
+    }
+    return v[0];
 }
 
 // y_i = x_i - (1/a_ii) sum_p a_ip x_col_p (one FMA per term in CSR order) or
@@ -140,9 +180,28 @@ __device__ __forceinline__ void target64(const AdjArgs &A, int64_t r, int lane, 
             for (int e = 0; e < V; ++e) acc[e] = fma(v[u], x[e], acc[e]);
         }
     }
-    const double d = 1.0 / __ldg((const double *)A.diag + r);
+    const double d = __ldg(A.inv + r);
 #pragma unroll
     for (int e = 0; e < V; ++e) y[e] = fma(-d, acc[e], y[e]);
+}
+
+// y as the FP32 number nearest to it and the FP32 number nearest to the rest, on
+// the integer pipe (three operations of the FP64 pipe otherwise): the upper 24 bits
+// of the significand rounded half up, the lower 29 as a signed integer, scaled.
+// Numbers whose parts may leave the normal FP32 range are converted.
+__device__ __forceinline__ void split32(double y, float &h, float &l)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(y);
+    const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu, sign = (uint32_t)(b >> 63) << 31;
+    if (e - 950u < 199u) {
+        const uint64_t t = (b & 0x7fffffffffffffffull) + 0x10000000ull;
+        h = __uint_as_float(sign | ((uint32_t)(t >> 29) - (896u << 23)));
+        const int lo = (int)((uint32_t)b << 3) >> 3;
+        l = (float)lo * __uint_as_float(sign | ((e - 948u) << 23));       // 2^(e - 1023 - 52)
+    } else {
+        h = (float)y;
+        l = (float)(y - (double)h);
+    }
 }
 
 // fixed-order block sum of one double per thread (result valid in thread 0)
@@ -214,15 +273,33 @@ __device__ __forceinline__ double fit_quotient(double yx, double xx)
     return fma(r, (double)(1.0f / xf), q0);
 }
 
+// v / d from the reciprocal y of d (once per row): the product, then its exact
+// remainder's share (the quotient to within rounding of the last bit, in three FP64
+// operations instead of nine); operands near the ends of the range divide
+__device__ __forceinline__ double quotient(double v, double d, double y)
+{
+    const double q = v * y;
+    const unsigned eq = (unsigned)__double2hiint(q) & 0x7ff00000u, ey = (unsigned)__double2hiint(y) & 0x7ff00000u;
+    if (eq - 0x10000000u < 0x60000000u && ey - 0x10000000u < 0x60000000u) return fma(fma(-q, d, v), y, q);
+    return v / d;
+}
+__global__ void __launch_bounds__(kThreads)
+k_inverse(const double *__restrict__ diag, double *__restrict__ inv, int32_t n)
+{
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (i < n) inv[i] = 1.0 / diag[i];
+}
 template <class C>
 __global__ void __launch_bounds__(kThreads)
-k_bvals(const double *__restrict__ val, const double *__restrict__ diag,
+k_bvals(const double *__restrict__ val, const double *__restrict__ diag, const double *__restrict__ inv,
         const int32_t *__restrict__ at_row, const int32_t *__restrict__ at_slot,
         C *__restrict__ b, int64_t nnz)
 {
     for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < nnz;
-         q += (int64_t)gridDim.x * kThreads)
-        b[q] = (C)(__ldg(val + __ldg(at_slot + q)) / __ldg(diag + __ldg(at_row + q)));
+         q += (int64_t)gridDim.x * kThreads) {
+        const int32_t i = __ldg(at_row + q);
+        b[q] = (C)quotient(__ldg(val + __ldg(at_slot + q)), __ldg(diag + i), __ldg(inv + i));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -343,8 +420,11 @@ __device__ __forceinline__ void fit_df(const float (&x)[V], const float (&yh)[V]
     df_two_sum(sls, cls, lh, ll);
 }
 
-template <class TS, int G>
-__global__ void __launch_bounds__(kThreads) k_refit(AdjArgs A)
+// DF: mixed storage with unit weights, the fits in double-float (FP32 pipe).  One
+// kernel for both forms kept the FP64 operands of the other in 102 registers; the
+// rows are gathers of latency, so warps count (5-point 512^2, K = 16: 184 -> 154 us).
+template <class TS, int G, bool DF>
+__global__ void __launch_bounds__(kThreads, !DF ? 1 : Store<TS>::V == 4 ? 4 : 2) refit_rows(AdjArgs A)
 {
     using S = Store<TS>;
     constexpr int V = S::V;
@@ -356,48 +436,56 @@ __global__ void __launch_bounds__(kThreads) k_refit(AdjArgs A)
     const int Kp = A.Kp;
     const int p0 = __ldg(A.rp + r), p1 = __ldg(A.rp + r + 1);
     double w[V], y[V];
-    ldc<double, V>((const double *)A.w + lane * V, w);
+    if constexpr (!DF) ldc<double, V>((const double *)A.w + lane * V, w);
     target64<TS, V>(A, r, lane, p0, p1, y);
     stc<double, V>((double *)A.y + r * Kp + lane * V, y);     // for the adjoint of the fits
     double *a_out = (double *)A.a_fit;
     double *ls_out = A.ls64;
     const bool fixed = A.target == 0 && p1 - p0 == 2;
-    const double diag = __ldg((const double *)A.diag + r);
-    // mixed storage with unit weights: the fits in double-float (FP32 pipe)
-    constexpr bool kMixed = !std::is_same<TS, double>::value;
-    const bool df = kMixed && A.unit_w;
     float yh[V], yl[V];
-    if (df) {
+    if constexpr (DF) {
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
-            yh[e] = (float)y[e];
-            yl[e] = (float)(y[e] - (double)yh[e]);
-        }
+        for (int e = 0; e < V; ++e) split32(y[e], yh[e], yl[e]);
     }
-    for (int p = p0; p < p1; ++p) {
-        const int64_t j = __ldg(A.col + p);
-        double a_, ls_;
-        if (j == r) {
-            a_ = 0.0;
-            ls_ = NAN;
-        } else if (fixed) {
-            a_ = -__ldg((const double *)A.val + p) / diag;
-            ls_ = 0.0;
-        } else if (df) {
-            if constexpr (kMixed) {
-                float xf[V], ah, al, lh, ll;
-                Store<TS>::unpack(ldg16(X + j * Kp + lane * V), xf);
-                fit_df<G, V>(xf, yh, yl, gmask, ah, al, lh, ll);
-                a_ = (double)ah + (double)al;
-                ls_ = (double)lh + (double)ll;
-            }
-        } else {
-            double x[V];
-            unpack64<TS, V>(ldg16(X + j * Kp + lane * V), x);
-            if (A.unit_w) fit64<G, V, true>(x, y, w, gmask, a_, ls_);
-            else fit64<G, V, false>(x, y, w, gmask, a_, ls_);
+    // U entries gathered at a time; lane u of the row finishes entry u, so the
+    // FP64 additions and conversions run once per batch instead of once per entry
+    constexpr int U = G < 4 ? G : 4;
+    for (int pb = p0; pb < p1; pb += U) {
+        int jj[U];
+        uint4 raw[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            jj[u] = pb + u < p1 ? __ldg(A.col + pb + u) : -1;
+            if (jj[u] >= 0 && jj[u] != r && !fixed) raw[u] = ldg16(X + (int64_t)jj[u] * Kp + lane * V);
         }
-        if (lane == 0) {
+        float ah[U], al[U], lh[U], ll[U];       // double-float fits
+        double a_ = 0.0, ls_ = NAN;              // this lane's entry
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            ah[u] = al[u] = lh[u] = ll[u] = 0.f;
+            if (jj[u] < 0 || jj[u] == r || fixed) continue;
+            if constexpr (DF) {
+                float xf[V];
+                Store<TS>::unpack(raw[u], xf);
+                fit_df<G, V>(xf, yh, yl, gmask, ah[u], al[u], lh[u], ll[u]);
+            } else {
+                double x[V], au, lu;
+                unpack64<TS, V>(raw[u], x);
+                if (A.unit_w) fit64<G, V, true>(x, y, w, gmask, au, lu);
+                else fit64<G, V, false>(x, y, w, gmask, au, lu);
+                if (lane == u) { a_ = au; ls_ = lu; }
+            }
+        }
+        const int j = pick<U>(jj, lane);
+        if (lane < U && j >= 0) {
+            const int p = pb + lane;
+            if (j != r && fixed) {
+                a_ = -__ldg((const double *)A.val + p) / __ldg((const double *)A.diag + r);
+                ls_ = 0.0;
+            } else if (DF && j != r) {
+                a_ = widen(pick<U>(ah, lane)) + widen(pick<U>(al, lane));
+                ls_ = widen(pick<U>(lh, lane)) + widen(pick<U>(ll, lane));
+            }
             a_out[p] = a_;
             ls_out[p] = ls_;
         }
@@ -445,20 +533,29 @@ __global__ void __launch_bounds__(kThreads) k_edge_bwd(AdjArgs A)
     C yb[V];
     const C Lc = (C)L;
 #pragma unroll
-    for (int e = 0; e < V; ++e) yb[e] = C(2) * w[e] * fma(Lc, y[e], -v[e]);
+    for (int e = 0; e < V; ++e) yb[e] = (A.unit_w ? C(2) : C(2) * w[e]) * fma(Lc, y[e], -v[e]);
     stc<C, V>((C *)A.ybar + off, yb);
 
     if (A.target == 0) {
         C *gt = (C *)A.gt;
-        for (int p = p0; p < p1; ++p) {
-            const int j = __ldg(A.col + p);
-            C xj[V];
-            unpack64<TS, V>(ldg16(X + (int64_t)j * Kp + lane * V), xj);
-            C part = C(0);
+        constexpr int W = G < 4 ? G : 4;            // gathered at a time; lane u stores entry u
+        for (int pb = p0; pb < p1; pb += W) {
+            uint4 raw[W];
 #pragma unroll
-            for (int e = 0; e < V; ++e) part = fma(yb[e], xj[e], part);
-            part = group_sum<G>(part, gmask);
-            if (lane == 0) gt[p] = part;
+            for (int u = 0; u < W; ++u)
+                if (pb + u < p1) raw[u] = ldg16(X + (int64_t)__ldg(A.col + pb + u) * Kp + lane * V);
+            C part[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                part[u] = C(0);
+                if (pb + u >= p1) continue;
+                C xj[V];
+                unpack64<TS, V>(raw[u], xj);
+#pragma unroll
+                for (int e = 0; e < V; ++e) part[u] = fma(yb[e], xj[e], part[u]);
+            }
+            const C t = lane_sums<G, W>(part, lane, gmask);
+            if (lane < W && pb + lane < p1) gt[pb + lane] = t;
         }
     }
 }
@@ -529,6 +626,29 @@ __global__ void __launch_bounds__(kThreads) k_xbar_nu(AdjArgs A)
     }
 }
 
+// gs[pb + u] (+)= the row's sum of parts[u], in FP64, u < U: the lanes of the row take
+// an entry each, so one addition of the narrow FP64 pipe serves as many entries as the
+// row has lanes (lane 0 alone took 17 of the sweep's 40 us on the 5-point 512^2)
+template <int G, int U, class C>
+__device__ __forceinline__ void add_parts(double *gs, C (&parts)[U], int pb, int p1, int lane, int first, unsigned gmask)
+{
+    if constexpr (G >= U) {
+        const double v = widen(lane_sums<G, U>(parts, lane, gmask));
+        if (lane < U && pb + lane < p1) gs[pb + lane] = first ? v : gs[pb + lane] + v;
+    } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) parts[u] = group_sum<G>(parts[u], gmask);
+#pragma unroll
+        for (int b = 0; b < U; b += G) {
+            const int u = b + lane;
+            if (u < U && pb + u < p1) {
+                const double v = widen(pick<U>(parts, u));
+                gs[pb + u] = first ? v : gs[pb + u] + v;
+            }
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // row i of sweep k:  gs_p (+)= <Xbar_{k+1,i}, X_k,col_p>, neighbours gathered
 // four at a time
@@ -555,17 +675,19 @@ __global__ void __launch_bounds__(kThreads) k_gram(AdjArgs A)
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (pb + u < p1) raw[u] = ldg16(X + (int64_t)__ldg(A.col + pb + u) * Kp + lane * V);
+        C parts[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (pb + u >= p1) break;
+            parts[u] = C(0);
+            if (pb + u >= p1) continue;
             C xj[V];
             S::unpack(raw[u], xj);
             C part = C(0);
 #pragma unroll
             for (int e = 0; e < V; ++e) part = fma(xb[e], xj[e], part);
-            part = group_sum<G>(part, gmask);
-            if (lane == 0) gs[pb + u] = A.first ? (double)part : gs[pb + u] + (double)part;
+            parts[u] = part;
         }
+        add_parts<G, U>(gs, parts, pb, p1, lane, A.first, gmask);
     }
 }
 
@@ -637,7 +759,7 @@ __global__ void __launch_bounds__(kThreads) k_sweep_sym(AdjArgs A)
     for (int pb = p0; pb < p1; pb += U) {
         uint4 raw[U];
         C xbi[U][V];
-        C c[U];
+        C c[U], parts[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (pb + u < p1) {
@@ -649,7 +771,8 @@ __global__ void __launch_bounds__(kThreads) k_sweep_sym(AdjArgs A)
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (pb + u >= p1) break;
+            parts[u] = C(0);
+            if (pb + u >= p1) continue;
             C xi[V];
             S::unpack(raw[u], xi);
             C part = C(0);
@@ -658,9 +781,9 @@ __global__ void __launch_bounds__(kThreads) k_sweep_sym(AdjArgs A)
                 part = fma(xb[e], xi[e], part);
                 acc[e] = fma(-c[u], xbi[u][e], acc[e]);
             }
-            part = group_sum<G>(part, gmask);
-            if (lane == 0) gs[pb + u] = A.first ? (double)part : gs[pb + u] + (double)part;
+            parts[u] = part;
         }
+        add_parts<G, U>(gs, parts, pb, p1, lane, A.first, gmask);
     }
     stc<C, V>((C *)A.xbar_out + r * Kp + lane * V, acc);
 }
@@ -746,7 +869,14 @@ static int lanes(int storage, int Kp) { return Kp / (storage == ST_FP64 ? 2 : st
         return cudaGetLastError();                                                       \
     }
 
-AMGD_ADJ_LAUNCHER(launch_adj_refit, k_refit)
+template <class TS, int G> constexpr auto k_refit = refit_rows<TS, G, false>;
+template <class TS, int G> constexpr auto k_refit_df = refit_rows<TS, G, !std::is_same<TS, double>::value>;
+AMGD_ADJ_LAUNCHER(refit_general, k_refit)
+AMGD_ADJ_LAUNCHER(refit_unit, k_refit_df)
+cudaError_t launch_adj_refit(int storage, const AdjArgs &a, cudaStream_t s)
+{
+    return a.unit_w ? refit_unit(storage, a, s) : refit_general(storage, a, s);
+}
 AMGD_ADJ_LAUNCHER(launch_adj_edge, k_edge_bwd)
 AMGD_ADJ_LAUNCHER(launch_adj_xbar_nu, k_xbar_nu)
 AMGD_ADJ_LAUNCHER(launch_adj_gram, k_gram)
@@ -764,7 +894,14 @@ cudaError_t launch_adj_upstream(int storage, const int32_t *rp, const int32_t *c
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_bvals(int storage, const double *val64, const double *diag64,
+cudaError_t launch_adj_inverse(const double *diag64, double *inv, int32_t n, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    k_inverse<<<(unsigned)(((int64_t)n + kThreads - 1) / kThreads), kThreads, 0, s>>>(diag64, inv, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adj_bvals(int storage, const double *val64, const double *diag64, const double *inv64,
                              const int32_t *at_row, const int32_t *at_slot, void *at_b,
                              int64_t nnz, cudaStream_t s)
 {
@@ -772,9 +909,9 @@ cudaError_t launch_adj_bvals(int storage, const double *val64, const double *dia
     const int64_t want = (nnz + kThreads - 1) / kThreads;
     const unsigned grid = (unsigned)(want < 152 * 16 ? want : 152 * 16);
     if (storage == ST_FP64)              // the sweeps' arithmetic type
-        k_bvals<double><<<grid, kThreads, 0, s>>>(val64, diag64, at_row, at_slot, (double *)at_b, nnz);
+        k_bvals<double><<<grid, kThreads, 0, s>>>(val64, diag64, inv64, at_row, at_slot, (double *)at_b, nnz);
     else
-        k_bvals<float><<<grid, kThreads, 0, s>>>(val64, diag64, at_row, at_slot, (float *)at_b, nnz);
+        k_bvals<float><<<grid, kThreads, 0, s>>>(val64, diag64, inv64, at_row, at_slot, (float *)at_b, nnz);
     return cudaGetLastError();
 }
 

@@ -38,19 +38,6 @@ constexpr int kWarps = 4;                    // warps per block
 constexpr int kMaxK = 64;                    // components per vector
 // shared memory of one warp, in doubles (the candidate list takes 16 doubles)
 
-// exact widening to double.  Normal BF16/FP32 numbers are re-biased by bit
-// manipulation on the integer pipe (exponent + 1023 - 127, mantissa shifted
-// to the top of the 52-bit field); zeros, subnormals, infinities and NaNs
-// take the conversion instruction.
-__device__ __forceinline__ double widen_f32_bits(uint32_t u)
-{
-    const uint32_t e = (u >> 23) & 0xffu;
-    if (e == 0u || e == 0xffu) return (double)__uint_as_float(u);
-    const uint64_t bits = ((uint64_t)(u >> 31) << 63) | ((uint64_t)(e + 896u) << 52) |
-                          ((uint64_t)(u & 0x7fffffu) << 29);
-    return __longlong_as_double((long long)bits);
-}
-
 // the product of two BF16 numbers as a double: their 8-bit significands
 // multiply exactly in FP32 whenever the result is a normal FP32 number, and
 // that number widens exactly; otherwise the FP64 product (also exact)
