@@ -425,6 +425,112 @@ __global__ void k_interp_list(InterpArgs A)
     }
 }
 
+// The subsets of a row with m <= MT candidates: columns cd, Gram entries Gm (row
+// stride MT), right-hand side bv and target yv in shared memory, element e of the
+// thread at [e * T].  Writes the row's selection, weights and LS.
+template <class TS, bool UNIT_W, int MT>
+__device__ __forceinline__ void search_row(const InterpArgs &A, const TS *X, int32_t i, int m, double syy,
+                                           const double *yv, const double *Gm, const double *bv, const int32_t *cd,
+                                           int T)
+{
+    const int K = A.K, Kp = A.Kp, C = A.caliber;
+    const float sy = sqrtf((float)syy) + 1e-22f;          // (never less than the norm)
+    // every subset of each size in lexicographic order; first smallest LS
+    double best_ls[kInterpMaxCaliber + 1];
+    int best_idx[kInterpMaxCaliber + 1][kInterpMaxCaliber];
+    double best_p[kInterpMaxCaliber + 1][kInterpMaxCaliber];
+    bool have[kInterpMaxCaliber + 1];
+    have[0] = true;
+    best_ls[0] = syy;
+#pragma unroll
+    for (int s = 1; s <= kInterpMaxCaliber; ++s) {
+        have[s] = false;
+        if (s > C || s > m) continue;
+        int idx[kInterpMaxCaliber];
+        for (int a = 0; a < s; ++a) idx[a] = a;
+        for (;;) {
+            double Gs[kInterpMaxCaliber * kInterpMaxCaliber], bs[kInterpMaxCaliber];
+            double p[kInterpMaxCaliber];
+            for (int a = 0; a < s; ++a) {
+                bs[a] = bv[idx[a] * T];
+                for (int c = 0; c < s; ++c) Gs[a * s + c] = Gm[(idx[a] * MT + idx[c]) * T];
+            }
+            bool exact = false;
+            if (solve_small(s, Gs, bs, p) == 0) {
+                exact = !have[s];
+                if (!exact) {
+                    // Pruning.  With S, b, G the stored sums, the value
+                    //   q = S - 2 p.b + p.G.p
+                    // and the explicit residual sum both approximate
+                    // sum_k w_k (y_k - p.x_k)^2; their rounding errors are
+                    // at most (s^2 + 5s + 2K + 6) u M^2 together, with
+                    // M = ||y||_w + sum_a |p_a| ||x_a||_w (Cauchy-Schwarz,
+                    // Minkowski).  If q minus four times that bound is not
+                    // below the best explicit value of this size, the
+                    // subset can neither beat nor tie it (a tie goes to
+                    // the earlier subset), and its explicit sum is skipped.
+                    double q = syy;
+                    float mf = sy;
+                    for (int a = 0; a < s; ++a) {
+                        q = __dsub_rn(q, __dmul_rn(__dmul_rn(2.0, p[a]), bv[idx[a] * T]));
+                        mf = fmaf(fabsf((float)p[a]), sqrtf((float)Gm[(idx[a] * MT + idx[a]) * T]) + 1e-22f, mf);
+                    }
+                    for (int a = 0; a < s; ++a)
+                        for (int c = 0; c < s; ++c)
+                            q = __dadd_rn(q, __dmul_rn(__dmul_rn(p[a], Gm[(idx[a] * MT + idx[c]) * T]), p[c]));
+                    // (M in FP32, its few roundings covered; not finite: no pruning)
+                    const double mm = (double)(mf * 1.0001f);
+                    const double bound = (double)(4 * (s * s + 6 * s + 2 * K + 8)) * 0x1p-53 * mm * mm;
+                    exact = !(__dsub_rn(q, bound) >= best_ls[s]);
+                }
+            }
+            if (exact) {
+                double r = 0.0;
+                for (int k = 0; k < K; ++k) {
+                    double ek = yv[k * T];
+                    for (int a = 0; a < s; ++a)
+                        ek = __dsub_rn(ek, __dmul_rn(p[a], widen<TS>(X + (int64_t)cd[idx[a] * T] * Kp, k)));
+                    const double we = UNIT_W ? ek : __dmul_rn(A.w64[k], ek);
+                    r = __dadd_rn(r, __dmul_rn(we, ek));
+                }
+                if (!have[s] || r < best_ls[s]) {
+                    have[s] = true;
+                    best_ls[s] = r;
+                    for (int a = 0; a < s; ++a) {
+                        best_idx[s][a] = idx[a];
+                        best_p[s][a] = p[a];
+                    }
+                }
+            }
+            // next subset in lexicographic order
+            int a = s - 1;
+            while (a >= 0 && idx[a] == m - s + a) --a;
+            if (a < 0) break;
+            ++idx[a];
+            for (int c = a + 1; c < s; ++c) idx[c] = idx[c - 1] + 1;
+        }
+    }
+    int chosen = 0;
+    if (syy > 0.0) {
+#pragma unroll
+        for (int s = 1; s <= kInterpMaxCaliber; ++s) {
+            if (!have[s]) continue;
+            const double cur = best_ls[chosen] / syy;
+            if (penalty_less(best_ls[s] / syy, cur, A.gamma * (double)(s - chosen))) chosen = s;
+        }
+    }
+    A.cnt[i] = chosen;
+    A.ls[i] = best_ls[chosen];
+#pragma unroll
+    for (int s = 1; s <= kInterpMaxCaliber; ++s) {
+        if (s != chosen) continue;
+        for (int a = 0; a < s; ++a) {
+            A.sel_col[(int64_t)i * kInterpMaxCaliber + a] = cd[best_idx[s][a] * T];
+            A.sel_val[(int64_t)i * kInterpMaxCaliber + a] = best_p[s][a];
+        }
+    }
+}
+
 // one thread per fine row with m <= kInterpRowCand candidates.  Per-thread
 // arrays live in shared memory, element e of thread t at [e * T + t] (T the
 // block size), so that a warp's accesses fall in distinct banks.
@@ -433,13 +539,12 @@ __global__ void __launch_bounds__(128) k_ls_interp_rows(InterpArgs A)
 {
     extern __shared__ __align__(16) double rsm[];
     const int T = blockDim.x, t = threadIdx.x;
-    const int K = A.K, Kp = A.Kp, C = A.caliber;
+    const int K = A.K, Kp = A.Kp;
     constexpr int MT = kInterpRowCand;
     double *yv = rsm + t;                        // y_k        at yv[k * T]
     double *Gm = yv + (size_t)K * T;              // G_ab       at Gm[(a * MT + b) * T]
     double *bv = Gm + (size_t)MT * MT * T;        // b_a        at bv[a * T]
-    double *sg = bv + (size_t)MT * T;             // sqrt(G_aa) at sg[a * T]
-    int32_t *cd = reinterpret_cast<int32_t *>(rsm + (size_t)(K + MT * MT + 2 * MT) * T) + t;
+    int32_t *cd = reinterpret_cast<int32_t *>(rsm + (size_t)(K + MT * MT + MT) * T) + t;
     const TS *X = (const TS *)A.x;
     int32_t nrows = 0;
     for (int q = 0; q <= MT; ++q) nrows += A.bcnt[q];
@@ -517,7 +622,6 @@ __global__ void __launch_bounds__(128) k_ls_interp_rows(InterpArgs A)
                 }
             }
             bv[a * T] = ba;
-            sg[a * T] = sqrt(Gm[(a * MT + a) * T]);
         }
         double syy = 0.0;
         for (int k = 0; k < K; ++k) {
@@ -525,99 +629,135 @@ __global__ void __launch_bounds__(128) k_ls_interp_rows(InterpArgs A)
             const double wy = UNIT_W ? yk : __dmul_rn(A.w64[k], yk);
             syy = __dadd_rn(syy, __dmul_rn(wy, yk));
         }
-        const double sy = sqrt(syy);
-        // every subset of each size in lexicographic order; first smallest LS
-        double best_ls[kInterpMaxCaliber + 1];
-        int best_idx[kInterpMaxCaliber + 1][kInterpMaxCaliber];
-        double best_p[kInterpMaxCaliber + 1][kInterpMaxCaliber];
-        bool have[kInterpMaxCaliber + 1];
-        have[0] = true;
-        best_ls[0] = syy;
-#pragma unroll
-        for (int s = 1; s <= kInterpMaxCaliber; ++s) {
-            have[s] = false;
-            if (s > C || s > m) continue;
-            int idx[kInterpMaxCaliber];
-            for (int a = 0; a < s; ++a) idx[a] = a;
-            for (;;) {
-                double Gs[kInterpMaxCaliber * kInterpMaxCaliber], bs[kInterpMaxCaliber];
-                double p[kInterpMaxCaliber];
-                for (int a = 0; a < s; ++a) {
-                    bs[a] = bv[idx[a] * T];
-                    for (int c = 0; c < s; ++c) Gs[a * s + c] = Gm[(idx[a] * MT + idx[c]) * T];
-                }
-                bool exact = false;
-                if (solve_small(s, Gs, bs, p) == 0) {
-                    exact = !have[s];
-                    if (!exact) {
-                        // Pruning.  With S, b, G the stored sums, the value
-                        //   q = S - 2 p.b + p.G.p
-                        // and the explicit residual sum both approximate
-                        // sum_k w_k (y_k - p.x_k)^2; their rounding errors are
-                        // at most (s^2 + 5s + 2K + 6) u M^2 together, with
-                        // M = ||y||_w + sum_a |p_a| ||x_a||_w (Cauchy-Schwarz,
-                        // Minkowski).  If q minus four times that bound is not
-                        // below the best explicit value of this size, the
-                        // subset can neither beat nor tie it (a tie goes to
-                        // the earlier subset), and its explicit sum is skipped.
-                        double q = syy, mm = sy;
-                        for (int a = 0; a < s; ++a) {
-                            q = __dsub_rn(q, __dmul_rn(__dmul_rn(2.0, p[a]), bv[idx[a] * T]));
-                            mm = __dadd_rn(mm, __dmul_rn(fabs(p[a]), sg[idx[a] * T]));
-                        }
-                        for (int a = 0; a < s; ++a)
-                            for (int c = 0; c < s; ++c)
-                                q = __dadd_rn(q, __dmul_rn(__dmul_rn(p[a], Gm[(idx[a] * MT + idx[c]) * T]), p[c]));
-                        const double bound = (double)(4 * (s * s + 6 * s + 2 * K + 8)) * 0x1p-53 * mm * mm;
-                        exact = !(__dsub_rn(q, bound) >= best_ls[s]);
-                    }
-                }
-                if (exact) {
-                    double r = 0.0;
-                    for (int k = 0; k < K; ++k) {
-                        double ek = yv[k * T];
-                        for (int a = 0; a < s; ++a)
-                            ek = __dsub_rn(ek, __dmul_rn(p[a], widen<TS>(X + (int64_t)cd[idx[a] * T] * Kp, k)));
-                        const double we = UNIT_W ? ek : __dmul_rn(A.w64[k], ek);
-                        r = __dadd_rn(r, __dmul_rn(we, ek));
-                    }
-                    if (!have[s] || r < best_ls[s]) {
-                        have[s] = true;
-                        best_ls[s] = r;
-                        for (int a = 0; a < s; ++a) {
-                            best_idx[s][a] = idx[a];
-                            best_p[s][a] = p[a];
-                        }
-                    }
-                }
-                // next subset in lexicographic order
-                int a = s - 1;
-                while (a >= 0 && idx[a] == m - s + a) --a;
-                if (a < 0) break;
-                ++idx[a];
-                for (int c = a + 1; c < s; ++c) idx[c] = idx[c - 1] + 1;
-            }
-        }
-        int chosen = 0;
-        if (syy > 0.0) {
-#pragma unroll
-            for (int s = 1; s <= kInterpMaxCaliber; ++s) {
-                if (!have[s]) continue;
-                const double cur = best_ls[chosen] / syy;
-                if (penalty_less(best_ls[s] / syy, cur, A.gamma * (double)(s - chosen))) chosen = s;
-            }
-        }
-        A.cnt[i] = chosen;
-        A.ls[i] = best_ls[chosen];
-#pragma unroll
-        for (int s = 1; s <= kInterpMaxCaliber; ++s) {
-            if (s != chosen) continue;
-            for (int a = 0; a < s; ++a) {
-                A.sel_col[(int64_t)i * kInterpMaxCaliber + a] = cd[best_idx[s][a] * T];
-                A.sel_val[(int64_t)i * kInterpMaxCaliber + a] = best_p[s][a];
-            }
-        }
+        search_row<TS, UNIT_W, MT>(A, X, i, m, syy, yv, Gm, bv, cd, T);
     }
+}
+
+// The same rows under unit weights, one launch per candidate count M (the rows
+// are grouped by it): the sums over the components run in registers, four
+// components of every candidate row at a time (32 bytes of an FP64 row per load),
+// and shared memory holds only what the subsets read.  The thread-per-row kernel
+// above keeps an 8 x 8 Gram matrix per thread in shared memory, which left two
+// blocks per SM and no L1 for its 8-byte gathers (call on the 9-point 512^2, K = 16
+// FP64, 157k fine rows: 1087 -> 1021 us).  Same rounding order.
+template <class TS> struct Chunk4;
+template <> struct Chunk4<double> {
+    double v[4];
+    __device__ __forceinline__ void load(const double *p)
+    {
+        uint4 a, b;
+        ldg32(p, a, b);
+        double lo[2], hi[2];
+        Store<double>::unpack(a, lo);
+        Store<double>::unpack(b, hi);
+        v[0] = lo[0]; v[1] = lo[1]; v[2] = hi[0]; v[3] = hi[1];
+    }
+};
+template <> struct Chunk4<float> {
+    float v[4];
+    __device__ __forceinline__ void load(const float *p)
+    {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    }
+};
+template <> struct Chunk4<__nv_bfloat16> {
+    __nv_bfloat16 v[4];
+    __device__ __forceinline__ void load(const __nv_bfloat16 *p)
+    {
+        const uint2 a = __ldg(reinterpret_cast<const uint2 *>(p));
+        v[0] = __ushort_as_bfloat16((unsigned short)a.x);
+        v[1] = __ushort_as_bfloat16((unsigned short)(a.x >> 16));
+        v[2] = __ushort_as_bfloat16((unsigned short)a.y);
+        v[3] = __ushort_as_bfloat16((unsigned short)(a.y >> 16));
+    }
+};
+
+template <class TS, int M>
+__global__ void __launch_bounds__(128) k_ls_interp_m(InterpArgs A)
+{
+    extern __shared__ __align__(16) double rsm[];
+    constexpr int T = 128, MT = M ? M : 1;
+    const int t = threadIdx.x, K = A.K, Kp = A.Kp;
+    double *yv = rsm + t;                        // y_k  at yv[k * T]
+    double *Gm = yv + (size_t)Kp * T;             // G_ab at Gm[(a * M + b) * T]
+    double *bv = Gm + (size_t)M * M * T;          // b_a  at bv[a * T]
+    int32_t *cd = reinterpret_cast<int32_t *>(rsm + (size_t)(Kp + M * M + M) * T) + t;
+    const TS *X = (const TS *)A.x;
+    int32_t first = 0;
+    for (int q = kInterpRowCand; q > M; --q) first += A.bcnt[q];
+    const int32_t last = first + A.bcnt[M];
+    // the launches of the other counts touch other rows: the next one may start at
+    // once, and this one only has to end after its predecessor
+    chain_release();
+    for (int32_t e = first + blockIdx.x * T + t; e < last; e += gridDim.x * T) {
+        const int32_t i = A.list[e];
+        const int p0 = A.rp[i], p1 = A.rp[i + 1];
+        double d = 1.0;
+        for (int p = p0; p < p1; ++p)
+            if (A.col[p] == i) d = A.val64[p];
+        const double c = -(1.0 / d);
+        int32_t cand[MT];
+        {
+            int m = 0;
+            const int q1 = A.prp[i + 1];
+            for (int q = A.prp[i]; q < q1; ++q) {
+                const int j = A.pcol[q];
+                if (A.coarse[j]) cd[(m++) * T] = j;
+            }
+#pragma unroll
+            for (int a = 0; a < M; ++a) cand[a] = cd[a * T];
+        }
+        double g[MT * (MT + 1) / 2], ba[MT], syy = 0.0;
+#pragma unroll
+        for (int a = 0; a < MT * (MT + 1) / 2; ++a) g[a] = 0.0;
+#pragma unroll
+        for (int a = 0; a < MT; ++a) ba[a] = 0.0;
+#pragma unroll 1
+        for (int k = 0; k < K; k += 4) {          // (components past K are zero in every row)
+            double y[4] = {0.0, 0.0, 0.0, 0.0};
+            Chunk4<TS> x;
+            if (A.target == 0)
+                for (int p = p0; p < p1; ++p) {
+                    x.load(X + (int64_t)A.col[p] * Kp + k);
+                    const double v = A.val64[p];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) y[q] = fma(v, widen_val<TS>(x.v[q]), y[q]);
+                }
+            x.load(X + (int64_t)i * Kp + k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const double xi = widen_val<TS>(x.v[q]);
+                y[q] = A.target == 0 ? fma(c, y[q], xi) : xi;
+                syy = __dadd_rn(syy, __dmul_rn(y[q], y[q]));
+                yv[(k + q) * T] = y[q];
+            }
+            Chunk4<TS> xc[MT];
+#pragma unroll
+            for (int a = 0; a < M; ++a) xc[a].load(X + (int64_t)cand[a] * Kp + k);
+#pragma unroll
+            for (int a = 0; a < M; ++a)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    ba[a] = __dadd_rn(ba[a], __dmul_rn(y[q], widen_val<TS>(xc[a].v[q])));
+#pragma unroll
+                    for (int b = a; b < M; ++b)
+                        g[b * (b + 1) / 2 + a] = __dadd_rn(g[b * (b + 1) / 2 + a],
+                                                           gram_term<TS, true>(xc[a].v[q], xc[b].v[q], 1.0));
+                }
+        }
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+            bv[a * T] = ba[a];
+#pragma unroll
+            for (int b = a; b < M; ++b) {
+                Gm[(a * M + b) * T] = g[b * (b + 1) / 2 + a];
+                Gm[(b * M + a) * T] = g[b * (b + 1) / 2 + a];
+            }
+        }
+        search_row<TS, true, M>(A, X, i, M, syy, yv, Gm, bv, cd, T);
+    }
+    chain_wait();
 }
 
 __global__ void k_interp_fill(const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ sel_col,
@@ -657,8 +797,8 @@ cudaError_t launch_rows_kernel(const InterpArgs &a, cudaStream_t s)
 {
     constexpr int T = 128;
     constexpr int MT = kInterpRowCand;
-    const size_t smem = (size_t)T * (8 * (a.K + MT * MT + 2 * MT) + 4 * MT);
-    constexpr size_t smem_max = (size_t)T * (8 * (kMaxK + MT * MT + 2 * MT) + 4 * MT);
+    const size_t smem = (size_t)T * (8 * (a.K + MT * MT + MT) + 4 * MT);
+    constexpr size_t smem_max = (size_t)T * (8 * (kMaxK + MT * MT + MT) + 4 * MT);
     static std::atomic<bool> opted[kOptDevices] = {};
     const cudaError_t e = opt_in_smem(k_ls_interp_rows<TS, UNIT_W>, opted, (int)smem_max);
     if (e != cudaSuccess) return e;
@@ -681,10 +821,33 @@ cudaError_t launch_warp_kernel(const InterpArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <class TS, int M>
+cudaError_t launch_m_kernels(const InterpArgs &a, cudaStream_t s)
+{
+    constexpr int T = 128;
+    auto bytes = [](int Kp) { return (size_t)T * (8 * (Kp + M * M + M) + 4 * M); };
+    static std::atomic<bool> opted[kOptDevices] = {};
+    cudaError_t e = opt_in_smem(k_ls_interp_m<TS, M>, opted, (int)bytes(kMaxK));
+    if (e != cudaSuccess) return e;
+    const int64_t want = ((int64_t)a.n + T - 1) / T;
+    const unsigned grid = (unsigned)(want < 152 * 6 ? want : 152 * 6);
+    if constexpr (M == kInterpRowCand) {
+        k_ls_interp_m<TS, M><<<grid, T, bytes(a.Kp), s>>>(a);
+        e = cudaGetLastError();
+    } else {
+        e = launch_chained(k_ls_interp_m<TS, M>, grid, T, bytes(a.Kp), s, a);
+    }
+    if (e != cudaSuccess) return e;
+    if constexpr (M > 0) return launch_m_kernels<TS, M - 1>(a, s);
+    return cudaSuccess;
+}
+
 template <class TS>
 cudaError_t launch_interp_typed(const InterpArgs &a, cudaStream_t s)
 {
-    cudaError_t e = a.unit_w ? launch_rows_kernel<TS, true>(a, s) : launch_rows_kernel<TS, false>(a, s);
+    // (rows of fewer than four components cannot be read four at a time)
+    cudaError_t e = a.unit_w && a.Kp >= 4 ? launch_m_kernels<TS, kInterpRowCand>(a, s)
+                  : a.unit_w ? launch_rows_kernel<TS, true>(a, s) : launch_rows_kernel<TS, false>(a, s);
     if (e != cudaSuccess) return e;
     return a.unit_w ? launch_warp_kernel<TS, true>(a, s) : launch_warp_kernel<TS, false>(a, s);
 }
