@@ -561,7 +561,6 @@ RelaxArgs sweep_args(amgd_ctx *h, double omega)
     a.diag = f64 ? (const void *)h->diag64 : (const void *)h->diag32;
     a.Kp = Kp_of(h->storage, h->K);
     a.omega = omega;
-    a.avg_nnz = h->n ? (float)((double)h->nnz / (double)h->n) : 0.f;
     a.nrows = (int32_t)h->n;
     if (h->sell_ok) {
         a.sell_ptr = h->sell_ptr;

@@ -286,7 +286,6 @@ struct RelaxArgs {
     int32_t split;        // rows < split take new values (earlier colors)
     int32_t Kp;           // padded row stride (elements)
     double omega;
-    float avg_nnz = 0.f;  // stored entries per row of the whole matrix
     int32_t nrows = 0;    // rows of the vector block (the range of a gather index)
     // sliced copy of the permuted matrix (NULL: none): slice q holds 32 rows of one
     // color, entry k of its row l at sell_ptr[q] + 32 k + l, column -1 past the row's end
@@ -392,9 +391,6 @@ cudaError_t launch_import(int storage, const double *src, void *x, const int32_t
                           int32_t n, int32_t K, int32_t Kp, cudaStream_t s);
 cudaError_t launch_export(int storage, const void *x, double *dst, const int32_t *perm,
                           int32_t n, int32_t K, int32_t Kp, cudaStream_t s);
-// convert vectors between storage types (same permutation and padding)
-cudaError_t launch_convert(int from, const void *src, int to, void *dst, int64_t count,
-                           cudaStream_t s);
 // per-slot outputs (arithmetic type of `storage`) -> doubles; NULL dst skipped
 cudaError_t launch_export_slots(int storage, const void *a_in, const void *ls_in,
                                 double *a, double *dist, double *ls, int64_t nnz,
@@ -405,10 +401,6 @@ cudaError_t launch_unpermute(int storage, const void *x, void *x_caller, const i
 // diagonal of every permuted row (double and float copies)
 cudaError_t launch_diagonal(const int32_t *rp_perm, const int32_t *col_perm, const double *vp64,
                             double *d64, float *d32, int32_t n, cudaStream_t s);
-// permuted values: vp[q] = v[slot of q in caller order] (double and float copies)
-cudaError_t launch_permute_values(const double *v, const int32_t *rp_orig,
-                                  const int32_t *perm, const int32_t *rp_perm, double *vp64,
-                                  float *vp32, int32_t n, cudaStream_t s);
 
 // every value copy that the queued kernels read, from caller-order values in
 // device memory, with the diagonals; NULL targets skipped; err (NULL: none) |= 1

@@ -205,13 +205,6 @@ __global__ void k_export(const TS *__restrict__ x, double *__restrict__ dst,
     dst[o * K + kappa] = to_double<TS>(x[r * Kp + kappa]);
 }
 
-template <class TF, class TT>
-__global__ void k_convert(const TF *__restrict__ src, TT *__restrict__ dst, int64_t count)
-{
-    const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (t < count) dst[t] = from_double<TT>(to_double<TF>(src[t]));
-}
-
 // 1 / l of an FP32 number in FP64 by long division in base 2^24: the FP32
 // reciprocal q1 is the first digit, the remainders 1 - l q1 and 1 - l (q1 + q2) are
 // exact FP32 numbers (one fused multiply-add each), their products with q1 the
@@ -262,22 +255,6 @@ __global__ void __launch_bounds__(kThreads) k_export_slots(const C *a_in, const 
         if (a) a[t] = widened(v[u]);
         if (ls) ls[t] = widened(l[u]);
         if (dist) dist[t] = reciprocal(l[u]);
-    }
-}
-
-__global__ void k_permute_values(const double *__restrict__ v, const int32_t *__restrict__ rp_orig,
-                                 const int32_t *__restrict__ perm, const int32_t *__restrict__ rp_perm,
-                                 double *__restrict__ vp64, float *__restrict__ vp32, int32_t n)
-{
-    const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (r >= n) return;
-    const int64_t o = perm ? perm[r] : r;
-    const int64_t s = rp_orig[o], d = rp_perm[r];
-    const int len = rp_orig[o + 1] - rp_orig[o];
-    for (int k = 0; k < len; ++k) {
-        const double x = v[s + k];
-        if (vp64) vp64[d + k] = x;
-        if (vp32) vp32[d + k] = (float)x;
     }
 }
 
@@ -546,34 +523,6 @@ cudaError_t launch_export(int storage, const void *x, double *dst, const int32_t
     return cudaGetLastError();
 }
 
-namespace {
-template <class TF>
-cudaError_t convert_to(const TF *src, int to, void *dst, int64_t count, cudaStream_t s)
-{
-    switch (to) {
-    case ST_FP64: k_convert<<<blocks(count), kThreads, 0, s>>>(src, (double *)dst, count); break;
-    case ST_FP32: k_convert<<<blocks(count), kThreads, 0, s>>>(src, (float *)dst, count); break;
-    case ST_BF16:
-        k_convert<<<blocks(count), kThreads, 0, s>>>(src, (__nv_bfloat16 *)dst, count);
-        break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-}  // namespace
-
-cudaError_t launch_convert(int from, const void *src, int to, void *dst, int64_t count,
-                           cudaStream_t s)
-{
-    if (count == 0) return cudaSuccess;
-    switch (from) {
-    case ST_FP64: return convert_to((const double *)src, to, dst, count, s);
-    case ST_FP32: return convert_to((const float *)src, to, dst, count, s);
-    case ST_BF16: return convert_to((const __nv_bfloat16 *)src, to, dst, count, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
 cudaError_t launch_export_slots(int storage, const void *a_in, const void *ls_in, double *a,
                                 double *dist, double *ls, int64_t nnz, cudaStream_t s)
 {
@@ -651,15 +600,6 @@ cudaError_t launch_diag_values(const double *v, const int32_t *diag_slot, const 
     if (n == 0) return cudaSuccess;
     k_diag_values<<<blocks(n), kThreads, 0, s>>>(v, diag_slot, perm, n, d64_o, d32_o, d64_p, d32_p,
                                                 err);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_permute_values(const double *v, const int32_t *rp_orig, const int32_t *perm,
-                                  const int32_t *rp_perm, double *vp64, float *vp32, int32_t n,
-                                  cudaStream_t s)
-{
-    if (n == 0) return cudaSuccess;
-    k_permute_values<<<blocks(n), kThreads, 0, s>>>(v, rp_orig, perm, rp_perm, vp64, vp32, n);
     return cudaGetLastError();
 }
 
