@@ -801,21 +801,21 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
     };
     bool on_device = mem == AMGD_MEM_DEVICE;
     if (on_device) {
-        // the entry counts; the rest of the matrix stays where it is
-        for (int32_t b = 0; b < nmat; ++b) {
-            if (!rp_in[b]) return fail(nullptr, AMGD_ERR_ARG, "NULL row_ptr");
+        // the entry counts; the rest of the matrix stays where it is.  What the host
+        // form refuses it refuses below, so that the first fault is the one named
+        for (int32_t b = 0; b < nmat && on_device; ++b) {
             int64_t ends[2] = {0, 0};
-            cudaError_t e = fetch(&ends[0], rp_in[b], sizeof(int64_t), mem);
-            if (e == cudaSuccess) e = fetch(&ends[1], rp_in[b] + n_in[b], sizeof(int64_t), mem);
+            cudaError_t e = cudaSuccess;
+            if (rp_in[b]) e = fetch(&ends[0], rp_in[b], sizeof(int64_t), mem);
+            if (rp_in[b] && e == cudaSuccess) e = fetch(&ends[1], rp_in[b] + n_in[b], sizeof(int64_t), mem);
             if (e != cudaSuccess) return cuda_fail(nullptr, e, "copy row_ptr");
-            if (ends[0] != 0) return fail(nullptr, AMGD_ERR_CSR, "row_ptr[0] != 0");
-            if (ends[1] < 0) return fail(nullptr, AMGD_ERR_CSR, "negative nnz");
-            if (slot_off.back() + ends[1] >= ((int64_t)1 << 31) - 16)
-                return fail(nullptr, AMGD_ERR_UNSUPPORTED, "nnz >= 2^31");
-            if (ends[1] > 0 && (!col_in[b] || !val_in[b])) return fail(nullptr, AMGD_ERR_ARG, "NULL col/val");
-            slot_off.push_back(slot_off.back() + ends[1]);
+            on_device = rp_in[b] && ends[0] == 0 && ends[1] >= 0 &&
+                        slot_off.back() + ends[1] < ((int64_t)1 << 31) - 16 &&
+                        (ends[1] == 0 || (col_in[b] && val_in[b]));
+            if (on_device) slot_off.push_back(slot_off.back() + ends[1]);
         }
-    } else {
+    }
+    if (!on_device) {
         const int rc = load_host();
         if (rc != AMGD_OK) return rc;
     }

@@ -1,0 +1,324 @@
+"""The kernels' dispatch edges on the GPU against the oracle.
+
+Sweeps keep the rounding order of the definition on every route (the row's own
+CSR entries or the sliced copy of the matrix that repeated sweeps read), so
+FP64 vectors are compared bit for bit with the oracle and FP32/BF16 vectors bit
+for bit between the two routes.  Distances are held to the parity rules of
+parity.py; strength patterns, interpolation and everything a handle built from
+device memory returns are compared exactly."""
+import ctypes
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1106_5990_gb300 import inputs
+from test_gpu_adjoint import rel, run_gpu, x0
+from test_gpu_parity import arrow, compare_fp64, gpu_build
+
+pytestmark = pytest.mark.gpu
+amgd = pytest.importorskip("paper_1106_5990_gb300.amgd")
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1106_5990_gb300 import _build
+    _build.build()
+
+
+# slices of 32 rows and their remainders; 2 to 9 entries in a slice's width;
+# rows sorted by length within windows (uneven rows); one row far too long for a
+# slice (the sweeps stay on the CSR)
+SWEEPS = {
+    "lap1d_31": lambda: inputs.lap1d(31),
+    "lap1d_33": lambda: inputs.lap1d(33),
+    "poisson5_37": lambda: inputs.poisson2d_5pt(37),
+    "aniso7_33": lambda: inputs.aniso2d_7pt(33, 0.1, -math.pi / 4),
+    "aniso9_66": lambda: inputs.aniso2d_9pt(66, 1e-3, math.pi / 6),
+    "graph_4129": lambda: inputs.graph_laplacian(4129, 8.0, 4),
+    "arrow_3001": lambda: arrow(3001),
+}
+
+
+@pytest.mark.parametrize("name", list(SWEEPS))
+@pytest.mark.parametrize("K", [1, 5, 8, 32, 64])
+@pytest.mark.parametrize("sweep", ["jacobi", "mcgs"])
+def test_repeated_sweeps_and_new_values(name, K, sweep):
+    rp, col, val = SWEEPS[name]()
+    n = len(rp) - 1
+    color = inputs.greedy_coloring(rp, col) if sweep == "mcgs" else None
+    mode, omode = (amgd.AMGD_SWEEP_MCGS, oracle.SWEEP_MCGS) if color is not None else (amgd.AMGD_SWEEP_JACOBI, 0)
+    rng = np.random.default_rng(8)
+    val2, val3, val4 = (val * (1 + 0.01 * rng.random(len(val))) for _ in range(3))
+    with amgd.Handle(rp, col, val, K, 7) as h:
+        if color is not None:
+            h.set_coloring(color)
+        X = oracle.tv_init(n, K, 7)
+        for v, nu in ((None, 1), (None, 2), (val2, 2)):
+            if v is not None:
+                h.set_values(v)
+            X = oracle.relax(rp, col, val if v is None else v, X, nu, 0.9, omode, color)
+            h.relax(nu, 0.9, mode)
+            assert np.array_equal(h.get_vectors(), X), nu
+        h.set_values_async(torch.from_numpy(val3).cuda())
+        h.relax(1, 0.9, mode)
+        h.sync()
+        X = oracle.relax(rp, col, val3, X, 1, 0.9, omode, color)
+        assert np.array_equal(h.get_vectors(), X)
+        # back to the CSR kernels, whose value copies the updates left out of date
+        G, NV, U, _ = h.kernel_shape(amgd.AMGD_KERNEL_RELAX)
+        try:
+            h.set_kernel_shape(amgd.AMGD_KERNEL_RELAX, G, NV, U, 1)
+        except amgd.AmgdError:
+            return                               # this shape's stage exceeds the shared memory
+        h.relax(1, 0.9, mode)
+        X = oracle.relax(rp, col, val3, X, 1, 0.9, omode, color)
+        assert np.array_equal(h.get_vectors(), X)
+        h.set_values(val4)
+        h.relax(1, 0.9, mode)
+        X = oracle.relax(rp, col, val4, X, 1, 0.9, omode, color)
+        assert np.array_equal(h.get_vectors(), X)
+
+
+@pytest.mark.parametrize("name", ["aniso9_66", "graph_4129", "lap1d_33"])
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("K", [3, 16, 64])
+def test_both_sweep_routes_round_alike(name, prec, K):
+    rp, col, val = SWEEPS[name]()
+    color = inputs.greedy_coloring(rp, col)
+    out = []
+    for parts in ((3,), (1, 2)):                 # the second call of a handle reads the sliced copy
+        with amgd.Handle(rp, col, val, K, 7) as h:
+            h.set_precision(prec)
+            h.set_coloring(color)
+            h.init_vectors(7)
+            for nu in parts:
+                h.relax(nu, 1.1, amgd.AMGD_SWEEP_MCGS)
+            out.append(h.get_vectors())
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("K", [2, 13, 33, 64])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("name", ["lap1d_31", "graph_4129", "arrow_3001"])
+def test_distances_with_zero_columns(name, K, weighted):
+    """Few and many rows, rows longer than a batch; some vectors' rows are zero
+    (S_xx = 0: a = 0, LS = S_yy).  LS in extended precision from the oracle's target:
+    the oracle's unfused products alone err by up to 1.2e-12 of an LS of 1e-8 S_yy."""
+    rp, col, val = SWEEPS[name]()
+    n = len(rp) - 1
+    w = np.random.default_rng(1).uniform(0.5, 2.0, K) if weighted else None
+    X = oracle.tv_init(n, K, 5)
+    X[::7] = 0.0
+    got = gpu_build(rp, col, val, K, 5, 0, 1.0, 0.5, w=w, X0=X)
+    Y = oracle.target(rp, col, val, X)
+    a, ls = oracle.edge_ls(rp, col, val, X, Y, w)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    fit = (rows != col) & (np.diff(rp)[rows] != 2)          # one off-diagonal: LS = 0 exactly
+    x, y = X[col[fit]].astype(np.longdouble), Y[rows[fit]].astype(np.longdouble)
+    wl = np.ones(K, np.longdouble) if w is None else w.astype(np.longdouble)
+    xx = (wl * x * x).sum(1)
+    q = (wl * x * y).sum(1) / np.where(xx == 0, 1, xx)
+    ls[fit] = (wl * (y - q[:, None] * x) ** 2).sum(1)
+    want = dict(X=X, Y=Y, a=a, ls=ls, flag=oracle.threshold(rp, col, ls, 0.5)[0])
+    compare_fp64(rp, col, val, got, want, 0.5, w)
+
+
+def test_reciprocals_of_the_fp32_range():
+    """dist = 1 / LS of the FP32 path over the type's whole range: equal to the
+    FP64 quotient of the exported LS to one unit of its last place."""
+    rp, col, val = inputs.graph_laplacian(4129, 8.0, 4)
+    n = len(rp) - 1
+    rng = np.random.default_rng(2)
+    X = rng.standard_normal((n, 4)) * 10.0 ** rng.uniform(-19, 18, (n, 1))
+    X[::50] = 0.0
+    with amgd.Handle(rp, col, val, 4, 1) as h:
+        h.set_precision("fp32")
+        h.set_target(1)
+        h.set_vectors(X)
+        d = h.distances(0.5)
+    ls, dist = d["ls"], d["dist"]
+    assert np.array_equal(np.isnan(ls), np.isnan(dist))
+    ok = ~np.isnan(ls)
+    assert (ls[ok] == 0).any() and (ls[ok] > 1e30).any() and ((ls[ok] > 0) & (ls[ok] < 1e-30)).any()
+    with np.errstate(divide="ignore"):
+        want = 1.0 / ls[ok]
+    inf = np.isinf(want)
+    assert np.array_equal(dist[ok][inf], want[inf])
+    assert np.all(np.abs(dist[ok][~inf] - want[~inf]) <= np.spacing(want[~inf]))
+
+
+@pytest.mark.parametrize("n", [32767, 32768, 32769, 2048 * 1024, 2048 * 1024 + 1])
+def test_strength_at_the_compaction_edges(n):
+    rp, col, val = inputs.lap1d(n)
+    with amgd.Handle(rp, col, val, 2, 3) as h:
+        h.relax(1, 0.7)
+        ls = h.distances(0.5, want=("ls",))["ls"]
+        s_rp, s_col = h.strength()
+    flag = oracle.threshold(rp, col, ls, 0.5)[0]
+    w_rp, w_col = oracle.strength_csr(rp, col, flag)
+    assert np.array_equal(s_rp, w_rp) and np.array_equal(s_col, w_col)
+
+
+def shuffled(rp, col, val, seed):
+    """The same rows with their entries in random order."""
+    rng = np.random.default_rng(seed)
+    rows = np.repeat(np.arange(len(rp) - 1), np.diff(rp))
+    o = np.lexsort((rng.random(len(col)), rows))
+    return rp, col[o], val[o]
+
+
+def device(m):
+    return [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in m]
+
+
+@pytest.mark.parametrize("name,order", [("aniso9_66", "sorted"), ("graph_4129", "shuffled"), ("arrow_3001", "shuffled"),
+                                        ("lap1d_31", "sorted")])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_create_from_device_memory(name, order, prec):
+    m = SWEEPS[name]()
+    if order == "shuffled":
+        m = shuffled(*m, 3)                      # arrow: a row of 3001 entries out of order
+    color = inputs.greedy_coloring(m[0], m[1])
+    out = []
+    for mat in (m, device(m)):
+        with amgd.Handle(*mat, 8, 4) as h:
+            h.set_precision(prec)
+            h.init_vectors(4)
+            h.relax(1, 0.8)
+            h.set_coloring(color)                # reads the pattern on the host
+            h.relax(2, 1.0, amgd.AMGD_SWEEP_MCGS)
+            d = h.distances(0.5)
+            s = h.strength()
+            h.set_search_depth(2)
+            d2 = h.distances(0.5, want=("ls",))
+            out.append([h.get_vectors(), d["a"], d["ls"], d["dist"], s[0], s[1], d2["ls"]])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16"])
+def test_batch_create_from_device_memory(prec):
+    mats = [inputs.graph_laplacian(k, 8.0, 4, b) for b, k in enumerate((700, 33, 1100))]
+    dev = [device(m) for m in mats]
+    L, hs = amgd.lib(), []
+    ns = np.array([len(m[0]) - 1 for m in mats], np.int64)
+    for group, ptr, mem in ((mats, lambda x: x.ctypes.data, amgd.AMGD_MEM_HOST),
+                            (dev, lambda x: x.data_ptr(), amgd.AMGD_MEM_DEVICE)):
+        arr = [(ctypes.c_void_p * 3)(*[ptr(m[k]) for m in group]) for k in range(3)]
+        h = amgd.Handle(batch=mats, row_ptr=None, col=None, val=None, K=16, seed=6)
+        if mem == amgd.AMGD_MEM_DEVICE:
+            h.close()
+            h.h = ctypes.c_void_p()
+            amgd.check(L.amgd_create_batch(3, *arr, ns.ctypes.data, 16, 6, mem, ctypes.byref(h.h)))
+        h.set_precision(prec)
+        h.init_vectors(6)
+        h.relax(3, 0.7)
+        hs.append((h.distances(0.5)["ls"], h.get_vectors(), *h.strength()))
+        h.close()
+    for a, b in zip(*hs):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
+def _bad(kind):
+    rp, col, val = (x.copy() for x in (arrow(2001) if kind == "duplicate_long" else inputs.aniso2d_9pt(40, 1e-3, 0.3)))
+    i = 0 if kind == "duplicate_long" else 700
+    a, b = int(rp[i]), int(rp[i + 1])
+    d = a + int(np.nonzero(col[a:b] == i)[0][0])
+    if kind == "row_ptr":
+        rp[i] = rp[i + 1] + 3
+    elif kind == "row_ptr_start":
+        rp[0] = 1
+    elif kind == "row_ptr_past_the_end":
+        rp[i] = rp[-1] + 5
+    elif kind == "column_high":
+        col[b - 1] = len(rp) - 1
+    elif kind == "column_negative":
+        col[a] = -1
+    elif kind.startswith("duplicate"):
+        col[a + 1 if d != a + 1 else a + 2] = col[b - 1]
+    elif kind == "nan":
+        val[a] = np.nan
+    elif kind == "inf":
+        val[b - 1] = np.inf
+    elif kind == "zero_diagonal":
+        val[d] = 0.0
+    elif kind == "no_diagonal":
+        j = np.setdiff1d(np.arange(len(rp) - 1), col[a:b])[0]
+        col[d] = j
+    return rp, col, val
+
+
+@pytest.mark.parametrize("kind", ["row_ptr", "row_ptr_start", "row_ptr_past_the_end", "column_high", "column_negative",
+                                  "duplicate", "duplicate_long", "nan", "inf", "zero_diagonal", "no_diagonal"])
+def test_create_refuses_alike_from_host_and_device(kind):
+    m = _bad(kind)
+    codes = []
+    for mat in (m, device(m)):
+        with pytest.raises(amgd.AmgdError) as e:
+            amgd.Handle(*mat, 4, 1)
+        codes.append(e.value.status)
+    assert codes[0] == codes[1]
+
+
+def test_a_batch_names_its_first_fault():
+    mats = [_bad("zero_diagonal"), _bad("row_ptr_start")]
+    dev = [device(m) for m in mats]
+    ns = np.array([len(m[0]) - 1 for m in mats], np.int64)
+    codes = []
+    for group, ptr, mem in ((mats, lambda x: x.ctypes.data, amgd.AMGD_MEM_HOST),
+                            (dev, lambda x: x.data_ptr(), amgd.AMGD_MEM_DEVICE)):
+        arr = [(ctypes.c_void_p * 2)(*[ptr(m[k]) for m in group]) for k in range(3)]
+        h = ctypes.c_void_p()
+        codes.append(amgd.lib().amgd_create_batch(2, *arr, ns.ctypes.data, 4, 1, mem, ctypes.byref(h)))
+    assert codes[0] == codes[1] != 0
+
+
+@pytest.mark.parametrize("K", [2, 3, 4, 6, 17, 64])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
+def test_interpolation_of_every_candidate_count(K, prec):
+    """Unit weights, 0 to 8 and more candidates in a row; K below, at and off the
+    four components that a load takes."""
+    rp, col, val = inputs.random_csr(700, 2.5, 21, symmetric_pattern=True)
+    n = len(rp) - 1
+    coarse = (np.random.default_rng(3).random(n) < 0.45).astype(np.uint8)
+    X = oracle.relax(rp, col, val, oracle.tv_init(n, K, 2), 2, 0.7)
+    if prec != "fp64":
+        X = torch.from_numpy(X).to(torch.bfloat16 if prec == "bf16" else torch.float32).to(torch.float64).numpy()
+    prp, pcol = oracle.distance_graph(rp, col, 2)
+    rows = np.repeat(np.arange(n), np.diff(prp))
+    m = np.bincount(rows[coarse[pcol] == 1], minlength=n)[coarse == 0]
+    assert set(range(9)) <= set(m.tolist())
+    Y = oracle.target(rp, col, val, X)
+    for caliber in (1, 3):
+        with amgd.Handle(rp, col, val, K, 2) as h:
+            h.set_precision(prec)
+            h.set_search_depth(2)
+            h.set_vectors(X)
+            got = h.ls_interpolation(coarse, caliber, 1.5)
+        for g, w_ in zip(got, oracle.ls_interp(X, Y, prp, pcol, coarse, caliber, 1.5)):
+            assert np.array_equal(g, w_)
+
+
+@pytest.mark.parametrize("K", [4, 8, 16, 32, 64])
+@pytest.mark.parametrize("pattern", ["symmetric", "general"])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_reverse_pass_of_every_row_width(K, pattern, weighted):
+    """1 to 32 lanes per row, the row's entries shared among them.  FP64 storage:
+    1e-11 of the oracle's gradient.  FP32 and BF16 storage without sweeps, from
+    start vectors that are exact in the type: the fits alone, in 48 bits or more
+    (2^-48 over sums of a few thousand terms: 1e-10)."""
+    mat = inputs.random_csr(300, 6.0, 9, symmetric_pattern=pattern == "symmetric")
+    w = np.random.default_rng(1).uniform(0.5, 2.0, K) if weighted else None
+    lsb = np.random.default_rng(5).standard_normal(len(mat[1]))
+    for prec, nu, tol in (("fp64", 3, 1e-11), ("fp32", 0, 1e-10), ("bf16", 0, 1e-10)):
+        g = run_gpu(mat, K, 7, nu, 0.6, 0.5, 2, prec=prec, w=w, ls_bar=lsb)
+        X0 = g["X0"]                             # the draws rounded to the type (its own tests pin them)
+        if prec == "fp64":
+            assert np.array_equal(X0, x0(mat, K, 7))
+        o = oracle.adjoint_jacobi(*mat, X0, nu, 0.6, 0.5, w, 0, ls_bar=lsb)
+        assert rel(g["val_bar"], o["val_bar"]) <= tol, prec
