@@ -324,8 +324,11 @@ int amgd_graph_launch(amgd_handle h);
  *   use (waits bounded to about one second; a wait that runs out makes the
  *   next synchronising call return AMGD_ERR_TIMEOUT); 2 warp-pipelined, CSR
  *   slices and neighbour rows copied with cp.async two and one row groups
- *   ahead (U must be 4); 3 accepted and kept, the same kernel as 0, which
- *   chooses its lanes, batch and blocks by the row's size and the matrix.
+ *   ahead (U must be 4); 3 one block per SM on a contiguous chunk of CSR rows.
+ *   Repeated sweeps of kernel 0 read a sliced copy of the matrix and choose
+ *   their lanes, batch and blocks by the row's size and the matrix, unless
+ *   amgd_autotune found the handle's sweeps faster on the CSR in a shape of
+ *   kernel 0, which they then run in.
  *   The distance pass has one kernel, chosen by the row's size alone: every
  *   shape in the range above (stage 2 with U in {2,4}, stage 3 with U in
  *   {4,8}) is accepted and kept, and all of them run it.  Shapes change speed
@@ -334,7 +337,8 @@ int amgd_graph_launch(amgd_handle h);
  *   storage precision.
  * amgd_autotune times every valid shape of the sweeps on the handle's own
  *   matrix and vectors (one sweep of sweep_type/omega into the spare vector
- *   buffer -- the current vectors are kept) and keeps the fastest, and times
+ *   buffer -- the current vectors are kept) on the CSR, and the sliced copy,
+ *   and keeps the fastest, and times
  *   the distance pass for the record (computed distances are invalidated).  cache_path
  *   (may be NULL): a text file of earlier results keyed by GPU name,
  *   storage, K, size buckets, sweep type and color count; a matching line

@@ -58,6 +58,7 @@ struct amgd_ctx {
     std::vector<int64_t> color_start;           // permuted row start of each color
     // sliced copy of the permuted matrix (built by ensure_sell for the sweeps)
     int64_t sweep_calls = 0;                     // sweep calls prepared so far
+    bool relax_csr[3] = {false, false, false};   // per storage: the tuner found kernel 0 faster on the CSR
     bool sell_tried = false;                     // for the current coloring
     bool sell_ok = false;                        // the copy exists (else its padding was too much)
     int64_t sell_entries = 0;
@@ -355,12 +356,11 @@ int upload_weights(amgd_ctx *h)
     return AMGD_OK;
 }
 
-// whether the sweeps read the row-permuted CSR (the staged kernels, or no sliced
+// whether the sweeps read the row-permuted CSR (a kernel chosen by stage, or no sliced
 // copy) instead of the sliced copy
 bool sweeps_use_csr(const amgd_ctx *h)
 {
-    const int st = h->relax_shape[h->storage].stage;
-    return st == 1 || st == 2 || !h->sell_ok;
+    return h->relax_shape[h->storage].stage != 0 || h->relax_csr[h->storage] || !h->sell_ok;
 }
 
 // Every value copy that queued work reads, from the caller-order values (src,
@@ -532,7 +532,7 @@ int prepare_sweeps(amgd_ctx *h, size_t bytes, cudaStream_t s)
     const int stage = h->relax_shape[h->storage].stage;
     const bool repeated = h->sweep_calls > 0 || bytes >= kWorth;
     ++h->sweep_calls;
-    if ((stage == 0 || stage == 3) && (repeated || h->sell_ok)) {
+    if (stage == 0 && !h->relax_csr[h->storage] && (repeated || h->sell_ok)) {
         const int rc = ensure_sell(h);
         if (rc != AMGD_OK) return rc;
     }
@@ -562,7 +562,7 @@ RelaxArgs sweep_args(amgd_ctx *h, double omega)
     a.Kp = Kp_of(h->storage, h->K);
     a.omega = omega;
     a.nrows = (int32_t)h->n;
-    if (h->sell_ok) {
+    if (!sweeps_use_csr(h)) {
         a.sell_ptr = h->sell_ptr;
         a.sell_col = h->sell_col;
         a.sell_val = f64 ? (const void *)h->sell_val64 : (const void *)h->sell_val32;
@@ -1646,25 +1646,30 @@ int amgd_autotune(amgd_handle h, int sweep_type, double omega, const char *cache
         if (f) {
             char buf[1024];
             Shape r{0, 0, 0, 0}, e{0, 0, 0, 0};
-            bool found = false;
+            bool found = false, csr = false;
             while (fgets(buf, sizeof buf, f)) {
                 std::string line(buf);
                 if (line.compare(0, key.size(), key) == 0 && line.size() > key.size() &&
                     line[key.size()] == ';' && parse_shape(line, "relax", r) &&
                     parse_shape(line, "edge", e) && shape_ok(h->storage, h->K, r) &&
                     shape_ok(h->storage, h->K, e) && edge_shape_ok(e) &&
-                    relax_shape_available(h->storage, r))
+                    relax_shape_available(h->storage, r)) {
                     found = true;       // the last matching line wins
+                    csr = line.find(";sliced=1") == std::string::npos;
+                }
             }
             fclose(f);
             if (found) {
                 h->relax_shape[h->storage] = r;
+                h->relax_csr[h->storage] = csr;
                 h->edge_shape[h->storage] = e;
                 return AMGD_OK;
             }
         }
     }
-    std::vector<Shape> cands;
+    const Shape keep_r = h->relax_shape[h->storage], best_e = h->edge_shape[h->storage];
+    // the sliced copy, whose kernel chooses its own shape, then every kernel on the CSR
+    std::vector<Shape> cands(1, Shape{keep_r.G, keep_r.NV, keep_r.U, 0});
     const int P = P_of(h->storage, h->K);
     for (int stage : {0, 1, 2, 3})
         for (int NV : {1, 2, 4})
@@ -1672,43 +1677,54 @@ int amgd_autotune(amgd_handle h, int sweep_type, double omega, const char *cache
                 if (P % NV == 0 && shape_ok(h->storage, h->K, Shape{P / NV, NV, U, stage}) &&
                     relax_shape_available(h->storage, Shape{P / NV, NV, U, stage}))
                     cands.push_back(Shape{P / NV, NV, U, stage});
-    const Shape keep_r = h->relax_shape[h->storage], best_e = h->edge_shape[h->storage];
     const int cur = h->cur;
     Shape best_r = keep_r;
+    bool &on_csr = h->relax_csr[h->storage];
+    const bool keep_csr = on_csr;
+    bool best_csr = false;
+    auto restore = [&](int rc) {
+        h->relax_shape[h->storage] = keep_r;
+        on_csr = keep_csr;
+        return rc;
+    };
     float tr = 1e30f, te = 1e30f;
     for (const Shape &c : cands) {
         float ms = 0.f;
         h->relax_shape[h->storage] = c;
+        on_csr = &c != &cands[0];
         {
             const int prc = prepare_sweeps(h, h->stream);
-            if (prc != AMGD_OK) { h->relax_shape[h->storage] = keep_r; return prc; }
+            if (prc != AMGD_OK) return restore(prc);
         }
+        if (!on_csr && sweeps_use_csr(h)) continue;            // no sliced copy of this matrix
         // one sweep from the current vectors into the spare buffer (the
         // current vectors are not touched), then restore the buffer index
         int rc = time_ms(h, [&]() { int q = run_relax(h, 1, omega, sweep_type, h->stream); h->cur = cur; return q; }, 5, ms);
-        if (rc != AMGD_OK) { h->relax_shape[h->storage] = keep_r; return rc; }
-        if (ms < tr) { tr = ms; best_r = c; }
+        if (rc != AMGD_OK) return restore(rc);
+        if (ms < tr) { tr = ms; best_r = c; best_csr = on_csr; }
         {
             const int prc = poll_status(h);
-            if (prc != AMGD_OK) { h->relax_shape[h->storage] = keep_r; return prc; }
+            if (prc != AMGD_OK) return restore(prc);
         }
     }
     // the distance pass has one kernel for every shape: timed once for the record
     {
         const int rc = time_ms(h, [&]() { return run_edge(h, 0.5, h->stream); }, 5, te);
-        if (rc != AMGD_OK) return rc;
+        if (rc != AMGD_OK) return restore(rc);
     }
     h->relax_shape[h->storage] = best_r;
     h->edge_shape[h->storage] = best_e;
+    on_csr = best_csr;
+    if (on_csr && !h->gexec) drop_sell(h);                // value updates need not keep it current
     h->cur = cur;
     h->have_dist = false;
     h->traj_valid = false;
     if (cache_path) {
         FILE *f = fopen(cache_path, "a");
         if (f) {
-            fprintf(f, "%s;relax=%d,%d,%d,%d;edge=%d,%d,%d,%d;relax_ms=%.5f;edge_ms=%.5f\n",
+            fprintf(f, "%s;relax=%d,%d,%d,%d;edge=%d,%d,%d,%d;sliced=%d;relax_ms=%.5f;edge_ms=%.5f\n",
                     key.c_str(), best_r.G, best_r.NV, best_r.U, best_r.stage, best_e.G, best_e.NV,
-                    best_e.U, best_e.stage, tr, te);
+                    best_e.U, best_e.stage, best_csr ? 0 : 1, tr, te);
             fclose(f);
         }
     }

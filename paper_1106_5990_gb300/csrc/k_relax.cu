@@ -690,6 +690,200 @@ __global__ void __launch_bounds__(SellShape<TS, P>::THREADS, 1) k_relax_sell(Rel
     }
 }
 
+// Chunked persistent variant (stage 3).  One block of kChunkThreads threads
+// per SM owns one contiguous chunk of rows; its warps walk the chunk side by
+// side in groups of RW = 32/G rows (group g of the chunk goes to warp g mod W),
+// so the whole SM moves through consecutive rows together.  On matrices whose
+// neighbours are close in the row order (stencils on grid lines, banded and
+// mesh orderings) the rows an SM gathers are then the few grid lines around
+// its current position, and a line fetched into L1 for one row serves the
+// rows of the next lines too: the L2 -> L1 traffic of the gathers drops from
+// one copy of each vector row per block that touches it towards one per SM.
+// Each warp also asks the L2 for the row-pointer line of its group after next
+// and for the column-index and value lines of its next group (their bounds
+// come from the row pointers prefetched one group earlier), so a row's first
+// two dependent round trips hit L2.  L2 policy: the test-vector block (read
+// by the gathers, written by the update) is loaded and stored with an
+// evict-last hint and the CSR, which streams through once per sweep, with an
+// evict-first hint, so the vectors of the next color phase and sweep tend to
+// stay in the 129 MB L2 instead of being pushed out by the matrix.  Same row
+// sums in the same order as k_relax: same bits.  The tuner times it, the direct
+// kernel and the sliced copy (us per color phase of a tuned handle: 9-point 1024^2
+// K = 16 FP32 31.3 against 32.4 of the sliced copy, BF16 20.2 / 21.4; 7-point 128^3
+// K = 32 FP32 194 of the direct kernel against 199; graphs and FP64 the sliced copy;
+// untuned sweeps always take it).  896 threads (28 warps): the
+// register budget of 72 per thread holds a batch of four 64-byte rows per lane
+// pair without spilling (at 1024 threads, 64 registers spilled and the sweep
+// was 10% slower; 768 threads were 4% slower, and at 640 the direct kernel
+// wins).
+constexpr int kChunkThreads = 896;
+
+__device__ __forceinline__ uint64_t policy_evict_last()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint64_t policy_evict_first()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint4 ldg16_hint(const void *p, uint64_t pol)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ void st16_hint(void *p, const uint4 &v, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(p), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
+                 : "memory");
+}
+// 32-byte vector load / store (sm_100 and later; the address is 32-byte aligned)
+__device__ __forceinline__ void ldg32_hint(const void *p, uint64_t pol, uint4 &a, uint4 &b)
+{
+    asm volatile("ld.global.nc.L2::cache_hint.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p), "l"(pol));
+}
+__device__ __forceinline__ void st32_hint(void *p, const uint4 &a, const uint4 &b, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;" ::"l"(p),
+                 "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "l"(pol)
+                 : "memory");
+}
+__device__ __forceinline__ int32_t ld32_hint(const int32_t *p, uint64_t pol)
+{
+    int32_t v;
+    asm volatile("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float ldv_hint(const float *p, uint64_t pol)
+{
+    float v;
+    asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ double ldv_hint(const double *p, uint64_t pol)
+{
+    double v;
+    asm volatile("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
+    return v;
+}
+
+template <class TS, int G, int NV, int U, bool SPLIT>
+__global__ void __launch_bounds__(kChunkThreads, 1) k_relax_chunk(RelaxArgs A, int32_t chunk)
+{
+    using S = Store<TS>;
+    using C = typename S::C;
+    using AV = typename S::A;
+    constexpr int V = S::V, RW = 32 / G, NW = kChunkThreads / 32;
+    constexpr int64_t STEP = (int64_t)NW * RW;            // rows between a warp's groups
+    const int warp = threadIdx.x / 32, lane32 = threadIdx.x % 32;
+    const int lane = lane32 % G, rig = lane32 / G;
+    const TS *xold = (const TS *)A.xold;
+    TS *xnew = (TS *)A.xnew;
+    const AV *val = (const AV *)A.val;
+    const int32_t *col = A.col;
+    const int Kp = A.Kp;
+    const int64_t c0 = (int64_t)A.r0 + (int64_t)blockIdx.x * chunk;
+    const int64_t c1 = min((int64_t)A.r1, c0 + chunk);
+    const uint64_t keep = policy_evict_last(), stream = policy_evict_first();
+    // a lane holding an even number of pieces holds them side by side and moves
+    // them two at a time (32-byte accesses: half the load instructions and
+    // cache wavefronts of a gather); otherwise the pieces interleave over the
+    // G lanes.  Every component keeps its own FMA chain, so both layouts give
+    // the same bits.
+    constexpr bool W32 = NV % 2 == 0;
+    auto piece = [&](int tt) { return W32 ? lane * NV + tt : tt * G + lane; };
+
+    for (int64_t wr0 = c0 + (int64_t)warp * RW; wr0 < c1; wr0 += STEP) {
+        // row pointers of this warp's group after next, into L2
+        if (lane32 == 0 && wr0 + 2 * STEP < c1) prefetch_l2(A.rp + wr0 + 2 * STEP);
+        // bounds of this warp's next group (its row pointers were prefetched)
+        int n0 = 0, n1 = 0;
+        if (wr0 + STEP < c1) {
+            n0 = ld32_hint(A.rp + wr0 + STEP, stream);
+            n1 = ld32_hint(A.rp + min(wr0 + STEP + RW, c1), stream);
+        }
+        const int64_t r = wr0 + rig;
+        if (r < c1) {
+            const int p0 = ld32_hint(A.rp + r, stream), p1 = ld32_hint(A.rp + r + 1, stream);
+            Acc<C, V> acc[NV];
+#pragma unroll
+            for (int tt = 0; tt < NV; ++tt) acc[tt].zero();
+            for (int pb = p0; pb < p1; pb += U) {
+                int jj[U];
+                C vv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool ok = pb + u < p1;
+                    jj[u] = ok ? ld32_hint(col + pb + u, stream) : -1;
+                    vv[u] = ok ? (C)ldv_hint(val + pb + u, stream) : C(0);
+                }
+                uint4 raw[U][NV];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (jj[u] >= 0) {
+                        const TS *src = (SPLIT && jj[u] < A.split ? (const TS *)xnew : xold) +
+                                        checked_row(jj[u], A.nrows, A.status) * Kp;
+                        if constexpr (W32) {
+#pragma unroll
+                            for (int tt = 0; tt < NV; tt += 2)
+                                ldg32_hint(src + piece(tt) * V, keep, raw[u][tt], raw[u][tt + 1]);
+                        } else {
+#pragma unroll
+                            for (int tt = 0; tt < NV; ++tt) raw[u][tt] = ldg16_hint(src + piece(tt) * V, keep);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (jj[u] < 0) break;
+#pragma unroll
+                    for (int tt = 0; tt < NV; ++tt) {
+                        C x[V];
+                        S::unpack(raw[u][tt], x);
+                        acc[tt].fma_piece(vv[u], x);
+                    }
+                }
+            }
+            const C c = (C)A.omega / ldv_hint((const AV *)A.diag + r, stream);
+            // x_i - (omega / a_ii) s_i, a pair of pieces (W32) or one piece at a time
+            constexpr int PW = W32 ? 2 : 1;
+#pragma unroll
+            for (int t0 = 0; t0 < NV; t0 += PW) {
+                uint4 own[PW];
+                if constexpr (W32) ldg32_hint(xold + r * Kp + piece(t0) * V, keep, own[0], own[1]);
+                else own[0] = ldg16_hint(xold + r * Kp + piece(t0) * V, keep);
+#pragma unroll
+                for (int h = 0; h < PW; ++h) {
+                    C xi[V], out[V];
+                    S::unpack(own[h], xi);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) out[e] = fma(-c, acc[t0 + h].get(e), xi[e]);
+                    own[h] = S::pack(out);
+                }
+                if constexpr (W32) st32_hint(xnew + r * Kp + piece(t0) * V, own[0], own[1], keep);
+                else st16_hint(xnew + r * Kp + piece(t0) * V, own[0], keep);
+            }
+        }
+        // column-index and value lines of this warp's next group, into L2
+        if (n1 > n0) {
+            const int64_t q0 = n0 & ~31, nq = ((int64_t)n1 - q0 + 31) / 32;     // 128-byte lines
+            for (int64_t q = lane32; q < nq; q += 32) prefetch_l2(col + q0 + 32 * q);
+            constexpr int EPL = 128 / (int)sizeof(AV);                          // values per line
+            const int64_t v0 = n0 & ~(int64_t)(EPL - 1), nv = ((int64_t)n1 - v0 + EPL - 1) / EPL;
+            for (int64_t q = lane32; q < nv; q += 32) prefetch_l2(val + v0 + EPL * q);
+        }
+    }
+}
+
 // Groups per block and threads of a block.  Small phases spread over the SMs in
 // blocks of two warps; otherwise one block per SM takes one chunk (one wave, with
 // as many warps as share its groups evenly),
@@ -759,6 +953,37 @@ cudaError_t dispatch_sell(const RelaxArgs &a, cudaStream_t s)
     case 32: if constexpr (32 * V <= 64) return go_sell<TS, 32>(a, s); break;
     }
     return cudaErrorInvalidValue;
+}
+
+template <class TS, int G, int NV, int U>
+cudaError_t go_chunk(const RelaxArgs &a, cudaStream_t s)
+{
+    const int64_t rows = (int64_t)a.r1 - a.r0;
+    if (rows <= 0) return cudaSuccess;
+    constexpr int RW = 32 / G;
+    auto kern = a.split > 0 ? k_relax_chunk<TS, G, NV, U, true> : k_relax_chunk<TS, G, NV, U, false>;
+    static PerDevice sm_count;
+    const int dev = current_device_index();
+    int sms = sm_count.get(dev);
+    if (sms == 0) {
+        int d = 0;
+        cudaGetDevice(&d);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
+        if (sms <= 0) sms = 1;
+        sm_count.set(dev, sms);
+    }
+    // 32-byte accesses (NV even) need 32-byte aligned rows: always true of the
+    // handle's buffers (P even), refused rather than faulted otherwise
+    if constexpr (NV % 2 == 0) {
+        if (!rows_aligned32(a.xold, a.Kp, sizeof(TS)) || !rows_aligned32(a.xnew, a.Kp, sizeof(TS)))
+            return cudaErrorMisalignedAddress;
+    }
+    // one chunk per SM, a whole number of warp groups each
+    int64_t chunk = (rows + sms - 1) / sms;
+    chunk = (chunk + RW - 1) / RW * RW;
+    const int64_t blocks = (rows + chunk - 1) / chunk;
+    kern<<<(unsigned)blocks, kChunkThreads, 0, s>>>(a, (int32_t)chunk);
+    return cudaGetLastError();
 }
 
 template <class TS, int G, int NV>
@@ -870,7 +1095,13 @@ cudaError_t go(const RelaxArgs &a, cudaStream_t s)
 template <class TS, int G, int NV>
 cudaError_t dispatch_u(int U, int stage, const RelaxArgs &a, cudaStream_t s)
 {
-    if (stage == 3) stage = 0;        // no sliced copy: the direct kernel
+    if (stage == 3) {
+        switch (U) {
+        case 4: return go_chunk<TS, G, NV, 4>(a, s);
+        case 8: return go_chunk<TS, G, NV, 8>(a, s);
+        }
+        return cudaErrorInvalidValue;
+    }
     switch (U) {
     case 4: return stage == 2 ? go_pipe<TS, G, NV>(a, s)
                  : stage ? go_staged<TS, G, NV, 4>(a, s) : go<TS, G, NV, 4>(a, s);
@@ -963,7 +1194,7 @@ bool relax_shape_available(int storage, Shape sh)
 
 cudaError_t launch_relax(int storage, Shape sh, const RelaxArgs &a, cudaStream_t s)
 {
-    if (a.sell_ptr && (sh.stage == 0 || sh.stage == 3)) {
+    if (a.sell_ptr && sh.stage == 0) {
         switch (storage) {
         case ST_FP64: return dispatch_sell<double>(a, s);
         case ST_FP32: return dispatch_sell<float>(a, s);

@@ -102,6 +102,40 @@ def test_both_sweep_routes_round_alike(name, prec, K):
     assert np.array_equal(out[0], out[1])
 
 
+@pytest.mark.parametrize("name", ["aniso9_66", "graph_4129", "arrow_3001"])
+@pytest.mark.parametrize("K", [8, 32])
+def test_tuned_handles_and_saved_lines(name, K, tmp_path):
+    """A tuned handle, then handles that load its line as it is, with the sliced copy
+    asked for, without the field (lines of before) and with the chunked kernel."""
+    import re
+    rp, col, val = SWEEPS[name]()
+    color = inputs.greedy_coloring(rp, col)
+    want = oracle.relax(rp, col, val, oracle.tv_init(len(rp) - 1, K, 7), 3, 1.0, oracle.SWEEP_MCGS, color)
+    val2 = val * 1.5
+    want2 = oracle.relax(rp, col, val2, want, 1, 1.0, oracle.SWEEP_MCGS, color)
+    cache = tmp_path / "tune.txt"
+
+    def run():
+        with amgd.Handle(rp, col, val, K, 7) as h:
+            h.set_coloring(color)
+            h.autotune(amgd.AMGD_SWEEP_MCGS, 1.0, str(cache))
+            for _ in range(3):
+                h.relax(1, 1.0, amgd.AMGD_SWEEP_MCGS)
+            assert np.array_equal(h.get_vectors(), want)
+            h.set_values(val2)
+            h.relax(1, 1.0, amgd.AMGD_SWEEP_MCGS)
+            assert np.array_equal(h.get_vectors(), want2)
+
+    run()
+    line = cache.read_text()
+    assert re.search(r";sliced=[01];", line)
+    for pattern, text in ((r"$^", ""), (r";sliced=[01]", ";sliced=1"), (r";sliced=[01]", ""),
+                          (r";relax=(\d+),(\d+),(\d+),\d+(.*);sliced=[01]", r";relax=\1,\2,\3,3\4;sliced=0")):
+        cache.write_text(re.sub(pattern, text, line))
+        run()
+        assert len(cache.read_text().splitlines()) == 1          # served from the file
+
+
 @pytest.mark.parametrize("K", [2, 13, 33, 64])
 @pytest.mark.parametrize("weighted", [False, True])
 @pytest.mark.parametrize("name", ["lap1d_31", "graph_4129", "arrow_3001"])
