@@ -962,11 +962,11 @@ def main():
     else:
         achieved = ab["relax_per_launch"] / (relax_launch_ms * 1e-3) / 1e9
         tkey = "relax/%s/K%d/%s" % (precision, w["K"], cfg)
-        traffic = recorded_traffic(tkey, source_sha("k_relax.cu", "rowops.cuh",
+        traffic = recorded_traffic(tkey, source_sha("k_relax.cu", "k_sell.cu", "rowops.cuh",
                                                     "amgd_internal.cuh"))
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak, "traffic": traffic,
-                    "kernel": "k_relax (one color phase of one sweep)",
+                    "kernel": "sweep kernel (one color phase of one sweep)",
                     "peak_source": "%s hbm_gbs" % peak_kind,
                     "algorithmic_bytes_per_launch": ab["relax_per_launch"],
                     "avg_launch_us": relax_launch_ms * 1e3}
@@ -989,9 +989,9 @@ def main():
                        "shapes": {"relax": list(r["shapes"][0]), "edge": list(r["shapes"][1]),
                                   "legend": "(lanes per row G, 16-byte vectors per lane NV, "
                                             "nonzeros per gather batch U, kernel: relaxation 0 "
-                                            "direct / 1 TMA-staged CSR / 2 cp.async pipelined / "
-                                            "3 chunked per SM; distances 0 rows / 1 tiles / "
-                                            "2 rows in place / 3 warp-staged in place), "
+                                            "sliced copy of the matrix, or direct on the CSR / "
+                                            "1 TMA-staged CSR / 2 cp.async pipelined / 3 chunked "
+                                            "per SM; the distance pass has one kernel), "
                                             "autotuned"}},
             "phase_ms": phases,
             "timed_region": ("start vectors (Philox) + nu recorded sweeps + distances + reverse "
@@ -1009,14 +1009,20 @@ def main():
         line["backward_phase_gbs"] = ab["backward"] / (r["phase_ms"][3] * 1e-3) / 1e9
         line["scalars"] = {"omega_bar": r["scalars"][0], "loss": r["scalars"][1]}
 
-    # kernels of ours per step
-    edge_launches = 2 if mixed else 1                     # + FP64 row fixup on mixed paths
+    # kernels of ours per step (one more where the sweeps read the sliced copy: their
+    # weights): the row norms and the fits, with the FP64 rows of the mixed paths
+    edge_launches = 3 if mixed else 2
     if adj:
+        # symmetric pattern: inverse diagonals, refit, upstream, quotients, the fits'
+        # adjoint and its column form; recomputed sweeps (weights per segment); one
+        # reverse sweep each; the finish and its reduction
         nck = -(-w["nu"] // adj)
-        bwd_launches = 4 + (w["nu"] - nck) + 2 * w["nu"] + 2
+        bwd_launches = 6 + (w["nu"] - nck) + w["nu"] + 2
         launches_per_step = 1 + launches_relax + edge_launches + bwd_launches
     else:
-        launches_per_step = 1 + launches_relax + (1 if permuted else 0) + edge_launches + 3
+        rows_c = 1 if n <= 32768 else 2 if n <= 2048 * 1024 else 3     # compaction
+        launches_per_step = 1 + launches_relax + (1 if depth > 1 and permuted else 0) + \
+            edge_launches + rows_c
     line["gpu_launches"] = launches_per_step * args.steps
 
     if not args.no_side and precision != "fp64":
