@@ -325,7 +325,9 @@ int amgd_graph_launch(amgd_handle h);
  *   next synchronising call return AMGD_ERR_TIMEOUT); 2 warp-pipelined, CSR
  *   slices and neighbour rows copied with cp.async two and one row groups
  *   ahead (U must be 4); 3 one block per SM on a contiguous chunk of CSR rows.
- *   Repeated sweeps of kernel 0 read a sliced copy of the matrix and choose
+ *   Repeated sweeps of kernel 0 (but for sweeps that the caller's own stream
+ *   capture records: those stay on the CSR, which value updates then keep
+ *   current for the graph) read a sliced copy of the matrix and choose
  *   their lanes, batch and blocks by the row's size and the matrix, unless
  *   amgd_autotune found the handle's sweeps faster on the CSR in a shape of
  *   kernel 0, which they then run in.

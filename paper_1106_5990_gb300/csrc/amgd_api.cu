@@ -69,6 +69,8 @@ struct amgd_ctx {
     std::vector<int64_t> color_slice;            // first slice of each color
     bool perm32_stale = false;                   // row-permuted FP32 values out of date
     bool graph_csr = false;                      // the captured graph reads the row-permuted CSR values
+    bool recording = false;                      // the current call is recorded by the caller's own capture
+    bool recorded_csr = false;                   // a caller's graph may read the row-permuted CSR values
     void *weight = nullptr;                      // omega / a_ii of a relaxation (8 bytes per row)
     // vectors
     void *x[2] = {nullptr, nullptr};
@@ -356,11 +358,12 @@ int upload_weights(amgd_ctx *h)
     return AMGD_OK;
 }
 
-// whether the sweeps read the row-permuted CSR (a kernel chosen by stage, or no sliced
-// copy) instead of the sliced copy
+// whether the sweeps read the row-permuted CSR (a kernel chosen by stage, no sliced
+// copy, or a call that the caller's own capture records: its graph outlives the
+// sliced copy) instead of the sliced copy
 bool sweeps_use_csr(const amgd_ctx *h)
 {
-    return h->relax_shape[h->storage].stage != 0 || h->relax_csr[h->storage] || !h->sell_ok;
+    return h->recording || h->relax_shape[h->storage].stage != 0 || h->relax_csr[h->storage] || !h->sell_ok;
 }
 
 // Every value copy that queued work reads, from the caller-order values (src,
@@ -375,7 +378,7 @@ int permute_values(amgd_ctx *h, const double *src = nullptr, uint32_t *err = nul
 {
     const bool in_place = src == nullptr;
     const bool mixed = h->storage != ST_FP64;
-    const bool csr = sweeps_use_csr(h) || (h->gexec && h->graph_csr);
+    const bool csr = sweeps_use_csr(h) || h->recorded_csr || (h->gexec && h->graph_csr);
     ValueArgs a = {};
     a.src = in_place ? h->val_o : src;
     a.rp = h->rp_o;
@@ -409,7 +412,7 @@ int refresh_perm64(amgd_ctx *h, cudaStream_t s)
                                     nullptr, nullptr, nullptr, s));
     CK(h, launch_diag_values(h->val_o, h->diag_slot, h->perm, (int32_t)h->n, nullptr, nullptr,
                              h->diag64, nullptr, s));
-    h->perm64_stale = false;
+    h->perm64_stale = h->recording;      // a recorded refresh has not run
     return AMGD_OK;
 }
 
@@ -420,7 +423,7 @@ int refresh_perm32(amgd_ctx *h, cudaStream_t s)
     if (h->perm)
         CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, nullptr, nullptr, h->val32,
                                     nullptr, nullptr, s));
-    h->perm32_stale = false;
+    h->perm32_stale = h->recording;
     return AMGD_OK;
 }
 
@@ -516,7 +519,13 @@ int ensure_sell(amgd_ctx *h)
                                       mixed ? nullptr : h->sell_val64, mixed ? h->sell_val32 : nullptr, s);
         if (e != cudaSuccess) return without(e);
     }
-    if (!h->weight) CK(h, cudaMalloc(&h->weight, (size_t)h->n * sizeof(double)));
+    if (!h->weight) {
+        e = cudaMalloc(&h->weight, (size_t)h->n * sizeof(double));
+        if (e != cudaSuccess) {
+            h->weight = nullptr;
+            return without(e);
+        }
+    }
     return AMGD_OK;
 }
 
@@ -532,7 +541,10 @@ int prepare_sweeps(amgd_ctx *h, size_t bytes, cudaStream_t s)
     const int stage = h->relax_shape[h->storage].stage;
     const bool repeated = h->sweep_calls > 0 || bytes >= kWorth;
     ++h->sweep_calls;
-    if (stage == 0 && !h->relax_csr[h->storage] && (repeated || h->sell_ok)) {
+    // into the caller's own graph: nothing is allocated or waited for, and value
+    // updates keep the CSR current for its replays from now on
+    if (h->recording) h->recorded_csr = true;
+    else if (stage == 0 && !h->relax_csr[h->storage] && (repeated || h->sell_ok)) {
         const int rc = ensure_sell(h);
         if (rc != AMGD_OK) return rc;
     }
@@ -1413,13 +1425,15 @@ int amgd_relax(amgd_handle h, int32_t nu, double omega, int sweep_type)
         return fail(h, AMGD_ERR_ARG, "unknown sweep type");
     if (sweep_type == AMGD_SWEEP_MCGS && !h->perm)
         return fail(h, AMGD_ERR_STATE, "MCGS needs amgd_set_coloring first");
-    if (nu > 0) {
-        const int rc = prepare_sweeps(h, sweep_bytes(h, nu), h->stream);
-        if (rc != AMGD_OK) return rc;
-    }
-    if (h->ckpt_every > 0 && sweep_type == AMGD_SWEEP_JACOBI && !h->perm)
-        return run_relax_recorded(h, nu, omega, h->stream);
-    return run_relax(h, nu, omega, sweep_type, h->stream);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    h->recording = cudaStreamIsCapturing(h->stream, &capture) == cudaSuccess && capture != cudaStreamCaptureStatusNone;
+    int rc = nu > 0 ? prepare_sweeps(h, sweep_bytes(h, nu), h->stream) : AMGD_OK;
+    if (rc == AMGD_OK)
+        rc = h->ckpt_every > 0 && sweep_type == AMGD_SWEEP_JACOBI && !h->perm
+                 ? run_relax_recorded(h, nu, omega, h->stream)
+                 : run_relax(h, nu, omega, sweep_type, h->stream);
+    h->recording = false;
+    return rc;
 }
 
 int amgd_distances(amgd_handle h, double theta, double *a, double *dist, double *ls, int mem)

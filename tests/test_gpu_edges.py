@@ -84,6 +84,47 @@ def test_repeated_sweeps_and_new_values(name, K, sweep):
         assert np.array_equal(h.get_vectors(), X)
 
 
+@pytest.mark.parametrize("built", [False, True])
+@pytest.mark.parametrize("sweep", ["jacobi", "mcgs"])
+def test_sweeps_in_a_graph_of_the_callers(built, sweep):
+    """Sweeps that the caller's own capture records neither allocate nor wait, and the
+    graph follows value updates, whichever copy of the matrix the handle's sweeps read."""
+    rp, col, val = SWEEPS["aniso9_66"]()
+    n, K = len(rp) - 1, 8
+    color = inputs.greedy_coloring(rp, col) if sweep == "mcgs" else None
+    mode, omode = (amgd.AMGD_SWEEP_MCGS, oracle.SWEEP_MCGS) if color is not None else (amgd.AMGD_SWEEP_JACOBI, 0)
+    s = torch.cuda.Stream()
+    with amgd.Handle(rp, col, val, K, 7) as h:
+        if color is not None:
+            h.set_coloring(color)
+        h.set_stream(s)
+        X = oracle.tv_init(n, K, 7)
+
+        def eager(v):
+            h.relax(2, 0.9, mode)
+            return oracle.relax(rp, col, v, X, 2, 0.9, omode, color)
+
+        X = eager(val)
+        if built:
+            X = eager(val)
+            val = val * 1.25
+            h.set_values(val)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            h.relax(2, 0.9, mode)
+        assert np.array_equal(h.get_vectors(), X)        # recorded, not run
+        for scale in (1.0, 1.5, 0.75):
+            h.set_values(val * scale)
+            with torch.cuda.stream(s):
+                g.replay()
+            s.synchronize()
+            X = oracle.relax(rp, col, val * scale, X, 2, 0.9, omode, color)
+            assert np.array_equal(h.get_vectors(), X), scale
+            X = eager(val * scale)
+            assert np.array_equal(h.get_vectors(), X), scale
+        h.set_stream(None)
+
+
 @pytest.mark.parametrize("name", ["aniso9_66", "graph_4129", "lap1d_33"])
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
 @pytest.mark.parametrize("K", [3, 16, 64])
