@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads) k_values(ValueArgs A, int cap)
         for (int q = tid; q < S1 - S0; q += kThreads) sp[q] = __ldg(A.slot_sell + S0 + q);
     chain_wait();
     bool bad = false;
-    for (int p = S0 + tid; p < S1; p += kThreads) {
+    for (int64_t p = (int64_t)S0 + tid; p < S1; p += kThreads) {   // 64 bits: the last stride may pass 2^31
         const double x = ld_plain(A.src + p);
         bad = bad || !isfinite(x);
         if (A.val_o) A.val_o[p] = x;
