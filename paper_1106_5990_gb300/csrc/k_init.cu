@@ -407,8 +407,12 @@ __global__ void __launch_bounds__(kThreads) k_values(ValueArgs A, int cap)
 
 // launch_create: one thread per row.  Rows in ascending order hold no duplicate;
 // others are compared entry by entry up to kPairRow entries (the same checks on
-// the host took most of the 17 ms of a one-call build of a 150k-row graph).
-constexpr int kPairRow = 1024;
+// the host took most of the 17 ms of a one-call build of a 150k-row graph).  The
+// comparisons of a row grow with its square and run in one thread, so longer
+// unordered rows go to the host check.  Creating a handle from unordered rows, us,
+// host check / here: 120 entries 2768 / 771, 300 entries 6044 / 3772 (thread per
+// row; 6243 by way of the host), 400 entries 2327 / 6627, 1000 entries 5531 / 33613.
+constexpr int kPairRow = 128;
 __global__ void __launch_bounds__(kThreads) k_create(CreateArgs A)
 {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
