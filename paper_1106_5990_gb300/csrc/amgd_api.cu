@@ -577,6 +577,7 @@ RelaxArgs sweep_args(amgd_ctx *h, double omega)
     if (!sweeps_use_csr(h)) {
         a.sell_ptr = h->sell_ptr;
         a.sell_col = h->sell_col;
+        a.sell_entries = h->sell_entries;
         a.sell_val = f64 ? (const void *)h->sell_val64 : (const void *)h->sell_val32;
         a.rowmap = h->sell_map;
         a.weight = h->weight;

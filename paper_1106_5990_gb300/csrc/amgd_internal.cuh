@@ -269,6 +269,18 @@ __device__ __forceinline__ int64_t checked_row(int64_t j, int64_t rows, uint32_t
     return j;
 }
 
+// the same test of the sliced copy's entries that a sweep asks the L2 for
+__device__ __forceinline__ bool checked_entry(int64_t p, int64_t entries, uint32_t *status)
+{
+#if AMGD_CHECKS
+    if (p < 0 || p >= entries) {
+        if (status) atomicOr(status, kStatusIndexRange);
+        return false;
+    }
+#endif
+    return true;
+}
+
 // ---------------------------------------------------------------------------
 // launch arguments
 // ---------------------------------------------------------------------------
@@ -294,6 +306,7 @@ struct RelaxArgs {
     const void *sell_val = nullptr;       // same type as val
     const int32_t *rowmap = nullptr;      // row of (q, l) at 32 q + l, -1: none (NULL: in order)
     int32_t sell_width = 0;               // entries of an average row of the sliced copy, padding included
+    int64_t sell_entries = 0;             // entries of the sliced copy
     int64_t slice0 = 0;                   // first slice of this color phase
     const void *weight = nullptr;         // omega / a_ii per row
 };

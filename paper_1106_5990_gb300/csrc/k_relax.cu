@@ -609,10 +609,15 @@ __global__ void __launch_bounds__(SellShape<TS, P>::THREADS, 1) k_relax_sell(Rel
         if (g + 2 * step < gend) {
             // the group after next: its lines into L2
             slice_of(g + 2 * step, fbase, fw);
+            auto ask = [&](int64_t p, bool col) {
+                if (!checked_entry(p, A.sell_entries, A.status)) return;
+                if (col) prefetch_l2(A.sell_col + p);
+                prefetch_l2((const AV *)A.sell_val + p);
+            };
             for (int q = lane32; q < fw; q += 32) {
-                prefetch_l2(A.sell_col + fbase + 32 * q);
-                prefetch_l2((const AV *)A.sell_val + fbase + 32 * q);
-                if constexpr (sizeof(AV) == 8) prefetch_l2((const AV *)A.sell_val + fbase + 32 * q + 16);
+                ask(fbase + 32 * (int64_t)q, true);
+                // 32 rows' FP64 values fill two lines, those of fewer rows lie in one
+                if constexpr (RW * sizeof(AV) > 128) ask(fbase + 32 * (int64_t)q + 16, false);
             }
         }
         Acc<C, V> acc[NV];

@@ -9,6 +9,8 @@ inside the kernel before its load.
 * A column index planted out of range after the handle's setup is caught by
   the sweep's test and reported as AMGD_ERR_CHECK by the next synchronising
   call; the load itself is redirected to row 0 and never leaves the buffer.
+* The entries of the sliced copy that a sweep asks the L2 for ahead of use are
+  tested in the same way: none lies past the copy's end.
 """
 import os
 import subprocess
@@ -73,3 +75,26 @@ with amgd.Handle(rp, col, val, 8, 1) as h:
 def test_planted_column_is_caught(checked_lib):
     p = _child(["-c", PLANTED], AMGD_TEST_BAD_COLUMN="77")
     assert p.returncode == 0 and p.stdout.strip().endswith("caught"), p.stdout + p.stderr
+
+
+# 16 rows of 64 bytes per group, three groups per warp, the last group in the upper
+# half of the last slice; and the other row widths at the same row counts
+AHEAD = r'''
+from paper_1106_5990_gb300 import amgd, inputs
+assert amgd.amgd_checked_build() == 1
+for n in (111872, 111872 - 16, 111872 - 37):
+    rp, col, val = inputs.lap1d(n)
+    for K in (2, 4, 8, 16, 32, 64):
+        for prec in ("fp64", "fp32"):
+            with amgd.Handle(rp, col, val, K, 1) as h:
+                h.set_precision(prec)
+                h.relax(1, 0.7)
+                h.relax(1, 0.7)                  # reads the sliced copy
+                h.get_vectors()                  # synchronises: reads the status
+print("in range")
+'''
+
+
+def test_entries_asked_for_ahead_stay_in_the_copy(checked_lib):
+    p = _child(["-c", AHEAD])
+    assert p.returncode == 0 and p.stdout.strip().endswith("in range"), p.stdout + p.stderr
