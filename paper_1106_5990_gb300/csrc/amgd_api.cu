@@ -63,7 +63,9 @@ struct amgd_ctx {
     bool sell_ok = false;                        // the copy exists (else its padding was too much)
     int64_t sell_entries = 0;
     int64_t *sell_ptr = nullptr, *sell_tab = nullptr;   // tab: first rows, then first slices of the colors
-    int32_t *sell_col = nullptr, *sell_slot = nullptr, *sell_map = nullptr;
+    int32_t *sell_col = nullptr, *sell_slot = nullptr;
+    int32_t *sell_map = nullptr;                 // row of every place of every slice (one color in row order: none)
+    bool sell_sorted = false;                    // its rows are sorted by length inside windows
     double *sell_val64 = nullptr;
     float *sell_val32 = nullptr;
     std::vector<int64_t> color_slice;            // first slice of each color
@@ -435,7 +437,7 @@ void drop_sell(amgd_ctx *h)
     h->sell_col = h->sell_slot = h->sell_map = nullptr;
     h->sell_val64 = nullptr;
     h->sell_val32 = nullptr;
-    h->sell_tried = h->sell_ok = false;
+    h->sell_tried = h->sell_ok = h->sell_sorted = false;
 }
 
 // The sliced copy of the current row order, and its values for the current
@@ -487,12 +489,17 @@ int ensure_sell(amgd_ctx *h)
         };
         measure();
         // rows of uneven length: sorted inside windows where the rows in order
-        // would store an eighth more than the matrix
+        // would store an eighth more than the matrix.  With several colors the rows
+        // of the slices are listed in any case: a color's last slice is padded, and a
+        // sweep over all rows at once has to know where
         const unsigned long long nnz = (unsigned long long)h->nnz;
-        if (e == cudaSuccess && total > nnz + nnz / 8 + 8192) {
-            e = dalloc(&h->sell_map, (size_t)nsl * kSellRows);
-            if (e == cudaSuccess) e = launch_sell_sort(a, h->sell_map, s);
+        h->sell_sorted = e == cudaSuccess && total > nnz + nnz / 8 + 8192;
+        if (e == cudaSuccess && (h->sell_sorted || nc > 1)) e = dalloc(&h->sell_map, (size_t)nsl * kSellRows);
+        if (e == cudaSuccess && h->sell_sorted) {
+            e = launch_sell_sort(a, h->sell_map, s);
             measure();
+        } else if (e == cudaSuccess && nc > 1) {
+            e = launch_sell_rows(a, h->sell_map, s);
         }
         const bool fits = total <= nnz + nnz / 2 + 32768 && total < (1ull << 31) - 64;
         if (e == cudaSuccess && fits) {
@@ -579,7 +586,7 @@ RelaxArgs sweep_args(amgd_ctx *h, double omega)
         a.sell_col = h->sell_col;
         a.sell_entries = h->sell_entries;
         a.sell_val = f64 ? (const void *)h->sell_val64 : (const void *)h->sell_val32;
-        a.rowmap = h->sell_map;
+        a.rowmap = h->sell_sorted ? h->sell_map : nullptr;
         a.weight = h->weight;
         a.sell_width = (int32_t)((h->sell_entries + 32 * h->color_slice.back() - 1) / (32 * h->color_slice.back()));
     }
@@ -617,6 +624,11 @@ int run_relax(amgd_ctx *h, int32_t nu, double omega, int sweep, cudaStream_t s)
             a.r0 = 0;
             a.r1 = (int32_t)h->n;
             a.split = 0;
+            if (sliced && h->sell_map) {
+                // places of the slices instead of rows: a color's last slice is padded
+                a.rowmap = h->sell_map;
+                a.r1 = (int32_t)(h->color_slice.back() * kSellRows);     // at most the copy's entries, < 2^31
+            }
             CK(h, launch_relax(h->storage, sh, a, s));
         } else {
             for (size_t c = 0; c + 1 < h->color_start.size(); ++c) {

@@ -294,7 +294,7 @@ struct RelaxArgs {
     const void *diag;     // permuted diagonal a_ii, same type as val
     const void *xold;     // iterate at the start of the sweep
     void *xnew;           // rows [r0, r1) written; rows < split read from here
-    int32_t r0, r1;       // rows of this color phase
+    int32_t r0, r1;       // rows of this color phase (sliced, rowmap: places from slice0 on)
     int32_t split;        // rows < split take new values (earlier colors)
     int32_t Kp;           // padded row stride (elements)
     double omega;
@@ -370,6 +370,8 @@ struct SellArgs {
 };
 // rowmap (sorted by length inside windows of kSellWindow rows; ties in row order)
 cudaError_t launch_sell_sort(const SellArgs &a, int32_t *rowmap, cudaStream_t s);
+// rowmap in row order (-1: padding at a color's end)
+cudaError_t launch_sell_rows(const SellArgs &a, int32_t *rowmap, cudaStream_t s);
 // entries of every slice (rowmap NULL: rows in order), width[nslices], and their sum
 cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t *width, unsigned long long *total,
                               cudaStream_t s);

@@ -51,6 +51,14 @@ __global__ void __launch_bounds__(kSellWindow) k_sell_sort(SellArgs a, int32_t *
     if (q * kSellRows + place < a.color_slice[c + 1] * kSellRows) rowmap[q * kSellRows + place] = t < rows ? (int32_t)(r0 + t) : -1;
 }
 
+// the rows of the slices in order
+__global__ void __launch_bounds__(kThreads) k_sell_rows(SellArgs a, int32_t *rowmap)
+{
+    const int64_t q = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / 32;
+    const int l = threadIdx.x % 32;
+    if (q < a.nslices) rowmap[q * kSellRows + l] = (int32_t)row_at(a, nullptr, q, l);
+}
+
 __global__ void __launch_bounds__(kThreads) k_sell_width(SellArgs a, const int32_t *rowmap, int32_t *width, unsigned long long *total)
 {
     const int64_t q = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / 32;
@@ -96,6 +104,13 @@ cudaError_t launch_sell_sort(const SellArgs &a, int32_t *rowmap, cudaStream_t s)
 {
     if (a.nslices == 0) return cudaSuccess;
     k_sell_sort<<<(unsigned)a.nslices, kSellWindow, 0, s>>>(a, rowmap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sell_rows(const SellArgs &a, int32_t *rowmap, cudaStream_t s)
+{
+    if (a.nslices == 0) return cudaSuccess;
+    k_sell_rows<<<slice_blocks(a.nslices), kThreads, 0, s>>>(a, rowmap);
     return cudaGetLastError();
 }
 

@@ -125,6 +125,47 @@ def test_sweeps_in_a_graph_of_the_callers(built, sweep):
         h.set_stream(None)
 
 
+@pytest.mark.parametrize("name", ["poisson5_37", "aniso9_66", "graph_4129", "arrow_3001"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
+@pytest.mark.parametrize("K", [4, 16, 64])
+def test_jacobi_sweeps_of_a_colored_handle(name, prec, K):
+    """Jacobi sweeps run over all rows at once; the sliced copy is padded where a color
+    ends (color sizes off the slices of 32 rows; rows in order and sorted by length)."""
+    rp, col, val = SWEEPS[name]()
+    n = len(rp) - 1
+    color = inputs.greedy_coloring(rp, col)
+    assert all(k % 32 for k in np.bincount(color))
+    s_rp = torch.empty(n + 1, dtype=torch.int64, device="cuda")
+    s_col = torch.empty(len(col), dtype=torch.int32, device="cuda")
+    want = None
+    if prec == "fp64":
+        want = oracle.relax(rp, col, val, oracle.tv_init(n, K, 7), 3, 0.8)
+    for colored in (False, True):
+        with amgd.Handle(rp, col, val, K, 7) as h:
+            h.set_precision(prec)
+            if colored:
+                h.set_coloring(color)
+            h.init_vectors(7)
+            parts = (1, 1, 1) if colored else (3,)
+            for nu in parts:                     # from the second call on: the sliced copy
+                h.relax(nu, 0.8)
+                if colored:
+                    h.set_values(val)
+            got = [h.get_vectors()]
+            if colored:
+                h.relax(1, 0.8, amgd.AMGD_SWEEP_MCGS)
+                h.graph_capture(7, 3, 0.8, amgd.AMGD_SWEEP_JACOBI, 0.5, s_rp, s_col)
+                h.graph_launch()
+                got.append(h.get_vectors())
+                h.autotune(amgd.AMGD_SWEEP_JACOBI, 0.8)
+                h.init_vectors(7)
+                h.relax(3, 0.8)
+                got.append(h.get_vectors())
+        want = got[0] if want is None else want
+        for g in got:
+            assert np.array_equal(g, want)
+
+
 @pytest.mark.parametrize("name", ["aniso9_66", "graph_4129", "lap1d_33"])
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
 @pytest.mark.parametrize("K", [3, 16, 64])
