@@ -69,6 +69,8 @@ struct amgd_ctx {
     double *sell_val64 = nullptr;
     float *sell_val32 = nullptr;
     std::vector<int64_t> color_slice;            // first slice of each color
+    bool sell_held = false;                      // a graph of the caller's may read the copy: kept when it is dropped
+    std::vector<void *> held;                    // such copies of before, freed with the handle
     bool perm32_stale = false;                   // row-permuted FP32 values out of date
     bool graph_csr = false;                      // the captured graph reads the row-permuted CSR values
     bool recording = false;                      // the current call is recorded by the caller's own capture
@@ -429,10 +431,33 @@ int refresh_perm32(amgd_ctx *h, cudaStream_t s)
     return AMGD_OK;
 }
 
+// Whether the caller captures the handle's stream: the work of the call is then
+// recorded into a graph of the caller's, which may be replayed at any later time.
+// Sweeps recorded there read the CSR, which is never freed.
+struct Recording {
+    amgd_ctx *h;
+    explicit Recording(amgd_ctx *c) : h(c)
+    {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        h->recording = cudaStreamIsCapturing(h->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+    }
+    ~Recording() { h->recording = false; }
+    Recording(const Recording &) = delete;
+};
+
+// array of a sliced copy that is given up; one that a graph of the caller's reads
+// stays until the handle goes
+void drop_part(amgd_ctx *h, void *p)
+{
+    if (p && h->sell_held) h->held.push_back(p);
+    else dfree(p);
+}
+
 void drop_sell(amgd_ctx *h)
 {
     void *ptrs[] = {h->sell_ptr, h->sell_tab, h->sell_col, h->sell_slot, h->sell_map, h->sell_val64, h->sell_val32};
-    for (void *p : ptrs) dfree(p);
+    for (void *p : ptrs) drop_part(h, p);
+    h->sell_held = false;
     h->sell_ptr = h->sell_tab = nullptr;
     h->sell_col = h->sell_slot = h->sell_map = nullptr;
     h->sell_val64 = nullptr;
@@ -1065,8 +1090,8 @@ int amgd_set_precision(amgd_handle h, int storage)
     if (slot_type_changes) {
         // the value copies of the new arithmetic type (the sliced one is remade
         // when a sweep next runs)
-        dfree(h->sell_val64);
-        dfree(h->sell_val32);
+        drop_part(h, h->sell_val64);
+        drop_part(h, h->sell_val32);
         h->sell_val64 = nullptr;
         h->sell_val32 = nullptr;
         rc = permute_values(h);
@@ -1438,15 +1463,12 @@ int amgd_relax(amgd_handle h, int32_t nu, double omega, int sweep_type)
         return fail(h, AMGD_ERR_ARG, "unknown sweep type");
     if (sweep_type == AMGD_SWEEP_MCGS && !h->perm)
         return fail(h, AMGD_ERR_STATE, "MCGS needs amgd_set_coloring first");
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    h->recording = cudaStreamIsCapturing(h->stream, &capture) == cudaSuccess && capture != cudaStreamCaptureStatusNone;
-    int rc = nu > 0 ? prepare_sweeps(h, sweep_bytes(h, nu), h->stream) : AMGD_OK;
-    if (rc == AMGD_OK)
-        rc = h->ckpt_every > 0 && sweep_type == AMGD_SWEEP_JACOBI && !h->perm
-                 ? run_relax_recorded(h, nu, omega, h->stream)
-                 : run_relax(h, nu, omega, sweep_type, h->stream);
-    h->recording = false;
-    return rc;
+    const Recording recording(h);
+    const int rc = nu > 0 ? prepare_sweeps(h, sweep_bytes(h, nu), h->stream) : AMGD_OK;
+    if (rc != AMGD_OK) return rc;
+    if (h->ckpt_every > 0 && sweep_type == AMGD_SWEEP_JACOBI && !h->perm)
+        return run_relax_recorded(h, nu, omega, h->stream);
+    return run_relax(h, nu, omega, sweep_type, h->stream);
 }
 
 int amgd_distances(amgd_handle h, double theta, double *a, double *dist, double *ls, int mem)
@@ -1779,6 +1801,8 @@ int amgd_graph_launch(amgd_handle h)
     AMGD_RANGE("amgd_graph_launch");
     if (!h) return AMGD_ERR_ARG;
     if (!h->gexec) return fail(h, AMGD_ERR_STATE, "no captured graph");
+    const Recording recording(h);
+    if (h->recording && !h->graph_csr) h->sell_held = true;      // becomes part of a graph of the caller's
     CK(h, cudaGraphLaunch(h->gexec, h->stream));
     h->cur = h->graph_cur_after;
     h->have_dist = true;
@@ -2354,6 +2378,7 @@ int amgd_backward(amgd_handle h, const double *ls_bar, int mem, double *val_bar,
     if (!val_bar && h->nnz) return fail(h, AMGD_ERR_ARG, "val_bar is NULL");
     int rc = backward_checks(h);
     if (rc != AMGD_OK) return rc;
+    const Recording recording(h);        // the recomputed sweeps, as in amgd_relax
     if ((rc = prepare_backward(h)) != AMGD_OK) return rc;
     cudaStream_t s = h->stream;
     const int64_t nnz = h->nnz;
@@ -2488,6 +2513,7 @@ int amgd_destroy(amgd_handle h)
         dfree(h->colx);
     }
     drop_sell(h);
+    for (void *p : h->held) dfree(p);
     dfree(h->weight);
     dfree(h->mat_id);
     if (h->depth > 1) {

@@ -125,6 +125,62 @@ def test_sweeps_in_a_graph_of_the_callers(built, sweep):
         h.set_stream(None)
 
 
+@pytest.mark.filterwarnings("ignore:DEBUG")
+@pytest.mark.parametrize("warmed", ["sliced", "staged"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_reverse_pass_in_a_graph_of_the_callers(warmed, prec, tmp_path):
+    """A training step that the caller records recomputes its sweeps on the CSR, which the
+    handle never frees, allocates nothing there, and follows value updates."""
+    rp, col, val = SWEEPS["aniso9_66"]()
+    K, nu, rng = 8, 4, np.random.default_rng(4)
+    s = torch.cuda.Stream()
+    vb = torch.zeros(len(val), dtype=torch.float64, device="cuda")
+
+    def step(h):
+        h.init_vectors(7)
+        h.relax(nu, 0.6)
+        amgd.check(amgd.amgd_distances(h.h, 0.5, None, None, None, amgd.AMGD_MEM_DEVICE), h.h)
+        amgd.check(amgd.amgd_backward(h.h, None, amgd.AMGD_MEM_DEVICE, vb.data_ptr(), None, None), h.h)
+
+    def handle(v):
+        h = amgd.Handle(rp, col, v, K, 7)
+        h.set_precision(prec)
+        h.set_checkpointing(2)
+        return h
+
+    with handle(val) as h:
+        h.set_stream(s)
+        G, NV, U, _ = h.kernel_shape(amgd.AMGD_KERNEL_RELAX)
+        if warmed == "staged":                   # the buffers exist, the sliced copy does not
+            h.set_kernel_shape(amgd.AMGD_KERNEL_RELAX, G, NV, U, 1)
+            step(h)
+            h.set_kernel_shape(amgd.AMGD_KERNEL_RELAX, G, NV, U, 0)
+        else:
+            for _ in range(3):
+                step(h)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(g, stream=s):
+            step(h)
+        g.debug_dump(str(tmp_path / "graph.dot"))
+        kernels = (tmp_path / "graph.dot").read_text()
+        assert "k_relax" in kernels and "k_relax_sell" not in kernels
+        for _ in range(2):
+            v = val * (1 + 0.3 * rng.random(len(val)))
+            h.set_values(v)
+            vb.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(s):
+                g.replay()
+            s.synchronize()
+            got = vb.cpu().numpy()
+            with handle(v) as h2:
+                step(h2)
+                torch.cuda.synchronize()
+            assert np.any(got) and np.array_equal(got, vb.cpu().numpy())
+        h.set_stream(None)
+
+
 @pytest.mark.parametrize("name", ["poisson5_37", "aniso9_66", "graph_4129", "arrow_3001"])
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
 @pytest.mark.parametrize("K", [4, 16, 64])
