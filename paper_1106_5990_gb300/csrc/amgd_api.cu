@@ -75,6 +75,7 @@ struct amgd_ctx {
     bool graph_csr = false;                      // the captured graph reads the row-permuted CSR values
     bool recording = false;                      // the current call is recorded by the caller's own capture
     bool recorded_csr = false;                   // a caller's graph may read the row-permuted CSR values
+    bool recorded_values = false;                // a caller's graph may replace the values at any time
     void *weight = nullptr;                      // omega / a_ii of a relaxation (8 bytes per row)
     // vectors
     void *x[2] = {nullptr, nullptr};
@@ -364,10 +365,11 @@ int upload_weights(amgd_ctx *h)
 
 // whether the sweeps read the row-permuted CSR (a kernel chosen by stage, no sliced
 // copy, or a call that the caller's own capture records: its graph outlives the
-// sliced copy) instead of the sliced copy
+// sliced copy; or values that a graph of the caller's replaces: it writes the copies
+// that there were when it was recorded) instead of the sliced copy
 bool sweeps_use_csr(const amgd_ctx *h)
 {
-    return h->recording || h->relax_shape[h->storage].stage != 0 || h->relax_csr[h->storage] || !h->sell_ok;
+    return h->recording || h->recorded_values || h->relax_shape[h->storage].stage != 0 || h->relax_csr[h->storage] || !h->sell_ok;
 }
 
 // Every value copy that queued work reads, from the caller-order values (src,
@@ -402,15 +404,17 @@ int permute_values(amgd_ctx *h, const double *src = nullptr, uint32_t *err = nul
     a.err = err;
     a.n = (int32_t)h->n;
     CK(h, launch_values(a, !mixed, h->nnz, h->stream));
-    h->perm64_stale = mixed || !csr;
-    h->perm32_stale = !(mixed && csr);
+    // (a recorded update has not run: what is out of date stays so)
+    h->perm64_stale = mixed || !csr || (h->recording && h->perm64_stale);
+    h->perm32_stale = !(mixed && csr) || (h->recording && h->perm32_stale);
     return AMGD_OK;
 }
 
 // bring the row-permuted FP64 values and diagonal up to date (stream order)
 int refresh_perm64(amgd_ctx *h, cudaStream_t s)
 {
-    if (!h->perm64_stale) return AMGD_OK;
+    // (an update in a graph of the caller's leaves these out of date on mixed storage)
+    if (!h->perm64_stale && !(h->recorded_values && h->storage != ST_FP64)) return AMGD_OK;
     if (h->perm)
         CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, nullptr, h->val64,
                                     nullptr, nullptr, nullptr, s));
@@ -576,7 +580,7 @@ int prepare_sweeps(amgd_ctx *h, size_t bytes, cudaStream_t s)
     // into the caller's own graph: nothing is allocated or waited for, and value
     // updates keep the CSR current for its replays from now on
     if (h->recording) h->recorded_csr = true;
-    else if (stage == 0 && !h->relax_csr[h->storage] && (repeated || h->sell_ok)) {
+    else if (stage == 0 && !h->relax_csr[h->storage] && !h->recorded_values && (repeated || h->sell_ok)) {
         const int rc = ensure_sell(h);
         if (rc != AMGD_OK) return rc;
     }
@@ -1355,7 +1359,13 @@ int amgd_set_values_async(amgd_handle h, const double *val, int mem)
     int rc = async_setup(h);
     if (rc != AMGD_OK) return rc;
     if (mem == AMGD_MEM_DEVICE) {
-        // read in place, in stream order: val stays unchanged until amgd_sync
+        // read in place, in stream order: val stays unchanged until amgd_sync.  A
+        // recorded update writes the copies there are now, the CSR always
+        const Recording recording(h);
+        if (h->recording) {
+            h->recorded_values = true;
+            h->sell_held = h->sell_held || h->sell_ok;
+        }
         rc = permute_values(h, val, h->async_err);
         if (rc != AMGD_OK) return rc;
     } else {

@@ -125,6 +125,54 @@ def test_sweeps_in_a_graph_of_the_callers(built, sweep):
         h.set_stream(None)
 
 
+@pytest.mark.parametrize("built", [False, True])
+@pytest.mark.parametrize("sweep", ["jacobi", "mcgs"])
+def test_value_updates_in_a_graph_of_the_callers(built, sweep):
+    """A recorded update reaches the sweeps of later calls, whether the sliced copy is there
+    when it is recorded, is asked for afterwards or is given up with its coloring."""
+    rp, col, val = SWEEPS["aniso9_66"]()
+    n, K = len(rp) - 1, 8
+    color = inputs.greedy_coloring(rp, col)
+    mode, omode = (amgd.AMGD_SWEEP_MCGS, oracle.SWEEP_MCGS) if sweep == "mcgs" else (amgd.AMGD_SWEEP_JACOBI, 0)
+    s = torch.cuda.Stream()
+    buf = torch.from_numpy(val).cuda()
+    with amgd.Handle(rp, col, val, K, 7) as h:
+        h.set_coloring(color)
+        h.set_stream(s)
+        X = oracle.tv_init(n, K, 7)
+
+        def eager(v):
+            h.relax(1, 0.9, mode)
+            return oracle.relax(rp, col, v, X, 1, 0.9, omode, color)
+
+        h.set_values_async(buf)
+        h.sync()
+        for _ in range(3 if built else 1):
+            X = eager(val)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            h.set_values_async(buf)
+        h.sync()
+        for _ in range(2):
+            X = eager(val)
+            assert np.array_equal(h.get_vectors(), X)    # recorded, not run
+        for scale in (1.5, 0.75):
+            v = val.copy()
+            v[col != np.repeat(np.arange(n), np.diff(rp))] *= scale
+            buf.copy_(torch.from_numpy(v))
+            torch.cuda.synchronize()
+            with torch.cuda.stream(s):
+                g.replay()
+            s.synchronize()
+            for _ in range(2):
+                X = eager(v)
+                assert np.array_equal(h.get_vectors(), X), scale
+            h.set_coloring((len(np.bincount(color)) - 1 - color).astype(np.int32))
+            h.set_coloring(color)
+        h.set_stream(None)
+
+
 @pytest.mark.filterwarnings("ignore:DEBUG")
 @pytest.mark.parametrize("warmed", ["sliced", "staged"])
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
