@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(128) k_ls_interp_m(InterpArgs A)
 #pragma unroll
         for (int a = 0; a < MT; ++a) ba[a] = 0.0;
 #pragma unroll 1
-        for (int k = 0; k < K; k += 4) {          // (components past K are zero in every row)
+        for (int k = 0; k < K; k += 4) {
             double y[4] = {0.0, 0.0, 0.0, 0.0};
             Chunk4<TS> x;
             if (A.target == 0)
@@ -729,6 +729,7 @@ __global__ void __launch_bounds__(128) k_ls_interp_m(InterpArgs A)
             for (int q = 0; q < 4; ++q) {
                 const double xi = widen_val<TS>(x.v[q]);
                 y[q] = A.target == 0 ? fma(c, y[q], xi) : xi;
+                if (k + q >= K) y[q] = 0.0;       // padding: zero in every row, but not times an infinite 1 / a_ii
                 syy = __dadd_rn(syy, __dmul_rn(y[q], y[q]));
                 yv[(k + q) * T] = y[q];
             }

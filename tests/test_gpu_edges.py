@@ -524,6 +524,22 @@ def test_interpolation_of_every_candidate_count(K, prec):
             assert np.array_equal(g, w_)
 
 
+@pytest.mark.parametrize("K", [6, 8, 13])
+def test_interpolation_with_tiny_diagonals(K):
+    """1 / a_ii overflows: infinite targets and LS in the components that there are."""
+    rp, col, val = inputs.random_csr(700, 2.5, 21, symmetric_pattern=True)
+    n = len(rp) - 1
+    val[np.nonzero(np.repeat(np.arange(n), np.diff(rp)) == col)[0][5::40]] = 1e-310
+    coarse = (np.random.default_rng(3).random(n) < 0.45).astype(np.uint8)
+    X = oracle.tv_init(n, K, 2)
+    want = oracle.ls_interp(X, oracle.target(rp, col, val, X), rp, col, coarse, 2, 1.5)
+    assert np.isinf(want[3]).any() and not np.isnan(want[3]).any()
+    with amgd.Handle(rp, col, val, K, 2) as h:
+        got = h.ls_interpolation(coarse, 2, 1.5)
+    for g, w_ in zip(got, want):
+        assert np.array_equal(g, w_)
+
+
 @pytest.mark.parametrize("K", [4, 8, 16, 32, 64])
 @pytest.mark.parametrize("pattern", ["symmetric", "general"])
 @pytest.mark.parametrize("weighted", [False, True])
