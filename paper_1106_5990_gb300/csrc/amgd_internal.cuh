@@ -336,6 +336,9 @@ struct EdgeArgs {                // everything in the caller's numbering
     int64_t nnz_p = 0;           // entries of the fits' pattern
     void *norms = nullptr;       // workspace, n rows: S_xx (FP32), or S_xx and 1 / S_xx (FP64)
     bool compensated = false;    // mixed paths: compensated FP32 LS sums
+    int32_t long_len = INT32_MAX;        // rows with more fits than this are listed in long_rows
+    const int32_t *long_rows = nullptr;
+    int32_t n_long = 0;
     uint32_t *status = nullptr;  // device status word (checked build: index range)
 };
 
@@ -379,6 +382,10 @@ cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t 
 cudaError_t launch_sell_fill(const SellArgs &a, const int32_t *rowmap, const int64_t *ptr, int32_t *sell_col,
                              int32_t *slot, cudaStream_t s);
 
+// rows with more than long_len entries (the first cap of them), in no order, and their
+// number (zero before the call)
+cudaError_t launch_long_rows(const int32_t *rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap,
+                             uint32_t *count, cudaStream_t s);
 // in_place: read the vectors in the sweeps' row order (search depth 1)
 cudaError_t launch_edge(int storage, bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s);

@@ -33,6 +33,7 @@
 
 #include "amgd_internal.cuh"
 #include "rowops.cuh"
+#include "staging.cuh"
 
 namespace amgd {
 namespace edge_impl {
@@ -500,9 +501,9 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
         for (int q = tid; q < S1 - S0; q += T) a_s[q] = (C)ld_plain(val + S0 + q);
     __syncthreads();
 
-    if (tid / width < nr) {
-        const int64_t r = R0 + tid / width;
-        const int q0 = __ldg(A.prp + r), q1 = __ldg(A.prp + r + 1);
+    const int64_t r = R0 + min(tid / width, nr - 1);
+    const int q0 = __ldg(A.prp + r), q1 = __ldg(A.prp + r + 1);
+    if (tid / width < nr && q1 - q0 <= A.long_len) {                 // longer rows: k_edge_long
         const int p0 = PX ? q0 : __ldg(A.rp + r), p1 = PX ? q1 : __ldg(A.rp + r + 1);
         const int64_t xr = (PX && A.xrow) ? checked_row(__ldg(A.xrow + r), A.n, A.status) : r;
         const C diag = (C)ld_plain((const AV *)A.diag + r);
@@ -664,6 +665,204 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
             a_out[S0 + q] = a_s[q];
             ls_out[S0 + q] = ls_s[q];
             A.flag_out[S0 + q] = fl_s[q];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Rows of more than A.long_len entries, one block each; same fits, same order
+// of every sum as k_edge_fit.  The target is a chain over the row's entries per
+// component (the sweeps' rounding): tiles of neighbour rows land in shared
+// memory with cp.async, one ahead, and one thread per component walks them.
+// Then every G lanes fit entries of their own.  Bound: latency, of a tile per 1 us for
+// the target and of a gather per 256 / G entries for the fits (a graph of 200k rows,
+// K = 16, with one row of 30000: FP32 418 us, 20302 with that row in one lane;
+// FP64 2524 / 78537).
+// ---------------------------------------------------------------------------
+constexpr int kLongThreads = 256;
+
+template <class TS, int P>
+struct LongLayout {
+    static constexpr int V = Store<TS>::V, KP = P * V;
+    static constexpr int TILE = P <= 2 ? 512 : 1024 / P;             // neighbour rows per tile
+    static constexpr int PPT = TILE * P / kLongThreads;               // 16-byte pieces per thread and tile
+    static_assert(TILE * P % kLongThreads == 0, "whole pieces per thread");
+};
+
+// component k of a stored row
+template <class TS>
+__device__ __forceinline__ typename Store<TS>::C component(const TS *x, int k)
+{
+    if constexpr (std::is_same<TS, __nv_bfloat16>::value) return __bfloat162float(x[k]);
+    else return x[k];
+}
+
+template <class TS, int P, bool UW, bool PX, bool COMP>
+__global__ void __launch_bounds__(kLongThreads) k_edge_long(EdgeArgs A)
+{
+    using S = Store<TS>;
+    using C = typename S::C;
+    using AV = typename S::A;
+    using L = FitLayout<TS, P>;
+    using LL = LongLayout<TS, P>;
+    constexpr int V = S::V, KP = L::KP, G = L::G, NP = L::NP, TILE = LL::TILE, PPT = LL::PPT, W = kLongThreads / 32;
+    constexpr bool kMixed = !std::is_same<C, double>::value;
+    __shared__ __align__(16) uint4 xs[2][TILE * P];                   // neighbour rows
+    __shared__ C vs[2][TILE];                                         // and the row's values
+    __shared__ C ys[KP], wsm[UW ? 1 : KP];
+    __shared__ C msm[W];
+    __shared__ int csm[W];
+    const int tid = threadIdx.x, gl = tid % G;
+    const unsigned gmask = G == 1 ? 1u << (tid % 32) : ((1u << G) - 1u) << ((tid % 32) / G * G);
+    const int np = G == 1 ? (A.K + V - 1) / V : NP;
+    const int32_t *__restrict__ xcol = PX ? A.xcol : A.col;
+    const int32_t *__restrict__ fcol = PX ? A.xcol : A.pcol;
+    const AV *val = (const AV *)A.val;
+    const TS *X = (const TS *)A.x;
+    C *a_out = (C *)A.a_out;
+    C *ls_out = (C *)A.ls_out;
+    chain_wait();
+    chain_release();
+    if constexpr (!UW)
+        for (int k = tid; k < KP; k += kLongThreads) wsm[k] = ((const C *)A.w)[k];
+    for (int li = blockIdx.x; li < A.n_long; li += gridDim.x) {
+        const int64_t r = A.long_rows[li];
+        const int q0 = __ldg(A.prp + r), q1 = __ldg(A.prp + r + 1);
+        const int p0 = PX ? q0 : __ldg(A.rp + r), p1 = PX ? q1 : __ldg(A.rp + r + 1);
+        const int64_t xr = (PX && A.xrow) ? checked_row(__ldg(A.xrow + r), A.n, A.status) : r;
+        const C diag = (C)ld_plain((const AV *)A.diag + r);
+
+        // ---- 1. target ------------------------------------------------------------
+        C acc = C(0);
+        if (A.target == 0) {
+            int jj[PPT];                                              // rows of this thread's pieces of a tile
+            auto indices = [&](int pb) {
+#pragma unroll
+                for (int u = 0; u < PPT; ++u) {
+                    const int p = pb + (tid + u * kLongThreads) / P;
+                    jj[u] = p < p1 ? __ldg(xcol + p) : -1;
+                }
+            };
+            auto copy = [&](int pb, int b) {
+#pragma unroll
+                for (int u = 0; u < PPT; ++u) {
+                    const int q = tid + u * kLongThreads;
+                    if (jj[u] >= 0) cp_async16(&xs[b][q], X + checked_row(jj[u], A.n, A.status) * KP + q % P * V);
+                }
+                cp_async_commit();
+                for (int q = tid; q < TILE && pb + q < p1; q += kLongThreads) vs[b][q] = (C)ld_plain(val + pb + q);
+            };
+            indices(p0);
+            copy(p0, 0);
+            indices(p0 + TILE);
+            for (int pb = p0, b = 0; pb < p1; pb += TILE, b ^= 1) {
+                if (pb + TILE < p1) {
+                    copy(pb + TILE, b ^ 1);
+                    indices(pb + 2 * TILE);
+                    cp_async_wait<1>();
+                } else {
+                    cp_async_wait<0>();
+                }
+                __syncthreads();                                      // the tile is in place
+                if (tid < KP) {
+                    const TS *x = (const TS *)xs[b] + tid;
+                    const int m = min(TILE, p1 - pb);
+#pragma unroll 8
+                    for (int q = 0; q < m; ++q) acc = fma(vs[b][q], component<TS>(x, q * KP), acc);
+                }
+                __syncthreads();                                      // and read out
+            }
+        }
+        const C d = C(1) / diag;
+        if (tid < KP) {
+            const C xi = component<TS>(X + xr * KP, tid);
+            ys[tid] = A.target == 0 ? fma(-d, acc, xi) : xi;
+        }
+        int j1 = -1;                                                  // (search depth > 1: a short row of A)
+        C a1 = C(0);
+        if (A.target == 0 && p1 - p0 == 2) {
+            const int pj = __ldg(xcol + p0) == xr ? p0 + 1 : p0;
+            j1 = __ldg(xcol + pj);
+            a1 = -(C)ld_plain(val + pj) / diag;
+        }
+        __syncthreads();
+        C y[NP][V];
+        auto w = [&](int q, int e) { return UW ? C(1) : wsm[fit_piece<G, NP>(gl, q) * V + e]; };
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+#pragma unroll
+            for (int e = 0; e < V; ++e) y[q][e] = ys[fit_piece<G, NP>(gl, q) * V + e];
+        float syy = 0.f;
+        if constexpr (kMixed) {
+            auto piece = [&](int q) {
+                float s = 0.f;
+#pragma unroll
+                for (int e = 0; e < V; ++e) s = fmaf(UW ? y[q][e] : w(q, e) * y[q][e], y[q][e], s);
+                return s;
+            };
+            if constexpr (NP == 1) {
+                syy = piece(0);
+            } else {
+                auto leaf = [&](int t) { return make_float2(piece(2 * t), piece(2 * t + 1)); };
+                auto join = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
+                syy = plain_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), gmask);
+            }
+        }
+
+        // ---- 2. one-point fits, G lanes per entry ------------------------------------
+        C m = C(INFINITY);
+        bool defer = false;
+        int j = q0 + tid / G < q1 ? __ldg(fcol + q0 + tid / G) : -1;
+        for (int p = q0 + tid / G; p < q1; p += kLongThreads / G) {
+            const int jn = p + kLongThreads / G < q1 ? __ldg(fcol + p + kLongThreads / G) : -1;
+            C a_ = C(0), ls_ = C(NAN);
+            if (j == xr) {
+            } else if (j == j1) {
+                a_ = a1;
+                ls_ = C(0);
+                m = fmin(m, ls_);
+            } else {
+                const int64_t row = checked_row(j, A.n, A.status);
+                const auto nr = ld_plain((const typename Norm<C>::T *)A.norms + row);
+                uint4 raw[NP];
+                if constexpr (NP == 1) {
+                    raw[0] = ld16(X + row * KP);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < NP; q += 2) ld32(X + row * KP + fit_piece<G, NP>(gl, q) * V, raw[q], raw[q + 1]);
+                }
+                fit_entry<TS, G, NP, UW, COMP>(raw, y, w, nr, np, gmask, a_, ls_);
+                m = fmin(m, ls_);
+                if constexpr (kMixed) defer = defer || ls_ < C(1e-4) * syy;
+            }
+            if (gl == 0) { a_out[p] = a_; ls_out[p] = ls_; }
+            j = jn;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (tid % 32 == 0) msm[tid / 32] = m;
+        if constexpr (kMixed) defer = __syncthreads_or(defer);
+        else __syncthreads();
+#pragma unroll
+        for (int k = 0; k < W; ++k) m = fmin(m, msm[k]);
+
+        // ---- 3. strength flags and counts --------------------------------------------
+        const C theta = (C)A.theta;
+        int cnt = 0;
+        for (int p = q0 + tid; p < q1; p += kLongThreads) {
+            const C l = ls_out[p];                                    // NaN on the diagonal
+            const bool strong = l == C(0) || theta * l < m;
+            A.flag_out[p] = (uint8_t)strong;
+            cnt += strong;
+        }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (tid % 32 == 0) csm[tid / 32] = cnt;
+        __syncthreads();
+        if (tid == 0) {
+            int total = 0;
+            for (int k = 0; k < W; ++k) total += csm[k];
+            A.count_out[r] = total;
+            if (kMixed && defer) A.defer_list[atomicAdd(A.defer_count, 1u)] = (int32_t)r;
         }
     }
 }
@@ -846,6 +1045,11 @@ cudaError_t go_fit(const EdgeArgs &a, cudaStream_t s)
     }
     e = launch_chained(kern, (unsigned)(((int64_t)a.n + rows - 1) / rows), T, smem, s, a, (int)cap, el);
     if (e != cudaSuccess) return e;
+    if (a.n_long > 0) {
+        e = launch_chained(k_edge_long<TS, P, UW, PX, COMP>, (unsigned)(a.n_long < 152 * 4 ? a.n_long : 152 * 4),
+                           kLongThreads, 0, s, a);
+        if (e != cudaSuccess) return e;
+    }
     if constexpr (!std::is_same<TS, double>::value)
         e = launch_chained(k_edge_fixup<TS, P, PX>, 152, kFixThreads, 0, s, a);
     return e;

@@ -454,6 +454,16 @@ __global__ void __launch_bounds__(kThreads) k_create(CreateArgs A)
     A.d32_p[r] = A.d32_o[r] = (float)diag;
 }
 
+// (cap: row pointers that do not pass the check of launch_create are listed too)
+__global__ void __launch_bounds__(kThreads)
+k_long_rows(const int32_t *__restrict__ rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap, uint32_t *count)
+{
+    const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (r >= n || rp[r + 1] - rp[r] <= long_len) return;
+    const uint32_t at = atomicAdd(count, 1u);
+    if (at < cap) rows[at] = (int32_t)r;
+}
+
 inline unsigned blocks(int64_t work) { return (unsigned)((work + kThreads - 1) / kThreads); }
 
 // priority keys of the coarse-point selection: one Philox4x64-10 block per
@@ -582,6 +592,14 @@ cudaError_t launch_create(const CreateArgs &a, cudaStream_t s)
 {
     if (a.n == 0) return cudaSuccess;
     k_create<<<blocks(a.n), kThreads, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_long_rows(const int32_t *rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap,
+                             uint32_t *count, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    k_long_rows<<<blocks(n), kThreads, 0, s>>>(rp, n, long_len, rows, cap, count);
     return cudaGetLastError();
 }
 

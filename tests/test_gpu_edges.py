@@ -348,6 +348,74 @@ def test_distances_with_zero_columns(name, K, weighted):
     compare_fp64(rp, col, val, got, want, 0.5, w)
 
 
+def hub(n, lengths, seed):
+    """A graph of some eleven entries a row, a row of each length first, and last a row
+    with row 0 as its one neighbour."""
+    rng = np.random.default_rng(seed)
+    adj = [set(rng.integers(0, n, 3).tolist()) | {i} for i in range(n)]
+    for i, m in enumerate(lengths):
+        adj[i] |= set(rng.choice(n, m, replace=False).tolist())
+    for i in range(n):
+        for j in list(adj[i]):
+            adj[j].add(i)
+    for i, m in enumerate(lengths):              # rows of just these lengths; columns stay symmetric enough
+        keep = sorted(adj[i] - {i}, key=lambda j: rng.random())[:m - 1]
+        adj[i] = set(keep) | {i}
+    adj[n - 1] = {0, n - 1}
+    rp = np.concatenate([[0], np.cumsum([len(a) for a in adj])]).astype(np.int64)
+    col = np.concatenate([sorted(a) for a in adj]).astype(np.int32)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    val = -rng.uniform(0.5, 1.5, len(col))
+    val[rows == col] = 1.5 * np.diff(rp)
+    return rp, col, val
+
+
+def dense(n, seed):
+    rng = np.random.default_rng(seed)
+    val = -rng.uniform(0.5, 1.5, (n, n)) + 2 * n * np.eye(n)
+    return (np.arange(n + 1) * n).astype(np.int64), np.tile(np.arange(n, dtype=np.int32), n), val.ravel()
+
+
+@pytest.mark.parametrize("K", [1, 7, 16, 32, 64])
+@pytest.mark.parametrize("prec,summation", [("fp64", "plain"), ("fp32", "compensated"), ("fp32", "plain"),
+                                            ("bf16", "compensated")])
+@pytest.mark.parametrize("form", ["colored", "weighted", "plain target", "depth 2"])
+def test_long_rows_round_alike(K, prec, summation, form):
+    """Rows of 64 to 600 entries, fitted by blocks of their own, and the same rows in a
+    handle whose other rows are so long that these are not: the same bits."""
+    if form == "depth 2":
+        m, extra = hub(6000, (300,), 2), dense(1500, 3)
+    else:
+        m, extra = hub(700, (64, 65, 66, 257, 513, 600), 2), dense(600, 3)
+    N = len(m[0]) - 1
+    X = np.random.default_rng(4).uniform(-1, 1, (N + len(extra[0]) - 1, K))
+    X[5::90] = 0.0
+    out = []
+    for mats in ([m], [m, extra]):
+        n = sum(len(t[0]) - 1 for t in mats)
+        with amgd.Handle(None, None, None, K, 1, batch=mats) as h:
+            h.set_precision(prec)
+            h.set_summation(summation)
+            if form == "colored":
+                h.set_coloring((np.arange(n) % 3).astype(np.int32))
+            elif form == "weighted":
+                h.set_weights(np.linspace(0.5, 1.5, K))
+            elif form == "plain target":
+                h.set_target(1)
+            else:
+                h.set_search_depth(2)
+            h.set_vectors(X[:n])
+            d = h.distances(0.5)
+            rp, col = h.strength()
+            if form == "depth 2":
+                last = int(h.distance_pattern()[0][N])
+            else:
+                last = len(m[1])
+            out.append([d["a"][:last], d["ls"][:last], rp[:N + 1], col[:rp[N]]])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
 def test_reciprocals_of_the_fp32_range():
     """dist = 1 / LS of the FP32 path over the type's whole range: equal to the
     FP64 quotient of the exported LS to one unit of its last place."""
