@@ -450,11 +450,17 @@ struct FitLayout {
     static constexpr bool LS_OVER = sizeof(C) == 4;                    // LS replaces the gather index
     static constexpr int SLOT = 4 + (LS_OVER ? 1 : 2) * (int)sizeof(C) + 1;
     static constexpr int UT = NP <= 2 || (sizeof(TS) == 8 && NP <= 4) ? 4 : (NP <= 4 ? 2 : 1);   // and in the target
-    static int bytes(int cap, bool unit_w) { return (unit_w ? 0 : WB) + cap * SLOT; }
+    static int bytes(int cap, bool unit_w, int shared_rows)           // of a block (shared_rows: with several shares)
+    {
+        return (unit_w ? 0 : WB) + shared_rows * KP * (int)sizeof(C) + cap * SLOT;
+    }
     static_assert(NP == 1 ? G == 1 : NP % 2 == 0, "pairs of pieces");
 };
 
-// SHARED: several shares per row (el of them; else one)
+// SHARED: several shares per row (el of them; else one).  Every lane of the row then
+// forms the target of pieces of its own, and y_i reaches the others by shared memory
+// (20000 rows of 70 entries, K = 16 FP64, four shares: 215 us, 420 with the whole
+// target in each).
 template <class TS, int P, bool UW, bool PX, bool COMP, bool SHARED>
 __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fit(EdgeArgs A, int cap, int shares)
 {
@@ -472,15 +478,16 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
     const int gl = tid % G, sub = tid / G % el, width = G * el;
     const unsigned gmask = G == 1 ? 1u << (tid % 32) : ((1u << G) - 1u) << ((tid % 32) / G * G);
     const unsigned rmask = width == 32 ? 0xffffffffu : ((1u << width) - 1u) << ((tid % 32) / width * width);
+    const int rows = T / width;
     C *ws = reinterpret_cast<C *>(esm);                              // weights (UW: none)
-    C *a_s = reinterpret_cast<C *>(esm + (UW ? 0 : L::WB));           // values, then a
+    C *ys = reinterpret_cast<C *>(esm + (UW ? 0 : L::WB));            // targets (SHARED)
+    C *a_s = ys + (SHARED ? rows * KP : 0);                          // values, then a
     C *lsep = a_s + cap;                                             // LS where it has its own place
     int32_t *x_s = reinterpret_cast<int32_t *>(L::LS_OVER ? lsep : lsep + cap);   // gather indices
     C *ls_s = L::LS_OVER ? reinterpret_cast<C *>(x_s) : lsep;
     uint8_t *fl_s = reinterpret_cast<uint8_t *>(x_s + cap);
 
     const int np = G == 1 ? (A.K + V - 1) / V : NP;                   // pieces that are not all padding
-    const int rows = T / width;
     const int64_t R0 = (int64_t)blockIdx.x * rows;
     const int nr = (int)min((int64_t)rows, A.n - R0);
     const int S0 = __ldg(A.prp + R0), S1 = __ldg(A.prp + R0 + nr);
@@ -523,7 +530,45 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
         float syy = 0.f;
         int j1 = -1;                 // exact rule: the row's one off-diagonal (gather index)
         C a1 = C(0);
-        {
+        if constexpr (SHARED) {
+            constexpr int US = 5;                                    // entries in flight
+            C *yr = ys + tid / width * KP;
+            const C d = C(1) / diag;
+            for (int t = tid % width; t < (G == 1 ? np : P); t += width) {
+                Acc<C, V> acc;
+                acc.zero();
+                if (A.target == 0) {
+                    for (int pb = p0; pb < p1; pb += US) {
+                        uint4 raw[US];
+                        C vv[US];
+#pragma unroll
+                        for (int u = 0; u < US; ++u) {
+                            const int p = pb + u;
+                            if (p >= p1) break;
+                            const int64_t j = PX && staged ? x_s[p - S0] : __ldg(xcol + p);
+                            vv[u] = PX && staged ? a_s[p - S0] : (C)ld_plain(val + p);
+                            raw[u] = ld16(X + checked_row(j, A.n, A.status) * KP + t * V);
+                        }
+#pragma unroll
+                        for (int u = 0; u < US; ++u) {
+                            if (pb + u >= p1) break;
+                            C x[V];
+                            S::unpack(raw[u], x);
+                            acc.fma_piece(vv[u], x);
+                        }
+                    }
+                }
+                C xi[V];
+                S::unpack(ld16(X + xr * KP + t * V), xi);
+#pragma unroll
+                for (int e = 0; e < V; ++e) yr[t * V + e] = A.target == 0 ? fma(-d, acc.get(e), xi[e]) : xi[e];
+            }
+            __syncwarp(rmask);
+#pragma unroll
+            for (int q = 0; q < NP; ++q)
+#pragma unroll
+                for (int e = 0; e < V; ++e) y[q][e] = yr[fit_piece<G, NP>(gl, q) * V + e];
+        } else {
             Acc<C, V> acc[NP];
 #pragma unroll
             for (int t = 0; t < NP; ++t) acc[t].zero();
@@ -571,6 +616,8 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
                     for (int e = 0; e < V; ++e) y[t][e] = fma(-d, acc[t].get(e), y[t][e]);
                 }
             }
+        }
+        {
             if constexpr (kMixed) {
                 // S_yy, in the order of the other sums
                 auto piece = [&](int q) {
@@ -998,14 +1045,30 @@ __global__ void __launch_bounds__(kFixThreads) k_edge_fixup(EdgeArgs A)
 
 // Shares of a row's entries and threads of a block.  A small matrix leaves most
 // of the chip idle at one lane group per row, and the pass is then the latency
-// of a row's entries one after the other: up to four shares (each forms the
-// target of its own) while the lanes fit in two warps per scheduler, and
+// of a row's entries one after the other: up to four shares, more for rows of more
+// than eight entries a share, while the lanes fit in two warps per scheduler, and
 // blocks of down to 32 threads while there are fewer than four per SM (64 x 64
-// 5-point, K = 8, FP64: 12.9 us with one share, 8.7 with four).
-inline int fit_shares(int64_t lanes, int G)
+// 5-point, K = 8, FP64: 12.9 us with one share, 8.7 with four; 2000 rows of 200,
+// K = 16 FP64: 272 with four, 108 with sixteen).
+// Long rows fill the shared memory of an SM with the slots of few threads: as many
+// shares as leave a block's slots within its part of it (100k rows of 100 entries,
+// K = 16 FP32: 528 us with one share, 264 with four; FP64 1545 / 1338).  Of six or
+// more blocks one may be lost rather than go from one share to two (9-point depth 2,
+// 25 a row, FP32: 112 / 118) or past a lane per piece of the target (20000 rows of
+// 100, FP32: 65 with four shares, 79 with eight); of four blocks it may not (of 70,
+// K = 16 FP64: 290 with four, 215 with eight).
+template <int P, int G>
+inline int fit_shares(int64_t n, int64_t nnz, int slot, int blocks)
 {
+    const int64_t avg = nnz / n, part = (int64_t)227 * 1024 / blocks;
     int el = 1;
-    while (el < 4 && G * el < 32 && lanes * el < (int64_t)152 * 256) el *= 2;
+    while (G * el < 32 && n * G * el < (int64_t)152 * 256 && (el < 4 || avg > 8 * el)) el *= 2;
+    while (G * el < 32) {
+        const int64_t bytes = (kFitThreads / (G * el) * avg * 5 / 4 + 32) * slot;
+        const bool lose_one = blocks >= 6 && (el == 1 || G * el >= P);
+        if (bytes <= (lose_one ? part * 115 / 100 : part)) break;
+        el *= 2;
+    }
     return el;
 }
 inline int fit_threads(int64_t lanes)
@@ -1028,13 +1091,13 @@ cudaError_t go_fit(const EdgeArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     // slots staged per block: the average rows' entries and a quarter more
     // (a block with longer rows works on global memory), at most 96 KB
-    const int el = fit_shares((int64_t)a.n * L::G, L::G);
+    const int el = fit_shares<P, L::G>(a.n, a.nnz_p, L::SLOT, L::MINB);
     const int T = fit_threads((int64_t)a.n * L::G * el);
-    const int rows = T / (L::G * el);
+    const int rows = T / (L::G * el), yrows = el > 1 ? rows : 0;
     int64_t cap = (int64_t)((double)a.nnz_p / a.n * rows * 1.25) + 32;
-    const int64_t most = (96 * 1024 - L::bytes(0, UW)) / L::SLOT;
+    const int64_t most = (96 * 1024 - L::bytes(0, UW, yrows)) / L::SLOT;
     cap = (cap < most ? cap : most) & ~(int64_t)15;
-    const int smem = L::bytes((int)cap, UW);
+    const int smem = L::bytes((int)cap, UW, yrows);
     const auto kern = el > 1 ? k_edge_fit<TS, P, UW, PX, COMP, true> : k_edge_fit<TS, P, UW, PX, COMP, false>;
     static PerDevice opted[2];               // shared-memory opt-in made on each device
     const int dev = current_device_index();

@@ -416,6 +416,47 @@ def test_long_rows_round_alike(K, prec, summation, form):
         assert np.array_equal(a, b, equal_nan=True)
 
 
+def circulant(n, m, seed):
+    """m entries in every row, the diagonal first among the column offsets."""
+    rng = np.random.default_rng(seed)
+    off = np.concatenate([[0], rng.choice(np.arange(1, n), m - 1, replace=False)])
+    col = np.sort((np.arange(n)[:, None] + off) % n, 1).astype(np.int32)
+    val = -rng.uniform(0.5, 1.5, (n, m))
+    val[col == np.arange(n)[:, None]] = 1.5 * m
+    return (np.arange(n + 1) * m).astype(np.int64), col.ravel(), val.ravel()
+
+
+@pytest.mark.parametrize("K", [1, 7, 16, 32, 64])
+@pytest.mark.parametrize("prec,summation", [("fp64", "plain"), ("fp32", "compensated"), ("fp32", "plain"),
+                                            ("bf16", "compensated"), ("bf16", "plain")])
+@pytest.mark.parametrize("n,m", [(97, 2), (301, 6), (301, 40), (700, 63), (301, 200)])
+@pytest.mark.parametrize("form", ["colored", "weighted", "plain target"])
+def test_shares_of_a_row_round_alike(n, m, prec, summation, K, form):
+    """Two to thirty-two lane groups per row in a small handle; one, or a block per row of
+    200 entries, in a large one: the same bits."""
+    M, extra = circulant(n, m, 2), inputs.lap1d(40001)
+    X = np.random.default_rng(4).uniform(-1, 1, (n + 40001, K))
+    X[5::90] = 0.0
+    out = []
+    for mats in ([M], [M, extra]):
+        rows = sum(len(t[0]) - 1 for t in mats)
+        with amgd.Handle(None, None, None, K, 1, batch=mats) as h:
+            h.set_precision(prec)
+            h.set_summation(summation)
+            if form == "colored":
+                h.set_coloring((np.arange(rows) % 3).astype(np.int32))
+            elif form == "weighted":
+                h.set_weights(np.linspace(0.5, 1.5, K))
+            else:
+                h.set_target(1)
+            h.set_vectors(X[:rows])
+            d = h.distances(0.5)
+            rp, col = h.strength()
+            out.append([d["a"][:n * m], d["ls"][:n * m], rp[:n + 1], col[:rp[n]]])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
 def test_reciprocals_of_the_fp32_range():
     """dist = 1 / LS of the FP32 path over the type's whole range: equal to the
     FP64 quotient of the exported LS to one unit of its last place."""
