@@ -155,6 +155,7 @@ struct amgd_ctx {
     // rows of the fits' pattern that are too long for the row-per-lanes kernel (find_long_rows)
     int32_t *long_rows = nullptr, *long_rows_p = nullptr;    // of A (in the slab) and of G_d
     int32_t long_len = INT32_MAX, n_long = 0;
+    bool uneven = false;                         // neighbouring rows differ much in length
     int32_t summation = AMGD_SUM_COMPENSATED;   // LS sums of the mixed paths (edge stage 2)
     int32_t *prp = nullptr, *pcol = nullptr;
     int64_t nnz_p = 0, E_p = 0;
@@ -781,6 +782,7 @@ int run_edge(amgd_ctx *h, double theta, cudaStream_t s)
     a.long_len = h->long_len;
     a.long_rows = h->depth > 1 ? h->long_rows_p : h->long_rows;
     a.n_long = h->n_long;
+    a.uneven = h->uneven;
     a.status = h->status;
     bool unit_w = true;
     for (double wk : h->h_w) unit_w = unit_w && wk == 1.0;
@@ -801,20 +803,20 @@ int alloc_slot_outputs(amgd_ctx *h, int st)
     return AMGD_OK;
 }
 
-// Lists the rows of the fits' pattern (prp, nnz_p set) that a block of their own
+// What the distance pass has to know of the rows' lengths.  Lists the rows of the fits' pattern (prp, nnz_p set) that a block of their own
 // fits: more than kLongRow entries and four times the average.  (Rows of 100 entries
 // in a graph of 17 a row, 20000 rows, K = 16: FP32 74 us among the others, 39 with
 // blocks of their own; FP64 318 / 168.  Where all rows are that long, a block each is
 // slower: 20000 rows of 100, FP32 78 / 232.)  rows: long_row_cap entries.  The first
 // form only enqueues; the second takes what it found to the host, with the error word.
 constexpr int32_t kLongRow = 64;
-constexpr int kErrWords = 2;                      // the error word of a check; long rows
+constexpr int kErrWords = 4;                      // the error word of a check; long rows; filled (64 bits)
 size_t long_row_cap(int64_t nnz_p) { return (size_t)(nnz_p / kLongRow + 1); }
 cudaError_t queue_long_rows(amgd_ctx *h, int32_t *rows)
 {
     h->long_len = (int32_t)std::max<int64_t>(kLongRow, h->n ? 4 * (h->nnz_p / h->n) : 0);
     return launch_long_rows(h->prp, (int32_t)h->n, h->long_len, rows, (uint32_t)long_row_cap(h->nnz_p),
-                            h->err_word + 1, h->stream);
+                            h->err_word + 1, (unsigned long long *)(h->err_word + 2), h->stream);
 }
 cudaError_t take_long_rows(amgd_ctx *h, uint32_t *err)
 {
@@ -823,6 +825,9 @@ cudaError_t take_long_rows(amgd_ctx *h, uint32_t *err)
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     *err = found[0];
     h->n_long = (int32_t)found[1];
+    unsigned long long filled = 0;
+    std::memcpy(&filled, found + 2, sizeof filled);
+    h->uneven = filled > (unsigned long long)(h->nnz_p + h->nnz_p / 8);
     return e;
 }
 int find_long_rows(amgd_ctx *h, int32_t *rows)

@@ -339,6 +339,7 @@ struct EdgeArgs {                // everything in the caller's numbering
     int32_t long_len = INT32_MAX;        // rows with more fits than this are listed in long_rows
     const int32_t *long_rows = nullptr;
     int32_t n_long = 0;
+    bool uneven = false;                 // neighbouring rows differ much in length
     uint32_t *status = nullptr;  // device status word (checked build: index range)
 };
 
@@ -383,9 +384,10 @@ cudaError_t launch_sell_fill(const SellArgs &a, const int32_t *rowmap, const int
                              int32_t *slot, cudaStream_t s);
 
 // rows with more than long_len entries (the first cap of them), in no order, and their
-// number (zero before the call)
+// number (zero before the call); filled (zero before the call): 32 times the longest of
+// the other rows of every 32
 cudaError_t launch_long_rows(const int32_t *rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap,
-                             uint32_t *count, cudaStream_t s);
+                             uint32_t *count, unsigned long long *filled, cudaStream_t s);
 // in_place: read the vectors in the sweeps' row order (search depth 1)
 cudaError_t launch_edge(int storage, bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s);

@@ -456,12 +456,23 @@ __global__ void __launch_bounds__(kThreads) k_create(CreateArgs A)
 
 // (cap: row pointers that do not pass the check of launch_create are listed too)
 __global__ void __launch_bounds__(kThreads)
-k_long_rows(const int32_t *__restrict__ rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap, uint32_t *count)
+k_long_rows(const int32_t *__restrict__ rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap, uint32_t *count,
+            unsigned long long *filled)
 {
+    __shared__ unsigned long long sum;
     const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (r >= n || rp[r + 1] - rp[r] <= long_len) return;
-    const uint32_t at = atomicAdd(count, 1u);
-    if (at < cap) rows[at] = (int32_t)r;
+    int len = r < n ? rp[r + 1] - rp[r] : 0;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    if (len > long_len) {
+        const uint32_t at = atomicAdd(count, 1u);
+        if (at < cap) rows[at] = (int32_t)r;
+        len = 0;
+    }
+    const unsigned longest = __reduce_max_sync(0xffffffffu, (unsigned)max(len, 0));
+    if (threadIdx.x % 32 == 0) atomicAdd(&sum, 32ull * longest);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(filled, sum);
 }
 
 inline unsigned blocks(int64_t work) { return (unsigned)((work + kThreads - 1) / kThreads); }
@@ -596,10 +607,10 @@ cudaError_t launch_create(const CreateArgs &a, cudaStream_t s)
 }
 
 cudaError_t launch_long_rows(const int32_t *rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap,
-                             uint32_t *count, cudaStream_t s)
+                             uint32_t *count, unsigned long long *filled, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_long_rows<<<blocks(n), kThreads, 0, s>>>(rp, n, long_len, rows, cap, count);
+    k_long_rows<<<blocks(n), kThreads, 0, s>>>(rp, n, long_len, rows, cap, count, filled);
     return cudaGetLastError();
 }
 

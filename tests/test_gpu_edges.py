@@ -457,6 +457,40 @@ def test_shares_of_a_row_round_alike(n, m, prec, summation, K, form):
         assert np.array_equal(a, b, equal_nan=True)
 
 
+@pytest.mark.parametrize("K", [1, 7, 16, 32, 64])
+@pytest.mark.parametrize("prec,summation", [("fp64", "plain"), ("fp32", "compensated"), ("fp32", "plain"),
+                                            ("bf16", "compensated")])
+@pytest.mark.parametrize("form", ["colored", "depth 2"])
+@pytest.mark.parametrize("rows", [4129, 40003])
+def test_sorted_rows_round_alike(rows, prec, summation, K, form):
+    """A graph whose rows are fitted in the order of their lengths, and the same graph in a
+    handle of rows so even that they are fitted as they come."""
+    side = 500 if rows < 10000 else 700
+    M, extra = inputs.graph_laplacian(rows, 4.0, 4), inputs.poisson2d_5pt(side)
+    X = np.random.default_rng(4).uniform(-1, 1, (rows + side * side, K))
+    if form == "depth 2":
+        if rows > 10000 or K > 16:
+            pytest.skip("one size of the wider pattern")
+        M = inputs.graph_laplacian(rows, 1.5, 4)
+    out = []
+    for mats in ([M], [M, extra]):
+        n = sum(len(t[0]) - 1 for t in mats)
+        with amgd.Handle(None, None, None, K, 1, batch=mats) as h:
+            h.set_precision(prec)
+            h.set_summation(summation)
+            if form == "colored":
+                h.set_coloring((np.arange(n) % 3).astype(np.int32))
+            else:
+                h.set_search_depth(2)
+            h.set_vectors(X[:n])
+            d = h.distances(0.5)
+            rp, col = h.strength()
+            last = int(h.distance_pattern()[0][rows])
+            out.append([d["a"][:last], d["ls"][:last], rp[:rows + 1], col[:rp[rows]]])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
 def test_reciprocals_of_the_fp32_range():
     """dist = 1 / LS of the FP32 path over the type's whole range: equal to the
     FP64 quotient of the exported LS to one unit of its last place."""
