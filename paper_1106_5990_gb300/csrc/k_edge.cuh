@@ -259,8 +259,9 @@ template <> struct Norm<double> { using T = double2; };
 
 // One fit: S_yx, a_ij and LS_ij from the lane's pieces of x_j (as stored), of
 // the target and of the weights (w, UW: unused), the first np of them not all
-// padding; every lane of the row ends with the result.
-template <class TS, int G, int NP, bool UW, bool COMP, class W>
+// padding; every lane of the row ends with the result.  OWN: S_xx is formed here,
+// in k_norms' order (plain sums; nr is not read).
+template <class TS, int G, int NP, bool UW, bool COMP, bool OWN, class W>
 __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
                                           const typename Store<TS>::C (&y)[NP][Store<TS>::V], const W &w,
                                           const typename Norm<typename Store<TS>::C>::T &nr, int np, unsigned mask,
@@ -300,6 +301,7 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
     } else if constexpr (NP == 1) {
         C x[V];
         S::unpack(raw[0], x);
+        float sxx = nr;
         auto wx = [&](int e) { return UW ? x[e] : w(0, e) * x[e]; };
         float syx;
         if constexpr (COMP) {
@@ -318,8 +320,15 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
             for (int e = 0; e < V; e += 2)
                 s = __ffma2_rn(make_float2(wx(e), wx(e + 1)), make_float2(y[0][e], y[0][e + 1]), s);
             syx = s.x + s.y;
+            if constexpr (OWN) {
+                float2 n2 = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int e = 0; e < V; e += 2)
+                    n2 = __ffma2_rn(make_float2(wx(e), wx(e + 1)), make_float2(x[e], x[e + 1]), n2);
+                sxx = n2.x + n2.y;
+            }
         }
-        a_ = (nr == 0.f) ? 0.f : divide(syx, nr);
+        a_ = (sxx == 0.f) ? 0.f : divide(syx, sxx);
         auto d2 = [&](int e) { return make_float2(fmaf(-a_, x[e], y[0][e]), fmaf(-a_, x[e + 1], y[0][e + 1])); };
         auto wd2 = [&](int e, float2 d) { return UW ? d : make_float2(w(0, e) * d.x, w(0, e + 1) * d.y); };
         if constexpr (COMP) {
@@ -329,16 +338,17 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
             });
             ls_ = comp_total<1>(v, mask);
         } else {
+            const float2 na = make_float2(-a_, -a_);
             float2 s = make_float2(0.f, 0.f);
 #pragma unroll
             for (int e = 0; e < V; e += 2) {
-                const float2 d = d2(e);
+                const float2 d = __ffma2_rn(na, make_float2(x[e], x[e + 1]), make_float2(y[0][e], y[0][e + 1]));
                 s = __ffma2_rn(wd2(e, d), d, s);
             }
             ls_ = s.x + s.y;
         }
     } else {
-        float syx;
+        float syx, sxx = nr;
         // products w x y of component e of the pair's two pieces
         auto xy = [&](const C (&x0)[V], const C (&x1)[V], int q, int e) {
             return make_float2(__fmul_rn(UW ? x0[e] : w(q, e) * x0[e], y[q][e]),
@@ -354,21 +364,26 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
             auto join = [](const Comp2 &a, const Comp2 &b) { return comp2_join(a, b); };
             syx = comp_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
         } else {
-            auto piece = [&](int q) {
+            // piece q's part of S_yx, or of S_xx
+            auto piece = [&](int q, bool norm) {
                 C x[V];
                 S::unpack(raw[q], x);
                 float2 s = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int e = 0; e < V; e += 2)
                     s = __ffma2_rn(UW ? make_float2(x[e], x[e + 1]) : make_float2(w(q, e) * x[e], w(q, e + 1) * x[e + 1]),
-                                   make_float2(y[q][e], y[q][e + 1]), s);
+                                   norm ? make_float2(x[e], x[e + 1]) : make_float2(y[q][e], y[q][e + 1]), s);
                 return s.x + s.y;
             };
-            auto leaf = [&](int t) { return make_float2(piece(2 * t), piece(2 * t + 1)); };
             auto join = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
+            auto leaf = [&](int t) { return make_float2(piece(2 * t, false), piece(2 * t + 1, false)); };
             syx = plain_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
+            if constexpr (OWN) {
+                auto nleaf = [&](int t) { return make_float2(piece(2 * t, true), piece(2 * t + 1, true)); };
+                sxx = plain_total<G>(tree_sum<0, 1, NP / 2>(nleaf, join), mask);
+            }
         }
-        a_ = (nr == 0.f) ? 0.f : divide(syx, nr);
+        a_ = (sxx == 0.f) ? 0.f : divide(syx, sxx);
         // residuals of component e of a pair's two pieces, times the weights
         auto terms = [&](int t, float2 (&d)[V], float2 (&wd)[V]) {
             C x0[V], x1[V];
@@ -392,17 +407,19 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
             auto join = [](const Comp2 &a, const Comp2 &b) { return comp2_join(a, b); };
             ls_ = comp_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
         } else {
-            auto leaf = [&](int t) {
-                float2 d[V], wd[V];
-                terms(t, d, wd);
-                float2 even = make_float2(0.f, 0.f), odd = make_float2(0.f, 0.f);
+            const float2 na = make_float2(-a_, -a_);
+            auto piece = [&](int q) {
+                C x[V];
+                S::unpack(raw[q], x);
+                float2 s = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int k = 0; k < V / 2; ++k) {
-                    even = __ffma2_rn(wd[2 * k], d[2 * k], even);
-                    odd = __ffma2_rn(wd[2 * k + 1], d[2 * k + 1], odd);
+                for (int e = 0; e < V; e += 2) {
+                    const float2 d = __ffma2_rn(na, make_float2(x[e], x[e + 1]), make_float2(y[q][e], y[q][e + 1]));
+                    s = __ffma2_rn(UW ? d : make_float2(w(q, e) * d.x, w(q, e + 1) * d.y), d, s);
                 }
-                return __fadd2_rn(even, odd);
+                return s.x + s.y;
             };
+            auto leaf = [&](int t) { return make_float2(piece(2 * t), piece(2 * t + 1)); };
             auto join = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
             ls_ = plain_total<G>(tree_sum<0, 1, NP / 2>(leaf, join), mask);
         }
@@ -436,8 +453,16 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
 // Before (G = P lanes per row, S_xx per entry) the two workloads took 193 (with
 // the best shape) and 1331 us (752 with the best), K = 13 FP64 7-point 333^2
 // 385 (150 now), 25 entries per row of BF16 K = 16 (512^2) 236 (92 now).
+//
+// Plain sums are half the arithmetic and bound by the gathers: they form S_xx from the
+// row at hand rather than read the vectors once more for it and gather the norms, and
+// run in more and smaller blocks.  us, in the compensated sums' layout -> in this one /
+// in the former row kernel's tuned shapes: 9-point 1024^2 K = 16 FP32 169 -> 150 / 149,
+// BF16 143 -> 119 / 120, K = 32 FP32 313 -> 275 / 268; 7-point 128^3 K = 32 FP32
+// 575 -> 484 / 460, K = 16 298 -> 256 / 234; 300k-row graph K = 16 FP32 187 -> 158 / 172.
+// Two entries at a time lose as above (152 -> 170).
 // ---------------------------------------------------------------------------
-template <class TS, int P>
+template <class TS, int P, bool COMP>
 struct FitLayout {
     using C = typename Store<TS>::C;
     static constexpr int V = Store<TS>::V, KP = P * V;
@@ -445,7 +470,13 @@ struct FitLayout {
     static constexpr int G = KP <= CL ? 1 : KP / CL;
     static constexpr int NP = P / G;
     static constexpr int U = sizeof(TS) == 8 && NP <= 4 ? 4 : 1;      // entries gathered at a time
-    static constexpr int MINB = sizeof(TS) == 8 ? 4 : sizeof(TS) == 4 ? 7 : NP * V <= 16 ? 6 : 5;   // resident blocks
+    // plain FP32 sums form S_xx with the fit, in blocks of 64 threads
+    static constexpr bool OWN = !COMP && sizeof(TS) < 8;
+    static constexpr int THREADS = OWN ? 64 : kFitThreads;
+    // resident blocks (of kFitThreads)
+    static constexpr int MINB = sizeof(TS) == 8 ? 4
+                              : OWN ? (NP * V <= 4 ? 10 : NP * V <= 16 ? 8 : 5)
+                              : sizeof(TS) == 4 ? 7 : NP * V <= 16 ? 6 : 5;
     static constexpr int WB = KP * (int)sizeof(C);                    // weights of the block
     static constexpr bool LS_OVER = sizeof(C) == 4;                    // LS replaces the gather index
     static constexpr int SLOT = 4 + (LS_OVER ? 1 : 2) * (int)sizeof(C) + 1;
@@ -462,12 +493,12 @@ struct FitLayout {
 // (20000 rows of 70 entries, K = 16 FP64, four shares: 215 us, 420 with the whole
 // target in each).
 template <class TS, int P, bool UW, bool PX, bool COMP, bool SHARED>
-__global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fit(EdgeArgs A, int cap, int shares)
+__global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P, COMP>::MINB) k_edge_fit(EdgeArgs A, int cap, int shares)
 {
     using S = Store<TS>;
     using C = typename S::C;
     using AV = typename S::A;
-    using L = FitLayout<TS, P>;
+    using L = FitLayout<TS, P, COMP>;
     constexpr int V = S::V, KP = L::KP, G = L::G, NP = L::NP, UT = L::UT, U = L::U;
     constexpr bool kMixed = !std::is_same<C, double>::value;
     extern __shared__ __align__(16) unsigned char esm[];
@@ -689,7 +720,7 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (jj[u] < 0 || jj[u] == xr) continue;
-                nr_j[u] = ld_plain((const typename Norm<C>::T *)A.norms + checked_row(jj[u], A.n, A.status));
+                if constexpr (!L::OWN) nr_j[u] = ld_plain((const typename Norm<C>::T *)A.norms + checked_row(jj[u], A.n, A.status));
                 gather(jj[u], raw[u]);
             }
             if constexpr (G > 1) __syncwarp(gmask);      // every lane has read these entries' indices
@@ -704,7 +735,7 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P>::MINB) k_edge_fi
                     ls_ = C(0);
                     m = fmin(m, ls_);
                 } else {
-                    fit_entry<TS, G, NP, UW, COMP>(raw[u], y, w, nr_j[u], np, gmask, a_, ls_);
+                    fit_entry<TS, G, NP, UW, COMP, L::OWN>(raw[u], y, w, nr_j[u], np, gmask, a_, ls_);
                     m = fmin(m, ls_);
                     if constexpr (kMixed) defer = defer || ls_ < C(1e-4) * syy;
                 }
@@ -781,7 +812,7 @@ __global__ void __launch_bounds__(kLongThreads) k_edge_long(EdgeArgs A)
     using S = Store<TS>;
     using C = typename S::C;
     using AV = typename S::A;
-    using L = FitLayout<TS, P>;
+    using L = FitLayout<TS, P, COMP>;
     using LL = LongLayout<TS, P>;
     constexpr int V = S::V, KP = L::KP, G = L::G, NP = L::NP, TILE = LL::TILE, PPT = LL::PPT, W = kLongThreads / 32;
     constexpr bool kMixed = !std::is_same<C, double>::value;
@@ -901,7 +932,8 @@ __global__ void __launch_bounds__(kLongThreads) k_edge_long(EdgeArgs A)
                 m = fmin(m, ls_);
             } else {
                 const int64_t row = checked_row(j, A.n, A.status);
-                const auto nr = ld_plain((const typename Norm<C>::T *)A.norms + row);
+                typename Norm<C>::T nr = {};
+                if constexpr (!L::OWN) nr = ld_plain((const typename Norm<C>::T *)A.norms + row);
                 uint4 raw[NP];
                 if constexpr (NP == 1) {
                     raw[0] = ld16(X + row * KP);
@@ -909,7 +941,7 @@ __global__ void __launch_bounds__(kLongThreads) k_edge_long(EdgeArgs A)
 #pragma unroll
                     for (int q = 0; q < NP; q += 2) ld32(X + row * KP + fit_piece<G, NP>(gl, q) * V, raw[q], raw[q + 1]);
                 }
-                fit_entry<TS, G, NP, UW, COMP>(raw, y, w, nr, np, gmask, a_, ls_);
+                fit_entry<TS, G, NP, UW, COMP, L::OWN>(raw, y, w, nr, np, gmask, a_, ls_);
                 m = fmin(m, ls_);
                 if constexpr (kMixed) defer = defer || ls_ < C(1e-4) * syy;
             }
@@ -1102,9 +1134,9 @@ inline int fit_shares(int64_t n, int64_t nnz, int slot, int blocks)
     }
     return el;
 }
-inline int fit_threads(int64_t lanes)
+inline int fit_threads(int64_t lanes, int most)
 {
-    int t = kFitThreads;
+    int t = most;
     while (t > 32 && lanes < (int64_t)152 * 4 * t) t /= 2;
     return t;
 }
@@ -1112,18 +1144,20 @@ inline int fit_threads(int64_t lanes)
 template <class TS, int P, bool UW, bool PX, bool COMP>
 cudaError_t go_fit(EdgeArgs a, cudaStream_t s)
 {
-    using L = FitLayout<TS, P>;
+    using L = FitLayout<TS, P, COMP>;
     if (a.Kp != L::KP || !a.norms) return cudaErrorInvalidValue;
     if constexpr (P % 2 == 0)                      // 32-byte row reads
         if (!rows_aligned32(a.x, a.Kp, sizeof(TS))) return cudaErrorMisalignedAddress;
     constexpr int per = sizeof(TS) == 8 ? kNormThreads : kNormThreads / P;    // rows per block
-    cudaError_t e = launch_chained(k_norms<TS, P, UW, COMP>, (unsigned)(((int64_t)a.n + per - 1) / per), kNormThreads,
+    cudaError_t e = cudaSuccess;
+    if constexpr (!L::OWN)
+        e = launch_chained(k_norms<TS, P, UW, COMP>, (unsigned)(((int64_t)a.n + per - 1) / per), kNormThreads,
                                    0, s, (const TS *)a.x, a.w, a.n, a.norms);
     if (e != cudaSuccess) return e;
     // slots staged per block: the average rows' entries and a quarter more
     // (a block with longer rows works on global memory), at most 96 KB
     const int el = fit_shares<P, L::G>(a.n, a.nnz_p, L::SLOT, L::MINB);
-    const int T = fit_threads((int64_t)a.n * L::G * el);
+    const int T = fit_threads((int64_t)a.n * L::G * el, L::THREADS);
     const int rows = T / (L::G * el), yrows = el > 1 ? rows : 0;
     // Rows of a graph differ in length (17 entries on average, the longest of 32 rows
     // 26).  Sorted, us: 400k rows FP64 K = 8 / 16 845 / 1426 -> 716 / 1179, FP32 207 /
