@@ -66,6 +66,7 @@ struct amgd_ctx {
     int32_t *sell_col = nullptr, *sell_slot = nullptr;
     int32_t *sell_map = nullptr;                 // row of every place of every slice (one color in row order: none)
     bool sell_sorted = false;                    // its rows are sorted by length inside windows
+    bool sell_one_type = false;                  // worth it in this arithmetic type only
     double *sell_val64 = nullptr;
     float *sell_val32 = nullptr;
     std::vector<int64_t> color_slice;            // first slice of each color
@@ -476,8 +477,9 @@ void drop_sell(amgd_ctx *h)
 // The sliced copy of the current row order, and its values for the current
 // storage.  Synchronises the handle's stream when something has to be built,
 // so it runs before a capture, never inside one.  Where the copy would be more
-// than half as large again as the matrix (rows of very uneven length), or does
-// not fit the device, the sweeps read the row-permuted CSR.
+// than half as large again as the matrix (rows of very uneven length), where one
+// row would hold up the rest, or where it does not fit the device, the sweeps read
+// the row-permuted CSR.
 int ensure_sell(amgd_ctx *h)
 {
     if (h->n == 0) return AMGD_OK;
@@ -504,7 +506,7 @@ int ensure_sell(amgd_ctx *h)
         const int64_t nsl = h->color_slice[(size_t)nc];
         std::vector<int64_t> tab(h->color_start.begin(), h->color_start.end());
         tab.insert(tab.end(), h->color_slice.begin(), h->color_slice.end());
-        // scratch: widths (padded for 16-byte loads), their tile sums, the total
+        // scratch: widths (padded for 16-byte loads), their tile sums, the total and the longest row
         const size_t wn = ((size_t)nsl + 8) & ~(size_t)7, tn = (size_t)(nsl / kTileRows + 2) & ~(size_t)1;
         int32_t *scratch = nullptr;
         e = dalloc(&h->sell_tab, tab.size());
@@ -513,11 +515,12 @@ int ensure_sell(amgd_ctx *h)
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h->sell_tab, tab.data(), tab.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
         int32_t *width = scratch, *tile = scratch + wn;
-        unsigned long long *dtotal = (unsigned long long *)(scratch + wn + tn), total = 0;
+        unsigned long long *dmeasure = (unsigned long long *)(scratch + wn + tn), measured[2] = {0, 0};
+        unsigned long long &total = measured[0];
         const SellArgs a{h->rp_p, h->col_p, h->rp_o, h->perm, h->sell_tab, h->sell_tab + nc + 1, nc, nsl, (int32_t)h->n};
         auto measure = [&]() {
-            if (e == cudaSuccess) e = launch_sell_width(a, h->sell_map, width, dtotal, s);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&total, dtotal, sizeof total, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = launch_sell_width(a, h->sell_map, width, dmeasure, s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(measured, dmeasure, sizeof measured, cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         };
         measure();
@@ -534,7 +537,22 @@ int ensure_sell(amgd_ctx *h)
         } else if (e == cudaSuccess && nc > 1) {
             e = launch_sell_rows(a, h->sell_map, s);
         }
-        const bool fits = total <= nnz + nnz / 2 + 32768 && total < (1ull << 31) - 64;
+        // A row is walked by the lanes of one row group, and a warp walks its groups one
+        // after the other: a row longer than a warp's share of a color's entries (16 rows
+        // a group, 20 warps an SM) sets the sweep's time, where the CSR kernels' blocks
+        // pass it by.  FP64 hides half as much again under its arithmetic; where a warp has
+        // next to no other rows, the mixed paths walk the long one as fast on the copy.  A
+        // row of m in a graph of 17 a row, us per four sweeps, CSR / sliced: 200k rows
+        // (share 70) m = 85 FP32 K = 16 118 / 107, K = 32 180 / 188, FP64 K = 16 620 / 513;
+        // m = 149 119 / 125, 177 / 215, FP64 K = 8 343 / 393, BF16 113 / 140; m = 3000, one
+        // sweep, FP32 277 / 326; 20k rows (7) m = 116 FP32 63 / 50, FP64 K = 16 127 / 186;
+        // 1M rows (350) m = 319 FP32 605 / 558.
+        const bool f64 = h->storage == ST_FP64;
+        const unsigned long long longest = measured[1], share = total / (16 * 20 * 152 * (unsigned long long)nc);
+        const bool uneven = longest > 24 && 2 * longest > 5 * (nnz / (unsigned long long)h->n);
+        const bool chain32 = uneven && share > 16 && longest > share, chain64 = uneven && 2 * longest > 3 * share;
+        const bool chain = f64 ? chain64 : chain32;
+        const bool fits = total <= nnz + nnz / 2 + 32768 && total < (1ull << 31) - 64 && !chain;
         if (e == cudaSuccess && fits) {
             e = launch_row_ptr(width, (int32_t)nsl, tile, h->sell_ptr, s);
             if (e == cudaSuccess) e = dalloc(&h->sell_col, (size_t)total);
@@ -545,6 +563,7 @@ int ensure_sell(amgd_ctx *h)
         dfree(scratch);
         if (e != cudaSuccess || !fits) return without(e);
         h->sell_entries = (int64_t)total;
+        h->sell_one_type = chain32 != chain64;
         h->sell_tried = h->sell_ok = true;
     }
     if (!h->sell_ok) return AMGD_OK;
@@ -1138,7 +1157,8 @@ int amgd_set_precision(amgd_handle h, int storage)
     h->storage = storage;
     if (slot_type_changes) {
         // the value copies of the new arithmetic type (the sliced one is remade
-        // when a sweep next runs)
+        // when a sweep next runs; whether there is one may depend on the type)
+        if (!h->sell_ok || h->sell_one_type) drop_sell(h);
         drop_part(h, h->sell_val64);
         drop_part(h, h->sell_val32);
         h->sell_val64 = nullptr;

@@ -376,8 +376,9 @@ struct SellArgs {
 cudaError_t launch_sell_sort(const SellArgs &a, int32_t *rowmap, cudaStream_t s);
 // rowmap in row order (-1: padding at a color's end)
 cudaError_t launch_sell_rows(const SellArgs &a, int32_t *rowmap, cudaStream_t s);
-// entries of every slice (rowmap NULL: rows in order), width[nslices], and their sum
-cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t *width, unsigned long long *total,
+// entries of every slice (rowmap NULL: rows in order), width[nslices], their sum and the
+// longest row (measured[2])
+cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t *width, unsigned long long *measured,
                               cudaStream_t s);
 // columns (-1: padding) and the position of every caller slot
 cudaError_t launch_sell_fill(const SellArgs &a, const int32_t *rowmap, const int64_t *ptr, int32_t *sell_col,

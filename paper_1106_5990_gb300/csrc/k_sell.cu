@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kThreads) k_sell_rows(SellArgs a, int32_t *row
     if (q < a.nslices) rowmap[q * kSellRows + l] = (int32_t)row_at(a, nullptr, q, l);
 }
 
-__global__ void __launch_bounds__(kThreads) k_sell_width(SellArgs a, const int32_t *rowmap, int32_t *width, unsigned long long *total)
+__global__ void __launch_bounds__(kThreads) k_sell_width(SellArgs a, const int32_t *rowmap, int32_t *width, unsigned long long *measured)
 {
     const int64_t q = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / 32;
     const int l = threadIdx.x % 32;
@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(kThreads) k_sell_width(SellArgs a, const int32
     const int w = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
     if (l == 0) {
         width[q] = w * kSellRows;            // wraps only where the 64-bit total is refused
-        atomicAdd(total, (unsigned long long)w * kSellRows);
+        atomicAdd(measured, (unsigned long long)w * kSellRows);
+        atomicMax(measured + 1, (unsigned long long)w);
     }
 }
 
@@ -114,12 +115,12 @@ cudaError_t launch_sell_rows(const SellArgs &a, int32_t *rowmap, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t *width, unsigned long long *total,
+cudaError_t launch_sell_width(const SellArgs &a, const int32_t *rowmap, int32_t *width, unsigned long long *measured,
                               cudaStream_t s)
 {
-    const cudaError_t e = cudaMemsetAsync(total, 0, sizeof *total, s);
+    const cudaError_t e = cudaMemsetAsync(measured, 0, 2 * sizeof *measured, s);
     if (e != cudaSuccess || a.nslices == 0) return e;
-    k_sell_width<<<slice_blocks(a.nslices), kThreads, 0, s>>>(a, rowmap, width, total);
+    k_sell_width<<<slice_blocks(a.nslices), kThreads, 0, s>>>(a, rowmap, width, measured);
     return cudaGetLastError();
 }
 
