@@ -25,7 +25,8 @@
  * - mem = AMGD_MEM_HOST: the pointers are host memory; the call copies
  *   through the handle's stream and returns when the data is in place.
  *   mem = AMGD_MEM_DEVICE: the pointers are device memory of the current
- *   device; the call only enqueues work on the handle's stream.
+ *   device; the call only enqueues work on the handle's stream (the first
+ *   use of a feature may also allocate its buffers and wait).
  * - Ordering: every call is ordered on the handle's stream (default: the
  *   legacy default stream).  A handle is not thread-safe; distinct handles
  *   are independent.
@@ -240,6 +241,14 @@ int amgd_sync(amgd_handle h);
  *   AMGD_SWEEP_JACOBI: x_i <- x_i - (omega / a_ii) sum_j a_ij x_j
  *   AMGD_SWEEP_MCGS:   as set by amgd_set_coloring, SOR weight omega
  *   Sweeps accumulate on the current vectors.  nu >= 0, omega finite.
+ *   Enqueued without synchronising, but for one call of a handle whose
+ *   sweeps go on: when they so far would have saved as much as a second,
+ *   sliced copy of the matrix costs to build (from some 120 us of savings for
+ *   a small matrix on), the call builds it -- it allocates device memory and
+ *   waits for the handle's stream, which no other stream's or thread's
+ *   capture sees.  amgd_backward, whose recomputed sweeps count too, may be
+ *   that call instead; amgd_graph_capture and amgd_autotune build the copy
+ *   at once.  A call on a stream that the caller captures does none of this.
  *   Errors: ARG, STATE (MCGS without coloring), CUDA.
  */
 int amgd_relax(amgd_handle h, int32_t nu, double omega, int sweep_type);
@@ -325,9 +334,11 @@ int amgd_graph_launch(amgd_handle h);
  *   next synchronising call return AMGD_ERR_TIMEOUT); 2 warp-pipelined, CSR
  *   slices and neighbour rows copied with cp.async two and one row groups
  *   ahead (U must be 4); 3 one block per SM on a contiguous chunk of CSR rows.
- *   Repeated sweeps of kernel 0 (but for sweeps that the caller's own stream
- *   capture records: those stay on the CSR, which value updates then keep
- *   current for the graph) read a sliced copy of the matrix and choose
+ *   Once built (see amgd_relax), a sliced copy of the matrix serves the sweeps
+ *   of kernel 0 (but for sweeps that the caller's own stream capture records,
+ *   those of amgd_backward among them: they stay on the CSR, which value
+ *   updates then keep current for the graph; and for every sweep after a value
+ *   update that the caller recorded).  The sweeps on it choose
  *   their lanes, batch and blocks by the row's size and the matrix, unless
  *   amgd_autotune found the handle's sweeps faster on the CSR in a shape of
  *   kernel 0, which they then run in.

@@ -57,11 +57,12 @@ struct amgd_ctx {
     int32_t *defer_list = nullptr;
     std::vector<int64_t> color_start;           // permuted row start of each color
     // sliced copy of the permuted matrix (built by ensure_sell for the sweeps)
-    int64_t sweep_calls = 0;                     // sweep calls prepared so far
+    double sweep_gain = 0.0;                     // us that the sweeps so far would have saved on the sliced copy
     bool relax_csr[3] = {false, false, false};   // per storage: the tuner found kernel 0 faster on the CSR
     bool sell_tried = false;                     // for the current coloring
     bool sell_ok = false;                        // the copy exists (else its padding was too much)
     int64_t sell_entries = 0;
+    void *sell_rows = nullptr, *sell_cells = nullptr;    // allocations of the arrays per slice and per entry
     int64_t *sell_ptr = nullptr, *sell_tab = nullptr;   // tab: first rows, then first slices of the colors
     int32_t *sell_col = nullptr, *sell_slot = nullptr;
     int32_t *sell_map = nullptr;                 // row of every place of every slice (one color in row order: none)
@@ -77,7 +78,6 @@ struct amgd_ctx {
     bool recording = false;                      // the current call is recorded by the caller's own capture
     bool recorded_csr = false;                   // a caller's graph may read the row-permuted CSR values
     bool recorded_values = false;                // a caller's graph may replace the values at any time
-    void *weight = nullptr;                      // omega / a_ii of a relaxation (8 bytes per row)
     // vectors
     void *x[2] = {nullptr, nullptr};
     int cur = 0;
@@ -149,7 +149,7 @@ struct amgd_ctx {
     bool async_pending = false;
     struct PendingOut { int64_t *rp; int mem; int64_t cap; };
     std::vector<PendingOut> pending_out;         // strength outputs checked at amgd_sync
-    void *norms = nullptr;                       // distance pass: S_xx of every vector row
+    void *norms = nullptr;                       // 16 bytes per row: S_xx of the distance pass, omega / a_ii of sweeps
     // pattern of the fits, threshold and strength graph: the graph G_d of A^d
     // (search depth d); for d = 1 these alias A's caller-order pattern
     int32_t depth = 1;
@@ -454,6 +454,15 @@ struct Recording {
     Recording(const Recording &) = delete;
 };
 
+// Allocations and waits on a stream of the handle's that no capture reaches: allowed
+// while another thread or stream captures in global mode, which they would break
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture &) = delete;
+};
+
 // array of a sliced copy that is given up; one that a graph of the caller's reads
 // stays until the handle goes
 void drop_part(amgd_ctx *h, void *p)
@@ -464,8 +473,9 @@ void drop_part(amgd_ctx *h, void *p)
 
 void drop_sell(amgd_ctx *h)
 {
-    void *ptrs[] = {h->sell_ptr, h->sell_tab, h->sell_col, h->sell_slot, h->sell_map, h->sell_val64, h->sell_val32};
+    void *ptrs[] = {h->sell_rows, h->sell_cells, h->sell_val64, h->sell_val32};
     for (void *p : ptrs) drop_part(h, p);
+    h->sell_rows = h->sell_cells = nullptr;
     h->sell_held = false;
     h->sell_ptr = h->sell_tab = nullptr;
     h->sell_col = h->sell_slot = h->sell_map = nullptr;
@@ -482,7 +492,8 @@ void drop_sell(amgd_ctx *h)
 // the row-permuted CSR.
 int ensure_sell(amgd_ctx *h)
 {
-    if (h->n == 0) return AMGD_OK;
+    if (h->n == 0 || (h->sell_tried && !h->sell_ok)) return AMGD_OK;
+    const RelaxedCapture relaxed;
     cudaStream_t s = h->stream;
     cudaError_t e = cudaSuccess;
     // gives the copy up; an allocation that fails leaves the CSR in use
@@ -506,17 +517,23 @@ int ensure_sell(amgd_ctx *h)
         const int64_t nsl = h->color_slice[(size_t)nc];
         std::vector<int64_t> tab(h->color_start.begin(), h->color_start.end());
         tab.insert(tab.end(), h->color_slice.begin(), h->color_slice.end());
-        // scratch: widths (padded for 16-byte loads), their tile sums, the total and the longest row
+        // one allocation: the total and the longest row, the colors, the slices' first
+        // entries and their rows, then scratch: widths (padded for 16-byte loads) and
+        // their tile sums
         const size_t wn = ((size_t)nsl + 8) & ~(size_t)7, tn = (size_t)(nsl / kTileRows + 2) & ~(size_t)1;
-        int32_t *scratch = nullptr;
-        e = dalloc(&h->sell_tab, tab.size());
-        if (e == cudaSuccess) e = dalloc(&h->sell_ptr, (size_t)nsl + 1);
-        if (e == cudaSuccess) e = dalloc(&scratch, wn + tn + 4);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h->sell_tab, tab.data(), tab.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
-        int32_t *width = scratch, *tile = scratch + wn;
-        unsigned long long *dmeasure = (unsigned long long *)(scratch + wn + tn), measured[2] = {0, 0};
-        unsigned long long &total = measured[0];
+        const size_t tabn = (tab.size() + 1) & ~(size_t)1, ptrn = ((size_t)nsl + 2) & ~(size_t)1;
+        const size_t mapn = (size_t)nsl * kSellRows;
+        unsigned long long measured[2] = {0, 0}, &total = measured[0];
+        e = cudaMalloc(&h->sell_rows, (2 + tabn + ptrn) * sizeof(int64_t) + (mapn + wn + tn) * sizeof(int32_t));
+        if (e != cudaSuccess) {
+            h->sell_rows = nullptr;
+            return without(e);
+        }
+        unsigned long long *dmeasure = (unsigned long long *)h->sell_rows;
+        h->sell_tab = (int64_t *)dmeasure + 2;
+        h->sell_ptr = h->sell_tab + tabn;
+        int32_t *map = (int32_t *)(h->sell_ptr + ptrn), *width = map + mapn, *tile = width + wn;
+        e = cudaMemcpyAsync(h->sell_tab, tab.data(), tab.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
         const SellArgs a{h->rp_p, h->col_p, h->rp_o, h->perm, h->sell_tab, h->sell_tab + nc + 1, nc, nsl, (int32_t)h->n};
         auto measure = [&]() {
             if (e == cudaSuccess) e = launch_sell_width(a, h->sell_map, width, dmeasure, s);
@@ -530,7 +547,7 @@ int ensure_sell(amgd_ctx *h)
         // sweep over all rows at once has to know where
         const unsigned long long nnz = (unsigned long long)h->nnz;
         h->sell_sorted = e == cudaSuccess && total > nnz + nnz / 8 + 8192;
-        if (e == cudaSuccess && (h->sell_sorted || nc > 1)) e = dalloc(&h->sell_map, (size_t)nsl * kSellRows);
+        if (h->sell_sorted || nc > 1) h->sell_map = map;
         if (e == cudaSuccess && h->sell_sorted) {
             e = launch_sell_sort(a, h->sell_map, s);
             measure();
@@ -555,12 +572,13 @@ int ensure_sell(amgd_ctx *h)
         const bool fits = total <= nnz + nnz / 2 + 32768 && total < (1ull << 31) - 64 && !chain;
         if (e == cudaSuccess && fits) {
             e = launch_row_ptr(width, (int32_t)nsl, tile, h->sell_ptr, s);
-            if (e == cudaSuccess) e = dalloc(&h->sell_col, (size_t)total);
-            if (e == cudaSuccess) e = dalloc(&h->sell_slot, (size_t)h->nnz);
+            if (e == cudaSuccess) e = cudaMalloc(&h->sell_cells, ((size_t)total + (size_t)h->nnz) * sizeof(int32_t));
+            if (e != cudaSuccess) h->sell_cells = nullptr;
+            h->sell_col = (int32_t *)h->sell_cells;
+            h->sell_slot = h->sell_col + total;
             if (e == cudaSuccess) e = launch_sell_fill(a, h->sell_map, h->sell_ptr, h->sell_col, h->sell_slot, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         }
-        dfree(scratch);
         if (e != cudaSuccess || !fits) return without(e);
         h->sell_entries = (int64_t)total;
         h->sell_one_type = chain32 != chain64;
@@ -578,28 +596,24 @@ int ensure_sell(amgd_ctx *h)
                                       mixed ? nullptr : h->sell_val64, mixed ? h->sell_val32 : nullptr, s);
         if (e != cudaSuccess) return without(e);
     }
-    if (!h->weight) {
-        e = cudaMalloc(&h->weight, (size_t)h->n * sizeof(double));
-        if (e != cudaSuccess) {
-            h->weight = nullptr;
-            return without(e);
-        }
-    }
     return AMGD_OK;
 }
 
-// What a sweep launch needs before it is queued or captured: the sliced copy,
-// or current CSR values for the kernels that read those.  `bytes`: vector bytes
-// the caller's sweeps gather.  Building the copy costs some 200 us and a pass
-// over the matrix, a sweep saves about a quarter of its time: it is built once a
-// handle's sweeps have gathered 2 GB, or when they are called a second time
-// (128 x 128 7-point, K = 8, FP64, one call of 4 sweeps: 30 us of sweeps).
-int prepare_sweeps(amgd_ctx *h, size_t bytes, cudaStream_t s)
+// What nu sweeps need before they are queued or captured: the sliced copy, or
+// current CSR values for the kernels that read those.  A sweep on the copy saves
+// some 1.2 us, and 60 us per GB of vectors that it gathers; building it costs about
+// 120 us and 35 us per million entries, allocates and waits for the stream.  It is
+// built when the handle's sweeps so far would have saved that much (nu = kMany: a
+// captured or tuned handle, whose sweeps repeat): a handle that is dropped before
+// has lost nothing, any other at most as much again.
+constexpr int32_t kMany = INT32_MAX;
+constexpr double kBuildUs = 120.0, kBuildUsPerEntry = 35e-6;
+int prepare_sweeps(amgd_ctx *h, int32_t nu, cudaStream_t s)
 {
-    constexpr size_t kWorth = (size_t)2 << 30;
     const int stage = h->relax_shape[h->storage].stage;
-    const bool repeated = h->sweep_calls > 0 || bytes >= kWorth;
-    ++h->sweep_calls;
+    const double gathered = (double)h->nnz * Kp_of(h->storage, h->K) * (double)esize(h->storage);
+    h->sweep_gain += (double)nu * (1.2 + 6e-8 * gathered);
+    const bool repeated = h->sweep_gain >= kBuildUs + kBuildUsPerEntry * (double)h->nnz;
     // into the caller's own graph: nothing is allocated or waited for, and value
     // updates keep the CSR current for its replays from now on
     if (h->recording) h->recorded_csr = true;
@@ -610,14 +624,6 @@ int prepare_sweeps(amgd_ctx *h, size_t bytes, cudaStream_t s)
     if (!sweeps_use_csr(h)) return AMGD_OK;
     return h->storage == ST_FP64 ? refresh_perm64(h, s) : refresh_perm32(h, s);
 }
-// of a captured graph or a tuned handle, whose sweeps repeat
-int prepare_sweeps(amgd_ctx *h, cudaStream_t s) { return prepare_sweeps(h, ~(size_t)0, s); }
-// vector bytes that nu sweeps gather
-size_t sweep_bytes(const amgd_ctx *h, int32_t nu)
-{
-    return (size_t)h->nnz * Kp_of(h->storage, h->K) * esize(h->storage) * (size_t)nu;
-}
-
 // the arguments shared by every sweep of the handle
 RelaxArgs sweep_args(amgd_ctx *h, double omega)
 {
@@ -639,7 +645,7 @@ RelaxArgs sweep_args(amgd_ctx *h, double omega)
         a.sell_entries = h->sell_entries;
         a.sell_val = f64 ? (const void *)h->sell_val64 : (const void *)h->sell_val32;
         a.rowmap = h->sell_sorted ? h->sell_map : nullptr;
-        a.weight = h->weight;
+        a.weight = h->norms;
         a.sell_width = (int32_t)((h->sell_entries + 32 * h->color_slice.back() - 1) / (32 * h->color_slice.back()));
     }
     return a;
@@ -668,7 +674,7 @@ int run_relax(amgd_ctx *h, int32_t nu, double omega, int sweep, cudaStream_t s)
     const Shape sh = h->relax_shape[h->storage];
     RelaxArgs a = sweep_args(h, omega);
     const bool sliced = !sweeps_use_csr(h);
-    if (sliced && nu > 0) CK(h, launch_weights(h->storage, a.diag, omega, h->weight, (int32_t)h->n, s));
+    if (sliced && nu > 0) CK(h, launch_weights(h->storage, a.diag, omega, h->norms, (int32_t)h->n, s));
     for (int32_t it = 0; it < nu; ++it) {
         a.xold = h->x[h->cur];
         a.xnew = h->x[1 - h->cur];
@@ -744,7 +750,7 @@ int run_relax_recorded(amgd_ctx *h, int32_t nu, double omega, cudaStream_t s)
     };
     if (nck > 0) CK(h, cudaMemcpyAsync(h->ckpt, h->x[c0], xb, cudaMemcpyDeviceToDevice, s));
     if (nu > 0 && !sweeps_use_csr(h))
-        CK(h, launch_weights(h->storage, sweep_args(h, omega).diag, omega, h->weight, (int32_t)h->n, s));
+        CK(h, launch_weights(h->storage, sweep_args(h, omega).diag, omega, h->norms, (int32_t)h->n, s));
     for (int32_t k = 0; k < nu; ++k) {
         const int rc = jacobi_step(h, loc(k), loc(k + 1), omega, s);
         if (rc != AMGD_OK) return rc;
@@ -1539,7 +1545,7 @@ int amgd_relax(amgd_handle h, int32_t nu, double omega, int sweep_type)
     if (sweep_type == AMGD_SWEEP_MCGS && !h->perm)
         return fail(h, AMGD_ERR_STATE, "MCGS needs amgd_set_coloring first");
     const Recording recording(h);
-    const int rc = nu > 0 ? prepare_sweeps(h, sweep_bytes(h, nu), h->stream) : AMGD_OK;
+    const int rc = nu > 0 ? prepare_sweeps(h, nu, h->stream) : AMGD_OK;
     if (rc != AMGD_OK) return rc;
     if (h->ckpt_every > 0 && sweep_type == AMGD_SWEEP_JACOBI && !h->perm)
         return run_relax_recorded(h, nu, omega, h->stream);
@@ -1627,7 +1633,7 @@ int amgd_graph_capture(amgd_handle h, uint64_t seed, int32_t nu, double omega, i
     if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
     if (h->graph) { cudaGraphDestroy(h->graph); h->graph = nullptr; }
     {
-        const int rc = prepare_sweeps(h, h->stream);
+        const int rc = prepare_sweeps(h, kMany, h->stream);
         if (rc != AMGD_OK) return rc;
     }
     h->graph_csr = sweeps_use_csr(h);
@@ -1817,7 +1823,7 @@ int amgd_autotune(amgd_handle h, int sweep_type, double omega, const char *cache
         h->relax_shape[h->storage] = c;
         on_csr = &c != &cands[0];
         {
-            const int prc = prepare_sweeps(h, h->stream);
+            const int prc = prepare_sweeps(h, kMany, h->stream);
             if (prc != AMGD_OK) return restore(prc);
         }
         if (!on_csr && sweeps_use_csr(h)) continue;            // no sliced copy of this matrix
@@ -2304,8 +2310,8 @@ int ensure_transpose(amgd_ctx *h)
 
 namespace {
 
-// device buffers of the reverse pass (allocated before any capture)
-int prepare_backward(amgd_ctx *h)
+// device buffers of the reverse pass of nu sweeps (allocated before any capture)
+int prepare_backward(amgd_ctx *h, int32_t nu)
 {
     const size_t cs = 8;                 // the reverse pass computes in FP64
     const size_t nk = (size_t)h->n * Kp_of(h->storage, h->K);
@@ -2313,7 +2319,9 @@ int prepare_backward(amgd_ctx *h)
     const int32_t S = h->ckpt_every > 0 ? h->ckpt_every : 1;
     int rc = ensure_transpose(h);
     if (rc != AMGD_OK) return rc;
-    if ((rc = prepare_sweeps(h, h->stream)) != AMGD_OK) return rc;
+    // the sweeps between checkpoints run once more
+    const int32_t again = nu - (int32_t)(((int64_t)nu + S - 1) / S);
+    if (again > 0 && (rc = prepare_sweeps(h, again, h->stream)) != AMGD_OK) return rc;
     CK(h, ensure_buf(&h->adj_vec, h->adj_vec_bytes, 4 * nk * cs));
     CK(h, ensure_buf(&h->adj_slot, h->adj_slot_bytes, (6 * (size_t)(h->nnz ? h->nnz : 1) + (size_t)h->n) * cs));
     CK(h, ensure_buf(&h->seg, h->seg_bytes, (size_t)(S - 1) * xb));
@@ -2401,7 +2409,7 @@ int run_backward(amgd_ctx *h, const double *lsb_in, double *vb, cudaStream_t s)
     // sweeps, last to first, one checkpoint segment at a time: the iterates
     // between two checkpoints are recomputed by the forward kernel
     if (nu > 0 && !sweeps_use_csr(h))
-        CK(h, launch_weights(st, sweep_args(h, h->traj_omega).diag, h->traj_omega, h->weight, n, s));
+        CK(h, launch_weights(st, sweep_args(h, h->traj_omega).diag, h->traj_omega, h->norms, n, s));
     int xc = 0;
     const int32_t nseg = (nu + S - 1) / S;
     for (int32_t c = nseg - 1; c >= 0; --c) {
@@ -2458,7 +2466,7 @@ int amgd_backward(amgd_handle h, const double *ls_bar, int mem, double *val_bar,
     int rc = backward_checks(h);
     if (rc != AMGD_OK) return rc;
     const Recording recording(h);        // the recomputed sweeps, as in amgd_relax
-    if ((rc = prepare_backward(h)) != AMGD_OK) return rc;
+    if ((rc = prepare_backward(h, h->traj_nu)) != AMGD_OK) return rc;
     cudaStream_t s = h->stream;
     const int64_t nnz = h->nnz;
     const double *lsb_in = ls_bar;
@@ -2510,14 +2518,14 @@ int amgd_graph_capture_backward(amgd_handle h, uint64_t seed, int32_t nu, double
         const size_t xb = (size_t)h->n * Kp_of(h->storage, h->K) * esize(h->storage);
         const int32_t nck = (nu + h->ckpt_every - 1) / h->ckpt_every;
         CK(h, ensure_buf(&h->ckpt, h->ckpt_bytes, (size_t)nck * xb));
-        const int rc = prepare_backward(h);
+        const int rc = prepare_backward(h, nu);
         if (rc != AMGD_OK) return rc;
     }
     if (!h->cap_stream) CK(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
     if (h->graph) { cudaGraphDestroy(h->graph); h->graph = nullptr; }
     {
-        const int rc = prepare_sweeps(h, h->stream);
+        const int rc = prepare_sweeps(h, kMany, h->stream);
         if (rc != AMGD_OK) return rc;
     }
     h->graph_csr = sweeps_use_csr(h);
@@ -2594,7 +2602,6 @@ int amgd_destroy(amgd_handle h)
     dfree(h->long_rows_p);
     drop_sell(h);
     for (void *p : h->held) dfree(p);
-    dfree(h->weight);
     dfree(h->mat_id);
     if (h->depth > 1) {
         dfree(h->prp);

@@ -61,16 +61,25 @@ __global__ void __launch_bounds__(kThreads) k_sell_rows(SellArgs a, int32_t *row
 
 __global__ void __launch_bounds__(kThreads) k_sell_width(SellArgs a, const int32_t *rowmap, int32_t *width, unsigned long long *measured)
 {
+    __shared__ int ws[kThreads / 32];
     const int64_t q = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / 32;
     const int l = threadIdx.x % 32;
-    if (q >= a.nslices) return;
-    const int64_t r = row_at(a, rowmap, q, l);
+    const int64_t r = q < a.nslices ? row_at(a, rowmap, q, l) : -1;
     const int len = r >= 0 ? a.rp[r + 1] - a.rp[r] : 0;
     const int w = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
     if (l == 0) {
-        width[q] = w * kSellRows;            // wraps only where the 64-bit total is refused
-        atomicAdd(measured, (unsigned long long)w * kSellRows);
-        atomicMax(measured + 1, (unsigned long long)w);
+        if (q < a.nslices) width[q] = w * kSellRows;   // wraps only where the 64-bit total is refused
+        ws[threadIdx.x / 32] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long sum = 0, longest = 0;
+        for (int k = 0; k < kThreads / 32; ++k) {
+            sum += (unsigned long long)ws[k] * kSellRows;
+            longest = max(longest, (unsigned long long)ws[k]);
+        }
+        atomicAdd(measured, sum);
+        atomicMax(measured + 1, longest);
     }
 }
 

@@ -80,6 +80,7 @@ def test_planted_column_is_caught(checked_lib):
 # 16 rows of 64 bytes per group, three groups per warp, the last group in the upper
 # half of the last slice; and the other row widths at the same row counts
 AHEAD = r'''
+import torch
 from paper_1106_5990_gb300 import amgd, inputs
 assert amgd.amgd_checked_build() == 1
 for n in (111872, 111872 - 16, 111872 - 37):
@@ -88,7 +89,8 @@ for n in (111872, 111872 - 16, 111872 - 37):
         for prec in ("fp64", "fp32"):
             with amgd.Handle(rp, col, val, K, 1) as h:
                 h.set_precision(prec)
-                h.relax(1, 0.7)
+                h.graph_capture(1, 1, 0.7, 0, 0.5, torch.empty(n + 1, dtype=torch.int64, device="cuda"),
+                                torch.empty(len(col), dtype=torch.int32, device="cuda"))
                 h.relax(1, 0.7)                  # reads the sliced copy
                 h.get_vectors()                  # synchronises: reads the status
 print("in range")

@@ -44,6 +44,111 @@ SWEEPS = {
 }
 
 
+def on_sliced_copy(h, sweep=amgd.AMGD_SWEEP_JACOBI):
+    """A captured build makes the sliced copy (if the matrix has one): the handle's sweeps
+    read it from there on.  The vectors stay."""
+    s_rp = torch.empty(h.n + 1, dtype=torch.int64, device="cuda")
+    s_col = torch.empty(max(h.E_p, 1), dtype=torch.int32, device="cuda")
+    h.graph_capture(1, 1, 1.0, sweep, 0.5, s_rp, s_col)
+
+
+@pytest.mark.parametrize("name", [*SWEEPS, "hub_3001"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
+@pytest.mark.parametrize("K", [1, 5, 8, 32, 64])
+@pytest.mark.parametrize("sweep", ["jacobi", "mcgs"])
+def test_sweeps_on_the_sliced_copy(name, prec, K, sweep):
+    """Against the CSR (one short call of a fresh handle) and, in FP64, the oracle; then
+    with new values."""
+    rp, col, val = hub(3001, (300,), 2) if name == "hub_3001" else SWEEPS[name]()
+    n = len(rp) - 1
+    color = inputs.greedy_coloring(rp, col) if sweep == "mcgs" else None
+    mode, omode = (amgd.AMGD_SWEEP_MCGS, oracle.SWEEP_MCGS) if color is not None else (amgd.AMGD_SWEEP_JACOBI, 0)
+    val2 = val * np.random.default_rng(8).uniform(1, 1.01, len(val))
+
+    def handle(v):
+        h = amgd.Handle(rp, col, v, K, 7)
+        h.set_precision(prec)
+        if color is not None:
+            h.set_coloring(color)
+        h.init_vectors(7)
+        return h
+
+    for v, update in ((val, False), (val2, True)):
+        with handle(v) as h:
+            h.relax(3, 0.9, mode)
+            want = h.get_vectors()
+        with handle(val) as h:
+            on_sliced_copy(h, mode)
+            if update:
+                h.set_values(v)
+            h.relax(1, 0.9, mode)
+            h.relax(2, 0.9, mode)
+            assert np.array_equal(h.get_vectors(), want)
+        if prec == "fp64":
+            assert np.array_equal(want, oracle.relax(rp, col, v, oracle.tv_init(n, K, 7), 3, 0.9, omode, color))
+
+
+def test_a_copy_for_one_arithmetic_type():
+    """A row of 300 entries in a small graph: the mixed sweeps read the copy, FP64 the CSR."""
+    rp, col, val = hub(3001, (300,), 2)
+    with amgd.Handle(rp, col, val, 8, 7) as h, amgd.Handle(rp, col, val, 8, 7) as fresh:
+        for prec in ("fp64", "fp32", "bf16", "fp64", "fp32"):
+            for k in (h, fresh):
+                k.set_precision(prec)
+                k.init_vectors(7)
+            on_sliced_copy(h)
+            h.set_values(val)
+            h.relax(3, 0.9)
+            fresh.relax(3, 0.9)
+            assert np.array_equal(h.get_vectors(), fresh.get_vectors()), prec
+
+
+def test_the_copy_is_built_when_it_has_paid():
+    """A handle that is swept a few times allocates nothing for it; one whose sweeps go on
+    gets the copy (11 MB of entries)."""
+    rp, col, val = inputs.poisson2d_5pt(512)
+    with amgd.Handle(rp, col, val, 8, 7) as h:
+        h.relax(2, 0.7)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        h.relax(2, 0.7)
+        h.relax(2, 0.7)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+        for _ in range(100):
+            h.relax(4, 0.7)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] <= free - (8 << 20)
+        X = oracle.relax(rp, col, val, oracle.tv_init(len(rp) - 1, 8, 7), 406, 0.7)
+        assert np.array_equal(h.get_vectors(), X)
+
+
+def test_the_copy_is_built_beside_a_capture():
+    """Another stream is captured in global mode while the handle's sweeps build the copy."""
+    rp, col, val = SWEEPS["aniso9_66"]()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    x = torch.zeros(8, device="cuda")
+    with amgd.Handle(rp, col, val, 8, 7) as h:   # every kernel is loaded
+        h.relax(400, 0.7)
+        h.relax(400, 0.7)
+        want = h.get_vectors()
+    with amgd.Handle(rp, col, val, 8, 7) as h:
+        h.set_stream(s2)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s1, capture_error_mode="global"):
+            x.add_(1)
+            h.relax(400, 0.7)
+            h.relax(400, 0.7)
+            x.add_(1)
+        s2.synchronize()
+        assert np.array_equal(h.get_vectors(), want)
+        g.replay()
+        torch.cuda.synchronize()
+        assert (x == 2).all()
+        h.set_stream(None)
+
+
 @pytest.mark.parametrize("name", list(SWEEPS))
 @pytest.mark.parametrize("K", [1, 5, 8, 32, 64])
 @pytest.mark.parametrize("sweep", ["jacobi", "mcgs"])
@@ -147,13 +252,17 @@ def test_value_updates_in_a_graph_of_the_callers(built, sweep):
 
         h.set_values_async(buf)
         h.sync()
-        for _ in range(3 if built else 1):
+        X = eager(val)
+        if built:
+            on_sliced_copy(h, mode)
             X = eager(val)
         torch.cuda.synchronize()
         g = torch.cuda.CUDAGraph()
         with torch.cuda.graph(g, stream=s):
             h.set_values_async(buf)
         h.sync()
+        if not built:
+            on_sliced_copy(h, mode)
         for _ in range(2):
             X = eager(val)
             assert np.array_equal(h.get_vectors(), X)    # recorded, not run
@@ -204,8 +313,8 @@ def test_reverse_pass_in_a_graph_of_the_callers(warmed, prec, tmp_path):
             step(h)
             h.set_kernel_shape(amgd.AMGD_KERNEL_RELAX, G, NV, U, 0)
         else:
-            for _ in range(3):
-                step(h)
+            on_sliced_copy(h)
+            step(h)
         s.synchronize()
         g = torch.cuda.CUDAGraph(keep_graph=True)
         with torch.cuda.graph(g, stream=s):
@@ -250,8 +359,9 @@ def test_jacobi_sweeps_of_a_colored_handle(name, prec, K):
             if colored:
                 h.set_coloring(color)
             h.init_vectors(7)
-            parts = (1, 1, 1) if colored else (3,)
-            for nu in parts:                     # from the second call on: the sliced copy
+            if colored:
+                on_sliced_copy(h)
+            for nu in (1, 1, 1) if colored else (3,):
                 h.relax(nu, 0.8)
                 if colored:
                     h.set_values(val)
