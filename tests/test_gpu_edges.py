@@ -123,6 +123,29 @@ def test_the_copy_is_built_when_it_has_paid():
         assert np.array_equal(h.get_vectors(), X)
 
 
+def test_a_saved_line_for_the_csr_gives_the_copy_back(tmp_path):
+    """A handle that has the copy and loads a line that says CSR: value updates need not
+    keep the copy current any more."""
+    import re
+    rp, col, val = inputs.poisson2d_5pt(512)
+    cache = tmp_path / "tune.txt"
+    with amgd.Handle(rp, col, val, 8, 7) as h:
+        h.autotune(amgd.AMGD_SWEEP_JACOBI, 0.7, str(cache))
+    cache.write_text(re.sub(r";relax=(\d+),(\d+),(\d+),\d+(.*);sliced=[01]", r";relax=\1,\2,\3,0\4;sliced=0", cache.read_text()))
+    with amgd.Handle(rp, col, val, 8, 7) as h:
+        h.relax(400, 0.7)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        h.autotune(amgd.AMGD_SWEEP_JACOBI, 0.7, str(cache))
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] >= free + (8 << 20)
+        h.set_values(2 * val)
+        h.relax(3, 0.7)
+        X = oracle.relax(rp, col, val, oracle.tv_init(len(rp) - 1, 8, 7), 403, 0.7)
+        assert np.array_equal(h.get_vectors(), X)
+    assert len(cache.read_text().splitlines()) == 1
+
+
 def test_the_copy_is_built_beside_a_capture():
     """Another stream is captured in global mode while the handle's sweeps build the copy."""
     rp, col, val = SWEEPS["aniso9_66"]()
