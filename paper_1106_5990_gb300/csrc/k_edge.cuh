@@ -152,6 +152,24 @@ struct CompJoin {
 // ---------------------------------------------------------------------------
 constexpr int kNormThreads = 256;
 
+// Chains of an FP64 sum (even and odd components of every M-th piece) joined.  Chains of
+// a few terms, for the rounding errors: with two over a lane's 16 components and two over
+// a whole row here, a was off by 1.13 (K = 16) to 1.40 (K = 64) units of its last place
+// (rms, against 80-bit sums of uniform vectors), by 1.03 as it is, as with a tree over
+// all pieces.
+template <int M>
+__device__ __forceinline__ double join_chains(const double (&c0)[M], const double (&c1)[M])
+{
+    double s[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) s[m] = c0[m] + c1[m];
+#pragma unroll
+    for (int h = M / 2; h > 0; h /= 2)
+#pragma unroll
+        for (int m = 0; m < h; ++m) s[m] += s[m + h];
+    return s[0];
+}
+
 template <class TS, int P, bool UW, bool COMP>
 __global__ void __launch_bounds__(kNormThreads) k_norms(const TS *X, const void *wv, int32_t n,
                                                         void *out)
@@ -164,16 +182,20 @@ __global__ void __launch_bounds__(kNormThreads) k_norms(const TS *X, const void 
         chain_wait();
         chain_release();
         if (r >= n) return;
-        double s = 0.0, s1 = 0.0;
+        constexpr int M = P < 4 ? 1 : P <= 8 ? 2 : P / 4;          // piece q belongs to chain q mod M
+        double c0[M] = {}, c1[M] = {};
 #pragma unroll 4
-        for (int q = 0; q < P; ++q) {
-            double x[V];
-            S::unpack(ld16(X + (r * P + q) * V), x);
-            const double2 w = UW ? make_double2(1.0, 1.0) : ld_plain((const double2 *)wv + q);
-            s = fma(UW ? x[0] : w.x * x[0], x[0], s);
-            s1 = fma(UW ? x[1] : w.y * x[1], x[1], s1);
-        }
-        s += s1;
+        for (int q0 = 0; q0 < P; q0 += M)
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                const int q = q0 + m;
+                double x[V];
+                S::unpack(ld16(X + (r * P + q) * V), x);
+                const double2 w = UW ? make_double2(1.0, 1.0) : ld_plain((const double2 *)wv + q);
+                c0[m] = fma(UW ? x[0] : w.x * x[0], x[0], c0[m]);
+                c1[m] = fma(UW ? x[1] : w.y * x[1], x[1], c1[m]);
+            }
+        const double s = join_chains(c0, c1);
         ((double2 *)out)[r] = make_double2(s, s > 1e-290 && s < 1e290 ? 1.0 / s : NAN);
     } else {
         const int lane = threadIdx.x % P;
@@ -271,33 +293,35 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
     using C = typename S::C;
     constexpr int V = S::V;
     if constexpr (std::is_same<C, double>::value) {
-        // two chains (even and odd components), joined once
-        double s0 = 0.0, s1 = 0.0;
+        // chains of at most four terms, joined once
+        constexpr int M = NP > 4 ? 2 : 1;
+        double s0[M] = {}, s1[M] = {};
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             if (q >= np) break;
             C x[V];
             S::unpack(raw[q], x);
-            s0 = fma(UW ? x[0] : w(q, 0) * x[0], y[q][0], s0);
-            s1 = fma(UW ? x[1] : w(q, 1) * x[1], y[q][1], s1);
+            s0[q % M] = fma(UW ? x[0] : w(q, 0) * x[0], y[q][0], s0[q % M]);
+            s1[q % M] = fma(UW ? x[1] : w(q, 1) * x[1], y[q][1], s1[q % M]);
         }
-        const double syx = group_sum<G>(s0 + s1, mask);
+        const double syx = group_sum<G>(join_chains(s0, s1), mask);
         // a = S_yx / S_xx: the product with the reciprocal, corrected by its
-        // exact remainder; operands outside its range divide
+        // exact remainder (Markstein's division step); operands outside its
+        // range divide
         a_ = syx * nr.y;
         if ((__double2hiint(a_) & 0x7fffffff) < 0x7f000000) a_ = fma(fma(-a_, nr.x, syx), nr.y, a_);
         else a_ = nr.x == 0.0 ? 0.0 : syx / nr.x;
-        double r0 = 0.0, r1 = 0.0;
+        double r0[M] = {}, r1[M] = {};
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             if (q >= np) break;
             C x[V];
             S::unpack(raw[q], x);
             const double d0 = fma(-a_, x[0], y[q][0]), d1 = fma(-a_, x[1], y[q][1]);
-            r0 = fma(UW ? d0 : w(q, 0) * d0, d0, r0);
-            r1 = fma(UW ? d1 : w(q, 1) * d1, d1, r1);
+            r0[q % M] = fma(UW ? d0 : w(q, 0) * d0, d0, r0[q % M]);
+            r1[q % M] = fma(UW ? d1 : w(q, 1) * d1, d1, r1[q % M]);
         }
-        ls_ = group_sum<G>(r0 + r1, mask);
+        ls_ = group_sum<G>(join_chains(r0, r1), mask);
     } else if constexpr (NP == 1) {
         C x[V];
         S::unpack(raw[0], x);
@@ -436,7 +460,7 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
 // is in flight while an entry is fitted.
 //
 // Bound: the FP32 pipe on the compensated mixed paths (8 FP32 operations per
-// component for S_yx and 9 for LS), the FP64 pipe on FP64 (3K + 3 operations
+// component for S_yx and 9 for LS), the FP64 pipe on FP64 (3K + 7 operations
 // per entry at two per clock and SM).  Few lanes per row keep y_i in registers
 // for all its entries and spend little on reductions; a lane per entry (y_i
 // from shared memory, row minima by shuffles) issued twice the instructions.
