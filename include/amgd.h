@@ -162,9 +162,9 @@ int amgd_set_target(amgd_handle h, int target);
  *   row combine their pairs with TwoSum in the shuffle reduction, and the two
  *   words are added once at the end.  AMGD_SUM_PLAIN: FP32 fused
  *   multiply-add chains.  Either way an edge whose LS falls below 1e-4 of
- *   sum_k w_k y_k^2 makes its row be redone in FP64 (cancellation).  Every
- *   distance kernel (each edge stage, any search depth) honours the
- *   setting; the FP64 path ignores it.  Drops computed distances and a
+ *   sum_k w_k y_k^2 makes its row be redone in FP64 (cancellation).  The
+ *   distance pass honours the setting at every search depth; the FP64 path
+ *   ignores it.  Drops computed distances and a
  *   captured graph.
  *   Errors: ARG.
  */

@@ -442,8 +442,9 @@ class Handle:
         """Stream-ordered value update (numpy array, pinned torch tensor or
         device tensor); val must stay unchanged until sync()."""
         if _is_torch(val):
-            # read by a copy that runs after this call returns: a converted
-            # temporary would be freed first, so the tensor must already match
+            # read after this call returns (host values by a copy, device values in
+            # place): a converted temporary would be freed first, so the tensor must
+            # already match
             v = arg_out(val, np.float64, self.nnz, "val")
         else:
             v = arg_in(val, np.float64, self.nnz, "val")

@@ -421,10 +421,8 @@ int refresh_perm64(amgd_ctx *h, cudaStream_t s)
     // (an update in a graph of the caller's leaves these out of date on mixed storage)
     if (!h->perm64_stale && !(h->recorded_values && h->storage != ST_FP64)) return AMGD_OK;
     if (h->perm)
-        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, nullptr, h->val64,
-                                    nullptr, nullptr, nullptr, s));
-    CK(h, launch_diag_values(h->val_o, h->diag_slot, h->perm, (int32_t)h->n, nullptr, nullptr,
-                             h->diag64, nullptr, s));
+        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, h->val64, nullptr, s));
+    CK(h, launch_diag_values(h->val_o, h->diag_slot, h->perm, (int32_t)h->n, h->diag64, s));
     h->perm64_stale = h->recording;      // a recorded refresh has not run
     return AMGD_OK;
 }
@@ -434,8 +432,7 @@ int refresh_perm32(amgd_ctx *h, cudaStream_t s)
 {
     if (!h->perm32_stale) return AMGD_OK;
     if (h->perm)
-        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, nullptr, nullptr, nullptr, h->val32,
-                                    nullptr, nullptr, s));
+        CK(h, launch_scatter_values(h->val_o, h->nnz, h->slot_perm, nullptr, h->val32, s));
     h->perm32_stale = h->recording;
     return AMGD_OK;
 }
@@ -592,8 +589,8 @@ int ensure_sell(amgd_ctx *h)
             e = cudaMemsetAsync(mixed ? (void *)h->sell_val32 : (void *)h->sell_val64, 0,
                                 (size_t)h->sell_entries * (mixed ? 4 : 8), s);
         if (e == cudaSuccess)
-            e = launch_scatter_values(h->val_o, h->nnz, nullptr, h->sell_slot, nullptr, nullptr, nullptr, nullptr,
-                                      mixed ? nullptr : h->sell_val64, mixed ? h->sell_val32 : nullptr, s);
+            e = launch_scatter_values(h->val_o, h->nnz, h->sell_slot, mixed ? nullptr : h->sell_val64,
+                                      mixed ? h->sell_val32 : nullptr, s);
         if (e != cudaSuccess) return without(e);
     }
     return AMGD_OK;

@@ -223,6 +223,11 @@ inline int current_device_index()
 // chain_release(), so the kernels before its predecessor are complete when it
 // starts.  chain_release() lets the next kernel start as soon as every block
 // has called it.  What it saves is the launch gap of the short kernels.
+// One kernel breaks the rule, k_ls_interp_m: it releases first, reads and writes, and
+// waits at its end.  That is right only because the first of its launches is not
+// chained (what they read is complete before any of them starts), they write disjoint
+// rows, every thread waits before it ends (the last of them ends after all others) and
+// a launch that is not chained follows.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... Args>
@@ -443,19 +448,13 @@ struct ValueArgs {
     int32_t n;
 };
 cudaError_t launch_values(const ValueArgs &a, bool f64, int64_t nnz, cudaStream_t s);
-// one coalesced pass over caller-order values src[nnz] into the caller FP64 /
-// FP32 copies, the row-permuted FP64 / FP32 copies (at slot_perm, NULL =
-// identity) and the sweeps' sliced copy (at slot_sell); NULL targets skipped;
-// err (NULL: none) |= 1 for a non-finite value
-cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *slot_perm, const int32_t *slot_sell,
-                                  double *val_o, float *val32_o, double *vp64, float *vp32, double *vs64,
-                                  float *vs32, cudaStream_t s, uint32_t *err = nullptr);
-// diagonals (diag_slot = caller slot of each row's diagonal) in caller order
-// and in permuted order (NULL targets skipped); err (NULL: none) |= 2 for a
-// zero diagonal
-cudaError_t launch_diag_values(const double *v, const int32_t *diag_slot, const int32_t *perm,
-                               int32_t n, double *d64_o, float *d32_o, double *d64_p, float *d32_p,
-                               cudaStream_t s, uint32_t *err = nullptr);
+// caller-order values src[nnz] at their places `to` (NULL = identity) of one other copy,
+// FP64 or FP32 (the other NULL)
+cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *to, double *v64, float *v32,
+                                  cudaStream_t s);
+// the diagonals (diag_slot = caller slot of each row's) in permuted order
+cudaError_t launch_diag_values(const double *v, const int32_t *diag_slot, const int32_t *perm, int32_t n, double *d64_p,
+                               cudaStream_t s);
 
 // value check of a staged val[nnz]: err |= 1 for a non-finite value, |= 2 for
 // a zero diagonal (diag_slot[n] = slot of each row's diagonal)

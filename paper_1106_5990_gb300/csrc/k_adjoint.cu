@@ -274,8 +274,9 @@ __device__ __forceinline__ double fit_quotient(double yx, double xx)
 }
 
 // v / d from the reciprocal y of d (once per row): the product, then its exact
-// remainder's share (the quotient to within rounding of the last bit, in three FP64
-// operations instead of nine); operands near the ends of the range divide
+// remainder's share (Markstein's division step: the quotient to within rounding of the
+// last bit, in three FP64 operations instead of nine); operands near the ends of the
+// range divide
 __device__ __forceinline__ double quotient(double v, double d, double y)
 {
     const double q = v * y;

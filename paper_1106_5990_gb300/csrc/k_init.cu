@@ -293,61 +293,23 @@ __global__ void k_check_values(const double *__restrict__ v, int64_t nnz,
     if (e && (threadIdx.x % 32) == 0) atomicOr(err, e);
 }
 
-// one pass over the stored values in caller order (coalesced): the FP64
-// caller copy, the FP32 caller copy, the row-permuted FP64 / FP32 copies
-// (slot_perm[p] = permuted slot of caller slot p) and the sliced copy
-// (slot_sell[p] = its position); NULL targets are skipped.  err (NULL: no
-// check): bit 0 set when a value is not finite.
-__global__ void k_scatter_values(const double *__restrict__ src, int64_t nnz,
-                                 const int32_t *__restrict__ slot_perm, const int32_t *__restrict__ slot_sell,
-                                 double *__restrict__ val_o, float *__restrict__ val32_o, double *__restrict__ vp64,
-                                 float *__restrict__ vp32, double *__restrict__ vs64, float *__restrict__ vs32,
-                                 uint32_t *__restrict__ err)
+// one pass over the stored values in caller order into one other copy (slot p at to[p])
+__global__ void k_scatter_values(const double *__restrict__ src, int64_t nnz, const int32_t *__restrict__ to,
+                                 double *__restrict__ v64, float *__restrict__ v32)
 {
-    bool bad = false;
-    for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < nnz;
-         p += (int64_t)gridDim.x * kThreads) {
-        const double x = src[p];
-        bad = bad || !isfinite(x);
-        const float f = (float)x;
-        if (val_o) val_o[p] = x;
-        if (val32_o) val32_o[p] = f;
-        if (vp64 || vp32) {
-            const int64_t q = slot_perm ? slot_perm[p] : p;
-            if (vp64) vp64[q] = x;
-            if (vp32) vp32[q] = f;
-        }
-        if (vs64 || vs32) {
-            const int64_t q = slot_sell[p];
-            if (vs64) vs64[q] = x;
-            if (vs32) vs32[q] = f;
-        }
+    for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * kThreads) {
+        const int64_t q = to ? to[p] : p;
+        if (v64) v64[q] = src[p];
+        else v32[q] = (float)src[p];
     }
-    if (err && __any_sync(0xffffffffu, bad) && (threadIdx.x % 32) == 0) atomicOr(err, 1u);
 }
 
-// diagonals in caller order and in permuted order (perm[r] = caller row of r);
-// NULL targets are skipped.  err (NULL: no check): bit 1 set on a zero
-// diagonal.
+// diagonals in permuted order (perm[r] = caller row of r)
 __global__ void k_diag_values(const double *__restrict__ v, const int32_t *__restrict__ diag_slot,
-                              const int32_t *__restrict__ perm, int32_t n, double *__restrict__ d64_o,
-                              float *__restrict__ d32_o, double *__restrict__ d64_p,
-                              float *__restrict__ d32_p, uint32_t *__restrict__ err)
+                              const int32_t *__restrict__ perm, int32_t n, double *__restrict__ d64_p)
 {
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    bool zero = false;
-    if (t < n) {
-        const double d = v[diag_slot[t]];
-        zero = d == 0.0;
-        if (d64_o) d64_o[t] = d;
-        if (d32_o) d32_o[t] = (float)d;
-        if (d64_p || d32_p) {
-            const double dp = perm ? v[diag_slot[perm[t]]] : d;
-            if (d64_p) d64_p[t] = dp;
-            if (d32_p) d32_p[t] = (float)dp;
-        }
-    }
-    if (err && __any_sync(0xffffffffu, zero) && (threadIdx.x % 32) == 0) atomicOr(err, 2u);
+    if (t < n) d64_p[t] = v[diag_slot[perm ? perm[t] : t]];
 }
 
 // Every copy of the values in one pass over them (launch_values).  A block takes
@@ -588,14 +550,12 @@ cudaError_t launch_check_values(const double *v, int64_t nnz, const int32_t *dia
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *slot_perm, const int32_t *slot_sell,
-                                  double *val_o, float *val32_o, double *vp64, float *vp32, double *vs64,
-                                  float *vs32, cudaStream_t s, uint32_t *err)
+cudaError_t launch_scatter_values(const double *src, int64_t nnz, const int32_t *to, double *v64, float *v32,
+                                  cudaStream_t s)
 {
     if (nnz == 0) return cudaSuccess;
     const int64_t want = (nnz + kThreads - 1) / kThreads;
-    k_scatter_values<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), kThreads, 0, s>>>(
-        src, nnz, slot_perm, slot_sell, val_o, val32_o, vp64, vp32, vs64, vs32, err);
+    k_scatter_values<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), kThreads, 0, s>>>(src, nnz, to, v64, v32);
     return cudaGetLastError();
 }
 
@@ -626,13 +586,11 @@ cudaError_t launch_values(const ValueArgs &a, bool f64, int64_t nnz, cudaStream_
     return launch_chained(k_values<float>, blocks(a.n), kThreads, (size_t)cap * slot, s, a, (int)cap);
 }
 
-cudaError_t launch_diag_values(const double *v, const int32_t *diag_slot, const int32_t *perm,
-                               int32_t n, double *d64_o, float *d32_o, double *d64_p, float *d32_p,
-                               cudaStream_t s, uint32_t *err)
+cudaError_t launch_diag_values(const double *v, const int32_t *diag_slot, const int32_t *perm, int32_t n, double *d64_p,
+                               cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_diag_values<<<blocks(n), kThreads, 0, s>>>(v, diag_slot, perm, n, d64_o, d32_o, d64_p, d32_p,
-                                                err);
+    k_diag_values<<<blocks(n), kThreads, 0, s>>>(v, diag_slot, perm, n, d64_p);
     return cudaGetLastError();
 }
 

@@ -832,7 +832,7 @@ cudaError_t launch_m_kernels(const InterpArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const int64_t want = ((int64_t)a.n + T - 1) / T;
     const unsigned grid = (unsigned)(want < 152 * 6 ? want : 152 * 6);
-    if constexpr (M == kInterpRowCand) {
+    if constexpr (M == kInterpRowCand) {         // the first: not chained (see launch_chained)
         k_ls_interp_m<TS, M><<<grid, T, bytes(a.Kp), s>>>(a);
         e = cudaGetLastError();
     } else {

@@ -473,7 +473,7 @@ k_relax_pipe(RelaxArgs A, int64_t chunk)
 }
 
 // ---------------------------------------------------------------------------
-// Sweep over the sliced copy of A (stages 0 and 3).  A slice is 32 consecutive
+// Sweep over the sliced copy of A (stage 0).  A slice is 32 consecutive
 // rows of one color phase; entry k of the slice's row l lies at
 // ptr[slice] + 32 k + l (column -1 where the row is shorter), so the lanes of a
 // warp read column indices and values of consecutive rows as one line and
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(SellShape<TS, P>::THREADS, 1) k_relax_sell(Rel
 // kernel and the sliced copy (us per color phase of a tuned handle: 9-point 1024^2
 // K = 16 FP32 31.3 against 32.4 of the sliced copy, BF16 20.2 / 21.4; 7-point 128^3
 // K = 32 FP32 194 of the direct kernel against 199; graphs and FP64 the sliced copy;
-// untuned sweeps always take it).  896 threads (28 warps): the
+// an untuned handle takes the copy once it is built).  896 threads (28 warps): the
 // register budget of 72 per thread holds a batch of four 64-byte rows per lane
 // pair without spilling (at 1024 threads, 64 registers spilled and the sweep
 // was 10% slower; 768 threads were 4% slower, and at 640 the direct kernel
