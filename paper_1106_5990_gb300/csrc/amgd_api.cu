@@ -826,20 +826,22 @@ int alloc_slot_outputs(amgd_ctx *h, int st)
     return AMGD_OK;
 }
 
-// What the distance pass has to know of the rows' lengths.  Lists the rows of the fits' pattern (prp, nnz_p set) that a block of their own
+// What the distance pass has to know of the rows' lengths: whether neighbours differ
+// much, and the rows of the fits' pattern (prp, nnz_p set) that a block of their own
 // fits: more than kLongRow entries and four times the average.  (Rows of 100 entries
 // in a graph of 17 a row, 20000 rows, K = 16: FP32 74 us among the others, 39 with
 // blocks of their own; FP64 318 / 168.  Where all rows are that long, a block each is
-// slower: 20000 rows of 100, FP32 78 / 232.)  rows: long_row_cap entries.  The first
-// form only enqueues; the second takes what it found to the host, with the error word.
+// slower: 20000 rows of 100, FP32 78 / 232.)  rows: long_row_cap entries.  Counted on
+// the device, by launch_create on its way or by find_long_rows; take_long_rows takes
+// what was found to the host, with the error word of a check.
 constexpr int32_t kLongRow = 64;
 constexpr int kErrWords = 4;                      // the error word of a check; long rows; filled (64 bits)
 size_t long_row_cap(int64_t nnz_p) { return (size_t)(nnz_p / kLongRow + 1); }
-cudaError_t queue_long_rows(amgd_ctx *h, int32_t *rows)
+LongArgs long_row_args(amgd_ctx *h, int32_t *rows)
 {
     h->long_len = (int32_t)std::max<int64_t>(kLongRow, h->n ? 4 * (h->nnz_p / h->n) : 0);
-    return launch_long_rows(h->prp, (int32_t)h->n, h->long_len, rows, (uint32_t)long_row_cap(h->nnz_p),
-                            h->err_word + 1, (unsigned long long *)(h->err_word + 2), h->stream);
+    return LongArgs{h->long_len, rows, (uint32_t)long_row_cap(h->nnz_p), h->err_word + 1,
+                    (unsigned long long *)(h->err_word + 2)};
 }
 cudaError_t take_long_rows(amgd_ctx *h, uint32_t *err)
 {
@@ -857,7 +859,7 @@ int find_long_rows(amgd_ctx *h, int32_t *rows)
 {
     uint32_t err = 0;
     CK(h, cudaMemsetAsync(h->err_word, 0, kErrWords * sizeof(uint32_t), h->stream));
-    CK(h, queue_long_rows(h, rows));
+    CK(h, launch_long_rows(h->prp, (int32_t)h->n, long_row_args(h, rows), h->stream));
     CK(h, take_long_rows(h, &err));
     return AMGD_OK;
 }
@@ -1007,12 +1009,12 @@ int create_impl(int32_t nmat, const int64_t *const *rp_in, const int32_t *const 
         for (int32_t b = 0; b < nmat; ++b) {
             const CreateArgs ca{rp_in[b], col_in[b], val_in[b], n_in[b], slot_off[(size_t)b + 1] - slot_off[(size_t)b],
                                 row_off[(size_t)b], slot_off[(size_t)b], h->rp_o, h->col_o, h->val_o, h->diag_slot,
-                                h->diag64, h->diag64_o, h->diag32, h->diag32_o, h->err_word};
+                                h->diag64, h->diag64_o, h->diag32, h->diag32_o, h->err_word,
+                                long_row_args(h, h->long_rows)};
             TRY(launch_create(ca, h->stream));
         }
         if (n == 0) TRY(cudaMemsetAsync(h->rp_o, 0, sizeof(int32_t), h->stream));
         uint32_t err = 0;
-        TRY(queue_long_rows(h, h->long_rows));
         TRY(take_long_rows(h, &err));
         if (err) {
             // a fault, or a long row in no order: the host check decides

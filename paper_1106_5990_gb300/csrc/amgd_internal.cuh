@@ -392,8 +392,14 @@ cudaError_t launch_sell_fill(const SellArgs &a, const int32_t *rowmap, const int
 // rows with more than long_len entries (the first cap of them), in no order, and their
 // number (zero before the call); filled (zero before the call): 32 times the longest of
 // the other rows of every 32
-cudaError_t launch_long_rows(const int32_t *rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap,
-                             uint32_t *count, unsigned long long *filled, cudaStream_t s);
+struct LongArgs {
+    int32_t long_len;
+    int32_t *rows;
+    uint32_t cap;
+    uint32_t *count;
+    unsigned long long *filled;
+};
+cudaError_t launch_long_rows(const int32_t *rp, int32_t n, const LongArgs &a, cudaStream_t s);
 // in_place: read the vectors in the sweeps' row order (search depth 1)
 cudaError_t launch_edge(int storage, bool in_place, bool unit_w, const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t s);
@@ -413,6 +419,7 @@ struct CreateArgs {
     double *d64_p, *d64_o;
     float *d32_p, *d32_o;
     uint32_t *err;
+    LongArgs rows;               // the rows' lengths are noted on the way
 };
 cudaError_t launch_create(const CreateArgs &a, cudaStream_t s);
 

@@ -367,6 +367,24 @@ __global__ void __launch_bounds__(kThreads) k_values(ValueArgs A, int cap)
     }
 }
 
+// a row and its length into what the distance pass has to know of them (every thread
+// of a block; length 0: no row).  cap: rows that a check refuses are listed too.
+__device__ __forceinline__ void note_row(const LongArgs &A, int64_t r, int64_t len)
+{
+    __shared__ unsigned long long sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    if (len > A.long_len) {
+        const uint32_t at = atomicAdd(A.count, 1u);
+        if (at < A.cap) A.rows[at] = (int32_t)r;
+        len = 0;
+    }
+    const unsigned longest = __reduce_max_sync(0xffffffffu, (unsigned)max(len, (int64_t)0));
+    if (threadIdx.x % 32 == 0) atomicAdd(&sum, 32ull * longest);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(A.filled, sum);
+}
+
 // launch_create: one thread per row.  Rows in ascending order hold no duplicate;
 // others are compared entry by entry up to kPairRow entries (the same checks on
 // the host took most of the 17 ms of a one-call build of a 150k-row graph).  The
@@ -378,9 +396,11 @@ constexpr int kPairRow = 128;
 __global__ void __launch_bounds__(kThreads) k_create(CreateArgs A)
 {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int64_t a = i < A.n ? A.rp[i] : 0, b = i < A.n ? A.rp[i + 1] : 0;
+    const bool rows_ok = a >= 0 && b >= a && b <= A.nnz;
+    note_row(A.rows, A.row0 + i, rows_ok ? b - a : 0);
     if (i >= A.n) return;
-    const int64_t a = A.rp[i], b = A.rp[i + 1];
-    if (a < 0 || b < a || b > A.nnz) {
+    if (!rows_ok) {
         atomicOr(A.err, 1u);
         return;
     }
@@ -416,25 +436,10 @@ __global__ void __launch_bounds__(kThreads) k_create(CreateArgs A)
     A.d32_p[r] = A.d32_o[r] = (float)diag;
 }
 
-// (cap: row pointers that do not pass the check of launch_create are listed too)
-__global__ void __launch_bounds__(kThreads)
-k_long_rows(const int32_t *__restrict__ rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap, uint32_t *count,
-            unsigned long long *filled)
+__global__ void __launch_bounds__(kThreads) k_long_rows(const int32_t *__restrict__ rp, int32_t n, LongArgs A)
 {
-    __shared__ unsigned long long sum;
     const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    int len = r < n ? rp[r + 1] - rp[r] : 0;
-    if (threadIdx.x == 0) sum = 0;
-    __syncthreads();
-    if (len > long_len) {
-        const uint32_t at = atomicAdd(count, 1u);
-        if (at < cap) rows[at] = (int32_t)r;
-        len = 0;
-    }
-    const unsigned longest = __reduce_max_sync(0xffffffffu, (unsigned)max(len, 0));
-    if (threadIdx.x % 32 == 0) atomicAdd(&sum, 32ull * longest);
-    __syncthreads();
-    if (threadIdx.x == 0) atomicAdd(filled, sum);
+    note_row(A, r, r < n ? rp[r + 1] - rp[r] : 0);
 }
 
 inline unsigned blocks(int64_t work) { return (unsigned)((work + kThreads - 1) / kThreads); }
@@ -566,11 +571,10 @@ cudaError_t launch_create(const CreateArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_long_rows(const int32_t *rp, int32_t n, int32_t long_len, int32_t *rows, uint32_t cap,
-                             uint32_t *count, unsigned long long *filled, cudaStream_t s)
+cudaError_t launch_long_rows(const int32_t *rp, int32_t n, const LongArgs &a, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_long_rows<<<blocks(n), kThreads, 0, s>>>(rp, n, long_len, rows, cap, count, filled);
+    k_long_rows<<<blocks(n), kThreads, 0, s>>>(rp, n, a);
     return cudaGetLastError();
 }
 
