@@ -34,6 +34,7 @@ import math
 import os
 import subprocess
 import sys
+import tempfile
 import time
 
 import numpy as np
@@ -313,7 +314,12 @@ def run_gpu_arm(mats, color, w, precision, steps, warmup, rank, flush, want_cloc
         sweep = amgd.AMGD_SWEEP_MCGS
     if w.get("depth", 1) > 1:
         h.set_search_depth(w["depth"])
-    shapes = h.autotune(sweep, w["omega"], tune_cache)   # kernel shapes; untimed
+    with tempfile.TemporaryDirectory() as tmp:
+        cache = tune_cache or os.path.join(tmp, "tune.txt")
+        shapes = h.autotune(sweep, w["omega"], cache)    # kernel shapes; untimed
+        # whether the sweeps read the sliced copy (its weights are a launch of their own)
+        lines = [l for l in open(cache) if ";relax=%d,%d,%d,%d;" % tuple(shapes[0]) in l]
+        sliced = bool(lines) and ";sliced=1" in lines[-1]
     h.init_vectors(w["seed"])
     d_rp = torch.empty(h.n + 1, dtype=torch.int64, device="cuda")
     d_col = torch.empty(max(h.E_p, 1), dtype=torch.int32, device="cuda")
@@ -351,7 +357,7 @@ def run_gpu_arm(mats, color, w, precision, steps, warmup, rank, flush, want_cloc
     E_s = int(d_rp[-1].item()) if d_vb is None else None
     scal = h.backward_scalars() if d_vb is not None else None
     return dict(h=h, step_ms=step_ms, phase_ms=phase / steps, E_s=E_s, ncolors=ncolors,
-                sweep=sweep, clocks=clk, d_rp=d_rp, d_col=d_col, shapes=shapes, d_vb=d_vb,
+                sweep=sweep, clocks=clk, d_rp=d_rp, d_col=d_col, shapes=shapes, sliced=sliced, d_vb=d_vb,
                 scalars=scal)
 
 
@@ -1009,19 +1015,20 @@ def main():
         line["backward_phase_gbs"] = ab["backward"] / (r["phase_ms"][3] * 1e-3) / 1e9
         line["scalars"] = {"omega_bar": r["scalars"][0], "loss": r["scalars"][1]}
 
-    # kernels of ours per step (one more where the sweeps read the sliced copy: their
-    # weights): the row norms and the fits, with the FP64 rows of the mixed paths
+    # kernels of ours per step: the row norms and the fits, with the FP64 rows of the
+    # mixed paths; the weights of a call's sweeps where they read the sliced copy
     edge_launches = 3 if mixed else 2
+    weights = 1 if r["sliced"] else 0
     if adj:
         # symmetric pattern: inverse diagonals, refit, upstream, quotients, the fits'
-        # adjoint and its column form; recomputed sweeps (weights per segment); one
+        # adjoint and its column form; recomputed sweeps (with their weights); one
         # reverse sweep each; the finish and its reduction
         nck = -(-w["nu"] // adj)
-        bwd_launches = 6 + (w["nu"] - nck) + w["nu"] + 2
-        launches_per_step = 1 + launches_relax + edge_launches + bwd_launches
+        bwd_launches = 6 + (weights if w["nu"] > nck else 0) + (w["nu"] - nck) + w["nu"] + 2
+        launches_per_step = 1 + weights + launches_relax + edge_launches + bwd_launches
     else:
         rows_c = 1 if n <= 32768 else 2 if n <= 2048 * 1024 else 3     # compaction
-        launches_per_step = 1 + launches_relax + (1 if depth > 1 and permuted else 0) + \
+        launches_per_step = 1 + weights + launches_relax + (1 if depth > 1 and permuted else 0) + \
             edge_launches + rows_c
     line["gpu_launches"] = launches_per_step * args.steps
 

@@ -351,7 +351,7 @@ int amgd_graph_launch(amgd_handle h);
  * amgd_autotune times every valid shape of the sweeps on the handle's own
  *   matrix and vectors (one sweep of sweep_type/omega into the spare vector
  *   buffer -- the current vectors are kept) on the CSR, and the sliced copy,
- *   and keeps the fastest, and times
+ *   and keeps the fastest (the copy if it wins by 3 % or more), and times
  *   the distance pass for the record (computed distances are invalidated).  cache_path
  *   (may be NULL): a text file of earlier results keyed by GPU name,
  *   storage, K, size buckets, sweep type and color count; a matching line

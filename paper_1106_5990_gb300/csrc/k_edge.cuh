@@ -494,9 +494,11 @@ struct FitLayout {
     static constexpr int G = KP <= CL ? 1 : KP / CL;
     static constexpr int NP = P / G;
     static constexpr int U = sizeof(TS) == 8 && NP <= 4 ? 4 : 1;      // entries gathered at a time
-    // plain FP32 sums form S_xx with the fit, in blocks of 64 threads
+    // plain FP32 sums form S_xx with the fit, in blocks of 64 threads, or 32 of 32
+    // components a lane (K = 32 BF16, us with 128 / 64 / 32 threads: 9-point 1024^2 205 /
+    // 201 / 197, 7-point 128^3 392 / 380 / 370)
     static constexpr bool OWN = !COMP && sizeof(TS) < 8;
-    static constexpr int THREADS = OWN ? 64 : kFitThreads;
+    static constexpr int THREADS = !OWN ? kFitThreads : NP * V < 32 ? 64 : 32;
     // resident blocks (of kFitThreads)
     static constexpr int MINB = sizeof(TS) == 8 ? 4
                               : OWN ? (NP * V <= 4 ? 10 : NP * V <= 16 ? 8 : 5)
