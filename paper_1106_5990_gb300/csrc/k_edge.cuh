@@ -494,14 +494,17 @@ struct FitLayout {
     static constexpr int G = KP <= CL ? 1 : KP / CL;
     static constexpr int NP = P / G;
     static constexpr int U = sizeof(TS) == 8 && NP <= 4 ? 4 : 1;      // entries gathered at a time
-    // plain FP32 sums form S_xx with the fit, in blocks of 64 threads, or 32 of 32
-    // components a lane (K = 32 BF16, us with 128 / 64 / 32 threads: 9-point 1024^2 205 /
-    // 201 / 197, 7-point 128^3 392 / 380 / 370)
-    static constexpr bool OWN = !COMP && sizeof(TS) < 8;
-    static constexpr int THREADS = !OWN ? kFitThreads : NP * V < 32 ? 64 : 32;
-    // resident blocks (of kFitThreads)
+    // plain FP32 sums form S_xx with the fit, in blocks of 64 threads (not with 32
+    // components a lane: BF16 K = 32, 2M-row graph 1212 us with the norms pass, 1417
+    // without; 9-point 1024^2 192 / 199, 7-point 128^3 372 / 370)
+    static constexpr bool OWN = !COMP && sizeof(TS) < 8 && NP * V <= 16;
+    static constexpr int THREADS = OWN ? 64 : kFitThreads;
+    static constexpr bool SORTS = sizeof(TS) == 8 || (sizeof(TS) == 2 && KP >= 16);   // uneven rows by length
+    // resident blocks (of kFitThreads); as many as spill nothing, and leave the gathers
+    // some L1 beside the slots (plain sums with 8 for K = 16 FP32: 2M-row graph 967 ->
+    // 1783 us)
     static constexpr int MINB = sizeof(TS) == 8 ? 4
-                              : OWN ? (NP * V <= 4 ? 10 : NP * V <= 16 ? 8 : 5)
+                              : OWN ? (NP == 1 ? 8 : 7)
                               : sizeof(TS) == 4 ? 7 : NP * V <= 16 ? 6 : 5;
     static constexpr int WB = KP * (int)sizeof(C);                    // weights of the block
     static constexpr bool LS_OVER = sizeof(C) == 4;                    // LS replaces the gather index
@@ -568,7 +571,7 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P, COMP>::MINB) k_e
     // uneven rows in the order of their lengths, so that the rows of a warp take as
     // long (launch: A.uneven)
     int place = min(tid / width, nr - 1);
-    if (A.uneven) {
+    if (L::SORTS && A.uneven) {
         __shared__ int bin[64];
         __shared__ uint8_t order[kFitThreads];
         for (int b = tid; b < 64; b += T) bin[b] = 0;
@@ -596,10 +599,18 @@ __global__ void __launch_bounds__(kFitThreads, FitLayout<TS, P, COMP>::MINB) k_e
         __syncthreads();
         place = order[place];
     }
-    const int64_t r = R0 + place;
-    const int q0 = __ldg(A.prp + r), q1 = __ldg(A.prp + r + 1);
-    if (tid / width < nr && q1 - q0 <= A.long_len) {                 // longer rows: k_edge_long
-        const int p0 = PX ? q0 : __ldg(A.rp + r), p1 = PX ? q1 : __ldg(A.rp + r + 1);
+    if (tid / width < nr) {
+        const int64_t r = R0 + place;
+        const int q0 = __ldg(A.prp + r);
+        int q1 = __ldg(A.prp + r + 1);
+        const int p0 = PX ? q0 : __ldg(A.rp + r);
+        int p1 = PX ? q1 : __ldg(A.rp + r + 1);
+        // k_edge_long fits the longer rows.  (No branch: what follows is requested without
+        // waiting for the row pointers; 7-point 128^3, K = 4 FP32 195 -> 170 us.)
+        if (q1 - q0 > A.long_len) {
+            q1 = q0;
+            p1 = p0;
+        }
         const int64_t xr = (PX && A.xrow) ? checked_row(__ldg(A.xrow + r), A.n, A.status) : r;
         const C diag = (C)ld_plain((const AV *)A.diag + r);
         auto gather = [&](int64_t j, uint4 (&raw)[NP]) {
@@ -1186,10 +1197,11 @@ cudaError_t go_fit(EdgeArgs a, cudaStream_t s)
     const int T = fit_threads((int64_t)a.n * L::G * el, L::THREADS);
     const int rows = T / (L::G * el), yrows = el > 1 ? rows : 0;
     // Rows of a graph differ in length (17 entries on average, the longest of 32 rows
-    // 26).  Sorted, us: 400k rows FP64 K = 8 / 16 845 / 1426 -> 716 / 1179, FP32 207 /
-    // 316 -> 204 / 304, BF16 171 / 297 -> 164 / 289; with several shares a row only FP64
-    // gains (20k rows FP64 69 / 148 -> 62 / 133, FP32 41 / 45 -> 42 / 47).
-    a.uneven = a.uneven && (el == 1 || sizeof(TS) == 8);
+    // 26).  Sorted, us: 400k rows FP64 K = 8 / 16 845 / 1426 -> 716 / 1179, BF16 K = 16 /
+    // 32 171 / 297 -> 164 / 289; FP64 gains with several shares a row, too (20k rows 69 /
+    // 148 -> 62 / 133).  FP32 and short BF16 rows wait for their gathers and lose the order
+    // of them (2M rows, K = 4 FP32 909 -> 1029, BF16 911 -> 981, K = 16 FP32 no change).
+    a.uneven = a.uneven && L::SORTS && (sizeof(TS) == 8 || el == 1);
     int64_t cap = (int64_t)((double)a.nnz_p / a.n * rows * 1.25) + 32;
     const int64_t most = (96 * 1024 - L::bytes(0, UW, yrows)) / L::SLOT;
     cap = (cap < most ? cap : most) & ~(int64_t)15;
