@@ -763,6 +763,7 @@ int run_relax_recorded(amgd_ctx *h, int32_t nu, double omega, cudaStream_t s)
 
 int run_edge(amgd_ctx *h, double theta, cudaStream_t s)
 {
+    if (!h->a || !h->ls || !h->flag) return fail(h, AMGD_ERR_STATE, "the search depth has no output arrays");
     // A's own pattern (search depth 1) is fitted on the vectors in the sweeps'
     // row order, in place; G_d on a caller-order copy
     const bool in_place = h->depth == 1;
@@ -1984,20 +1985,29 @@ int amgd_set_search_depth(amgd_handle h, int32_t d)
         h->depth = d;
     }
     h->E_p = h->nnz_p - h->n;
-    dfree(h->long_rows_p);
-    h->long_rows_p = nullptr;
-    if (h->depth > 1) CK(h, dalloc(&h->long_rows_p, long_row_cap(h->nnz_p)));
-    int rc = find_long_rows(h, h->depth > 1 ? h->long_rows_p : h->long_rows);
-    if (rc != AMGD_OK) return rc;
-    if ((rc = alloc_slot_outputs(h, h->storage)) != AMGD_OK) return rc;
-    dfree(h->flag);
-    h->flag = nullptr;
-    CK(h, dalloc(&h->flag, (size_t)h->nnz_p + 16));
-    dfree(h->s_col_tmp);
-    h->s_col_tmp = nullptr;
     h->have_dist = false;
     h->traj_valid = false;
-    return AMGD_OK;
+    // nothing of the former pattern stays in use where an allocation below fails
+    // (run_edge refuses without its outputs; without the list no row is left to it)
+    h->long_len = INT32_MAX;
+    h->n_long = 0;
+    h->uneven = false;
+    dfree(h->flag);
+    h->flag = nullptr;
+    dfree(h->s_col_tmp);
+    h->s_col_tmp = nullptr;
+    dfree(h->long_rows_p);
+    h->long_rows_p = nullptr;
+    int rc = alloc_slot_outputs(h, h->storage);
+    if (rc != AMGD_OK) return rc;
+    CK(h, dalloc(&h->flag, (size_t)h->nnz_p + 16));
+    if (h->depth > 1) CK(h, dalloc(&h->long_rows_p, long_row_cap(h->nnz_p)));
+    rc = find_long_rows(h, h->depth > 1 ? h->long_rows_p : h->long_rows);
+    if (rc != AMGD_OK) {
+        h->long_len = INT32_MAX;
+        h->n_long = 0;
+    }
+    return rc;
 }
 
 int amgd_distance_pattern(amgd_handle h, int64_t *row_ptr, int32_t *col, int64_t cap,
