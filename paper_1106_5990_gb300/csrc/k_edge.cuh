@@ -499,7 +499,9 @@ struct FitLayout {
     // without; 9-point 1024^2 192 / 199, 7-point 128^3 372 / 370)
     static constexpr bool OWN = !COMP && sizeof(TS) < 8 && NP * V <= 16;
     static constexpr int THREADS = OWN ? 64 : kFitThreads;
-    static constexpr bool SORTS = sizeof(TS) == 8 || (sizeof(TS) == 2 && KP >= 16);   // uneven rows by length
+    // uneven rows may be taken by length (go_fit; FP32 of K = 16 has the form for its shared
+    // memory alone: without those 384 bytes a 2M-row graph took 1356 us instead of 1212)
+    static constexpr bool SORTS = sizeof(TS) == 8 || KP >= 16;
     // resident blocks (of kFitThreads); as many as spill nothing, and leave the gathers
     // some L1 beside the slots (plain sums with 8 for K = 16 FP32: 2M-row graph 967 ->
     // 1783 us)
@@ -1198,10 +1200,11 @@ cudaError_t go_fit(EdgeArgs a, cudaStream_t s)
     const int rows = T / (L::G * el), yrows = el > 1 ? rows : 0;
     // Rows of a graph differ in length (17 entries on average, the longest of 32 rows
     // 26).  Sorted, us: 400k rows FP64 K = 8 / 16 845 / 1426 -> 716 / 1179, BF16 K = 16 /
-    // 32 171 / 297 -> 164 / 289; FP64 gains with several shares a row, too (20k rows 69 /
-    // 148 -> 62 / 133).  FP32 and short BF16 rows wait for their gathers and lose the order
-    // of them (2M rows, K = 4 FP32 909 -> 1029, BF16 911 -> 981, K = 16 FP32 no change).
-    a.uneven = a.uneven && L::SORTS && (sizeof(TS) == 8 || el == 1);
+    // 32 171 / 297 -> 164 / 289, FP32 K = 32 316 -> 304; FP64 gains with several shares a
+    // row, too (20k rows 69 / 148 -> 62 / 133).  Shorter rows wait for their gathers and
+    // lose the order of them (2M rows, K = 4 FP32 909 -> 1029, BF16 911 -> 981; 300k rows,
+    // K = 16 FP32 166 -> 172).
+    a.uneven = a.uneven && L::SORTS && (sizeof(TS) == 8 || (el == 1 && L::KP >= (sizeof(TS) == 2 ? 16 : 32)));
     int64_t cap = (int64_t)((double)a.nnz_p / a.n * rows * 1.25) + 32;
     const int64_t most = (96 * 1024 - L::bytes(0, UW, yrows)) / L::SLOT;
     cap = (cap < most ? cap : most) & ~(int64_t)15;
