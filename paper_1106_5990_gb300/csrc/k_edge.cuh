@@ -481,9 +481,9 @@ __device__ __forceinline__ void fit_entry(const uint4 (&raw)[NP],
 // Plain sums are half the arithmetic and bound by the gathers: they form S_xx from the
 // row at hand rather than read the vectors once more for it and gather the norms, and
 // run in more and smaller blocks.  us, in the compensated sums' layout -> in this one /
-// in the former row kernel's tuned shapes: 9-point 1024^2 K = 16 FP32 169 -> 150 / 149,
-// BF16 143 -> 119 / 120, K = 32 FP32 313 -> 275 / 268; 7-point 128^3 K = 32 FP32
-// 575 -> 484 / 460, K = 16 298 -> 256 / 234; 300k-row graph K = 16 FP32 187 -> 158 / 172.
+// in the former row kernel's tuned shapes: 9-point 1024^2 K = 16 FP32 169 -> 147 / 149,
+// BF16 143 -> 117 / 120, K = 32 FP32 313 -> 287 / 268; 7-point 128^3 K = 32 FP32
+// 575 -> 484 / 460, K = 16 298 -> 249 / 234; 300k-row graph K = 16 FP32 187 -> 148 / 172.
 // Two entries at a time lose as above (152 -> 170).
 // ---------------------------------------------------------------------------
 template <class TS, int P, bool COMP>
